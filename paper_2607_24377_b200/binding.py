@@ -1,7 +1,8 @@
-"""ctypes binding of the C ABI in include/mxattn.h: same names, argument marshalling only.
+"""Binding of the C ABI in include/mxattn.h: same names, argument marshalling only.
 
 Tensors are torch CUDA tensors used purely as device-memory handles (``data_ptr()``); the stream
-is torch's current stream.  Nothing here computes.
+is torch's current stream.  Nothing here computes.  The calls of a user's inner loop go through a small CPython module
+(csrc/pycall.cpp), the rest through ctypes; both call the same library.
 """
 from __future__ import annotations
 
@@ -17,6 +18,7 @@ FLAG_UOS, FLAG_PNQ, FLAG_OUT_FP32, FLAG_HADAMARD = 1, 2, 4, 8
 LAYOUT_CANONICAL, LAYOUT_TILE = 0, 1
 
 _lib = None
+_call = None
 
 
 class MxAttnError(RuntimeError):
@@ -80,6 +82,19 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+def _calls():
+    """The CPython module of the inner-loop calls (loaded once; like the library, there is nothing to fall back to)."""
+    global _call
+    if _call is None:
+        lib()
+        from . import _mxcall
+        if not hasattr(torch._C, "_cuda_getCurrentRawStream"):
+            raise ImportError("this torch build has no CUDA support")
+        _mxcall.init(torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+        _call = _mxcall
+    return _call
+
+
 def strerror(code: int) -> str:
     return lib().mxattn_strerror(int(code)).decode()
 
@@ -98,28 +113,33 @@ def _ptr(t) -> int:
 
 
 def quantize_mxfp4(inp, codes, e8m0_scales, rows, cols, block_axis, mode):
-    _check(lib().mxattn_quantize_mxfp4(_ptr(inp), _ptr(codes), _ptr(e8m0_scales), rows, cols,
-                                       block_axis, mode, _stream()), "mxattn_quantize_mxfp4")
+    rc = (_call or _calls()).quantize_mxfp4(inp, codes, e8m0_scales, rows, cols, block_axis, mode)
+    if rc:
+        raise MxAttnError(rc, "mxattn_quantize_mxfp4")
 
 
 def quantize_mxfp4_batched(inp, codes, e8m0_scales, batch, rows, cols, block_axis, mode, layout):
-    _check(lib().mxattn_quantize_mxfp4_batched(_ptr(inp), _ptr(codes), _ptr(e8m0_scales), batch, rows,
-                                               cols, block_axis, mode, layout, _stream()),
-           "mxattn_quantize_mxfp4_batched")
+    rc = (_call or _calls()).quantize_mxfp4_batched(inp, codes, e8m0_scales, batch, rows, cols, block_axis, mode, layout)
+    if rc:
+        raise MxAttnError(rc, "mxattn_quantize_mxfp4_batched")
 
 
 def quantize_mxfp4_qmax(inp, codes, e8m0_scales, batch, rows, cols, block_axis, qmax, layout):
-    _check(lib().mxattn_quantize_mxfp4_qmax(_ptr(inp), _ptr(codes), _ptr(e8m0_scales), batch, rows, cols,
-                                            block_axis, qmax, layout, _stream()), "mxattn_quantize_mxfp4_qmax")
+    rc = (_call or _calls()).quantize_mxfp4_qmax(inp, codes, e8m0_scales, batch, rows, cols, block_axis, qmax, layout)
+    if rc:
+        raise MxAttnError(rc, "mxattn_quantize_mxfp4_qmax")
 
 
 def tensor_amax(inp, amax, batch, rows, cols):
-    _check(lib().mxattn_tensor_amax(_ptr(inp), _ptr(amax), batch, rows, cols, _stream()), "mxattn_tensor_amax")
+    rc = (_call or _calls()).tensor_amax(inp, amax, batch, rows, cols)
+    if rc:
+        raise MxAttnError(rc, "mxattn_tensor_amax")
 
 
 def quantize_nvfp4(inp, codes, e4m3_scales, tensor_amax, tensor_scale, batch, rows, cols, block_axis, layout):
-    _check(lib().mxattn_quantize_nvfp4(_ptr(inp), _ptr(codes), _ptr(e4m3_scales), _ptr(tensor_amax), _ptr(tensor_scale),
-                                       batch, rows, cols, block_axis, layout, _stream()), "mxattn_quantize_nvfp4")
+    rc = (_call or _calls()).quantize_nvfp4(inp, codes, e4m3_scales, tensor_amax, tensor_scale, batch, rows, cols, block_axis, layout)
+    if rc:
+        raise MxAttnError(rc, "mxattn_quantize_nvfp4")
 
 
 def forward_workspace_bytes(B, H, Nq, Nkv, d) -> int:
@@ -133,8 +153,9 @@ def set_workspace(ws, nbytes=None):
 
 
 def forward(q, k, v, o, B, H, Nq, Nkv, d, softmax_scale, flags):
-    _check(lib().mxattn_forward(_ptr(q), _ptr(k), _ptr(v), _ptr(o), B, H, Nq, Nkv, d,
-                                softmax_scale, flags, _stream()), "mxattn_forward")
+    rc = (_call or _calls()).forward(q, k, v, o, B, H, Nq, Nkv, d, softmax_scale, flags)
+    if rc:
+        raise MxAttnError(rc, "mxattn_forward")
 
 
 STATIC_SCRATCH_BYTES = 32 << 20
@@ -143,21 +164,21 @@ STATIC_SCRATCH_BYTES = 32 << 20
 def forward_static(q, k, v, o, B, H, Nq, Nkv, d, softmax_scale, flags):
     """mxattn_forward_static: the forward pass for callers that may not allocate device memory;
     its scratch is a fixed 32 MiB array inside the library (see include/mxattn.h for the rules)."""
-    _check(lib().mxattn_forward_static(_ptr(q), _ptr(k), _ptr(v), _ptr(o), B, H, Nq, Nkv, d,
-                                       softmax_scale, flags, _stream()), "mxattn_forward_static")
+    rc = (_call or _calls()).forward_static(q, k, v, o, B, H, Nq, Nkv, d, softmax_scale, flags)
+    if rc:
+        raise MxAttnError(rc, "mxattn_forward_static")
 
 
 def forward_ws(q, k, v, o, B, H, Nq, Nkv, d, softmax_scale, flags, workspace):
-    _check(lib().mxattn_forward_ws(_ptr(q), _ptr(k), _ptr(v), _ptr(o), B, H, Nq, Nkv, d, softmax_scale,
-                                   flags, _ptr(workspace),
-                                   0 if workspace is None else workspace.numel() * workspace.element_size(),
-                                   _stream()), "mxattn_forward_ws")
+    rc = (_call or _calls()).forward_ws(q, k, v, o, B, H, Nq, Nkv, d, softmax_scale, flags, workspace)
+    if rc:
+        raise MxAttnError(rc, "mxattn_forward_ws")
 
 
 def rowsum_diagnostic(q, k, out, B, H, Nq, Nkv, d, softmax_scale, flags, workspace):
-    _check(lib().mxattn_rowsum_diagnostic(_ptr(q), _ptr(k), _ptr(out), B, H, Nq, Nkv, d, softmax_scale, flags,
-                                          _ptr(workspace), 0 if workspace is None else workspace.numel() * workspace.element_size(),
-                                          _stream()), "mxattn_rowsum_diagnostic")
+    rc = (_call or _calls()).rowsum_diagnostic(q, k, out, B, H, Nq, Nkv, d, softmax_scale, flags, workspace)
+    if rc:
+        raise MxAttnError(rc, "mxattn_rowsum_diagnostic")
 
 
 def forward_debug_dump_bytes(B, H, Nq, Nkv, d) -> int:
@@ -187,9 +208,9 @@ def forward_bf16_workspace_bytes(B, H, Nq, Nkv, d) -> int:
 
 
 def forward_bf16(q, k, v, o, B, H, Nq, Nkv, d, softmax_scale, flags, workspace):
-    _check(lib().mxattn_forward_bf16(_ptr(q), _ptr(k), _ptr(v), _ptr(o), B, H, Nq, Nkv, d, softmax_scale, flags,
-                                     _ptr(workspace), workspace.numel() * workspace.element_size(), _stream()),
-           "mxattn_forward_bf16")
+    rc = (_call or _calls()).forward_bf16(q, k, v, o, B, H, Nq, Nkv, d, softmax_scale, flags, workspace)
+    if rc:
+        raise MxAttnError(rc, "mxattn_forward_bf16")
 
 
 def forward_nvfp4_workspace_bytes(B, H, Nq, Nkv, d) -> int:
@@ -197,17 +218,17 @@ def forward_nvfp4_workspace_bytes(B, H, Nq, Nkv, d) -> int:
 
 
 def forward_nvfp4(q, k, v, o, B, H, Nq, Nkv, d, softmax_scale, flags, workspace):
-    _check(lib().mxattn_forward_nvfp4(_ptr(q), _ptr(k), _ptr(v), _ptr(o), B, H, Nq, Nkv, d, softmax_scale, flags,
-                                      _ptr(workspace), 0 if workspace is None else workspace.numel() * workspace.element_size(),
-                                      _stream()), "mxattn_forward_nvfp4")
+    rc = (_call or _calls()).forward_nvfp4(q, k, v, o, B, H, Nq, Nkv, d, softmax_scale, flags, workspace)
+    if rc:
+        raise MxAttnError(rc, "mxattn_forward_nvfp4")
 
 
 def forward_prequantized(q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, o,
                          B, H, Nq, Nkv, d, softmax_scale, flags, status):
-    _check(lib().mxattn_forward_prequantized(_ptr(q_codes), _ptr(q_scales), _ptr(k_codes), _ptr(k_scales),
-                                             _ptr(v_codes), _ptr(v_scales), _ptr(o), B, H, Nq, Nkv, d,
-                                             softmax_scale, flags, _ptr(status), _stream()),
-           "mxattn_forward_prequantized")
+    rc = (_call or _calls()).forward_prequantized(q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, o,
+                                            B, H, Nq, Nkv, d, softmax_scale, flags, status)
+    if rc:
+        raise MxAttnError(rc, "mxattn_forward_prequantized")
 
 
 def forward_host_arena_bytes(B, H, Nq, Nkv, d, flags) -> int:
@@ -216,10 +237,9 @@ def forward_host_arena_bytes(B, H, Nq, Nkv, d, flags) -> int:
 
 def forward_host(q_host, k_host, v_host, o_host, B, H, Nq, Nkv, d, softmax_scale, flags, arena):
     """q_host.. are CPU tensors (pinned recommended); arena is a CUDA byte tensor."""
-    _check(lib().mxattn_forward_host(q_host.data_ptr(), k_host.data_ptr(), v_host.data_ptr(),
-                                     o_host.data_ptr(), B, H, Nq, Nkv, d, softmax_scale, flags,
-                                     _ptr(arena), arena.numel() * arena.element_size(), _stream()),
-           "mxattn_forward_host")
+    rc = (_call or _calls()).forward_host(q_host, k_host, v_host, o_host, B, H, Nq, Nkv, d, softmax_scale, flags, arena)
+    if rc:
+        raise MxAttnError(rc, "mxattn_forward_host")
 
 
 def probe_fp4_gemm(a_codes, a_scales, b_codes, b_scales, c, M, N, K, k_steps, resident, out_fp32, status, tile_n=256):

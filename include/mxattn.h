@@ -157,8 +157,8 @@ int mxattn_set_workspace(void* dev_ptr, size_t bytes);
  * when MXATTN_FLAG_HADAMARD is set).  q [B,H,Nq,d], k, v [B,H,Nkv,d] bf16; o [B,H,Nq,d] bf16 (fp32 with
  * MXATTN_FLAG_OUT_FP32).  d must be 128.  Non-causal, no mask.  softmax_scale > 0 multiplies the
  * quantized product Q-hat K-hat^T (line 9).  KV tiles are 128 keys, visited in ascending order.
- * Enqueues three quantize launches (Q, K along d; V along tokens) and one fused attention
- * launch.  Uses the workspace registered with mxattn_set_workspace. */
+ * Enqueues the quantization of Q, K (along d) and V (along tokens), in one to three launches, and
+ * one fused attention launch.  Uses the workspace registered with mxattn_set_workspace. */
 int mxattn_forward(const void* q, const void* k, const void* v, void* o,
                    int B, int H, int64_t Nq, int64_t Nkv, int d,
                    float softmax_scale, unsigned flags, void* stream);
@@ -363,7 +363,9 @@ int mxattn_selftest_bounded_wait(void* status, int64_t limit_cycles, void* strea
  * in status[1] -- `meetings` if no warp was left stranded.  `status`: 4 device ints, zeroed by the caller. */
 int mxattn_selftest_pair_abandon(void* status, int64_t limit_cycles, int meetings, void* stream);
 
-/* Number of kernel launches the last forward call of this process enqueued (for accounting). */
+/* Number of stages the last forward call of this process enqueued (for accounting): one per operand quantized (or
+ * re-tiled), one per tensor maximum, one for the attention kernel.  Stages may share a kernel launch: short problems
+ * quantize Q, K and V in one. */
 int mxattn_last_launch_count(void);
 
 const char* mxattn_strerror(int status);

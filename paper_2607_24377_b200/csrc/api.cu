@@ -1,6 +1,7 @@
 // C-ABI entry points that orchestrate the kernels: workspace carving, the three quantize
 // launches plus the fused attention launch (paper Algorithm 2, lines 3-19), and the host-buffer
 // end-to-end form.
+#include <atomic>
 #include <vector>
 
 #include "common.cuh"
@@ -22,6 +23,42 @@ static void* g_workspace = nullptr;
 static size_t g_workspace_bytes = 0;
 
 void count_launch(int n) { g_launches += n; }
+
+constexpr int kMaxDevices = 64;
+static int current_device() {
+  int dev = -1;
+  return (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices) ? dev : -1;
+}
+
+int sm_count() {
+  static std::atomic<int> n[kMaxDevices];
+  const int dev = current_device();
+  if (dev < 0) return 0;
+  int v = n[dev].load(std::memory_order_relaxed);
+  if (v == 0) {
+    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) return 0;
+    n[dev].store(v, std::memory_order_relaxed);
+  }
+  return v;
+}
+
+bool ensure_dynamic_smem(const void* kern, int bytes) {
+  // one entry per kernel (a few dozen): the devices on which its limit has been raised, one bit each
+  struct Entry { std::atomic<const void*> kern; std::atomic<uint64_t> devices; };
+  static Entry table[128];
+  const int dev = current_device();
+  if (dev < 0) return false;
+  for (Entry& e : table) {
+    const void* k = e.kern.load(std::memory_order_acquire);
+    if (k == nullptr && e.kern.compare_exchange_strong(k, kern, std::memory_order_acq_rel)) k = kern;
+    if (k != kern) continue;                        // (a failed exchange left another thread's kernel in k)
+    if (e.devices.load(std::memory_order_acquire) >> dev & 1) return true;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
+    e.devices.fetch_or((uint64_t)1 << dev, std::memory_order_release);
+    return true;
+  }
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
+}
 
 struct WorkspaceLayout {
   size_t q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, status, total;
@@ -68,14 +105,12 @@ static int forward_ws(const void* q, const void* k, const void* v, void* o, int 
   const int qk_mode = mode | ((flags & MXATTN_FLAG_HADAMARD) ? MXATTN_MODE_HADAMARD : 0);   // Algorithm 2 lines 1-2
   const int64_t bh = (int64_t)B * H;
   cudaStream_t qs = qstream ? qstream : stream;
-  if (cudaMemsetAsync(ws + w.status, 0, 16, qs) != cudaSuccess) return MXATTN_ECUDA;
-  int rc;
-  // Algorithm 2 lines 3-5: Q-hat, K-hat (blocks along d), V-hat (blocks along tokens)
+  // Algorithm 2 lines 3-5: Q-hat, K-hat (blocks along d), V-hat (blocks along tokens); the launch clears the status word
   {
     TraceRange tr("mxattn quantize Q K V");
-    if ((rc = launch_quantize(q, ws + w.q_codes, ws + w.q_scales, bh, Nq, d, 1, qk_mode, MXATTN_LAYOUT_TILE, qs))) return rc;
-    if ((rc = launch_quantize(k, ws + w.k_codes, ws + w.k_scales, bh, Nkv, d, 1, qk_mode, MXATTN_LAYOUT_TILE, qs))) return rc;
-    if ((rc = launch_quantize(v, ws + w.v_codes, ws + w.v_scales, bh, Nkv, d, 0, mode, MXATTN_LAYOUT_TILE, qs))) return rc;
+    const int rc = launch_quantize_qkv(q, ws + w.q_codes, ws + w.q_scales, k, ws + w.k_codes, ws + w.k_scales, v, ws + w.v_codes,
+                                       ws + w.v_scales, bh, Nq, Nkv, qk_mode, reinterpret_cast<int*>(ws + w.status), qs);
+    if (rc != MXATTN_OK) return rc;
   }
   if (qstream) {
     if (cudaEventRecord(qdone, qstream) != cudaSuccess || cudaStreamWaitEvent(stream, qdone, 0) != cudaSuccess) return MXATTN_ECUDA;
@@ -136,10 +171,9 @@ extern "C" int mxattn_rowsum_diagnostic(const void* q, const void* k, void* out,
   const int mode = (flags & MXATTN_FLAG_UOS) ? MXATTN_MODE_UOS : MXATTN_MODE_OCP;
   const int qk_mode = mode | ((flags & MXATTN_FLAG_HADAMARD) ? MXATTN_MODE_HADAMARD : 0);
   const int64_t bh = (int64_t)B * H;
-  if (cudaMemsetAsync(ws + w.status, 0, 16, stream) != cudaSuccess) return MXATTN_ECUDA;
-  int rc;
-  if ((rc = launch_quantize(q, ws + w.q_codes, ws + w.q_scales, bh, Nq, d, 1, qk_mode, MXATTN_LAYOUT_TILE, stream))) return rc;
-  if ((rc = launch_quantize(k, ws + w.k_codes, ws + w.k_scales, bh, Nkv, d, 1, qk_mode, MXATTN_LAYOUT_TILE, stream))) return rc;
+  const int rc = launch_quantize_qkv(q, ws + w.q_codes, ws + w.q_scales, k, ws + w.k_codes, ws + w.k_scales, nullptr, nullptr, nullptr,
+                                     bh, Nq, Nkv, qk_mode, reinterpret_cast<int*>(ws + w.status), stream);
+  if (rc != MXATTN_OK) return rc;
   return launch_rowsum_diag(ws + w.q_codes, ws + w.q_scales, ws + w.k_codes, ws + w.k_scales, out, B, H, Nq, Nkv,
                             softmax_scale, (flags & MXATTN_FLAG_UOS) ? kRuleUos : kRuleOcp,
                             reinterpret_cast<int*>(ws + w.status), stream);
@@ -360,7 +394,6 @@ static __device__ __align__(256) unsigned char g_static_scratch[MXATTN_STATIC_SC
 
 // In host code `g_static_scratch` is only a handle for the runtime, not a device address, so the
 // address is looked up once per device (with that device current) and cached.
-constexpr int kMaxDevices = 64;
 static void* g_static_scratch_ptr[kMaxDevices] = {nullptr};
 
 extern "C" int mxattn_forward_static(const void* q, const void* k, const void* v, void* o, int B, int H,

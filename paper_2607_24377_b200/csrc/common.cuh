@@ -85,12 +85,38 @@ __device__ __host__ __forceinline__ int tile_scale_offset(int r, int c) {
   return (r & 31) * 16 + (r >> 5) * 4 + c;
 }
 
+// Programmatic dependent launch.  Every kernel of this library that is launched with launch_pdl starts with pdl_wait():
+// nothing is read or written before all work queued earlier on the stream has completed and is visible, so the launch
+// behaves as in plain stream order.  What overlaps is the launch itself: the CTAs are placed, and their set-up that
+// touches no global memory runs, while the predecessor drains (pdl_trigger lets the successor's CTAs be placed as soon as
+// every CTA of this grid has started).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t stream, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = dim3(block); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
+}
+// Raises a kernel's dynamic shared memory limit, once per kernel and device (a driver call per launch otherwise).
+bool ensure_dynamic_smem(const void* kern, int bytes);
+int sm_count();              // of the current device (0 on error)
+
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // Internal launchers (defined in quantize.cu / forward.cu); all return an mxattn_status.
 int launch_quantize(const void* in, void* codes, void* scales, int64_t batch, int64_t rows,
                     int64_t cols, int block_axis, int mode, int layout, cudaStream_t stream,
                     uint32_t rule_override = 0xFFFFFFFFu);
+// Q, K (block axis 1) and V (block axis 0) of `bh` heads in tile layout; mode may carry MXATTN_MODE_HADAMARD for Q and K.
+// v may be null (two operands).  Also clears status[0..3].
+int launch_quantize_qkv(const void* q, void* q_codes, void* q_scales, const void* k, void* k_codes, void* k_scales,
+                        const void* v, void* v_codes, void* v_scales, int64_t bh, int64_t Nq, int64_t Nkv, int mode,
+                        int* status, cudaStream_t stream);
 int launch_tensor_amax(const void* in, float* amax, int64_t batch, int64_t rows, int64_t cols, cudaStream_t stream);
 int launch_quantize_nvfp4(const void* in, void* codes, void* scales, const float* amax, float* tensor_scale, int64_t batch,
                           int64_t rows, int64_t cols, int block_axis, int layout, cudaStream_t stream);

@@ -160,7 +160,6 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kOffMisc + 8);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (*reinterpret_cast<volatile int*>(p.status) != 0) return;   // an earlier CTA gave up: drain the grid quickly
   const int T = p.kv_tiles;
   const int bh0 = blockIdx.x / p.q_pairs, pair0 = blockIdx.x - bh0 * p.q_pairs;
 
@@ -176,7 +175,6 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
     mbar_init(bar(BAR_PFULL + 0), 4 * kSplit); mbar_init(bar(BAR_PFULL + 1), 4 * kSplit);   // one arrival per softmax warp
     mbar_init(bar(BAR_ODONE + 0), 1); mbar_init(bar(BAR_ODONE + 1), 1);
     abort_flag[0] = 0;
-    abort_flag[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   // constant rows of ones appended to every V stage (E2M1 code 2 = 1.0) and their scale atom (2^0)
@@ -192,12 +190,16 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  pdl_wait();                                        // the operands and the status word are ready (everything above overlapped their quantization)
+  if (tid == 0) abort_flag[1] = *reinterpret_cast<volatile int*>(p.status);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_trigger();
   const uint32_t tmem = *tmem_slot;
+  const int role = abort_flag[1] != 0 ? kSoftmaxWarps + 2 : warp;     // an earlier CTA gave up: drain the grid quickly
 
-  if (warp == kSoftmaxWarps) {
+  if (role == kSoftmaxWarps) {
     // =============================== producer ===============================================
     if (lane == 0) {
       int F = 0;                                   // tiles issued so far, over all items of this CTA
@@ -246,7 +248,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
         }
       }
     }
-  } else if (warp == kSoftmaxWarps + 1) {
+  } else if (role == kSoftmaxWarps + 1) {
     // =============================== MMA issuer =============================================
     if (lane == 0) {
       if (kProf) prof_prev = clock64();
@@ -444,7 +446,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
         prof_t[9] = kPersist ? (long long)((p.total_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x) * T : T;
       }
     }
-  } else if (warp < kSoftmaxWarps) {
+  } else if (role < kSoftmaxWarps) {
     // =============================== softmax groups =========================================
     const int t = warp >> 3;                       // query tile of this group
     const int h = (warp >> 2) & 1;                 // which 64 key columns of the tile
@@ -860,13 +862,8 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
   // Short key/value sequences with more work items than SMs: one CTA per SM walks the items, so that the set-up,
   // the first loads and the epilogue of one item overlap the tiles of its neighbours.  Long sequences keep one
   // item per CTA (the hardware's block scheduler then balances the tail better than a static assignment).
-  static int n_sm = 0;
-  if (n_sm == 0) {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0)
-      return MXATTN_ECUDA;
-    n_sm = v;
-  }
+  const int n_sm = sm_count();
+  if (n_sm == 0) return MXATTN_ECUDA;
   const bool persist = (!dump || profile) && grid > n_sm && kt <= kPersistMaxTiles;
   // Descriptor of the bf16 output as a [B H][Nq][128] tensor with boxes of 32 rows x 64 columns (the epilogue's copies).
   CUtensorMap out_map;
@@ -906,11 +903,9 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
     PICKD(false, false) PICKD(false, true) PICKD(true, false) PICKD(true, true)
 #undef PICKD
   }
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess)
-    return MXATTN_ECUDA;
-  kern<<<(unsigned)(persist ? n_sm : grid), kThreads, kSmemBytes, stream>>>(p, out_map);
+  if (!ensure_dynamic_smem((const void*)kern, kSmemBytes)) return MXATTN_ECUDA;
   count_launch(1);
-  return cudaGetLastError() == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
+  return launch_pdl(kern, dim3((unsigned)(persist ? n_sm : grid)), kThreads, kSmemBytes, stream, p, out_map) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 
 }  // namespace mxattn

@@ -50,6 +50,7 @@ quantize_axis1_kernel(const uint4* __restrict__ in, uint32_t* __restrict__ codes
   // (c = 4 blk + k per thread) touch every bank group once per quarter warp.
   __shared__ uint4 s_v[kQThreads * kQChunksPerThread];
   const int tid = threadIdx.x, lane = tid & 31;
+  pdl_wait(); pdl_trigger();
   const int64_t base = (int64_t)blockIdx.x * (kQThreads * kQChunksPerThread);
   auto pos = [](int c) { return c ^ ((c >> 3) & 7); };
 #pragma unroll
@@ -93,18 +94,15 @@ quantize_axis1_kernel(const uint4* __restrict__ in, uint32_t* __restrict__ codes
 }
 
 // ------------------------------------------------------------------------------------------
-// Axis 1, tile layout (cols == 128).  grid = (2 x row tiles, batch); one CTA quantizes half a 128-row tile
-// (64 rows, 16 KiB in) the same way: asynchronous copies into shared memory, one block (row r, 32 columns c) per
-// thread, one 16-byte store into the tile image, one 32-bit scale store per row.
-__global__ void __launch_bounds__(kQThreads)
-quantize_axis1_tile_kernel(const uint4* __restrict__ in, uint8_t* __restrict__ codes,
-                           uint8_t* __restrict__ scales, int64_t rows, uint32_t rule) {
-  __shared__ uint4 s_v[kQThreads * 4];
+// Axis 1, tile layout (cols == 128).  One CTA quantizes half a 128-row tile (64 rows, 16 KiB in) the same way: asynchronous
+// copies into shared memory (`s_v`, 16 KiB), one block (row r, 32 columns c) per thread, one 16-byte store into the tile
+// image, one 32-bit scale store per row.  Tile t of matrix m; `tile` = its index in the output.
+__device__ __forceinline__ void quantize_axis1_half_tile(uint4* s_v, const uint4* __restrict__ in, uint8_t* __restrict__ codes,
+                                                         uint8_t* __restrict__ scales, int64_t rows, uint32_t rule,
+                                                         int64_t m, int64_t t, int64_t tile, int half) {
   const int tid = threadIdx.x;
-  const int64_t tile = (int64_t)blockIdx.y * (gridDim.x >> 1) + (blockIdx.x >> 1);
-  const int half = blockIdx.x & 1;
-  const int64_t row0 = (int64_t)(blockIdx.x >> 1) * kTile + half * 64;
-  const uint4* src = in + ((int64_t)blockIdx.y * rows + row0) * 16;     // 16 chunks per row
+  const int64_t row0 = t * kTile + half * 64;
+  const uint4* src = in + (m * rows + row0) * 16;                       // 16 chunks per row
   const int rows_here = (int)max((int64_t)0, min((int64_t)64, rows - row0));
   auto pos = [](int c) { return c ^ ((c >> 3) & 7); };
 #pragma unroll
@@ -120,8 +118,8 @@ quantize_axis1_tile_kernel(const uint4* __restrict__ in, uint8_t* __restrict__ c
   uint4 v[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) v[k] = s_v[pos(4 * tid + k)];
-  const uint32_t m = max(max(absmax_bf16x8(v[0]), absmax_bf16x8(v[1])), max(absmax_bf16x8(v[2]), absmax_bf16x8(v[3])));
-  const int e = shared_exponent_rule(m << 16, rule);
+  const uint32_t mx = max(max(absmax_bf16x8(v[0]), absmax_bf16x8(v[1])), max(absmax_bf16x8(v[2]), absmax_bf16x8(v[3])));
+  const int e = shared_exponent_rule(mx << 16, rule);
   const float inv = pow2_neg(e);
   const uint32_t eb = (uint32_t)(e + 127);
   const uint32_t b1 = __shfl_down_sync(0xFFFFFFFFu, eb, 1);
@@ -131,6 +129,15 @@ quantize_axis1_tile_kernel(const uint4* __restrict__ in, uint8_t* __restrict__ c
       make_uint4(quantize_bf16x8(v[0], inv), quantize_bf16x8(v[1], inv), quantize_bf16x8(v[2], inv), quantize_bf16x8(v[3], inv));
   if (c == 0)
     *reinterpret_cast<uint32_t*>(scales + tile * kTileScaleBytes + tile_scale_offset(r, 0)) = eb | (b1 << 8) | (b2 << 16) | (b3 << 24);
+}
+
+__global__ void __launch_bounds__(kQThreads)
+quantize_axis1_tile_kernel(const uint4* __restrict__ in, uint8_t* __restrict__ codes,
+                           uint8_t* __restrict__ scales, int64_t rows, uint32_t rule) {
+  __shared__ uint4 s_v[kQThreads * 4];
+  pdl_wait(); pdl_trigger();
+  const int64_t t = blockIdx.x >> 1;                 // grid = (2 x row tiles, batch)
+  quantize_axis1_half_tile(s_v, in, codes, scales, rows, rule, blockIdx.y, t, (int64_t)blockIdx.y * (gridDim.x >> 1) + t, blockIdx.x & 1);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -156,12 +163,15 @@ __device__ int g_status = 0;                               // non-zero if a boun
 
 __device__ __forceinline__ int half_chunk_offset(int r, int c) { return r * 128 + ((c ^ (r & 7)) << 4); }
 
+struct Operand { const uint4* in; uint8_t* codes; uint8_t* scales; int64_t rows; int tiles_per_matrix, n_tiles; };
+
 template <bool kTileLayout, int kRuleKind>
 __global__ void __launch_bounds__(kThreads, 2)
-quantize_axis1_rot_tc_kernel(const uint4* __restrict__ in, uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
-                             int64_t rows, int tiles_per_matrix, int n_tiles, uint32_t rule) {
-  // tile layout: `rows` per matrix of the batch, tile = matrix * tiles_per_matrix + tile within the matrix;
-  // canonical: one matrix of `rows` rows (the batch is contiguous), tiles_per_matrix == n_tiles
+quantize_axis1_rot_tc_kernel(const Operand op0, const Operand op1, uint32_t rule) {
+  // two operands (the second may have no tiles), walked as one sequence of tiles.  Tile layout: `rows` per matrix of the
+  // batch, tile = matrix * tiles_per_matrix + tile within the matrix; canonical: one matrix of `rows` rows (the batch is
+  // contiguous), tiles_per_matrix == n_tiles
+  const int n_tiles = op0.n_tiles + op1.n_tiles;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t sbase = smem_u32(smem);
@@ -171,14 +181,16 @@ quantize_axis1_rot_tc_kernel(const uint4* __restrict__ in, uint8_t* __restrict__
   const int tid = threadIdx.x, warp = tid >> 5;
   const int n_my = ((int)blockIdx.x < n_tiles) ? (n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
 
-  auto tile_rows = [&](int tile, int64_t* first_row) {       // rows of the input this tile covers
-    const int m = tile / tiles_per_matrix, t = tile - m * tiles_per_matrix;
-    *first_row = (int64_t)m * rows + (int64_t)t * kTile;
-    return (int)min((int64_t)kTile, rows - (int64_t)t * kTile);
+  auto tile_rows = [&](const Operand& op, int tile, int64_t* first_row) {       // rows of the input this tile covers
+    const int m = tile / op.tiles_per_matrix, t = tile - m * op.tiles_per_matrix;
+    *first_row = (int64_t)m * op.rows + (int64_t)t * kTile;
+    return (int)min((int64_t)kTile, op.rows - (int64_t)t * kTile);
   };
   auto fetch = [&](int tile, int buf) {                       // X tile -> shared memory, zero beyond the matrix
     int64_t first;
-    const int here = tile_rows(tile, &first);
+    const Operand& op = tile < op0.n_tiles ? op0 : op1;
+    const int here = tile_rows(op, tile < op0.n_tiles ? tile : tile - op0.n_tiles, &first);
+    const uint4* in = op.in;
     const uint4* src = in + first * 16;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
@@ -200,7 +212,6 @@ quantize_axis1_rot_tc_kernel(const uint4* __restrict__ in, uint8_t* __restrict__
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(smem_u32(tmem_slot)) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  if (n_my > 0) fetch(blockIdx.x, 0);
   // H as the B operand: B[n][k] = H[k][n] = (-1)^popcount(n & k); chunk (n, cc) holds k = 8 cc .. 8 cc + 7
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
@@ -219,12 +230,19 @@ quantize_axis1_rot_tc_kernel(const uint4* __restrict__ in, uint8_t* __restrict__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_wait();
+  pdl_trigger();                                      // after the tensor-memory allocation: a dependent CTA must not get it first
+  if (n_my > 0) fetch(blockIdx.x, 0);
 
   // epilogue of one tile: this thread's half row (row r, columns 64 h .. 64 h + 63) out of accumulator `buf`
   const int r = (warp & 3) * 32 + (tid & 31), h = warp >> 2;
   auto quantize_tile = [&](int tile, int buf) {
     int64_t first;
-    const int here = tile_rows(tile, &first);
+    const Operand& op = tile < op0.n_tiles ? op0 : op1;
+    if (tile >= op0.n_tiles) tile -= op0.n_tiles;
+    const int here = tile_rows(op, tile, &first);
+    uint8_t* codes = op.codes;
+    uint8_t* scales = op.scales;
     const uint32_t t_row = tmem + 128 * buf + ((uint32_t)((warp & 3) * 32) << 16) + 64 * h;
     uint32_t sf = 0;
 #pragma unroll
@@ -320,23 +338,28 @@ quantize_axis1_rot_tc_kernel(const uint4* __restrict__ in, uint8_t* __restrict__
 //                 (and 8 scale bytes) instead of two 64-byte ones; grid = (ceil(cols/64), ceil(rows_pad/256), batch)
 constexpr int kVThreads = 256;
 
+struct __align__(16) Axis0Smem {
+  uint16_t in[128 * 128];                 // [token][column] raw bf16
+  uint8_t codes[kTileCodeBytes];          // [column][code bytes], 16-byte chunks swizzled
+  uint8_t scales[kTileScaleBytes];
+};
+
+// slab (cx, ry) of matrix b; n_ry: slabs along the tokens
 template <bool kTileLayout>
-__global__ void __launch_bounds__(kVThreads)
-quantize_axis0_kernel(const uint16_t* __restrict__ in, uint8_t* __restrict__ codes,
-                      uint8_t* __restrict__ scales, int64_t rows, int64_t cols, int64_t rows_pad,
-                      uint32_t rule) {
+__device__ __forceinline__ void quantize_axis0_slab(Axis0Smem& sm, const uint16_t* __restrict__ in, uint8_t* __restrict__ codes,
+                                                    uint8_t* __restrict__ scales, int64_t rows, int64_t cols, int64_t rows_pad,
+                                                    uint32_t rule, int64_t cx, int64_t ry, int64_t n_ry, int64_t b) {
   constexpr int kTok = kTileLayout ? 128 : 256;                   // tokens per slab
   constexpr int kCol = kTileLayout ? 128 : 64;                    // columns per slab
   constexpr int kColBytes = kTok / 2;                             // code bytes per column of the slab
   constexpr int kColBlocks = kTok / kBlock;                       // blocks (scale bytes) per column of the slab
-  __shared__ __align__(16) uint16_t s_in[kTok][kCol];             // [token][column] raw bf16
-  __shared__ __align__(16) uint8_t s_codes[kTileCodeBytes];       // [column][kColBytes], 16-byte chunks swizzled
-  __shared__ __align__(16) uint8_t s_scales[kTileScaleBytes];
+  uint16_t(*s_in)[kCol] = reinterpret_cast<uint16_t(*)[kCol]>(sm.in);
+  uint8_t* s_codes = sm.codes;
+  uint8_t* s_scales = sm.scales;
 
   const int tid = threadIdx.x;
-  const int64_t col0 = (int64_t)blockIdx.x * kCol;
-  const int64_t row0 = (int64_t)blockIdx.y * kTok;
-  const int64_t b = blockIdx.z;
+  const int64_t col0 = cx * kCol;
+  const int64_t row0 = ry * kTok;
   const uint16_t* src = in + b * rows * cols;
   // staging offset of the 16-byte chunk c of column n: the tile image's own swizzle, or (canonical) the
   // chunk index XORed with the column pair so that the 8 threads of a store phase hit 8 different bank groups
@@ -389,7 +412,7 @@ quantize_axis0_kernel(const uint16_t* __restrict__ in, uint8_t* __restrict__ cod
 
   // phase 3: staged slab -> global
   if (kTileLayout) {
-    const int64_t tile = b * gridDim.y + blockIdx.y;            // cols == 128: one column tile
+    const int64_t tile = b * n_ry + ry;                         // cols == 128: one column tile
     uint4* dst = reinterpret_cast<uint4*>(codes + tile * kTileCodeBytes);
 #pragma unroll
     for (int k = 0; k < kTileCodeBytes / 16 / kVThreads; ++k)
@@ -420,16 +443,85 @@ quantize_axis0_kernel(const uint16_t* __restrict__ in, uint8_t* __restrict__ cod
   }
 }
 
+template <bool kTileLayout>
+__global__ void __launch_bounds__(kVThreads)
+quantize_axis0_kernel(const uint16_t* __restrict__ in, uint8_t* __restrict__ codes,
+                      uint8_t* __restrict__ scales, int64_t rows, int64_t cols, int64_t rows_pad,
+                      uint32_t rule) {
+  __shared__ Axis0Smem sm;
+  pdl_wait(); pdl_trigger();
+  quantize_axis0_slab<kTileLayout>(sm, in, codes, scales, rows, cols, rows_pad, rule, blockIdx.x, blockIdx.y, gridDim.y, blockIdx.z);
+}
+
 // ------------------------------------------------------------------------------------------
-// persistent grid of the rotating quantizer: two CTAs per SM
-static int rot_grid() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) v = 148;
-    n = 2 * v;
+// All operands of a forward call in one launch (tile layout, cols == 128): the half tiles of Q, then those of K, then the
+// tiles of V; a count of zero leaves an operand out (the rotating quantizer handles Q and K then).  Short problems are
+// bound by launches and their latency, not by bytes: three launches and a memset of the status word took 12 us of a
+// 31 us call at 2 heads of 1024 tokens.  Thread 0 of the first CTA clears the status word.
+struct QkvOperand { const void* in; uint8_t* codes; uint8_t* scales; int64_t rows; int64_t tiles; int64_t ctas; };   // tiles per matrix
+__global__ void __launch_bounds__(kQThreads)
+quantize_qkv_kernel(const QkvOperand q, const QkvOperand k, const QkvOperand v, uint32_t rule, int* status) {
+  __shared__ Axis0Smem sm;
+  pdl_wait(); pdl_trigger();
+  int64_t i = blockIdx.x;
+  if (i == 0 && threadIdx.x < 4 && status) status[threadIdx.x] = 0;
+  if (i < q.ctas + k.ctas) {
+    const QkvOperand& o = i < q.ctas ? q : k;
+    if (i >= q.ctas) i -= q.ctas;
+    const int64_t tile = i >> 1, m = tile / o.tiles;
+    quantize_axis1_half_tile(reinterpret_cast<uint4*>(sm.in), (const uint4*)o.in, o.codes, o.scales, o.rows, rule, m, tile - m * o.tiles, tile, (int)(i & 1));
+  } else if (i < q.ctas + k.ctas + v.ctas) {
+    i -= q.ctas + k.ctas;
+    const int64_t m = i / v.tiles;
+    quantize_axis0_slab<true>(sm, (const uint16_t*)v.in, v.codes, v.scales, v.rows, kHeadDim, v.tiles * kTile, rule, 0, i - m * v.tiles, v.tiles, m);
   }
-  return n;
+}
+
+// ------------------------------------------------------------------------------------------
+// the rotating quantizer on one or two operands: persistent grid, two CTAs per SM
+static int launch_rot(const rot::Operand& a, const rot::Operand& b, bool tile, uint32_t rule, cudaStream_t stream) {
+  auto kern = tile ? (rule == kRuleOcp ? rot::quantize_axis1_rot_tc_kernel<true, 0>
+                    : rule == kRuleUos ? rot::quantize_axis1_rot_tc_kernel<true, 1> : rot::quantize_axis1_rot_tc_kernel<true, 2>)
+                   : (rule == kRuleOcp ? rot::quantize_axis1_rot_tc_kernel<false, 0>
+                    : rule == kRuleUos ? rot::quantize_axis1_rot_tc_kernel<false, 1> : rot::quantize_axis1_rot_tc_kernel<false, 2>);
+  if (!ensure_dynamic_smem((const void*)kern, rot::kSmemBytes)) return MXATTN_ECUDA;
+  const int64_t n = (int64_t)a.n_tiles + b.n_tiles, most = 2 * (int64_t)sm_count();
+  return launch_pdl(kern, dim3((unsigned)min(most > 0 ? most : (int64_t)296, n)), rot::kThreads, rot::kSmemBytes, stream, a, b, rule) == cudaSuccess
+             ? MXATTN_OK : MXATTN_ECUDA;
+}
+
+int launch_quantize_qkv(const void* q, void* q_codes, void* q_scales, const void* k, void* k_codes, void* k_scales,
+                        const void* v, void* v_codes, void* v_scales, int64_t bh, int64_t Nq, int64_t Nkv, int mode,
+                        int* status, cudaStream_t stream) {
+  const uint32_t rule = (mode & ~MXATTN_MODE_HADAMARD) == MXATTN_MODE_UOS ? kRuleUos : kRuleOcp;
+  const bool rotate = (mode & MXATTN_MODE_HADAMARD) != 0;
+  const int64_t qt = (Nq + kTile - 1) / kTile, kt = (Nkv + kTile - 1) / kTile;
+  if (bh * (2 * qt + 3 * kt) > 0x7FFFFFFF) return MXATTN_EUNSUPPORTED;
+  QkvOperand oq{q, (uint8_t*)q_codes, (uint8_t*)q_scales, Nq, qt, rotate ? 0 : 2 * bh * qt};
+  QkvOperand ok{k, (uint8_t*)k_codes, (uint8_t*)k_scales, Nkv, kt, rotate ? 0 : 2 * bh * kt};
+  QkvOperand ov{v, (uint8_t*)v_codes, (uint8_t*)v_scales, Nkv, kt, v ? bh * kt : 0};
+  // Long problems are bound by bandwidth: Q and K then run in the kernel of their own, which has six CTAs per SM where the
+  // shared one has four (its registers and shared memory are sized for V) -- 774 MB of Q: 0.12 against 0.14 ms.  From 24
+  // CTAs per SM on that outweighs the two further launches.
+  const int n_sm = sm_count();
+  if (n_sm == 0) return MXATTN_ECUDA;
+  if (!rotate && oq.ctas + ok.ctas > 24 * (int64_t)n_sm && bh <= 65535) {
+    for (const QkvOperand* o : {&oq, &ok})
+      if (launch_pdl(quantize_axis1_tile_kernel, dim3((unsigned)(2 * o->tiles), (unsigned)bh), kQThreads, 0, stream, (const uint4*)o->in,
+                     o->codes, o->scales, o->rows, rule) != cudaSuccess) return MXATTN_ECUDA;
+    oq.ctas = ok.ctas = 0;
+  }
+  const int64_t ctas = oq.ctas + ok.ctas + ov.ctas;
+  // with the rotation and no V there is nothing for the plain kernel but the status word: one CTA does it
+  if (launch_pdl(quantize_qkv_kernel, dim3((unsigned)(ctas > 0 ? ctas : 1)), kQThreads, 0, stream, oq, ok, ov, rule, status) != cudaSuccess) return MXATTN_ECUDA;
+  if (rotate) {
+    const rot::Operand a{(const uint4*)q, (uint8_t*)q_codes, (uint8_t*)q_scales, Nq, (int)qt, (int)(bh * qt)};
+    const rot::Operand b{(const uint4*)k, (uint8_t*)k_codes, (uint8_t*)k_scales, Nkv, (int)kt, (int)(bh * kt)};
+    const int rc = launch_rot(a, b, true, rule, stream);
+    if (rc != MXATTN_OK) return rc;
+  }
+  count_launch(v ? 3 : 2);
+  return MXATTN_OK;
 }
 
 int launch_quantize(const void* in, void* codes, void* scales, int64_t batch, int64_t rows,
@@ -450,6 +542,7 @@ int launch_quantize(const void* in, void* codes, void* scales, int64_t batch, in
   const uint32_t rule = rule_override != 0xFFFFFFFFu ? rule_override : (mode == MXATTN_MODE_UOS ? kRuleUos : kRuleOcp);
   const int64_t rows_pad = (rows + kTile - 1) / kTile * kTile;
 
+  cudaError_t e = cudaSuccess;
   if (block_axis == 1) {
     const bool tile = (layout == MXATTN_LAYOUT_TILE);
     const int64_t n_chunks = tile ? batch * rows_pad * 16 : batch * rows * (cols / 8);
@@ -459,27 +552,21 @@ int launch_quantize(const void* in, void* codes, void* scales, int64_t batch, in
       if (rows_pad / kTile > 0x3FFFFFFF || batch > 65535) return MXATTN_EUNSUPPORTED;
       dim3 grid((unsigned)(2 * (rows_pad / kTile)), (unsigned)batch);       // the plain tile kernel takes half a tile per CTA
       if (rotate) {
-        auto kern = rule == kRuleOcp ? rot::quantize_axis1_rot_tc_kernel<true, 0>
-                  : rule == kRuleUos ? rot::quantize_axis1_rot_tc_kernel<true, 1> : rot::quantize_axis1_rot_tc_kernel<true, 2>;
         const int64_t n_tiles = batch * (rows_pad / kTile);
         if (n_tiles > 0x7FFFFFFF) return MXATTN_EUNSUPPORTED;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, rot::kSmemBytes) != cudaSuccess) return MXATTN_ECUDA;
-        kern<<<(unsigned)min((int64_t)rot_grid(), n_tiles), rot::kThreads, rot::kSmemBytes, stream>>>(
-            (const uint4*)in, (uint8_t*)codes, (uint8_t*)scales, rows, (int)(rows_pad / kTile), (int)n_tiles, rule);
+        const rot::Operand a{(const uint4*)in, (uint8_t*)codes, (uint8_t*)scales, rows, (int)(rows_pad / kTile), (int)n_tiles};
+        if (launch_rot(a, rot::Operand{}, true, rule, stream) != MXATTN_OK) return MXATTN_ECUDA;
       } else
-        quantize_axis1_tile_kernel<<<grid, kQThreads, 0, stream>>>((const uint4*)in, (uint8_t*)codes,
+        e = launch_pdl(quantize_axis1_tile_kernel, grid, kQThreads, 0, stream, (const uint4*)in, (uint8_t*)codes,
                                                                           (uint8_t*)scales, rows, rule);
     } else {
       if (rotate) {                                  // cols == 128 here: batch * rows rows of 16 chunks
         const int64_t groups = (batch * rows + kTile - 1) / kTile;
         if (groups > 0x7FFFFFFF) return MXATTN_EUNSUPPORTED;
-        auto kern = rule == kRuleOcp ? rot::quantize_axis1_rot_tc_kernel<false, 0>
-                  : rule == kRuleUos ? rot::quantize_axis1_rot_tc_kernel<false, 1> : rot::quantize_axis1_rot_tc_kernel<false, 2>;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, rot::kSmemBytes) != cudaSuccess) return MXATTN_ECUDA;
-        kern<<<(unsigned)min((int64_t)rot_grid(), groups), rot::kThreads, rot::kSmemBytes, stream>>>(
-            (const uint4*)in, (uint8_t*)codes, (uint8_t*)scales, batch * rows, (int)groups, (int)groups, rule);
+        const rot::Operand a{(const uint4*)in, (uint8_t*)codes, (uint8_t*)scales, batch * rows, (int)groups, (int)groups};
+        if (launch_rot(a, rot::Operand{}, false, rule, stream) != MXATTN_OK) return MXATTN_ECUDA;
       } else
-        quantize_axis1_kernel<<<(unsigned)blocks, kQThreads, 0, stream>>>(
+        e = launch_pdl(quantize_axis1_kernel, dim3((unsigned)blocks), kQThreads, 0, stream, 
             (const uint4*)in, (uint32_t*)codes, (uint8_t*)scales, n_chunks, rule);
     }
   } else {
@@ -488,14 +575,14 @@ int launch_quantize(const void* in, void* codes, void* scales, int64_t batch, in
     if (ct > 0x7FFFFFFF || rt > 65535 || batch > 65535) return MXATTN_EUNSUPPORTED;
     dim3 grid((unsigned)ct, (unsigned)rt, (unsigned)batch);
     if (tile)
-      quantize_axis0_kernel<true><<<grid, kVThreads, 0, stream>>>(
+      e = launch_pdl(quantize_axis0_kernel<true>, grid, kVThreads, 0, stream, 
           (const uint16_t*)in, (uint8_t*)codes, (uint8_t*)scales, rows, cols, rows_pad, rule);
     else
-      quantize_axis0_kernel<false><<<grid, kVThreads, 0, stream>>>(
+      e = launch_pdl(quantize_axis0_kernel<false>, grid, kVThreads, 0, stream, 
           (const uint16_t*)in, (uint8_t*)codes, (uint8_t*)scales, rows, cols, rows_pad, rule);
   }
   count_launch(1);
-  return cudaGetLastError() == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
+  return e == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 
 }  // namespace mxattn

@@ -124,6 +124,10 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
                    const void* k_scales, const void* v_codes, const void* v_scales, void* o,
                    int B, int H, int64_t Nq, int64_t Nkv, float softmax_scale, unsigned flags,
                    int* status, cudaStream_t stream, void* dump = nullptr, bool profile = false);
+int forward_rows_replication(int64_t bh, int64_t Nq, int64_t Nkv);
+int launch_forward_rows(int R, const void* q_codes, const void* q_scales, const void* k_codes, const void* k_scales,
+                        const void* v_codes, const void* v_scales, void* o, int B, int H, int64_t Nq, int64_t Nkv,
+                        float softmax_scale, unsigned flags, int* status, cudaStream_t stream);
 size_t forward_dump_bytes(int B, int H, int64_t Nq, int64_t Nkv);
 size_t forward_profile_bytes(int B, int H, int64_t Nq, int64_t Nkv);
 size_t bf16_workspace_bytes(int B, int H, int64_t Nq, int64_t Nkv);

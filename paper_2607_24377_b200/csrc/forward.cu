@@ -864,6 +864,10 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
   // item per CTA (the hardware's block scheduler then balances the tail better than a static assignment).
   const int n_sm = sm_count();
   if (n_sm == 0) return MXATTN_ECUDA;
+  if (!dump) {
+    const int r = forward_rows_replication((int64_t)B * H, Nq, Nkv);
+    if (r > 0) return launch_forward_rows(r, q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, o, B, H, Nq, Nkv, softmax_scale, flags, status, stream);
+  }
   const bool persist = (!dump || profile) && grid > n_sm && kt <= kPersistMaxTiles;
   // Descriptor of the bf16 output as a [B H][Nq][128] tensor with boxes of 32 rows x 64 columns (the epilogue's copies).
   CUtensorMap out_map;

@@ -150,6 +150,40 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
                ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
+// ---------------------------------------------------------------------------------------------
+// An MMA issuer that runs as a converged warp: all its lanes walk the loop, so that loop counters, addresses and descriptors
+// live in uniform registers, and one elected lane issues each tcgen05 instruction under a predicate.  In code that only
+// one lane executes, every descriptor word is moved from a vector to a uniform register in front of each instruction
+// (about 100 cycles per tcgen05 instruction).
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0); }   // uniform for the compiler too
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+  return r;
+}
+static __device__ __noinline__ bool mbar_wait_warp_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status, int code) {
+  return __all_sync(0xFFFFFFFFu, mbar_wait_loop(bar, parity, abort_flag, status, code, kWaitLimitCycles, nullptr));
+}
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status, int code) {
+  if (__all_sync(0xFFFFFFFFu, mbar_try(bar, parity))) return true;
+  return mbar_wait_warp_slow(bar, parity, abort_flag, status, code);
+}
+__device__ __forceinline__ void tc_cp_sf_if(uint32_t leader, uint32_t taddr, uint32_t saddr) {
+  const uint64_t d = ((uint64_t)((128u >> 4) | (1u << 14)) << 32) | (saddr >> 4);
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t"
+               "@p tcgen05.cp.cta_group::1.32x128b.warpx4 [%0], %1;\n\t}" ::"r"(taddr), "l"(d), "r"(leader) : "memory");
+}
+__device__ __forceinline__ void tc_commit_if(uint32_t leader, uint32_t bar) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %1, 0;\n\t"
+               "@p tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar), "r"(leader) : "memory");
+}
+__device__ __forceinline__ void tc_mma_if(uint32_t leader, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                          uint32_t sfa, uint32_t sfb, uint32_t accumulate) {
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %7, 0;\n\t"
+               "@q tcgen05.mma.cta_group::1.kind::mxf4.block_scale.block32 [%0], %1, %2, %3, [%5], [%6], p;\n\t}"
+               ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(sfa), "r"(sfb), "r"(leader) : "memory");
+}
+
 __device__ __forceinline__ void tc_cp_sf(uint32_t taddr, uint32_t saddr) {   // 512-byte scale atom -> 4 columns
   const uint64_t d = ((uint64_t)((128u >> 4) | (1u << 14)) << 32) | (saddr >> 4);   // no swizzle, 8-row groups 128 B apart
   asm volatile("tcgen05.cp.cta_group::1.32x128b.warpx4 [%0], %1;" ::"r"(taddr), "l"(d) : "memory");
@@ -219,6 +253,60 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// tcgen05.wait::ld that names registers of the loads it waits for, so that no use of them can move ahead of it
+#define TMEM_LD_WAIT32(r)                                                                                              \
+  asm volatile("tcgen05.wait::ld.sync.aligned;"                                                                        \
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),       \
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), \
+                 "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]),            \
+                 "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]),            \
+                 "+r"(r[30]), "+r"(r[31])::"memory")
+__device__ __forceinline__ int lds_volatile(uint32_t addr) {
+  int v;
+  asm volatile("ld.volatile.shared.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+// A wait after which the caller goes on in any case: it gives up on its own limit (about two seconds; the code then goes
+// into the CTA's abort flag, from where it reaches `status` at the end) or when the abort flag is up, and every later wait
+// of the CTA then returns at once.  For warps that meet at named barriers: none of them ever leaves its loop early, so none
+// can be stranded there.
+template <int kCode>
+__device__ __forceinline__ void mbar_wait_soft(uint32_t bar, uint32_t parity, uint32_t abort_addr) {
+  // one block of assembly, so that the usual case is a probe, a vote and a branch, and the rest costs no registers
+  asm volatile("{\n\t.reg .pred p;\n\t.reg .u64 t0, t1;\n\t.reg .u32 a;\n\t"
+               "mbarrier.try_wait.parity.shared::cta.b64 p, [%0], %1, 20000;\n\t"
+               "vote.sync.all.pred p, p, 0xffffffff;\n\t"
+               "@p bra.uni DONE;\n\t"
+               "mov.u64 t0, %%clock64;\n"
+               "AGAIN:\n\t"
+               "ld.volatile.shared.u32 a, [%2];\n\t"
+               "setp.ne.u32 p, a, 0;\n\t"
+               "vote.sync.any.pred p, p, 0xffffffff;\n\t"
+               "@p bra.uni DONE;\n\t"
+               "mbarrier.try_wait.parity.shared::cta.b64 p, [%0], %1, 20000;\n\t"
+               "vote.sync.all.pred p, p, 0xffffffff;\n\t"
+               "@p bra.uni DONE;\n\t"
+               "mov.u64 t1, %%clock64;\n\t"
+               "sub.u64 t1, t1, t0;\n\t"
+               "setp.lt.u64 p, t1, 4000000000;\n\t"
+               "vote.sync.any.pred p, p, 0xffffffff;\n\t"
+               "@p bra.uni AGAIN;\n\t"
+               "st.volatile.shared.u32 [%2], %3;\n"
+               "DONE:\n\t}"
+               ::"r"(bar), "r"(parity), "r"(abort_addr), "n"(kCode) : "memory");
+}
+
+__device__ __forceinline__ void sts8(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared.b8 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+// (a0, a1) * ss, two IEEE fp32 multiplications in one instruction
+__device__ __forceinline__ void mul2(uint32_t& a0, uint32_t& a1, uint64_t ss) {
+  uint64_t ab, r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(ab) : "r"(a0), "r"(a1));
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(ab), "l"(ss));
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(a0), "=r"(a1) : "l"(r));
+}
 
 
 }  // namespace fwd

@@ -1,0 +1,50 @@
+"""The attention kernel for few query rows (32 or 64 rows per CTA, replicated down the operand tile): against the oracle at
+its edges, and bit for bit against the 256-row kernel, which the same heads reach when many copies of them fill the GPU."""
+import numpy as np
+import pytest
+import torch
+
+import synth_inputs as si
+from oracle import attention
+from tests import util
+
+pytestmark = pytest.mark.gpu
+
+
+def run(cfg, q, k, v, flags):
+    import paper_2607_24377_b200 as mx
+    f32 = bool(flags & mx.FLAG_OUT_FP32)
+    out = util.guarded((cfg.B, cfg.H, cfg.Nq, 128), torch.float32 if f32 else torch.bfloat16, float("nan"))
+    ws = util.guarded(mx.forward_workspace_bytes(cfg.B, cfg.H, cfg.Nq, cfg.Nkv, 128), torch.uint8)
+    mx.forward_ws(*(util.to_dev_bf16(x) for x in (q, k, v)), out.t, cfg.B, cfg.H, cfg.Nq, cfg.Nkv, 128, cfg.softmax_scale, flags, ws.t)
+    assert mx.device_status(ws.t) == 0
+    out.check(); ws.check()
+    return out.t.clone()
+
+
+# rows per CTA 32 (few heads) or 64 (the last three); query counts around the row groups, key counts around blocks and tiles
+@pytest.mark.parametrize("H,nq,nkv", [(1, 1, 1), (2, 31, 33), (2, 33, 128), (1, 97, 129), (3, 64, 640), (1, 160, 1100),
+                                      (50, 127, 300), (70, 65, 31), (20, 449, 257)])
+@pytest.mark.parametrize("uos,pnq", [(True, True), (False, False)])
+def test_against_the_oracle(H, nq, nkv, uos, pnq):
+    import paper_2607_24377_b200 as mx
+    cfg = si.custom_config("rw", 1, H, nq, nkv, 17 + nq + nkv)
+    q, k, v = si.make_all(cfg)
+    got = run(cfg, q, k, v, (mx.FLAG_UOS if uos else 0) | (mx.FLAG_PNQ if pnq else 0) | mx.FLAG_OUT_FP32).double().cpu().numpy()
+    want = attention.forward(*(util.bits_to_f64(x) for x in (q, k, v)), cfg.softmax_scale, uos, pnq)
+    assert np.isfinite(got).all()
+    assert np.linalg.norm(got - want) <= 1e-3 * np.linalg.norm(want) and np.abs(got - want).max() <= 4e-3
+
+
+@pytest.mark.parametrize("heads", [2, 40])
+@pytest.mark.parametrize("f32", [False, True])
+def test_bit_identical_to_the_256_row_kernel(heads, f32):
+    import paper_2607_24377_b200 as mx
+    flags = mx.FLAG_UOS | mx.FLAG_PNQ | (mx.FLAG_OUT_FP32 if f32 else 0)
+    one = si.custom_config("rb", 1, heads, 300, 700, 5)
+    q, k, v = si.make_all(one)
+    want = run(one, q, k, v, flags)                                    # 32 (2 heads) or 64 rows (40 heads) per CTA
+    many = si.custom_config("rm", 640 // heads, heads, 300, 700, 5)    # 1280 pairs of query tiles
+    rep = lambda x: np.ascontiguousarray(np.broadcast_to(x, (many.B,) + x.shape[1:]))
+    got = run(many, rep(q), rep(k), rep(v), flags)
+    assert torch.equal(got, want.expand_as(got))

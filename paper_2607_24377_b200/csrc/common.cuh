@@ -2,6 +2,8 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <cuda.h>              // CUtensorMap and the enumerations of its encoder (types only: nothing links libcuda)
+#include <cudaTypedefs.h>
 
 #include "../../include/mxattn.h"
 
@@ -104,6 +106,7 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, unsigned block,
 }
 // Raises a kernel's dynamic shared memory limit, once per kernel and device (a driver call per launch otherwise).
 bool ensure_dynamic_smem(const void* kern, int bytes);
+PFN_cuTensorMapEncodeTiled tensor_map_encoder();      // null if the driver has none
 int sm_count();              // of the current device (0 on error)
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }

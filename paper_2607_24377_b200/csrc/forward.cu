@@ -51,10 +51,9 @@
 // them (template flag kPersist).
 //
 // Every mbarrier wait is bounded; on expiry the CTA records a code in `status`, drains and exits.
-#include <cuda.h>              // CUtensorMap and the enumerations of its encoder (types only: nothing links libcuda)
-#include <cudaTypedefs.h>
-
 #include <string.h>
+
+#include <atomic>
 
 #include <type_traits>
 
@@ -841,6 +840,19 @@ size_t forward_dump_bytes(int B, int H, int64_t Nq, int64_t Nkv) {
   return (size_t)((int64_t)B * H * qt * kt * fwd::kDumpTileBytes + (int64_t)B * H * qt * kTile * 4);
 }
 
+PFN_cuTensorMapEncodeTiled tensor_map_encoder() {
+  static std::atomic<void*> cached{nullptr};
+  void* fn = cached.load(std::memory_order_acquire);
+  if (!fn) {
+    cudaDriverEntryPointQueryResult qres;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) != cudaSuccess ||
+        qres != cudaDriverEntryPointSuccess || !fn)
+      return nullptr;
+    cached.store(fn, std::memory_order_release);
+  }
+  return reinterpret_cast<PFN_cuTensorMapEncodeTiled>(fn);
+}
+
 int launch_forward(const void* q_codes, const void* q_scales, const void* k_codes, const void* k_scales,
                    const void* v_codes, const void* v_scales, void* o, int B, int H, int64_t Nq, int64_t Nkv,
                    float softmax_scale, unsigned flags, int* status, cudaStream_t stream, void* dump, bool profile) {
@@ -873,15 +885,8 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
   CUtensorMap out_map;
   memset(&out_map, 0, sizeof(out_map));
   if (!f32) {
-    static PFN_cuTensorMapEncodeTiled encode = nullptr;
-    if (!encode) {
-      void* fn = nullptr;
-      cudaDriverEntryPointQueryResult qres;
-      if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) != cudaSuccess ||
-          qres != cudaDriverEntryPointSuccess || !fn)
-        return MXATTN_ECUDA;
-      encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled>(fn);
-    }
+    const auto encode = tensor_map_encoder();
+    if (!encode) return MXATTN_ECUDA;
     if (Nq > 0x7FFFFFFFLL || (uint64_t)Nq * kHeadDim * 2 >= (1ULL << 40)) return MXATTN_EUNSUPPORTED;
     const cuuint64_t dims[3] = {(cuuint64_t)kHeadDim, (cuuint64_t)Nq, (cuuint64_t)B * H};
     const cuuint64_t strides[2] = {(cuuint64_t)kHeadDim * 2, (cuuint64_t)Nq * kHeadDim * 2};     // bytes, dimensions 1 and 2

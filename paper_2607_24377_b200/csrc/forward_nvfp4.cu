@@ -53,7 +53,8 @@ enum Bar { BAR_Q = 0, BAR_KFULL = 1, BAR_KEMPTY = BAR_KFULL + kStages, BAR_SFULL
            BAR_PFULL = BAR_SFREE + 1, BAR_ODONE = BAR_PFULL + 2, kNumBars = BAR_ODONE + 2 };
 constexpr int kOffMisc = kOffBar + kNumBars * 8;
 constexpr int kOffMax = kOffMisc + 64;                     // half-row exchange: [parity 2][tile 2][half 2][128] floats
-constexpr int kSmemBytes = kOffMax + 2 * 2 * 2 * 128 * 4 + 1024;
+constexpr int kOffTab = kOffMax + 2 * 2 * 2 * 128 * 4;           // per E4M3 code: log2(2688 / d), d / 2688
+constexpr int kSmemBytes = kOffTab + 128 * 8 + 1024;
 static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
 
 // tensor-memory columns: per operand tile 8 scale columns (atom of K half 0, atom of K half 1); a V slot interleaves
@@ -107,8 +108,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kOffMisc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kOffMisc + 8);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (*reinterpret_cast<volatile int*>(p.status) != 0) return;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int T = p.kv_tiles;
   const int bh = blockIdx.x / p.q_pairs, pair = blockIdx.x - bh * p.q_pairs;
 
@@ -120,7 +120,6 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
     mbar_init(bar(BAR_PFULL + 0), 8); mbar_init(bar(BAR_PFULL + 1), 8);
     mbar_init(bar(BAR_ODONE + 0), 1); mbar_init(bar(BAR_ODONE + 1), 1);
     abort_flag[0] = 0;
-    abort_flag[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   // rows of ones appended to every V stage (E2M1 code 2 = 1.0) and their scale atom (E4M3 1.0 = 0x38)
@@ -131,17 +130,27 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
   }
   for (int i = tid; i < kTileScaleBytes / 16; i += kThreads)
     reinterpret_cast<uint4*>(smem + kOffSFOnes)[i] = make_uint4(0x38383838u, 0x38383838u, 0x38383838u, 0x38383838u);
+  // what a softmax thread needs of a block's scale code (E4M3, never negative): the logarithm of the element multiplier, and
+  // for the direct placement its inverse.  d = 0 keeps multiplier 1 (see below).
+  if (tid < 128) {
+    const float d = e4m3_decode((uint32_t)tid);
+    reinterpret_cast<float2*>(smem + kOffTab)[tid] = (tid == 0 || tid == 127) ? make_float2(0.0f, 1.0f) : make_float2(log2f(2688.0f / d), d * kInvTensorRangeP);
+  }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   if (warp == kSoftmaxWarps + 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  pdl_wait();                                        // the operands and the status word are ready
+  if (tid == 0) abort_flag[1] = *reinterpret_cast<volatile int*>(p.status);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_trigger();
   const uint32_t tmem = *tmem_slot;
+  const int role = abort_flag[1] != 0 ? kSoftmaxWarps + 2 : warp;     // an earlier CTA gave up: drain the grid quickly
 
-  if (warp == kSoftmaxWarps) {
+  if (role == kSoftmaxWarps) {
     // =============================== producer ===============================================
     if (lane == 0) {
       const int64_t qt0 = (int64_t)bh * p.q_tiles + 2 * pair;
@@ -171,7 +180,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
         while (!mbar_try(bar(BAR_Q), 0u) && clock64() - t0 < 200000000LL) {}
       }
     }
-  } else if (warp == kSoftmaxWarps + 1) {
+  } else if (role == kSoftmaxWarps + 1) {
     // =============================== MMA issuer =============================================
     if (lane == 0) {
       bool ok = mbar_wait(bar(BAR_Q), 0, abort_flag, p.status, 21);
@@ -261,7 +270,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
         }
       }
     }
-  } else {
+  } else if (role < kSoftmaxWarps) {
     // =============================== softmax groups =========================================
     const int t = warp >> 3;
     const int h = (warp >> 2) & 1;
@@ -277,6 +286,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
     const uint32_t aSF = sbase + kOffSFP + t * kSF + h * kTileScaleBytes + tile_scale_offset(row, 0);   // atom h: this thread's 4 blocks
     const uint32_t aMaxOwn = sbase + kOffMax + (t * 256 + h * 128 + row) * 4;
     const uint32_t aMaxPartner = sbase + kOffMax + (t * 256 + (h ^ 1) * 128 + row) * 4;
+    const uint32_t aTab = sbase + kOffTab;
     const int pair_bar = 1 + (warp & 3) + 4 * t;
     volatile int* const own_limit_only = abort_flag + 1;
     bool ok = true;
@@ -329,31 +339,28 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
       tc_fence_after();
       const bool rescale = __any_sync(0xFFFFFFFFu, moved);
       float alpha = 1.0f;
-      // block scales: the block's largest probability by the elements' own expression, then the two-level recipe.
-      // The element multiplier 2688 / d_b is folded into the exponent as its logarithm (one lg2.approx per block in
-      // place of a division per block and a multiply per element; relative difference about 2e-7, the order of
-      // ex2.approx itself).  A block whose scale rounds to zero keeps multiplier 1: its probabilities are below
-      // 2.2e-6 and round to code 0 either way, and the direct placement still sums them.
+      // Block scales: the block's largest probability by the elements' own expression, then the two-level recipe, two blocks
+      // per conversion.  The element multiplier 2688 / d_b is folded into the exponent as its logarithm, which (like
+      // d_b / 2688) comes from a table of the 127 codes, correctly rounded: relative difference about 2e-7, the order of
+      // ex2.approx itself.  (Computed per block -- decode, lg2.approx on the mantissa, two additions and the selections for
+      // subnormal and zero codes -- it was 22 instructions per block instead of 8.)  A block whose scale rounds to zero
+      // keeps multiplier 1: its probabilities are below 2.2e-6 and round to code 0 either way, and the direct placement
+      // still sums them.
       float nb[4], inv_r[4];
       uint32_t sf4 = 0;
 #pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const float pm = ex2(fmaf(bmax[b], c, nmc));
-        const float y = __fmul_rn(__fmul_rn(pm, kTensorRangeP), kOneSixth);
-        const uint32_t code = e4m3_encode(y);
-        const float d = e4m3_decode(code);
-        // log2(2688 / d) from the code's fields: d = (1 + k/8) 2^(E-7), so only the mantissa's logarithm is approximated,
-        // on an argument in [1, 2) where lg2.approx is good to 2^-22 absolute (on d itself its error is relative to
-        // log2 d, about 2e-6 for the blocks that matter, which moves codes across rounding boundaries); the integer part
-        // and log2(2688) = 11 + 0.39231742 are added exactly enough that the sum rounds once at its own magnitude
-        const uint32_t fe = code >> 3, fk = code & 7u;
-        float lgm;
-        asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lgm) : "f"(fe ? __uint_as_float(0x3F800000u | (fk << 20)) : d * 512.0f));
-        const float fef = __uint_as_float(0x4B400000u + fe) - 12582912.0f;           // (float)E without a conversion instruction
-        const float lr = (fe ? 18.0f - fef : 20.0f) + (0.39231742f - lgm);           // subnormal d = k 2^-9
-        nb[b] = d == 0.0f ? nmc : fmaf(-m_new, c, lr);     // one rounding: -(m_new c) + log2(2688 / d)
-        inv_r[b] = d == 0.0f ? 1.0f : d * kInvTensorRangeP;
-        sf4 |= code << (8 * b);
+      for (int b = 0; b < 4; b += 2) {
+        const float y0 = __fmul_rn(__fmul_rn(ex2(fmaf(bmax[b], c, nmc)), kTensorRangeP), kOneSixth);
+        const float y1 = __fmul_rn(__fmul_rn(ex2(fmaf(bmax[b + 1], c, nmc)), kTensorRangeP), kOneSixth);
+        uint16_t code2;
+        asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(code2) : "f"(y1), "f"(y0));
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          float lr;
+          asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(lr), "=f"(inv_r[b + u]) : "r"(aTab + ((u ? (uint32_t)code2 >> 8 : (uint32_t)code2 & 0xFFu) << 3)));
+          nb[b + u] = fmaf(-m_new, c, lr);         // one rounding: -(m_new c) + log2(2688 / d)
+        }
+        sf4 |= (uint32_t)code2 << (8 * b);
       }
       asm volatile("st.shared.b32 [%0], %1;" ::"r"(aSF), "r"(sf4) : "memory");
       float l_tile = 0.0f;
@@ -361,6 +368,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
       auto tile_body = [&](auto resc_tag) {
         constexpr bool kResc = decltype(resc_tag)::value;
         if (kResc) alpha = ex2((m_old - m_new) * c);
+        const uint64_t al2 = dup2(alpha);
 #pragma unroll
         for (int b32 = 0; b32 < 2; ++b32) {           // one 16-byte chunk of codes = 32 elements = two blocks
           uint4 w;
@@ -387,7 +395,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
             if (kResc) {
               tmem_ld_wait();
 #pragma unroll
-              for (int i = 0; i < 8; ++i) oc[i] = __float_as_uint(__uint_as_float(oc[i]) * alpha);
+              for (int i = 0; i < 8; i += 2) mul2(oc[i], oc[i + 1], al2);
               TMEM_ST8(t_oc, oc);
             }
           }
@@ -518,15 +526,10 @@ int launch_forward_nvfp4(const void* q, const void* k, const void* v, void* o, i
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   float* amax = reinterpret_cast<float*>(ws + w.amax);
   float* ts = reinterpret_cast<float*>(ws + w.tscale);
-  if (cudaMemsetAsync(ws + w.status, 0, 16, stream) != cudaSuccess) return MXATTN_ECUDA;
-  int rc;
-  // one tensor-level scale per head matrix (Q, K, V each), then the block quantizers
-  if ((rc = launch_tensor_amax(q, amax, bh, Nq, kHeadDim, stream))) return rc;
-  if ((rc = launch_tensor_amax(k, amax + bh, bh, Nkv, kHeadDim, stream))) return rc;
-  if ((rc = launch_tensor_amax(v, amax + 2 * bh, bh, Nkv, kHeadDim, stream))) return rc;
-  if ((rc = launch_quantize_nvfp4(q, ws + w.q_codes, ws + w.q_scales, amax, ts, bh, Nq, kHeadDim, 1, MXATTN_LAYOUT_TILE, stream))) return rc;
-  if ((rc = launch_quantize_nvfp4(k, ws + w.k_codes, ws + w.k_scales, amax + bh, ts + bh, bh, Nkv, kHeadDim, 1, MXATTN_LAYOUT_TILE, stream))) return rc;
-  if ((rc = launch_quantize_nvfp4(v, ws + w.v_codes, ws + w.v_scales, amax + 2 * bh, ts + 2 * bh, bh, Nkv, kHeadDim, 0, MXATTN_LAYOUT_TILE, stream))) return rc;
+  if (cudaMemsetAsync(ws + w.status, 0, w.tscale - w.status, stream) != cudaSuccess) return MXATTN_ECUDA;      // status word and tensor maxima
+  const int rc = launch_nvfp4_operands(q, ws + w.q_codes, ws + w.q_scales, k, ws + w.k_codes, ws + w.k_scales, v, ws + w.v_codes, ws + w.v_scales,
+                                       amax, ts, bh, Nq, Nkv, stream);
+  if (rc != MXATTN_OK) return rc;
   Params p;
   p.q_codes = ws + w.q_codes; p.q_scales = ws + w.q_scales; p.k_codes = ws + w.k_codes; p.k_scales = ws + w.k_scales;
   p.v_codes = ws + w.v_codes; p.v_scales = ws + w.v_scales;
@@ -537,10 +540,9 @@ int launch_forward_nvfp4(const void* q, const void* k, const void* v, void* o, i
   const bool pnq = flags & MXATTN_FLAG_PNQ, f32 = flags & MXATTN_FLAG_OUT_FP32;
   void (*kern)(const Params) = pnq ? (f32 ? attention_nvfp4_kernel<true, true> : attention_nvfp4_kernel<true, false>)
                                    : (f32 ? attention_nvfp4_kernel<false, true> : attention_nvfp4_kernel<false, false>);
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess) return MXATTN_ECUDA;
-  kern<<<(unsigned)grid, kThreads, kSmemBytes, stream>>>(p);
+  if (!ensure_dynamic_smem((const void*)kern, kSmemBytes)) return MXATTN_ECUDA;
   count_launch(1);
-  return cudaGetLastError() == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
+  return launch_pdl(kern, dim3((unsigned)grid), kThreads, kSmemBytes, stream, p) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 
 }  // namespace mxattn

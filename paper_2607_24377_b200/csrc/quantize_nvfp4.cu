@@ -55,23 +55,41 @@ __device__ __forceinline__ uint32_t quantize_bf16x8(const uint4& v, float r) {
 }
 
 // ------------------------------------------------------------------------------------------
-// Largest magnitude of each matrix of the batch: amax[b] (fp32; must be zero on entry).  grid = (chunks, batch).
-__global__ void __launch_bounds__(kThreads) tensor_amax_kernel(const uint4* __restrict__ in, uint32_t* __restrict__ amax,
-                                                               int64_t chunks_per_matrix) {
-  const uint4* src = in + (int64_t)blockIdx.y * chunks_per_matrix;
+// Largest magnitude of each matrix of the batch: amax[b] (fp32; must be zero on entry).  grid = (chunks, batch); a forward
+// call takes the matrices of Q, K and V in one grid of three operands.  Eight loads of 16 bytes are in flight per thread.
+constexpr int kAmaxUnroll = 8;
+struct AmaxOperand { const uint4* in; uint32_t* amax; int64_t chunks; };       // chunks of 16 bytes per matrix
+__device__ __forceinline__ void tensor_amax_part(const AmaxOperand& o, int64_t b, int part, int parts) {
+  const uint4* src = o.in + b * o.chunks;
   uint32_t m = 0;
-  for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < chunks_per_matrix; i += (int64_t)gridDim.x * kThreads)
-    m = max(m, absmax_bf16x8(__ldg(src + i)));
+  const int64_t step = (int64_t)parts * kThreads;
+  int64_t i = (int64_t)part * kThreads + threadIdx.x;
+  for (; i + (kAmaxUnroll - 1) * step < o.chunks; i += kAmaxUnroll * step) {
+    uint4 v[kAmaxUnroll];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+    for (int u = 0; u < kAmaxUnroll; ++u) v[u] = __ldg(src + i + u * step);
+#pragma unroll
+    for (int u = 0; u < kAmaxUnroll; ++u) m = max(m, absmax_bf16x8(v[u]));
+  }
+  for (; i < o.chunks; i += step) m = max(m, absmax_bf16x8(__ldg(src + i)));
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, s));
   __shared__ uint32_t s[kThreads / 32];
   if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = m;
   __syncthreads();
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int w = 1; w < kThreads / 32; ++w) m = max(m, s[w]);
-    atomicMax(amax + blockIdx.y, m << 16);          // non-negative floats order like their bit patterns
+    atomicMax(o.amax + b, m << 16);                 // non-negative floats order like their bit patterns
   }
+}
+__global__ void __launch_bounds__(kThreads) tensor_amax_kernel(const AmaxOperand o) {
+  pdl_wait(); pdl_trigger();
+  tensor_amax_part(o, blockIdx.y, blockIdx.x, gridDim.x);
+}
+__global__ void __launch_bounds__(kThreads) tensor_amax_qkv_kernel(const AmaxOperand q, const AmaxOperand k, const AmaxOperand v) {
+  pdl_wait(); pdl_trigger();
+  tensor_amax_part(blockIdx.z == 0 ? q : blockIdx.z == 1 ? k : v, blockIdx.y, blockIdx.x, gridDim.x);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -83,18 +101,15 @@ __global__ void __launch_bounds__(kThreads) tensor_amax_kernel(const uint4* __re
 // (cols == 128): chunks = rows_pad * 16, rows beyond `rows` read as zero.
 constexpr int kA1ChunksPerCta = kThreads * 4;
 template <bool kTileLayout>
-__global__ void __launch_bounds__(kThreads)
-quantize_nvfp4_axis1_kernel(const uint4* __restrict__ in, uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
-                            const float* __restrict__ amax, float* __restrict__ tensor_scale, int64_t rows, int64_t cols,
-                            int64_t rows_pad) {
-  __shared__ uint4 s_v[kA1ChunksPerCta];
+__device__ __forceinline__ void quantize_nvfp4_axis1_part(uint4* s_v, const uint4* __restrict__ in, uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
+                                                          const float* __restrict__ amax, float* __restrict__ tensor_scale, int64_t rows, int64_t cols,
+                                                          int64_t rows_pad, int64_t part, int64_t b) {
   const int tid = threadIdx.x;
-  const int64_t b = blockIdx.y;
   const int64_t chunks_per_row = cols / 8;
   const int64_t n_valid = rows * chunks_per_row;                                  // chunks that exist in the input
   const int64_t n_out = (kTileLayout ? rows_pad : rows) * chunks_per_row;         // chunks that are written
   const uint4* src = in + b * n_valid;
-  const int64_t base = (int64_t)blockIdx.x * kA1ChunksPerCta;
+  const int64_t base = part * kA1ChunksPerCta;
   auto pos = [](int c) { return c ^ ((c >> 3) & 7); };
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
@@ -104,7 +119,7 @@ quantize_nvfp4_axis1_kernel(const uint4* __restrict__ in, uint8_t* __restrict__ 
                  "l"(inside ? src + base + c : in), "r"(inside ? 16 : 0) : "memory");
   }
   const float g = encode_scale(amax[b]);
-  if (blockIdx.x == 0 && tid == 0 && tensor_scale) tensor_scale[b] = __fdiv_rn(1.0f, g);
+  if (part == 0 && tid == 0 && tensor_scale) tensor_scale[b] = __fdiv_rn(1.0f, g);
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   const int64_t i = base + 4 * tid;                 // first of this thread's four chunks (n_out is even: whole blocks only)
@@ -148,22 +163,36 @@ quantize_nvfp4_axis1_kernel(const uint4* __restrict__ in, uint8_t* __restrict__ 
   }
 }
 
+template <bool kTileLayout>
+__global__ void __launch_bounds__(kThreads)
+quantize_nvfp4_axis1_kernel(const uint4* __restrict__ in, uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
+                            const float* __restrict__ amax, float* __restrict__ tensor_scale, int64_t rows, int64_t cols,
+                            int64_t rows_pad) {
+  __shared__ uint4 s_v[kA1ChunksPerCta];
+  pdl_wait(); pdl_trigger();
+  quantize_nvfp4_axis1_part<kTileLayout>(s_v, in, codes, scales, amax, tensor_scale, rows, cols, rows_pad, blockIdx.x, blockIdx.y);
+}
+
 // ------------------------------------------------------------------------------------------
 // Axis 0 (V: blocks of 16 along the rows = tokens), outputs transposed (column-major, token-contiguous).
 // A CTA stages a 128-token x 128-column slab; thread -> (column pair, chunk of 32 tokens = two blocks).
 // grid = (ceil(cols / 128), rows_pad / 128, batch).
+struct __align__(16) Axis0Smem {
+  uint16_t in[kTile][kTile];
+  uint8_t codes[kTileCodeBytes];
+  uint8_t scales[kNvTileScaleBytes];
+};
 template <bool kTileLayout>
-__global__ void __launch_bounds__(kThreads)
-quantize_nvfp4_axis0_kernel(const uint16_t* __restrict__ in, uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
-                            const float* __restrict__ amax, float* __restrict__ tensor_scale, int64_t rows, int64_t cols,
-                            int64_t rows_pad) {
-  __shared__ __align__(16) uint16_t s_in[kTile][kTile];
-  __shared__ __align__(16) uint8_t s_codes[kTileCodeBytes];
-  __shared__ __align__(16) uint8_t s_scales[kNvTileScaleBytes];
+__device__ __forceinline__ void quantize_nvfp4_axis0_slab(Axis0Smem& sm, const uint16_t* __restrict__ in, uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
+                                                          const float* __restrict__ amax, float* __restrict__ tensor_scale, int64_t rows, int64_t cols,
+                                                          int64_t rows_pad, int64_t cx, int64_t ry, int64_t b) {
+  uint16_t(*s_in)[kTile] = sm.in;
+  uint8_t* s_codes = sm.codes;
+  uint8_t* s_scales = sm.scales;
   const int tid = threadIdx.x;
-  const int64_t col0 = (int64_t)blockIdx.x * kTile, row0 = (int64_t)blockIdx.y * kTile, b = blockIdx.z;
+  const int64_t col0 = cx * kTile, row0 = ry * kTile;
   const float g = encode_scale(amax[b]);
-  if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0 && tensor_scale) tensor_scale[b] = __fdiv_rn(1.0f, g);
+  if (cx == 0 && ry == 0 && tid == 0 && tensor_scale) tensor_scale[b] = __fdiv_rn(1.0f, g);
   const uint16_t* src = in + b * rows * cols;
 #pragma unroll
   for (int k = 0; k < (kTile * kTile / 8) / kThreads; ++k) {
@@ -212,7 +241,7 @@ quantize_nvfp4_axis0_kernel(const uint16_t* __restrict__ in, uint8_t* __restrict
   }
   __syncthreads();
   if (kTileLayout) {
-    const int64_t tile = b * gridDim.y + blockIdx.y;
+    const int64_t tile = b * (rows_pad / kTile) + ry;
     uint4* dst = reinterpret_cast<uint4*>(codes + tile * kTileCodeBytes);
 #pragma unroll
     for (int k = 0; k < kTileCodeBytes / 16 / kThreads; ++k)
@@ -235,7 +264,66 @@ quantize_nvfp4_axis0_kernel(const uint16_t* __restrict__ in, uint8_t* __restrict
   }
 }
 
+template <bool kTileLayout>
+__global__ void __launch_bounds__(kThreads)
+quantize_nvfp4_axis0_kernel(const uint16_t* __restrict__ in, uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
+                            const float* __restrict__ amax, float* __restrict__ tensor_scale, int64_t rows, int64_t cols,
+                            int64_t rows_pad) {
+  __shared__ Axis0Smem sm;
+  pdl_wait(); pdl_trigger();
+  quantize_nvfp4_axis0_slab<kTileLayout>(sm, in, codes, scales, amax, tensor_scale, rows, cols, rows_pad, blockIdx.x, blockIdx.y, blockIdx.z);
+}
+
+// Q, K (axis 1) and V (axis 0) of a forward call in one launch (tile layout), as in quantize.cu; amax and tensor_scale are
+// indexed by operand and head.
+struct QkvOperand { const void* in; uint8_t* codes; uint8_t* scales; const float* amax; float* tensor_scale; int64_t rows, tiles, ctas; };
+__global__ void __launch_bounds__(kThreads) quantize_nvfp4_qkv_kernel(const QkvOperand q, const QkvOperand k, const QkvOperand v) {
+  __shared__ Axis0Smem sm;
+  pdl_wait(); pdl_trigger();
+  int64_t i = blockIdx.x;
+  if (i < q.ctas + k.ctas) {                       // half a tile per CTA
+    const QkvOperand& o = i < q.ctas ? q : k;
+    if (i >= q.ctas) i -= q.ctas;
+    const int64_t b = i / (2 * o.tiles);
+    quantize_nvfp4_axis1_part<true>(reinterpret_cast<uint4*>(sm.in), (const uint4*)o.in, o.codes, o.scales, o.amax, o.tensor_scale, o.rows, kHeadDim,
+                                    o.tiles * kTile, i - b * 2 * o.tiles, b);
+  } else if (i < q.ctas + k.ctas + v.ctas) {
+    i -= q.ctas + k.ctas;
+    const int64_t b = i / v.tiles;
+    quantize_nvfp4_axis0_slab<true>(sm, (const uint16_t*)v.in, v.codes, v.scales, v.amax, v.tensor_scale, v.rows, kHeadDim, v.tiles * kTile, 0, i - b * v.tiles, b);
+  }
+}
+
 }  // namespace nv
+
+int launch_nvfp4_operands(const void* q, void* q_codes, void* q_scales, const void* k, void* k_codes, void* k_scales,
+                          const void* v, void* v_codes, void* v_scales, float* amax, float* tensor_scale, int64_t bh,
+                          int64_t Nq, int64_t Nkv, cudaStream_t stream) {
+  using namespace nv;
+  const int64_t qt = (Nq + kTile - 1) / kTile, kt = (Nkv + kTile - 1) / kTile;
+  if (bh > 65535 || bh * (2 * qt + 3 * kt) > 0x7FFFFFFF) return MXATTN_EUNSUPPORTED;
+  const int n_sm = sm_count();
+  if (n_sm == 0) return MXATTN_ECUDA;
+  // one tensor-level scale per head matrix (Q, K, V each), then the block quantizers
+  const int64_t cq = Nq * kHeadDim / 8, ck = Nkv * kHeadDim / 8;
+  int64_t parts = ((cq > ck ? cq : ck) + kThreads * kAmaxUnroll - 1) / (kThreads * kAmaxUnroll);
+  const int64_t most = (8 * n_sm + 3 * bh - 1) / (3 * bh) > 1 ? (8 * n_sm + 3 * bh - 1) / (3 * bh) : 1;    // about one wave of CTAs
+  if (parts > most) parts = most;
+  if (launch_pdl(tensor_amax_qkv_kernel, dim3((unsigned)parts, (unsigned)bh, 3), kThreads, 0, stream, AmaxOperand{(const uint4*)q, (uint32_t*)amax, cq},
+                 AmaxOperand{(const uint4*)k, (uint32_t*)amax + bh, ck}, AmaxOperand{(const uint4*)v, (uint32_t*)amax + 2 * bh, ck}) != cudaSuccess) return MXATTN_ECUDA;
+  QkvOperand oq{q, (uint8_t*)q_codes, (uint8_t*)q_scales, amax, tensor_scale, Nq, qt, 2 * bh * qt};
+  QkvOperand ok{k, (uint8_t*)k_codes, (uint8_t*)k_scales, amax + bh, tensor_scale + bh, Nkv, kt, 2 * bh * kt};
+  QkvOperand ov{v, (uint8_t*)v_codes, (uint8_t*)v_scales, amax + 2 * bh, tensor_scale + 2 * bh, Nkv, kt, bh * kt};
+  if (oq.ctas + ok.ctas > 24 * (int64_t)n_sm) {    // long problems: a kernel of their own for Q and K (quantize.cu has the reason)
+    for (const QkvOperand* o : {&oq, &ok})
+      if (launch_pdl(quantize_nvfp4_axis1_kernel<true>, dim3((unsigned)(2 * o->tiles), (unsigned)bh), kThreads, 0, stream, (const uint4*)o->in, o->codes, o->scales,
+                     o->amax, o->tensor_scale, o->rows, (int64_t)kHeadDim, o->tiles * kTile) != cudaSuccess) return MXATTN_ECUDA;
+    oq.ctas = ok.ctas = 0;
+  }
+  if (launch_pdl(quantize_nvfp4_qkv_kernel, dim3((unsigned)(oq.ctas + ok.ctas + ov.ctas)), kThreads, 0, stream, oq, ok, ov) != cudaSuccess) return MXATTN_ECUDA;
+  count_launch(6);
+  return MXATTN_OK;
+}
 
 int launch_tensor_amax(const void* in, float* amax, int64_t batch, int64_t rows, int64_t cols, cudaStream_t stream) {
   if (!in || !amax) return MXATTN_EINVAL;
@@ -247,10 +335,9 @@ int launch_tensor_amax(const void* in, float* amax, int64_t batch, int64_t rows,
   int64_t blocks = (chunks + nv::kThreads * 8 - 1) / (nv::kThreads * 8);
   if (blocks > 1184) blocks = 1184;                 // 8 CTAs per SM at most: the loop strides over the rest
   if (cudaMemsetAsync(amax, 0, (size_t)batch * sizeof(float), stream) != cudaSuccess) return MXATTN_ECUDA;
-  nv::tensor_amax_kernel<<<dim3((unsigned)blocks, (unsigned)batch), nv::kThreads, 0, stream>>>(
-      (const uint4*)in, reinterpret_cast<uint32_t*>(amax), chunks);
   count_launch(1);
-  return cudaGetLastError() == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
+  return launch_pdl(nv::tensor_amax_kernel, dim3((unsigned)blocks, (unsigned)batch), nv::kThreads, 0, stream,
+                    nv::AmaxOperand{(const uint4*)in, reinterpret_cast<uint32_t*>(amax), chunks}) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 
 int launch_quantize_nvfp4(const void* in, void* codes, void* scales, const float* amax, float* tensor_scale, int64_t batch,
@@ -267,30 +354,31 @@ int launch_quantize_nvfp4(const void* in, void* codes, void* scales, const float
   if (batch > 65535) return MXATTN_EUNSUPPORTED;
   const int64_t rows_pad = (rows + kTile - 1) / kTile * kTile;
   const bool tile = (layout == MXATTN_LAYOUT_TILE);
+  cudaError_t e = cudaSuccess;
   if (block_axis == 1) {
     const int64_t n_out = (tile ? rows_pad : rows) * (cols / 8);
     const int64_t blocks = (n_out + nv::kA1ChunksPerCta - 1) / nv::kA1ChunksPerCta;
     if (blocks > 0x7FFFFFFF) return MXATTN_EUNSUPPORTED;
     dim3 grid((unsigned)blocks, (unsigned)batch);
     if (tile)
-      nv::quantize_nvfp4_axis1_kernel<true><<<grid, nv::kThreads, 0, stream>>>((const uint4*)in, (uint8_t*)codes, (uint8_t*)scales,
+      e = launch_pdl(nv::quantize_nvfp4_axis1_kernel<true>, grid, nv::kThreads, 0, stream, (const uint4*)in, (uint8_t*)codes, (uint8_t*)scales,
                                                                                amax, tensor_scale, rows, cols, rows_pad);
     else
-      nv::quantize_nvfp4_axis1_kernel<false><<<grid, nv::kThreads, 0, stream>>>((const uint4*)in, (uint8_t*)codes, (uint8_t*)scales,
+      e = launch_pdl(nv::quantize_nvfp4_axis1_kernel<false>, grid, nv::kThreads, 0, stream, (const uint4*)in, (uint8_t*)codes, (uint8_t*)scales,
                                                                                 amax, tensor_scale, rows, cols, rows_pad);
   } else {
     const int64_t ct = (cols + kTile - 1) / kTile, rt = rows_pad / kTile;
     if (ct > 0x7FFFFFFF || rt > 65535) return MXATTN_EUNSUPPORTED;
     dim3 grid((unsigned)ct, (unsigned)rt, (unsigned)batch);
     if (tile)
-      nv::quantize_nvfp4_axis0_kernel<true><<<grid, nv::kThreads, 0, stream>>>((const uint16_t*)in, (uint8_t*)codes, (uint8_t*)scales,
+      e = launch_pdl(nv::quantize_nvfp4_axis0_kernel<true>, grid, nv::kThreads, 0, stream, (const uint16_t*)in, (uint8_t*)codes, (uint8_t*)scales,
                                                                                amax, tensor_scale, rows, cols, rows_pad);
     else
-      nv::quantize_nvfp4_axis0_kernel<false><<<grid, nv::kThreads, 0, stream>>>((const uint16_t*)in, (uint8_t*)codes, (uint8_t*)scales,
+      e = launch_pdl(nv::quantize_nvfp4_axis0_kernel<false>, grid, nv::kThreads, 0, stream, (const uint16_t*)in, (uint8_t*)codes, (uint8_t*)scales,
                                                                                 amax, tensor_scale, rows, cols, rows_pad);
   }
   count_launch(1);
-  return cudaGetLastError() == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
+  return e == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 
 }  // namespace mxattn

@@ -87,10 +87,6 @@ constexpr int kOffBar = kOffSFP + 2 * kTileScaleBytes;     // barriers
 constexpr int kNumBars = 4 + 2 * kStages + 2 + 1 + 2 + 2;  // Q full/empty[2], K/V stage full+empty, S_full[2], S_free, P_full[2], O_done[2]
 constexpr int kOffMisc = kOffBar + kNumBars * 8;           // tmem slot, abort flag
 constexpr int kOffMax = kOffMisc + 64;                     // half-row maxima: [parity 2][tile 2][half 2][128] floats
-#ifndef MXATTN_PERSIST_MAX_T
-#define MXATTN_PERSIST_MAX_T 48
-#endif
-constexpr int kPersistMaxTiles = MXATTN_PERSIST_MAX_T;    // longest key/value sequence (in tiles) run by the persistent variant
 constexpr int kOffOut = (kOffMax + 2 * 2 * 2 * 128 * 4 + 1023) & ~1023;   // bf16 output staging: one box per softmax warp
 constexpr int kOutBoxBytes = 32 * kCols * 2;               // 32 rows x 64 bf16 (128 bytes, the span of the 128-byte swizzle)
 constexpr int kSmemBytes = kOffOut + kSoftmaxWarps * kOutBoxBytes + 1024;   // + slack for the 1024 alignment
@@ -557,10 +553,8 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
 #pragma unroll
       for (int b = 0; b < kBlocksPerThread; ++b) {
         const float d = (bmax[b] - m_new) * c;
-        const float rn = (d + 12582912.0f) - 12582912.0f;              // round to nearest integer
-        const float fl = rn > d ? rn - 1.0f : rn;                       // floor(d)
-        float ef = fl - 2.0f;
-        if (kUos && (d - fl) > 0.85798097f) ef += 1.0f;
+        const float fl = __fadd_rd(d, 12582912.0f) - 12582912.0f;       // floor(d)
+        float ef = fl + ((kUos && (d - fl) > 0.85798097f) ? -1.0f : -2.0f);
         ef = fmaxf(ef, -127.0f);
         if (d < -126.0f) ef = 0.0f;
         const int e = __float_as_int(ef + 12582912.0f) - 0x4B400000;    // exact small-integer conversion
@@ -876,11 +870,18 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
   // item per CTA (the hardware's block scheduler then balances the tail better than a static assignment).
   const int n_sm = sm_count();
   if (n_sm == 0) return MXATTN_ECUDA;
-  if (!dump) {
-    const int r = forward_rows_replication((int64_t)B * H, Nq, Nkv);
-    if (r > 0) return launch_forward_rows(r, q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, o, B, H, Nq, Nkv, softmax_scale, flags, status, stream);
-  }
-  const bool persist = (!dump || profile) && grid > n_sm && kt <= kPersistMaxTiles;
+  // query tiles that would leave SMs idle (a problem smaller than the GPU, or a last wave that is nearly empty) go to the
+  // kernel for few query rows
+  const RowSplit split = dump ? RowSplit{grid, 0} : forward_row_split((int64_t)B * H, Nq, Nkv, pnq);
+  count_launch(1);
+  auto rest = [&]() {
+    return split.R == 0 ? (int)MXATTN_OK
+                        : launch_forward_rows(split.R, split.pairs_256, q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, o, B, H, Nq, Nkv,
+                                              softmax_scale, flags, status, stream);
+  };
+  if (split.pairs_256 == 0) return rest();
+  p.total_items = (int)split.pairs_256;
+  const bool persist = (!dump || profile) && split.pairs_256 > n_sm && kt <= kWalkMaxTiles;
   // Descriptor of the bf16 output as a [B H][Nq][128] tensor with boxes of 32 rows x 64 columns (the epilogue's copies).
   CUtensorMap out_map;
   memset(&out_map, 0, sizeof(out_map));
@@ -913,8 +914,8 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
 #undef PICKD
   }
   if (!ensure_dynamic_smem((const void*)kern, kSmemBytes)) return MXATTN_ECUDA;
-  count_launch(1);
-  return launch_pdl(kern, dim3((unsigned)(persist ? n_sm : grid)), kThreads, kSmemBytes, stream, p, out_map) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
+  if (launch_pdl(kern, dim3((unsigned)(persist ? n_sm : split.pairs_256)), kThreads, kSmemBytes, stream, p, out_map) != cudaSuccess) return MXATTN_ECUDA;
+  return rest();
 }
 
 }  // namespace mxattn

@@ -1,5 +1,5 @@
 // MXFP4 attention forward for few query rows (paper Algorithm 2, lines 6-19): the kernel that forward.cu hands a problem
-// to when its query tiles cannot fill the GPU.
+// to when its query tiles cannot fill the GPU, or could not fill its last wave.
 //
 // KV tiles must be visited one after the other (P-hat depends on the history of the running maximum), so what counts for a
 // short problem is the latency of one tile, and the only way to use idle SMs is to give each CTA fewer query rows.  A CTA of
@@ -16,8 +16,8 @@
 // of block kb: one thread per row and block.  The four warps of a row group exchange their block maxima through shared
 // memory at a named barrier once per tile.  S is double-buffered, so the next tile's scores are ready when a warp gets
 // there (loading them before the hand-over instead makes the hand-over's fence wait for the load: 5 % slower).  Measured
-// (B200, 1965 MHz, row maxima moving in most tiles): 1120 cycles per tile with R = 4, 1430 with R = 2; 2 heads of
-// 1024 x 1024: attention launch 14 -> 6 us.
+// (B200, 1965 MHz): 1200 cycles per tile with R = 4, 1530 with R = 2, 2125 with R = 1 (one query tile of 128 rows, 16 warps);
+// 2 heads of 1024 x 1024: attention launch 14 -> 6 us.
 #include <string.h>
 
 #include "common.cuh"
@@ -40,13 +40,18 @@ constexpr int kOffSFK = kOffSFQ + kTileScaleBytes;
 constexpr int kOffSFV = kOffSFK + kStages * kTileScaleBytes;
 constexpr int kOffSFP = kOffSFV + kStages * kTileScaleBytes;     // 2 buffers
 constexpr int kOffSFOnes = kOffSFP + 2 * kTileScaleBytes;
-constexpr int kOffX = kOffSFOnes + kTileScaleBytes;              // block maxima: [2 buffers][row group 2][block 4][32] floats
-constexpr int kOffXL = kOffX + 2 * 2 * 4 * 32 * 4;               // row sums of a tile by block (direct placement), laid out alike
-constexpr int kOffBar = kOffXL + 2 * 2 * 4 * 32 * 4;
+constexpr int kOffX = kOffSFOnes + kTileScaleBytes;              // block maxima: [2 buffers][row group 4][block 4][32] floats
+constexpr int kXBuf = 4 * 4 * 32 * 4;
+constexpr int kOffXL = kOffX + 2 * kXBuf;               // row sums of a tile by block (direct placement), laid out alike
+constexpr int kOffBar = kOffXL + 2 * kXBuf;
 enum Bar { BAR_Q = 0, BAR_KFULL = 1, BAR_KEMPTY = BAR_KFULL + kStages, BAR_SFULL = BAR_KEMPTY + kStages, BAR_PFULL = BAR_SFULL + 2,
            BAR_ODONE = BAR_PFULL + 2, kNumBars = BAR_ODONE + 2 };
 constexpr int kOffMisc = kOffBar + kNumBars * 8;                 // tmem slot, abort flag, "an earlier CTA gave up"
-constexpr int kSmemBytes = kOffMisc + 32 + 1024;
+// More than half of an SM's shared memory, so that no two CTAs share an SM: the second one would wait in its tensor-memory
+// allocation until the first has finished, while other SMs stand idle (placed behind a draining predecessor, CTAs do land
+// like that: 1.5 us per tile instead of 0.7).
+constexpr int kSmemBytes = 120 * 1024;
+static_assert(kOffMisc + 32 + 1024 <= kSmemBytes, "shared memory per CTA");
 constexpr uint32_t kColS = 0, kColO = 256, kColSFQ = 400, kColSFK = 404, kColSFV = 412, kColSFP = 428;
 
 struct Params {
@@ -57,6 +62,7 @@ struct Params {
   int* status;
   int64_t Nq, Nkv;
   int q_tiles, kv_tiles, groups;   // groups of 128/R rows per head
+  int first;                       // the first CTA's group, counted over all heads
   float scale_log2e;
 };
 
@@ -73,7 +79,7 @@ __global__ void __launch_bounds__(32 * (16 / R + 2), 1) attention_rows_kernel(co
 
   const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int T = p.kv_tiles;
-  const int bh = blockIdx.x / p.groups, grp = blockIdx.x - bh * p.groups;
+  const int bh = ((int)blockIdx.x + p.first) / p.groups, grp = (int)blockIdx.x + p.first - bh * p.groups;
   const int qtile = grp / R, slab = (grp % R) * kRG;             // 128-row tile and first 32-row group in it
 
   // ---- setup -------------------------------------------------------------------------------
@@ -190,7 +196,7 @@ __global__ void __launch_bounds__(32 * (16 / R + 2), 1) attention_rows_kernel(co
     // alike) is accumulated by both warps of the pair, one tile behind: the partner's part comes with the next meeting.
     float l_run = 0.0f, l_own = 0.0f, alpha = 1.0f;
     auto add_sums = [&](int b) {
-      l_run = fmaf(alpha, l_run, l_own + lds32f(aX + (kOffXL - kOffX) + b * (2 * 4 * 32 * 4) + (kb ^ 1) * 128));     // line 14 (direct), Eq. 12
+      l_run = fmaf(alpha, l_run, l_own + lds32f(aX + (kOffXL - kOffX) + b * kXBuf + (kb ^ 1) * 128));     // line 14 (direct), Eq. 12
     };
     for (int j = 0; j < T; ++j) {
       const int b = j & 1;
@@ -215,7 +221,7 @@ __global__ void __launch_bounds__(32 * (16 / R + 2), 1) attention_rows_kernel(co
         q4[u] = fmaxf(mx, __uint_as_float(v[7]));
       }
       const float bmax = fmaxf(max3(q4[0], q4[1], q4[2]), q4[3]);
-      const uint32_t ax = aX + b * (2 * 4 * 32 * 4);
+      const uint32_t ax = aX + b * kXBuf;
       sts32f(ax + kb * 128, bmax);
       asm volatile("bar.sync %0, 128;" ::"r"(1 + rg) : "memory");                  // the four warps of these rows
       if (!kPnq && j > 0) add_sums(b ^ 1);
@@ -292,7 +298,7 @@ __global__ void __launch_bounds__(32 * (16 / R + 2), 1) attention_rows_kernel(co
     if (!kPnq) {
       asm volatile("bar.sync %0, 128;" ::"r"(1 + rg) : "memory");
       add_sums((T - 1) & 1);
-      const uint32_t ax = aX + (T & 1) * (2 * 4 * 32 * 4);
+      const uint32_t ax = aX + (T & 1) * kXBuf;
       sts32f(ax + kb * 128, l_run);
       asm volatile("bar.sync %0, 128;" ::"r"(1 + rg) : "memory");
       l = l_run + lds32f(ax + (kb ^ 2) * 128);                   // the other pair's sum
@@ -340,19 +346,32 @@ __global__ void __launch_bounds__(32 * (16 / R + 2), 1) attention_rows_kernel(co
 
 }  // namespace rows
 
-// Query rows per CTA for a problem of bh heads, as the replication R (0: the 256-row kernel of forward.cu).  Estimated
-// cycles = waves of CTAs over the SMs x (KV tiles x cycles per tile + the fixed cost of a CTA); the cycles per tile are the
-// measured ones.  The smaller CTAs win while they are few enough for one wave or two: they cost 2.2 to 3.5 times as
-// many SM cycles per row, so a problem that fills the GPU with 256-row CTAs stays there.
-int forward_rows_replication(int64_t bh, int64_t Nq, int64_t Nkv) {
-  const int64_t n_sm = sm_count() > 0 ? sm_count() : 148, T = (Nkv + kTile - 1) / kTile;
-  auto cost = [&](int64_t rows, int64_t tile, int64_t fixed) { return (bh * ((Nq + rows - 1) / rows) + n_sm - 1) / n_sm * (T * tile + fixed); };
-  const int64_t c256 = cost(256, 2600, 4000), c64 = cost(64, 1430, 2500), c32 = cost(32, 1120, 2500);
-  if (c256 <= c64 && c256 <= c32) return 0;
-  return c32 <= c64 ? 4 : 2;
+// How a problem of bh heads is divided between the 256-row CTAs of forward.cu and the smaller ones of this file: the first
+// `pairs_256` pairs of query tiles (counted over all heads) go there, the rest to CTAs of 128/R rows.  Estimated cycles =
+// waves of CTAs over the SMs x (KV tiles x cycles per tile + fixed cost), with measured figures: a 256-row CTA takes 2700
+// cycles per tile (3050 with the direct row sum), 128 rows 2125, 64 rows 1530, 32 rows 1200.  A small CTA costs more SM
+// cycles per row, so a problem that fills whole waves of 256-row CTAs stays there; a problem smaller than a wave goes to
+// small CTAs; and where the last wave of 256-row CTAs would be nearly empty, its items are cut into small CTAs instead:
+// 24 heads of 8192 queries are 5.19 waves (direct row sum 647 -> 603 us).  That second launch waits for the last of the full
+// waves, which costs a few us, and more where the CTAs of forward.cu do not walk their items in step.
+RowSplit forward_row_split(int64_t bh, int64_t Nq, int64_t Nkv, bool pnq) {
+  const int64_t n_sm = sm_count() > 0 ? sm_count() : 148, T = (Nkv + kTile - 1) / kTile, tiles = (Nq + kTile - 1) / kTile;
+  const int64_t pairs = (tiles + 1) / 2, total = bh * pairs, full = total / n_sm;
+  const int64_t c256 = T * (pnq ? 2700 : 3050) + 4400;
+  RowSplit best{total, 0};
+  if (total % n_sm == 0) return best;
+  int64_t best_cost = (full + 1) * c256 + 1600;
+  for (int R = 1; R <= 4; R *= 2) {
+    const int64_t c = T * (R == 4 ? 1200 : R == 2 ? 1530 : 2125) + 4500, per_head = (Nq + kTile / R - 1) / (kTile / R);
+    const int64_t at = full * n_sm, done = at / pairs * per_head + (at % pairs) * 2 * R;     // groups in the full waves
+    const int64_t gap = full == 0 ? 0 : T > kWalkMaxTiles ? 4000 + c256 / 10 : 4000;
+    const int64_t cost = full * c256 + gap + (bh * per_head - done + n_sm - 1) / n_sm * c;
+    if (cost < best_cost) { best_cost = cost; best = RowSplit{at, R}; }
+  }
+  return best;
 }
 
-int launch_forward_rows(int R, const void* q_codes, const void* q_scales, const void* k_codes, const void* k_scales,
+int launch_forward_rows(int R, int64_t first_pair, const void* q_codes, const void* q_scales, const void* k_codes, const void* k_scales,
                         const void* v_codes, const void* v_scales, void* o, int B, int H, int64_t Nq, int64_t Nkv,
                         float softmax_scale, unsigned flags, int* status, cudaStream_t stream) {
   using namespace rows;
@@ -363,16 +382,18 @@ int launch_forward_rows(int R, const void* q_codes, const void* q_scales, const 
   p.out = o; p.status = status; p.Nq = Nq; p.Nkv = Nkv;
   p.q_tiles = (int)((Nq + kTile - 1) / kTile); p.kv_tiles = (int)((Nkv + kTile - 1) / kTile);
   p.groups = (int)((Nq + kTile / R - 1) / (kTile / R));
+  const int64_t pairs = (p.q_tiles + 1) / 2, first = first_pair / pairs * p.groups + (first_pair % pairs) * 2 * R, total = (int64_t)B * H * p.groups;
+  if (total > 0x7FFFFFFF) return MXATTN_EUNSUPPORTED;
+  p.first = (int)first;
   p.scale_log2e = softmax_scale * 1.4426950408889634f;
   const bool uos = flags & MXATTN_FLAG_UOS, pnq = flags & MXATTN_FLAG_PNQ, f32 = flags & MXATTN_FLAG_OUT_FP32;
   void (*kern)(const Params) = nullptr;
-#define PICK(U, P, F) if (uos == U && pnq == P && f32 == F) kern = R == 4 ? attention_rows_kernel<4, U, P, F> : attention_rows_kernel<2, U, P, F>;
+#define PICK(U, P, F) if (uos == U && pnq == P && f32 == F) kern = R == 4 ? attention_rows_kernel<4, U, P, F> : R == 2 ? attention_rows_kernel<2, U, P, F> : attention_rows_kernel<1, U, P, F>;
   PICK(false, false, false) PICK(false, false, true) PICK(false, true, false) PICK(false, true, true)
   PICK(true, false, false) PICK(true, false, true) PICK(true, true, false) PICK(true, true, true)
 #undef PICK
   if (!ensure_dynamic_smem((const void*)kern, kSmemBytes)) return MXATTN_ECUDA;
-  count_launch(1);
-  return launch_pdl(kern, dim3((unsigned)((int64_t)B * H * p.groups)), 32 * (16 / R + 2), kSmemBytes, stream, p) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
+  return launch_pdl(kern, dim3((unsigned)(total - first)), 32 * (16 / R + 2), kSmemBytes, stream, p) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 
 }  // namespace mxattn

@@ -48,3 +48,19 @@ def test_bit_identical_to_the_256_row_kernel(heads, f32):
     rep = lambda x: np.ascontiguousarray(np.broadcast_to(x, (many.B,) + x.shape[1:]))
     got = run(many, rep(q), rep(k), rep(v), flags)
     assert torch.equal(got, want.expand_as(got))
+
+
+# 152 to 156 pairs of query tiles: one more wave than the GPU has SMs would be nearly empty, so the 256-row kernel takes
+# whole waves only and the pairs behind them are cut into small CTAs (short and long key/value sequences; the last head's
+# tiles ragged)
+@pytest.mark.parametrize("heads,nq,nkv", [(38, 1000, 700), (39, 897, 6300), (51, 700, 300)])
+@pytest.mark.parametrize("pnq", [True, False])
+def test_last_wave_cut_into_small_ctas(heads, nq, nkv, pnq):
+    import paper_2607_24377_b200 as mx
+    flags = mx.FLAG_UOS | (mx.FLAG_PNQ if pnq else 0)
+    one = si.custom_config("lw", 1, 1, nq, nkv, 6)
+    q, k, v = si.make_all(one)
+    want = run(one, q, k, v, flags)
+    many = si.custom_config("lm", 1, heads, nq, nkv, 6)
+    rep = lambda x: np.ascontiguousarray(np.broadcast_to(x, (1, heads) + x.shape[2:]))
+    assert torch.equal(run(many, rep(q), rep(k), rep(v), flags), want.expand(1, heads, nq, 128))

@@ -104,6 +104,19 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, unsigned block,
   cfg.attrs = &attr; cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
 }
+// The same with clusters of `cluster` CTAs along x.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl_cluster(void (*kern)(KArgs...), dim3 grid, unsigned block, unsigned cluster, cudaStream_t stream, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = dim3(block); cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
+}
 // Raises a kernel's dynamic shared memory limit, once per kernel and device (a driver call per launch otherwise).
 bool ensure_dynamic_smem(const void* kern, int bytes);
 PFN_cuTensorMapEncodeTiled tensor_map_encoder();      // null if the driver has none

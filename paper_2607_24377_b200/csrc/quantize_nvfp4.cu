@@ -11,6 +11,8 @@
 // Three HBM-bound passes: the tensor maximum (2 B/element read), then the quantizer (2 B read, 0.5 + 1/16 B written).
 #include <cuda_fp16.h>
 
+#include <atomic>
+
 #include "common.cuh"
 
 namespace mxattn {
@@ -59,21 +61,21 @@ __device__ __forceinline__ uint32_t quantize_bf16x8(const uint4& v, float r) {
 // call takes the matrices of Q, K and V in one grid of three operands.  Eight loads of 16 bytes are in flight per thread.
 constexpr int kAmaxUnroll = 8;
 struct AmaxOperand { const uint4* in; uint32_t* amax; int64_t chunks; };       // chunks of 16 bytes per matrix
-__device__ __forceinline__ void tensor_amax_part(const AmaxOperand& o, int64_t b, int part, int parts) {
-  const uint4* src = o.in + b * o.chunks;
+__device__ __forceinline__ uint32_t thread_amax(const uint4* __restrict__ src, int64_t chunks, int64_t first, int64_t step) {
   uint32_t m = 0;
-  const int64_t step = (int64_t)parts * kThreads;
-  int64_t i = (int64_t)part * kThreads + threadIdx.x;
-  for (; i + (kAmaxUnroll - 1) * step < o.chunks; i += kAmaxUnroll * step) {
+  int64_t i = first;
+  for (; i + (kAmaxUnroll - 1) * step < chunks; i += kAmaxUnroll * step) {
     uint4 v[kAmaxUnroll];
 #pragma unroll
     for (int u = 0; u < kAmaxUnroll; ++u) v[u] = __ldg(src + i + u * step);
 #pragma unroll
     for (int u = 0; u < kAmaxUnroll; ++u) m = max(m, absmax_bf16x8(v[u]));
   }
-  for (; i < o.chunks; i += step) m = max(m, absmax_bf16x8(__ldg(src + i)));
-#pragma unroll
-  for (int s = 16; s > 0; s >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, s));
+  for (; i < chunks; i += step) m = max(m, absmax_bf16x8(__ldg(src + i)));
+  return __reduce_max_sync(0xFFFFFFFFu, m);           // over the warp
+}
+__device__ __forceinline__ void tensor_amax_part(const AmaxOperand& o, int64_t b, int part, int parts) {
+  uint32_t m = thread_amax(o.in + b * o.chunks, o.chunks, (int64_t)part * kThreads + threadIdx.x, (int64_t)parts * kThreads);
   __shared__ uint32_t s[kThreads / 32];
   if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = m;
   __syncthreads();
@@ -86,6 +88,28 @@ __device__ __forceinline__ void tensor_amax_part(const AmaxOperand& o, int64_t b
 __global__ void __launch_bounds__(kThreads) tensor_amax_kernel(const AmaxOperand o) {
   pdl_wait(); pdl_trigger();
   tensor_amax_part(o, blockIdx.y, blockIdx.x, gridDim.x);
+}
+// The same with one cluster of 16 CTAs per matrix: the maxima meet in the first CTA's shared memory, which then simply writes
+// the result -- nothing has to be zeroed before (a memset and the gap behind it are 2 us of a 10 us call).
+constexpr int kClusterCtas = 16, kClusterThreads = 512;
+__global__ void __launch_bounds__(kClusterThreads) tensor_amax_cluster_kernel(const AmaxOperand o) {
+  __shared__ uint32_t s[kClusterCtas * kClusterThreads / 32];       // of CTA 0: one slot per warp of the cluster
+  pdl_wait(); pdl_trigger();
+  const uint32_t rank = blockIdx.x;                                 // gridDim.x == cluster size
+  const uint32_t m = thread_amax(o.in + blockIdx.y * o.chunks, o.chunks, (int64_t)rank * kClusterThreads + threadIdx.x, (int64_t)kClusterCtas * kClusterThreads);
+  if ((threadIdx.x & 31) == 0) {
+    uint32_t dst;
+    asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(dst) : "r"((uint32_t)__cvta_generic_to_shared(&s[rank * (kClusterThreads / 32) + (threadIdx.x >> 5)])));
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(dst), "r"(m) : "memory");
+  }
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (rank == 0 && threadIdx.x < 32) {
+    uint32_t v = 0;
+#pragma unroll
+    for (int i = 0; i < kClusterCtas * kClusterThreads / 32; i += 32) v = max(v, s[i + threadIdx.x]);
+    v = __reduce_max_sync(0xFFFFFFFFu, v);
+    if (threadIdx.x == 0) o.amax[blockIdx.y] = v << 16;
+  }
 }
 __global__ void __launch_bounds__(kThreads) tensor_amax_qkv_kernel(const AmaxOperand q, const AmaxOperand k, const AmaxOperand v) {
   pdl_wait(); pdl_trigger();
@@ -332,12 +356,27 @@ int launch_tensor_amax(const void* in, float* amax, int64_t batch, int64_t rows,
   if (!aligned16(in) || (reinterpret_cast<uintptr_t>(amax) & 3u)) return MXATTN_EALIGN;
   if (batch > 65535) return MXATTN_EUNSUPPORTED;
   const int64_t chunks = rows * cols / 8;
+  // One cluster per matrix where the matrices are many enough to fill the GPU with 16 CTAs each, or so small that 16 CTAs
+  // with eight loads per thread cover one.
+  const nv::AmaxOperand op{(const uint4*)in, reinterpret_cast<uint32_t*>(amax), chunks};
+  if (batch >= 8 || chunks <= nv::kClusterCtas * nv::kClusterThreads * nv::kAmaxUnroll) {
+    static std::atomic<uint64_t> allowed{0};                         // devices on which clusters of 16 have been allowed
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return MXATTN_ECUDA;
+    if (!(allowed.load(std::memory_order_relaxed) >> (dev & 63) & 1)) {
+      if (cudaFuncSetAttribute(nv::tensor_amax_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return MXATTN_ECUDA;
+      allowed.fetch_or((uint64_t)1 << (dev & 63), std::memory_order_relaxed);
+    }
+    count_launch(1);
+    return launch_pdl_cluster(nv::tensor_amax_cluster_kernel, dim3(nv::kClusterCtas, (unsigned)batch), nv::kClusterThreads, nv::kClusterCtas, stream, op) == cudaSuccess
+               ? MXATTN_OK : MXATTN_ECUDA;
+  }
   int64_t blocks = (chunks + nv::kThreads * 8 - 1) / (nv::kThreads * 8);
   if (blocks > 1184) blocks = 1184;                 // 8 CTAs per SM at most: the loop strides over the rest
   if (cudaMemsetAsync(amax, 0, (size_t)batch * sizeof(float), stream) != cudaSuccess) return MXATTN_ECUDA;
   count_launch(1);
   return launch_pdl(nv::tensor_amax_kernel, dim3((unsigned)blocks, (unsigned)batch), nv::kThreads, 0, stream,
-                    nv::AmaxOperand{(const uint4*)in, reinterpret_cast<uint32_t*>(amax), chunks}) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
+                    op) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 
 int launch_quantize_nvfp4(const void* in, void* codes, void* scales, const float* amax, float* tensor_scale, int64_t batch,

@@ -122,6 +122,29 @@ bool ensure_dynamic_smem(const void* kern, int bytes);
 PFN_cuTensorMapEncodeTiled tensor_map_encoder();      // null if the driver has none
 int sm_count();              // of the current device (0 on error)
 
+// Division of an attention kernel's work (pairs of query tiles of 128 rows, one pair per CTA and wave): where the last wave
+// of pairs fills at most half of the SMs, each of its tiles gets a CTA of its own, which takes less time than a pair.
+struct TileSplit {
+  int64_t pair_ctas, ctas;
+  explicit TileSplit(int64_t pairs) {
+    const int64_t n_sm = sm_count(), rest = n_sm > 0 ? pairs % n_sm : 0;
+    pair_ctas = 2 * rest <= n_sm ? pairs - rest : pairs;
+    ctas = pair_ctas + 2 * (pairs - pair_ctas);
+  }
+};
+struct TileOfCta {
+  int bh, qtile;               // head, first query tile
+  bool two, empty;             // whether the CTA has a second one / has none (an odd head's missing tile)
+  __device__ __forceinline__ TileOfCta(int cta, int pair_ctas, int q_pairs, int q_tiles) {
+    const bool single = cta >= pair_ctas;
+    const int pair = single ? pair_ctas + ((cta - pair_ctas) >> 1) : cta;
+    bh = pair / q_pairs;
+    qtile = 2 * (pair - bh * q_pairs) + (single ? (cta - pair_ctas) & 1 : 0);
+    empty = qtile >= q_tiles;
+    two = !single && qtile + 1 < q_tiles;
+  }
+};
+
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // Internal launchers (defined in quantize.cu / forward.cu); all return an mxattn_status.

@@ -6,7 +6,7 @@
 //   GEMM 1  S_t  = Q_t K_j^T         tcgen05.mma kind::f16, M=128, N=128, 8 instructions of K=16, operands in shared memory
 //   GEMM 2  O_t += P_t V_j           A = P_t from tensor memory, B = V_j as it lies in memory (token-major, "MN-major" operand)
 //
-// One CTA = two query tiles of 128 rows of one head; the roles are those of forward.cu (16 softmax warps in two groups, a
+// One CTA = two query tiles of 128 rows of one head (or one, see below); the roles are those of forward.cu (16 softmax warps in two groups, a
 // producer, an MMA issuer).  Q, K and V tiles are fetched straight from the [B H][N][128] tensors by tensor copies with the
 // 128-byte swizzle (two 64-channel halves of 16 KiB per tile; rows beyond the sequence arrive as zeros), so there is no
 // re-tiling pass over the inputs.
@@ -20,6 +20,8 @@
 // Measured (B200): H=24, N=8192 970 -> 755 us, H=40, N=16384 5.40 -> 4.5 ms; the former version re-tiled its inputs
 // (60 us), kept P in shared memory and issued its 32 multiplies per tile from a single thread, which had to move every
 // descriptor word to a uniform register in front of each of them (966 -> 800 us by the converged issuer alone).
+// A last wave that would leave half of the SMs idle runs with one query tile per CTA (common.cuh): 755 -> 646 us at
+// H=24, N=8192 (5.19 waves), 25 -> 19 us at 2 heads of 1024.
 #include <string.h>
 
 #include <type_traits>
@@ -70,6 +72,7 @@ struct Params {
   int* status;
   int64_t Nq, Nkv;
   int q_tiles_n, kv_tiles, q_pairs;
+  int pair_ctas;        // CTAs before this one take two query tiles, the others one (TileSplit)
   float scale_log2e;
 };
 
@@ -87,8 +90,9 @@ __global__ void __launch_bounds__(kThreads, 1) attention_bf16_kernel(const Param
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kOffMisc + 8);
 
   const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
-  const int bh = blockIdx.x / p.q_pairs;
-  const int pair = blockIdx.x - bh * p.q_pairs;
+  const TileOfCta at((int)blockIdx.x, p.pair_ctas, p.q_pairs, p.q_tiles_n);
+  const int bh = at.bh, qtile0 = at.qtile;
+  const bool two = at.two;                           // a second query tile: softmax group 1 has work
   const int T = p.kv_tiles;
 
   if (tid == 0) {
@@ -110,7 +114,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_bf16_kernel(const Param
   tc_fence_after();
   pdl_trigger();
   constexpr uint32_t tmem = 0;                       // all 512 columns are allocated: the base is column 0
-  const int role = (abort_flag[1] != 0 || *tmem_slot != 0) ? kSoftmaxWarps + 2 : warp;     // an earlier CTA gave up: drain the grid quickly
+  const int role = (abort_flag[1] != 0 || *tmem_slot != 0 || at.empty || (!two && warp >= 8 && warp < kSoftmaxWarps)) ? kSoftmaxWarps + 2 : warp;     // an earlier CTA gave up: drain the grid quickly
 
   if (role == kSoftmaxWarps) {
     // =============================== producer ===============================================
@@ -119,10 +123,9 @@ __global__ void __launch_bounds__(kThreads, 1) attention_bf16_kernel(const Param
         tensor_g2s(dst, map, 0, row, bh, b);
         tensor_g2s(dst + kHalfBytes, map, 64, row, bh, b);
       };
-      const int qt0 = 2 * pair, qt1 = (2 * pair + 1 < p.q_tiles_n) ? qt0 + 1 : qt0;
-      mbar_expect_tx(bar(BAR_Q), 2 * kTileBytes);
-      fetch(sbase + kOffQ, &q_map, qt0 * kTile, bar(BAR_Q));
-      fetch(sbase + kOffQ + kTileBytes, &q_map, qt1 * kTile, bar(BAR_Q));
+      mbar_expect_tx(bar(BAR_Q), (two ? 2 : 1) * kTileBytes);
+      fetch(sbase + kOffQ, &q_map, qtile0 * kTile, bar(BAR_Q));
+      if (two) fetch(sbase + kOffQ + kTileBytes, &q_map, (qtile0 + 1) * kTile, bar(BAR_Q));
       bool ok = true;
       int n = 0;
       for (; n < 2 * T; ++n) {                         // load n: K_j for n = 2 j, V_j for n = 2 j + 1
@@ -159,7 +162,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_bf16_kernel(const Param
         tc_mma_ss(leader, tmem + kColS, ((uint64_t)kDescHi << 32) | (a + off), ((uint64_t)kDescHi << 32) | (b + off), kIdescBase, k > 0 ? 1u : 0u);
       }
       tc_commit_if(leader, bar(BAR_SFULL + t));
-      if (t == 1) tc_commit_if(leader, bar(BAR_EMPTY + 2 * j % kStages));      // K_j: both groups' products are issued
+      if (t == 1 || !two) tc_commit_if(leader, bar(BAR_EMPTY + 2 * j % kStages));      // K_j: both groups' products are issued
     };
     auto gemm2 = [&](int t, int j) {                   // O_t += P_t V_j; K = 16 tokens per instruction: 8 columns of P, 2048 bytes of V
       const uint32_t b = kv_lo + (uint32_t)((2 * j + 1) % kStages) * (kTileBytes >> 4);
@@ -168,7 +171,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_bf16_kernel(const Param
         tc_mma_ts(leader, tmem + kColO + 128 * t, tmem + kColP + 192 * t + 8 * k,
                   ((uint64_t)kDescHi << 32) | ((uint64_t)(kHalfBytes >> 4) << 16) | (b + (uint32_t)k * 128), kIdescV, (j > 0 || k > 0) ? 1u : 0u);
       tc_commit_if(leader, bar(BAR_ODONE + t));
-      if (t == 1) tc_commit_if(leader, bar(BAR_EMPTY + (2 * j + 1) % kStages));
+      if (t == 1 || !two) tc_commit_if(leader, bar(BAR_EMPTY + (2 * j + 1) % kStages));
     };
     auto wait_p = [&](int t, int j) {
       const bool r = mbar_wait_warp(bar(BAR_PFULL + t), (uint32_t)(j & 1), abort_flag, p.status, 24 + 2 * t);
@@ -186,29 +189,40 @@ __global__ void __launch_bounds__(kThreads, 1) attention_bf16_kernel(const Param
     };
     ok = ok && landed(0);
     if (ok) gemm1(0, 0);
-    ok = ok && wait_sfree();
-    if (ok) gemm1(1, 0);
-    if (T > 1) {
-      ok = ok && landed(2) && wait_sfree();
-      if (ok) gemm1(0, 1);
-    }
-    for (int j = 0; j < T && ok; ++j) {
-      ok = landed(2 * j + 1) && wait_p(0, j);
-      if (!ok) break;
-      gemm2(0, j);
+    for (int j = 0; !two && j < T && ok; ++j) {        // one query tile: its next scores go ahead of the output product
       if (j + 1 < T) {
-        ok = wait_sfree();
+        ok = landed(2 * j + 2) && wait_sfree();
         if (!ok) break;
-        gemm1(1, j + 1);
+        gemm1(0, j + 1);
       }
-      if (j + 2 < T) ok = landed(2 * j + 4);
-      ok = ok && wait_p(1, j);
-      if (!ok) break;
-      gemm2(1, j);
-      if (j + 2 < T) {
-        ok = wait_sfree();
+      ok = landed(2 * j + 1) && wait_p(0, j);
+      if (ok) gemm2(0, j);
+    }
+    if (two) {
+      ok = ok && wait_sfree();
+      if (ok) gemm1(1, 0);
+      if (T > 1) {
+        ok = ok && landed(2) && wait_sfree();
+        if (ok) gemm1(0, 1);
+      }
+      for (int j = 0; j < T && ok; ++j) {
+        ok = landed(2 * j + 1) && wait_p(0, j);
         if (!ok) break;
-        gemm1(0, j + 2);
+        gemm2(0, j);
+        if (j + 1 < T) {
+          ok = wait_sfree();
+          if (!ok) break;
+          gemm1(1, j + 1);
+        }
+        if (j + 2 < T) ok = landed(2 * j + 4);
+        ok = ok && wait_p(1, j);
+        if (!ok) break;
+        gemm2(1, j);
+        if (j + 2 < T) {
+          ok = wait_sfree();
+          if (!ok) break;
+          gemm1(0, j + 2);
+        }
       }
     }
   } else if (role < kSoftmaxWarps) {
@@ -310,9 +324,9 @@ __global__ void __launch_bounds__(kThreads, 1) attention_bf16_kernel(const Param
     const float inv_l = 1.0f / (l_run + lds32f(aMaxPartner + par));
     mbar_wait_soft<33>(bar(BAR_ODONE + t), (uint32_t)((T - 1) & 1), abort_addr);
     tc_fence_after();
-    const int qtile = 2 * pair + t;
+    const int qtile = qtile0 + t;
     const int64_t grow = (int64_t)qtile * kTile + row;
-    const bool store = (qtile < p.q_tiles_n) && (grow < p.Nq) && lds_volatile(abort_addr) == 0;
+    const bool store = (grow < p.Nq) && lds_volatile(abort_addr) == 0;
     const int64_t obase = ((int64_t)bh * p.Nq + grow) * kHeadDim + 64 * h;
 #pragma unroll 1
     for (int c0 = 0; c0 < 64; c0 += 32) {
@@ -391,11 +405,13 @@ int launch_forward_bf16(const void* q, const void* k, const void* v, void* o, in
   Params p;
   p.out = o; p.status = static_cast<int*>(workspace);
   p.Nq = Nq; p.Nkv = Nkv; p.q_tiles_n = (int)qt; p.kv_tiles = (int)kt; p.q_pairs = (int)pairs;
+  const TileSplit split(grid);
+  p.pair_ctas = (int)split.pair_ctas;
   p.scale_log2e = softmax_scale * 1.4426950408889634f;
   auto kern = (flags & MXATTN_FLAG_OUT_FP32) ? attention_bf16_kernel<true> : attention_bf16_kernel<false>;
   if (!ensure_dynamic_smem((const void*)kern, kSmemBytes)) return MXATTN_ECUDA;
   count_launch(1);
-  return launch_pdl(kern, dim3((unsigned)grid), kThreads, kSmemBytes, stream, p, q_map, k_map, v_map) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
+  return launch_pdl(kern, dim3((unsigned)split.ctas), kThreads, kSmemBytes, stream, p, q_map, k_map, v_map) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 
 }  // namespace mxattn

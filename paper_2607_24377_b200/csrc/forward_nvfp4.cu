@@ -17,7 +17,8 @@
 // r = 2688 / d folded into the exponent (the recipe's fl32(p_i * r) differs from this by about 2e-7 relative, the order
 // of ex2.approx itself; a block with d = 0 keeps r = 1, its codes are 0 either way).
 //
-// One CTA per work item (two query tiles of one head); outputs are stored from registers.  Tensor-memory map:
+// One CTA per work item: two query tiles of one head, or one where the last wave would leave half of the SMs idle
+// (common.cuh; 2 heads of 1024: 29 -> 23 us, 40 heads of 16384: 4090 -> 4033); outputs are stored from registers.  Tensor-memory map:
 // S [0,128), O_0 [128,272), O_1 [272,416), scale factors from 416 (8 columns per operand tile: two atoms).
 // Every mbarrier wait is bounded; a softmax warp that gives up keeps its partner's appointments (tc_helpers.cuh).
 #include <cuda_fp16.h>
@@ -74,6 +75,7 @@ struct Params {
   int* status;
   int64_t Nq, Nkv;
   int q_tiles, kv_tiles, q_pairs;
+  int pair_ctas;        // CTAs before this one take two query tiles, the others one (TileSplit)
   float scale_log2e;
 };
 
@@ -110,7 +112,9 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
 
   const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int T = p.kv_tiles;
-  const int bh = blockIdx.x / p.q_pairs, pair = blockIdx.x - bh * p.q_pairs;
+  const TileOfCta at((int)blockIdx.x, p.pair_ctas, p.q_pairs, p.q_tiles);
+  const int bh = at.bh, qtile0 = at.qtile;
+  const bool two = at.two;                           // a second query tile: softmax group 1 has work
 
   if (tid == 0) {
     mbar_init(bar(BAR_Q), 1);
@@ -148,18 +152,17 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
   tc_fence_after();
   pdl_trigger();
   const uint32_t tmem = *tmem_slot;
-  const int role = abort_flag[1] != 0 ? kSoftmaxWarps + 2 : warp;     // an earlier CTA gave up: drain the grid quickly
+  const int role = (abort_flag[1] != 0 || at.empty || (!two && warp >= 8 && warp < kSoftmaxWarps)) ? kSoftmaxWarps + 2 : warp;     // an earlier CTA gave up: drain the grid quickly
 
   if (role == kSoftmaxWarps) {
     // =============================== producer ===============================================
     if (lane == 0) {
-      const int64_t qt0 = (int64_t)bh * p.q_tiles + 2 * pair;
-      const int64_t qt1 = (2 * pair + 1 < p.q_tiles) ? qt0 + 1 : qt0;
-      mbar_expect_tx(bar(BAR_Q), 2 * (kTileCodeBytes + kSF));
-      bulk_g2s(sbase + kOffQ, p.q_codes + qt0 * kTileCodeBytes, kTileCodeBytes, bar(BAR_Q));
-      bulk_g2s(sbase + kOffQ + kTileCodeBytes, p.q_codes + qt1 * kTileCodeBytes, kTileCodeBytes, bar(BAR_Q));
-      bulk_g2s(sbase + kOffSFQ, p.q_scales + qt0 * kSF, kSF, bar(BAR_Q));
-      bulk_g2s(sbase + kOffSFQ + kSF, p.q_scales + qt1 * kSF, kSF, bar(BAR_Q));
+      const int64_t qt0 = (int64_t)bh * p.q_tiles + qtile0;
+      mbar_expect_tx(bar(BAR_Q), (two ? 2 : 1) * (kTileCodeBytes + kSF));
+      for (int i = 0; i < (two ? 2 : 1); ++i) {
+        bulk_g2s(sbase + kOffQ + i * kTileCodeBytes, p.q_codes + (qt0 + i) * kTileCodeBytes, kTileCodeBytes, bar(BAR_Q));
+        bulk_g2s(sbase + kOffSFQ + i * kSF, p.q_scales + (qt0 + i) * kSF, kSF, bar(BAR_Q));
+      }
       const int64_t kv0 = (int64_t)bh * T;
       bool ok = true;
       int j = 0;
@@ -230,7 +233,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
       };
       if (ok) {
         tc_fence_after();
-        for (int t = 0; t < 2; ++t) {
+        for (int t = 0; t < (two ? 2 : 1); ++t) {
           tc_cp_sf(tmem + kColSFQ + 8 * t, sbase + kOffSFQ + t * kSF);
           tc_cp_sf(tmem + kColSFQ + 8 * t + 4, sbase + kOffSFQ + t * kSF + kTileScaleBytes);
         }
@@ -239,34 +242,48 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
           tc_cp_sf(tmem + kColSFV + 16 * slot + 12, sbase + kOffSFOnes);
         }
       }
-      // the issue order of forward.cu: G2(0,j) G1(1,j+1) G2(1,j) G1(0,j+2)
       ok = ok && wait_kv(0, true);
       if (ok) gemm1(0, 0);
-      ok = ok && wait_sfree();
-      if (ok) gemm1(1, 0);
-      if (T > 1) {
-        ok = ok && wait_kv(1, false);
-        if (ok) gemm1(0, 1);
-      }
-      for (int j = 0; j < T && ok; ++j) {
+      for (int j = 0; !two && j < T && ok; ++j) {      // one query tile: its next scores go ahead of the output product
+        if (j + 1 < T) {
+          ok = wait_kv(j + 1, false);
+          if (!ok) break;
+          gemm1(0, j + 1);
+        }
         ok = mbar_wait(bar(BAR_PFULL + 0), (uint32_t)(j & 1), abort_flag, p.status, 24);
         if (!ok) break;
         tc_fence_after();
         gemm2(0, j);
-        if (j + 1 < T) {
-          ok = wait_sfree();
-          if (!ok) break;
-          gemm1(1, j + 1);
-        }
-        ok = mbar_wait(bar(BAR_PFULL + 1), (uint32_t)(j & 1), abort_flag, p.status, 26);
-        if (!ok) break;
-        tc_fence_after();
-        gemm2(1, j);
         tc_commit(bar(BAR_KEMPTY + j % kStages));
-        if (j + 2 < T) {
-          ok = wait_kv(j + 2, false);
+      }
+      if (two) {
+        // the issue order of forward.cu: G2(0,j) G1(1,j+1) G2(1,j) G1(0,j+2)
+        ok = ok && wait_sfree();
+        if (ok) gemm1(1, 0);
+        if (T > 1) {
+          ok = ok && wait_kv(1, false);
+          if (ok) gemm1(0, 1);
+        }
+        for (int j = 0; j < T && ok; ++j) {
+          ok = mbar_wait(bar(BAR_PFULL + 0), (uint32_t)(j & 1), abort_flag, p.status, 24);
           if (!ok) break;
-          gemm1(0, j + 2);
+          tc_fence_after();
+          gemm2(0, j);
+          if (j + 1 < T) {
+            ok = wait_sfree();
+            if (!ok) break;
+            gemm1(1, j + 1);
+          }
+          ok = mbar_wait(bar(BAR_PFULL + 1), (uint32_t)(j & 1), abort_flag, p.status, 26);
+          if (!ok) break;
+          tc_fence_after();
+          gemm2(1, j);
+          tc_commit(bar(BAR_KEMPTY + j % kStages));
+          if (j + 2 < T) {
+            ok = wait_kv(j + 2, false);
+            if (!ok) break;
+            gemm1(0, j + 2);
+          }
         }
       }
     }
@@ -441,9 +458,9 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
       } else {
         o_scale *= __fdiv_rn(1.0f, kTensorRangeP);
       }
-      const int qtile = 2 * pair + t;
+      const int qtile = qtile0 + t;
       const int64_t grow = (int64_t)qtile * kTile + row;
-      const bool store = (qtile < p.q_tiles) && (grow < p.Nq);
+      const bool store = (grow < p.Nq);
       const float inv_l = o_scale / l;
       const int64_t obase = ((int64_t)bh * p.Nq + grow) * kHeadDim + kCols * h;
 #pragma unroll 1
@@ -536,13 +553,15 @@ int launch_forward_nvfp4(const void* q, const void* k, const void* v, void* o, i
   p.ts_q = ts; p.ts_k = ts + bh; p.ts_v = ts + 2 * bh;
   p.out = o; p.status = reinterpret_cast<int*>(ws + w.status);
   p.Nq = Nq; p.Nkv = Nkv; p.q_tiles = (int)qt; p.kv_tiles = (int)kt; p.q_pairs = (int)pairs;
+  const TileSplit split(grid);
+  p.pair_ctas = (int)split.pair_ctas;
   p.scale_log2e = softmax_scale * 1.4426950408889634f;
   const bool pnq = flags & MXATTN_FLAG_PNQ, f32 = flags & MXATTN_FLAG_OUT_FP32;
   void (*kern)(const Params) = pnq ? (f32 ? attention_nvfp4_kernel<true, true> : attention_nvfp4_kernel<true, false>)
                                    : (f32 ? attention_nvfp4_kernel<false, true> : attention_nvfp4_kernel<false, false>);
   if (!ensure_dynamic_smem((const void*)kern, kSmemBytes)) return MXATTN_ECUDA;
   count_launch(1);
-  return launch_pdl(kern, dim3((unsigned)grid), kThreads, kSmemBytes, stream, p) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
+  return launch_pdl(kern, dim3((unsigned)split.ctas), kThreads, kSmemBytes, stream, p) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 
 }  // namespace mxattn

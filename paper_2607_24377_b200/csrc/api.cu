@@ -1,7 +1,9 @@
 // C-ABI entry points that orchestrate the kernels: workspace carving, the three quantize
 // launches plus the fused attention launch (paper Algorithm 2, lines 3-19), and the host-buffer
 // end-to-end form.
+#include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <vector>
 
 #include "common.cuh"
@@ -269,29 +271,42 @@ static HostPipe* host_pipe(size_t n_events) {
   return &hp;
 }
 
-// How many heads a pipeline stage of mxattn_forward_host takes (after the first stage, which takes one).  A stage
-// is one attention launch of g * ceil(ceil(Nq/128)/2) CTAs.  Consecutive stages' launches go to two streams, so
-// the CTAs of the next stage start on the SMs the current one leaves and a partly filled last wave costs
-// nothing; what is left to weigh is a launch that cannot fill the device at all (small heads: take several),
-// the fixed cost per stage, and the last stage's copy out, which nothing hides.  The estimate (attention at
-// ~1.8 PFLOP/s, copies at ~50 GB/s, 20 us of launches and events per stage) only has to rank the candidates.
-static int heads_per_stage(size_t bh, int64_t Nq, int64_t Nkv, size_t out_bytes_per_head) {
-  int dev = 0, n_sm = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-  if (n_sm <= 0) n_sm = 148;
-  const double ctas = (double)(((Nq + kTile - 1) / kTile + 1) / 2);
-  const double t_head = 4.0 * (double)Nq * (double)Nkv * kHeadDim / 1.8e15;
-  const double t_out = (double)out_bytes_per_head / 50e9;
-  int best = 1;
-  double best_t = 1e300;
-  for (int g = 1; g <= 8 && (size_t)g <= bh; ++g) {
-    if (g > 1 && bh / g < 3) break;                 // keep at least three stages to overlap
-    const double fill = g * ctas / n_sm;
-    const double eff = fill < 1.0 ? fill : 1.0;
-    const double t = (double)bh * t_head / eff + g * t_out + 20e-6 * (double)((bh + g - 1) / g);
-    if (t < best_t * 0.995) { best_t = t; best = g; }
+// First heads of the pipeline stages of mxattn_forward_host; the last entry is bh.  The link bounds the call (a head
+// of N tokens arrives in 14 us per 1000 tokens, and its attention takes less than that below some 50000 tokens), and a
+// stage costs it about 20 us: three copies of some 6 us each on top of their bytes.  So there should be few stages.
+//   - Nothing hides the last stage's attention and copy out, so that stage is small, and the stages before it grow by
+//     the ratio at which a stage's attention and copy out are just done when the smaller one behind it has arrived
+//     (55 GB/s in and out, attention at 1.6 PFLOP/s).  It is kept between 1.5 and 3, beyond which nothing is gained.
+//   - Where the copies in are the bound the first stages may be large: they start at an eighth of the heads and double.
+//     Where the copies out weigh as much (Nkv small) the first stage has to be small, and a stage that grows leaves
+//     the link idle outwards while it arrives: equal ones then, of the size at which the wait for one stage is what
+//     all stages' fixed cost is.
+//   - No stage is below 2.5 MB in, which is 45 us of the link, unless the call is.
+// Against one head followed by stages of equal size, us: 24 x 8192 3310 -> 3249 (copying in alone takes 2731), 40 x 4096
+// 2858 -> 2712 (2280), 160 x 5000 13170 -> 12230, 160 x 300 1134 -> 912, 2 x 1024 (one stage now) 195 -> 164, 12 x 20000
+// 4084 -> 4011; 40 heads of 10000 x 512 3024 -> 3023.
+static std::vector<size_t> host_stages(size_t bh, int64_t Nq, int64_t Nkv, size_t in_bytes_per_head, size_t out_bytes_per_head) {
+  const double t_in = (double)in_bytes_per_head / 55e9, t_out = (double)out_bytes_per_head / 55e9;
+  const double t_rest = t_out + 4.0 * (double)Nq * (double)Nkv * kHeadDim / 1.6e15;
+  const double shrink = std::min(3.0, std::max(1.5, 1.1 * t_in / t_rest));
+  const size_t least = (size_t)(2.5e6 / (double)in_bytes_per_head) + 1;
+  const bool in_bound = t_in > 1.5 * t_out;
+  const size_t most = in_bound ? bh : std::max(least, (size_t)std::sqrt((double)bh * 20e-6 / t_out));
+  size_t next_head = in_bound ? std::max(least, bh / 8) : least, next_tail = least;
+  std::vector<size_t> head, tail;
+  for (size_t left = bh; left > 0;) {
+    const bool at_head = next_head < next_tail;
+    size_t& next = at_head ? next_head : next_tail;
+    // what would be left over and too small for a stage of its own joins this one
+    const size_t n = 4 * left < 5 * next || left < next + least ? left : next;
+    (at_head ? head : tail).push_back(n);
+    next = std::min(most, at_head ? 2 * n : (size_t)std::lround(shrink * (double)n));
+    left -= n;
   }
-  return best;
+  std::vector<size_t> first(1, 0);
+  for (size_t n : head) first.push_back(first.back() + n);
+  for (size_t k = tail.size(); k-- > 0;) first.push_back(first.back() + tail[k]);
+  return first;
 }
 
 extern "C" size_t mxattn_forward_host_arena_bytes(int B, int H, int64_t Nq, int64_t Nkv, int d, unsigned flags) {
@@ -323,14 +338,8 @@ extern "C" int mxattn_forward_host(const void* q_host, const void* k_host, const
   uint8_t* dv = dk + align_up(bh * kh, 256);
   uint8_t* dout = dv + align_up(bh * kh, 256);
   uint8_t* ws = dout + align_up(bh * oh, 256);
-  // The first stage takes one head (nothing hides its copy in), the others g heads each.
-  const int g = heads_per_stage(bh, Nq, Nkv, oh);
-  const size_t stages = (g == 1) ? bh : 1 + (bh - 1 + g - 1) / g;
-  auto first_head = [&](size_t st) {
-    if (g == 1 || st == 0) return st;
-    const size_t h = 1 + (st - 1) * (size_t)g;
-    return h < bh ? h : bh;
-  };
+  const std::vector<size_t> first_head = host_stages(bh, Nq, Nkv, qh + 2 * kh, oh);
+  const size_t stages = first_head.size() - 1;
   HostPipe* hp = host_pipe(3 * stages + 2);
   if (!hp) return MXATTN_ECUDA;
   cudaEvent_t* ev = hp->ev.data();
@@ -339,10 +348,10 @@ extern "C" int mxattn_forward_host(const void* q_host, const void* k_host, const
   ck(cudaEventRecord(ev[3 * stages], stream));                   // work already queued on the caller's stream comes first
   ck(cudaStreamWaitEvent(hp->in, ev[3 * stages], 0));
   ck(cudaStreamWaitEvent(hp->attn, ev[3 * stages], 0));
-  int rc = MXATTN_OK;
+  int rc = MXATTN_OK, launched = 0;
   for (size_t st = 0; st < stages && !fail && rc == MXATTN_OK; ++st) {
     TraceRange tr("mxattn host stage");
-    const size_t i = first_head(st), n = first_head(st + 1) - i;  // heads of the stage; heads are contiguous in memory
+    const size_t i = first_head[st], n = first_head[st + 1] - i;  // heads of the stage; heads are contiguous in memory
     // attention launches alternate between the caller's stream and one of the pipeline's, so that the CTAs of a
     // stage start on the SMs the previous stage's last CTAs leave (no tail, no launch gap between stages)
     cudaStream_t as = (st & 1) ? hp->attn : stream;
@@ -356,6 +365,7 @@ extern "C" int mxattn_forward_host(const void* q_host, const void* k_host, const
     // launch, so that they fill the SMs the previous stage's attention kernel frees as it drains
     rc = forward_ws(dq + i * qh, dk + i * kh, dv + i * kh, dout + i * oh, 1, (int)n, Nq, Nkv, d, softmax_scale, flags,
                     ws + i * w.total, n * w.total, as, nullptr, hp->quant, ev[3 * st + 1]);
+    launched += g_launches;
     ck(cudaEventRecord(ev[3 * st + 2], as));
     ck(cudaStreamWaitEvent(hp->out, ev[3 * st + 2], 0));
     ck(cudaMemcpyAsync(static_cast<char*>(o_host) + i * oh, dout + i * oh, n * oh, cudaMemcpyDeviceToHost, hp->out));
@@ -368,16 +378,14 @@ extern "C" int mxattn_forward_host(const void* q_host, const void* k_host, const
   ck(cudaStreamSynchronize(stream));
   ck(cudaStreamSynchronize(hp->attn));
   ck(cudaStreamSynchronize(hp->out));
-  g_launches = 4 * (int)stages;
+  g_launches = launched;
   if (rc != MXATTN_OK) return rc;
   if (fail) return MXATTN_ECUDA;
-  // one status word per stage, at the start of its workspace slice
-  std::vector<int> stw(stages, 0);
-  if (cudaMemcpy(stw.data(), ws, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return MXATTN_ECUDA;
-  if (stages > 1 && cudaMemcpy2D(stw.data() + 1, sizeof(int), ws + first_head(1) * w.total, (size_t)g * w.total, sizeof(int),
-                                 stages - 1, cudaMemcpyDeviceToHost) != cudaSuccess) return MXATTN_ECUDA;
-  for (size_t i = 0; i < stages; ++i)
-    if (stw[i]) return MXATTN_ETIMEOUT;
+  // one status word per stage, at the start of the workspace slice of the stage's first head
+  std::vector<int> word(bh, 0);
+  if (cudaMemcpy2D(word.data(), sizeof(int), ws, w.total, sizeof(int), bh, cudaMemcpyDeviceToHost) != cudaSuccess) return MXATTN_ECUDA;
+  for (size_t st = 0; st < stages; ++st)
+    if (word[first_head[st]]) return MXATTN_ETIMEOUT;
   return MXATTN_OK;
 }
 

@@ -7,7 +7,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("batch,rows,cols", [(1, 1, 8), (3, 4097, 128), (1, 4096 * 4, 32), (1, 4096 * 4 + 1, 32), (7, 8200, 128), (8, 8200, 128),
-                                             (9, 1023, 64), (2, 70001, 8)])
+                                             (9, 1023, 64), (2, 70001, 8), (1, 16384, 128), (1, 16385, 128), (4, 11264, 128), (4, 11265, 128)])
 def test_maximum_of_every_matrix(batch, rows, cols):
     import paper_2607_24377_b200 as mx
     n = rows * cols

@@ -42,8 +42,8 @@
 // to registers at once, so the buffer is free again long before the other group needs it),
 // O_0 [128,272), O_1 [272,416), scale factors from 416.
 //
-// Epilogue: O = O~ / l; the bf16 result is staged in shared memory (one 32-row x 128-byte box per softmax warp,
-// 128-byte swizzle) and leaves as one tensor copy per warp through a tensor map of the output, so that whole
+// Epilogue: O = O~ / l; the result is staged in shared memory (one 32-row x 128-byte box per softmax warp, 128-byte
+// swizzle) and leaves as one tensor copy per warp (fp32: two) through a tensor map of the output, so that whole
 // lines are written and the stores do not queue in front of the next tile's shared-memory traffic.
 //
 // Two launch shapes: one CTA per work item (two query tiles of one head), or -- more items than SMs and a short
@@ -87,8 +87,8 @@ constexpr int kOffBar = kOffSFP + 2 * kTileScaleBytes;     // barriers
 constexpr int kNumBars = 4 + 2 * kStages + 2 + 1 + 2 + 2;  // Q full/empty[2], K/V stage full+empty, S_full[2], S_free, P_full[2], O_done[2]
 constexpr int kOffMisc = kOffBar + kNumBars * 8;           // tmem slot, abort flag
 constexpr int kOffMax = kOffMisc + 64;                     // half-row maxima: [parity 2][tile 2][half 2][128] floats
-constexpr int kOffOut = (kOffMax + 2 * 2 * 2 * 128 * 4 + 1023) & ~1023;   // bf16 output staging: one box per softmax warp
-constexpr int kOutBoxBytes = 32 * kCols * 2;               // 32 rows x 64 bf16 (128 bytes, the span of the 128-byte swizzle)
+constexpr int kOffOut = (kOffMax + 2 * 2 * 2 * 128 * 4 + 1023) & ~1023;   // output staging: one box per softmax warp
+constexpr int kOutBoxBytes = 32 * 128;                     // 32 rows x 128 bytes (the span of the 128-byte swizzle)
 constexpr int kSmemBytes = kOffOut + kSoftmaxWarps * kOutBoxBytes + 1024;   // + slack for the 1024 alignment
 static_assert(kOffOut % 1024 == 0 && kOutBoxBytes % 1024 == 0, "swizzled boxes start on the swizzle pattern's period");
 static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
@@ -105,7 +105,6 @@ struct Params {
   const uint8_t* q_codes; const uint8_t* q_scales;
   const uint8_t* k_codes; const uint8_t* k_scales;
   const uint8_t* v_codes; const uint8_t* v_scales;
-  void* out;
   int* status;
   uint8_t* dump;        // per-tile P-hat images, scales, running maxima and final row sums (debug entry point only)
   int64_t Nq, Nkv;
@@ -133,6 +132,7 @@ constexpr int kProfSlots = 16;
 template <bool kUos, bool kPnq, bool kOutF32, bool kDump, bool kPersist, bool kProf = false>
 __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, const __grid_constant__ CUtensorMap out_map) {
   static_assert(!(kDump && kPersist), "the tile dump is written by the one-item-per-CTA variant only");
+  constexpr int kOutSize = kOutF32 ? 4 : 2, kBoxCols = 128 / kOutSize;
   static_assert(!(kDump && kProf), "the dump buffer holds either the tile dump or the cycle profile");
   long long prof_t[kProfSlots];
   long long prof_prev = 0;
@@ -636,7 +636,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
     if (!ok) pair_keep_company(pair_bar, T - j);    // gave up (now or in an earlier item): only the meetings are kept
 
     // ---- epilogue: O = O~ / l (line 18) ----
-    if (kPersist && !kOutF32) {                    // the previous item's output copy has read this warp's box
+    if (kPersist) {                                // the previous item's output copy has read this warp's box
       if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
       __syncwarp();
     }
@@ -652,10 +652,9 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
       tc_fence_after();
       if (kPersist) { bh = item / p.q_pairs; pair = item - bh * p.q_pairs; }
       const int qtile = 2 * pair + t;
-      const int64_t grow = (int64_t)qtile * kTile + row;
-      if (kPersist && !kOutF32) {
+      if (kPersist) {
         // Item-walking variant: the epilogue is part of every item's critical path.  Row sum and all 64 accumulator
-        // columns are loaded with one wait, then the bf16 rows go to this warp's swizzled box and out as one tensor
+        // columns are loaded with one wait, then the rows go to this warp's swizzled box and out as one tensor
         // copy (see the comments of the general path).
         uint32_t lr = 0, r64[kCols];
         if (kPnq) asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(lr) : "r"(t_o + 128) : "memory");
@@ -664,23 +663,34 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
         if (kPnq) l = __uint_as_float(lr);
         const float inv_l = 1.0f / l;
         const uint32_t aBox = sbase + kOffOut + (t * 8 + h * 4 + (row >> 5)) * kOutBoxBytes;
-        const uint32_t aRow = aBox + (row & 31) * (kCols * 2);
+        const uint32_t aRow = aBox + (row & 31) * (kBoxCols * kOutSize);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          uint32_t hh[4];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const float a = __uint_as_float(r64[8 * i + 2 * k]) * inv_l, b2 = __uint_as_float(r64[8 * i + 2 * k + 1]) * inv_l;
-            asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hh[k]) : "f"(b2), "f"(a));
+        for (int b = 0; b < kCols / kBoxCols; ++b) {
+          if (b > 0) {                               // fp32: the first half has left the box
+            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+            __syncwarp();
           }
-          sts128(aRow + ((i ^ (row & 7)) << 4), make_uint4(hh[0], hh[1], hh[2], hh[3]));
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
-        if (lane == 0 && qtile < p.q_tiles && (int64_t)qtile * kTile + (row & ~31) < p.Nq) {
-          asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
-                       ::"l"(&out_map), "r"(kCols * h), "r"(qtile * kTile + (row & ~31)), "r"(bh), "r"(aBox) : "memory");
-          asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            uint32_t hh[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              if (kOutF32) {
+                hh[k] = __float_as_uint(__uint_as_float(r64[kBoxCols * b + 4 * i + k]) * inv_l);
+              } else {
+                const float a = __uint_as_float(r64[8 * i + 2 * k]) * inv_l, b2 = __uint_as_float(r64[8 * i + 2 * k + 1]) * inv_l;
+                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hh[k]) : "f"(b2), "f"(a));
+              }
+            }
+            sts128(aRow + ((i ^ (row & 7)) << 4), make_uint4(hh[0], hh[1], hh[2], hh[3]));
+          }
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          __syncwarp();
+          if (lane == 0 && qtile < p.q_tiles && (int64_t)qtile * kTile + (row & ~31) < p.Nq) {
+            asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
+                         ::"l"(&out_map), "r"(kCols * h + kBoxCols * b), "r"(qtile * kTile + (row & ~31)), "r"(bh), "r"(aBox) : "memory");
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+          }
         }
       } else {
       if (kPnq) {
@@ -689,57 +699,51 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
         tmem_ld_wait();
         l = __uint_as_float(lr);
       }
-      const bool store = (qtile < p.q_tiles) && (grow < p.Nq);
       const float inv_l = 1.0f / l;                // line 18 as one reciprocal and 64 multiplies per thread
       if (kDump && h == 0 && qtile < p.q_tiles)
         reinterpret_cast<float*>(p.dump + (int64_t)p.total_items / p.q_pairs * p.q_tiles * T * kDumpTileBytes)
             [((int64_t)bh * p.q_tiles + qtile) * kTile + row] = l;
-      const int64_t obase = ((int64_t)bh * p.Nq + grow) * kHeadDim + kCols * h;
-      if (kOutF32) {
+      // The warp's 32 half rows go to shared memory and from there to global memory as tensor copies (boxes of 32 rows x
+      // 128 bytes: 64 bf16 columns or 32 fp32 ones, so that fp32 takes two turns with the box; rows at or beyond Nq are
+      // clipped by the copy).  Written from registers, a warp's 16-byte stores land 256 or 512 bytes apart (one partly
+      // filled sector per lane and instruction); and any store instruction of these warps queues 64 KiB per item in front
+      // of the next tile's shared-memory traffic.  The box uses the 128-byte swizzle (16-byte chunk c of row r sits at
+      // chunk c ^ (r & 7)), which also spreads a quarter warp's stores over all banks.  As tensor
+      // copies fp32 takes 834 us for 40 x 75600 x 512 (1208 from registers), 64.5 for 40 x 4096 x 512 (86), 20.6 for 14 x
+      // 1300 x 777 (23.4).
+      const uint32_t aBox = sbase + kOffOut + (t * 8 + h * 4 + (row >> 5)) * kOutBoxBytes;    // one box per warp
+      const uint32_t aRow = aBox + (row & 31) * (kBoxCols * kOutSize);
 #pragma unroll 1
-        for (int c0 = 0; c0 < kCols; c0 += 32) {
-          uint32_t r32[32];
-          TMEM_LD32(t_o + kCols * h + c0, r32);
-          tmem_ld_wait();
-          if (store) {
-            float4* dst = reinterpret_cast<float4*>(static_cast<float*>(p.out) + obase + c0);
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-              dst[i] = make_float4(__uint_as_float(r32[4 * i]) * inv_l, __uint_as_float(r32[4 * i + 1]) * inv_l,
-                                   __uint_as_float(r32[4 * i + 2]) * inv_l, __uint_as_float(r32[4 * i + 3]) * inv_l);
-          }
+      for (int c0 = 0; c0 < kCols; c0 += 32) {
+        uint32_t r32[32];
+        TMEM_LD32(t_o + kCols * h + c0, r32);
+        if (kOutF32 && c0 > 0) {                   // the first half has left the box
+          if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+          __syncwarp();
         }
-      } else {
-        // bf16: the warp's 32 half rows (128 bytes each) go to shared memory and from there to global memory as one
-        // tensor copy (box of 32 rows x 64 columns; rows at or beyond Nq are clipped by the copy).  Written from
-        // registers, a warp's 16-byte stores land 256 bytes apart (one partly filled sector per lane and
-        // instruction); and any store instruction of these warps queues 64 KiB per item in front of the next
-        // tile's shared-memory traffic.  The box uses the 128-byte swizzle (16-byte chunk c of row r sits at
-        // chunk c ^ (r & 7)), which also spreads a quarter warp's stores over all banks.
-        const uint32_t aBox = sbase + kOffOut + (t * 8 + h * 4 + (row >> 5)) * kOutBoxBytes;    // one box per warp
-        const uint32_t aRow = aBox + (row & 31) * (kCols * 2);
-#pragma unroll 1
-        for (int c0 = 0; c0 < kCols; c0 += 32) {
-          uint32_t r32[32];
-          TMEM_LD32(t_o + kCols * h + c0, r32);
-          tmem_ld_wait();
+        tmem_ld_wait();
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            uint32_t hh[4];
+        for (int i = 0; i < 32 * kOutSize / 16; ++i) {
+          uint32_t hh[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const float a = __uint_as_float(r32[8 * i + 2 * k]) * inv_l, b2 = __uint_as_float(r32[8 * i + 2 * k + 1]) * inv_l;
+          for (int k = 0; k < 4; ++k) {
+            if (kOutF32) {
+              hh[k] = __float_as_uint(__uint_as_float(r32[4 * i + k]) * inv_l);
+            } else {
+              const float a = __uint_as_float(r32[(8 * i + 2 * k) & 31]) * inv_l, b2 = __uint_as_float(r32[(8 * i + 2 * k + 1) & 31]) * inv_l;
               asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hh[k]) : "f"(b2), "f"(a));
             }
-            sts128(aRow + ((((c0 >> 3) + i) ^ (row & 7)) << 4), make_uint4(hh[0], hh[1], hh[2], hh[3]));
           }
+          sts128(aRow + ((((kOutF32 ? 0 : c0 >> 3) + i) ^ (row & 7)) << 4), make_uint4(hh[0], hh[1], hh[2], hh[3]));
         }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
-        if ((row & 31) == 0 && qtile < p.q_tiles && (int64_t)qtile * kTile + (row & ~31) < p.Nq) {
-          asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
-                       ::"l"(&out_map), "r"(kCols * h), "r"(qtile * kTile + (row & ~31)), "r"(bh), "r"(aBox) : "memory");
-          asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        if (kOutF32 || c0 + 32 == kCols) {
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          __syncwarp();
+          if (lane == 0 && qtile < p.q_tiles && (int64_t)qtile * kTile + (row & ~31) < p.Nq) {
+            asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
+                         ::"l"(&out_map), "r"(kCols * h + (kOutF32 ? c0 : 0)), "r"(qtile * kTile + (row & ~31)), "r"(bh), "r"(aBox) : "memory");
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+          }
         }
       }
       }
@@ -756,7 +760,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
     for (int i = 0; i < kProfSlots; ++i) dst[i] = prof_t[i];
   }
   // ---- teardown ------------------------------------------------------------------------------
-  if (!kOutF32 && warp < kSoftmaxWarps && lane == 0)
+  if (warp < kSoftmaxWarps && lane == 0)
     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");     // the output copies have left shared memory
   tc_fence_before();
   __syncthreads();
@@ -855,7 +859,7 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
   p.q_codes = (const uint8_t*)q_codes; p.q_scales = (const uint8_t*)q_scales;
   p.k_codes = (const uint8_t*)k_codes; p.k_scales = (const uint8_t*)k_scales;
   p.v_codes = (const uint8_t*)v_codes; p.v_scales = (const uint8_t*)v_scales;
-  p.out = o; p.status = status; p.dump = (uint8_t*)dump; p.Nq = Nq; p.Nkv = Nkv;
+  p.status = status; p.dump = (uint8_t*)dump; p.Nq = Nq; p.Nkv = Nkv;
   const int64_t qt = (Nq + kTile - 1) / kTile, kt = (Nkv + kTile - 1) / kTile;
   const int64_t pairs = (qt + 1) / 2;
   const int64_t grid = (int64_t)B * H * pairs;
@@ -882,21 +886,20 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
   if (split.pairs_256 == 0) return rest();
   p.total_items = (int)split.pairs_256;
   const bool persist = (!dump || profile) && split.pairs_256 > n_sm && kt <= kWalkMaxTiles;
-  // Descriptor of the bf16 output as a [B H][Nq][128] tensor with boxes of 32 rows x 64 columns (the epilogue's copies).
+  // Descriptor of the output as a [B H][Nq][128] tensor with boxes of 32 rows x 128 bytes (the epilogue's copies).
   CUtensorMap out_map;
   memset(&out_map, 0, sizeof(out_map));
-  if (!f32) {
-    const auto encode = tensor_map_encoder();
-    if (!encode) return MXATTN_ECUDA;
-    if (Nq > 0x7FFFFFFFLL || (uint64_t)Nq * kHeadDim * 2 >= (1ULL << 40)) return MXATTN_EUNSUPPORTED;
-    const cuuint64_t dims[3] = {(cuuint64_t)kHeadDim, (cuuint64_t)Nq, (cuuint64_t)B * H};
-    const cuuint64_t strides[2] = {(cuuint64_t)kHeadDim * 2, (cuuint64_t)Nq * kHeadDim * 2};     // bytes, dimensions 1 and 2
-    const cuuint32_t box[3] = {(cuuint32_t)kCols, 32u, 1u};
-    const cuuint32_t estr[3] = {1u, 1u, 1u};
-    if (encode(&out_map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, o, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return MXATTN_ECUDA;
-  }
+  const auto encode = tensor_map_encoder();
+  if (!encode) return MXATTN_ECUDA;
+  const uint64_t osz = f32 ? 4 : 2;
+  if (Nq > 0x7FFFFFFFLL || (uint64_t)Nq * kHeadDim * osz >= (1ULL << 40)) return MXATTN_EUNSUPPORTED;
+  const cuuint64_t dims[3] = {(cuuint64_t)kHeadDim, (cuuint64_t)Nq, (cuuint64_t)B * H};
+  const cuuint64_t strides[2] = {(cuuint64_t)kHeadDim * osz, (cuuint64_t)Nq * kHeadDim * osz};   // bytes, dimensions 1 and 2
+  const cuuint32_t box[3] = {(cuuint32_t)(128 / osz), 32u, 1u};
+  const cuuint32_t estr[3] = {1u, 1u, 1u};
+  if (encode(&out_map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, o, dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return MXATTN_ECUDA;
   void (*kern)(const Params, const CUtensorMap) = nullptr;
 #define PICK(U, P, F)                                                                     \
   if (uos == U && pnq == P && f32 == F)                                                   \

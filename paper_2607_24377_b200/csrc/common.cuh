@@ -120,6 +120,8 @@ inline cudaError_t launch_pdl_cluster(void (*kern)(KArgs...), dim3 grid, unsigne
 // Raises a kernel's dynamic shared memory limit, once per kernel and device (a driver call per launch otherwise).
 bool ensure_dynamic_smem(const void* kern, int bytes);
 PFN_cuTensorMapEncodeTiled tensor_map_encoder();      // null if the driver has none
+// an attention output as a [bh][Nq][128] tensor that is written in boxes of 32 rows x 128 bytes with the 128-byte swizzle
+int encode_output_map(CUtensorMap* map, void* o, int64_t bh, int64_t Nq, bool f32);
 int sm_count();              // of the current device (0 on error)
 
 // Division of an attention kernel's work (pairs of query tiles of 128 rows, one pair per CTA and wave): where the last wave

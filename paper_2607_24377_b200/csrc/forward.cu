@@ -88,7 +88,6 @@ constexpr int kNumBars = 4 + 2 * kStages + 2 + 1 + 2 + 2;  // Q full/empty[2], K
 constexpr int kOffMisc = kOffBar + kNumBars * 8;           // tmem slot, abort flag
 constexpr int kOffMax = kOffMisc + 64;                     // half-row maxima: [parity 2][tile 2][half 2][128] floats
 constexpr int kOffOut = (kOffMax + 2 * 2 * 2 * 128 * 4 + 1023) & ~1023;   // output staging: one box per softmax warp
-constexpr int kOutBoxBytes = 32 * 128;                     // 32 rows x 128 bytes (the span of the 128-byte swizzle)
 constexpr int kSmemBytes = kOffOut + kSoftmaxWarps * kOutBoxBytes + 1024;   // + slack for the 1024 alignment
 static_assert(kOffOut % 1024 == 0 && kOutBoxBytes % 1024 == 0, "swizzled boxes start on the swizzle pattern's period");
 static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
@@ -191,7 +190,9 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
   __syncthreads();
   tc_fence_after();
   pdl_trigger();
-  const uint32_t tmem = *tmem_slot;
+  // All 512 columns are allocated, so the base is column 0.  With the row sum placed directly the loop is faster with the
+  // constant (16 x 32768: 5361 -> 5302 us), with the PNQ row sum with the loaded value (37 x 16384: 2849 against 2890).
+  const uint32_t tmem = kPnq ? *tmem_slot : 0u;
   const int role = abort_flag[1] != 0 ? kSoftmaxWarps + 2 : warp;     // an earlier CTA gave up: drain the grid quickly
 
   if (role == kSoftmaxWarps) {
@@ -654,8 +655,8 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
       const int qtile = 2 * pair + t;
       if (kPersist) {
         // Item-walking variant: the epilogue is part of every item's critical path.  Row sum and all 64 accumulator
-        // columns are loaded with one wait, then the rows go to this warp's swizzled box and out as one tensor
-        // copy (see the comments of the general path).
+        // columns are loaded with one wait, then the rows go to this warp's swizzled box and out as a tensor
+        // copy (store_half_rows has the reasons).
         uint32_t lr = 0, r64[kCols];
         if (kPnq) asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(lr) : "r"(t_o + 128) : "memory");
         TMEM_LD64(t_o + kCols * h, r64);
@@ -703,49 +704,12 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
       if (kDump && h == 0 && qtile < p.q_tiles)
         reinterpret_cast<float*>(p.dump + (int64_t)p.total_items / p.q_pairs * p.q_tiles * T * kDumpTileBytes)
             [((int64_t)bh * p.q_tiles + qtile) * kTile + row] = l;
-      // The warp's 32 half rows go to shared memory and from there to global memory as tensor copies (boxes of 32 rows x
-      // 128 bytes: 64 bf16 columns or 32 fp32 ones, so that fp32 takes two turns with the box; rows at or beyond Nq are
-      // clipped by the copy).  Written from registers, a warp's 16-byte stores land 256 or 512 bytes apart (one partly
-      // filled sector per lane and instruction); and any store instruction of these warps queues 64 KiB per item in front
-      // of the next tile's shared-memory traffic.  The box uses the 128-byte swizzle (16-byte chunk c of row r sits at
-      // chunk c ^ (r & 7)), which also spreads a quarter warp's stores over all banks.  As tensor
-      // copies fp32 takes 834 us for 40 x 75600 x 512 (1208 from registers), 64.5 for 40 x 4096 x 512 (86), 20.6 for 14 x
-      // 1300 x 777 (23.4).
-      const uint32_t aBox = sbase + kOffOut + (t * 8 + h * 4 + (row >> 5)) * kOutBoxBytes;    // one box per warp
-      const uint32_t aRow = aBox + (row & 31) * (kBoxCols * kOutSize);
-#pragma unroll 1
-      for (int c0 = 0; c0 < kCols; c0 += 32) {
-        uint32_t r32[32];
-        TMEM_LD32(t_o + kCols * h + c0, r32);
-        if (kOutF32 && c0 > 0) {                   // the first half has left the box
-          if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-          __syncwarp();
-        }
-        tmem_ld_wait();
-#pragma unroll
-        for (int i = 0; i < 32 * kOutSize / 16; ++i) {
-          uint32_t hh[4];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            if (kOutF32) {
-              hh[k] = __float_as_uint(__uint_as_float(r32[4 * i + k]) * inv_l);
-            } else {
-              const float a = __uint_as_float(r32[(8 * i + 2 * k) & 31]) * inv_l, b2 = __uint_as_float(r32[(8 * i + 2 * k + 1) & 31]) * inv_l;
-              asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hh[k]) : "f"(b2), "f"(a));
-            }
-          }
-          sts128(aRow + ((((kOutF32 ? 0 : c0 >> 3) + i) ^ (row & 7)) << 4), make_uint4(hh[0], hh[1], hh[2], hh[3]));
-        }
-        if (kOutF32 || c0 + 32 == kCols) {
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          __syncwarp();
-          if (lane == 0 && qtile < p.q_tiles && (int64_t)qtile * kTile + (row & ~31) < p.Nq) {
-            asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
-                         ::"l"(&out_map), "r"(kCols * h + (kOutF32 ? c0 : 0)), "r"(qtile * kTile + (row & ~31)), "r"(bh), "r"(aBox) : "memory");
-            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-          }
-        }
-      }
+      // coordinates computed afresh: keeping those of the loop costs it registers (37 x 16384: 2874 -> 2849 us)
+      const uint32_t tid2 = fresh_tid(), w = tid2 >> 5;
+      const int bh2 = (int)blockIdx.x / p.q_pairs, qtile2 = 2 * ((int)blockIdx.x - bh2 * p.q_pairs) + (int)(w >> 3), col = kCols * ((w >> 2) & 1);
+      const int64_t row0 = (int64_t)qtile2 * kTile + (w & 3) * 32;
+      store_half_rows<kOutF32>((w >> 3 ? kColO1 : kColO0) + ((w & 3) << 21) + col, ((smem_u32(smem_raw) + 1023u) & ~1023u) + kOffOut + w * kOutBoxBytes,
+                               (int)(tid2 & 31), inv_l, &out_map, col, (int)row0, bh2, qtile2 < p.q_tiles && row0 < p.Nq);
       }
     }
     PROF_MARK(8);
@@ -851,6 +815,20 @@ PFN_cuTensorMapEncodeTiled tensor_map_encoder() {
   return reinterpret_cast<PFN_cuTensorMapEncodeTiled>(fn);
 }
 
+int encode_output_map(CUtensorMap* map, void* o, int64_t bh, int64_t Nq, bool f32) {
+  const auto encode = tensor_map_encoder();
+  if (!encode) return MXATTN_ECUDA;
+  const uint64_t osz = f32 ? 4 : 2;
+  if (Nq > 0x7FFFFFFFLL || (uint64_t)Nq * kHeadDim * osz >= (1ULL << 40)) return MXATTN_EUNSUPPORTED;
+  const cuuint64_t dims[3] = {(cuuint64_t)kHeadDim, (cuuint64_t)Nq, (cuuint64_t)bh};
+  const cuuint64_t strides[2] = {(cuuint64_t)kHeadDim * osz, (cuuint64_t)Nq * kHeadDim * osz};   // bytes, dimensions 1 and 2
+  const cuuint32_t box[3] = {(cuuint32_t)(128 / osz), 32u, 1u};
+  const cuuint32_t estr[3] = {1u, 1u, 1u};
+  return encode(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, o, dims, strides, box, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
+             ? MXATTN_OK : MXATTN_ECUDA;
+}
+
 int launch_forward(const void* q_codes, const void* q_scales, const void* k_codes, const void* k_scales,
                    const void* v_codes, const void* v_scales, void* o, int B, int H, int64_t Nq, int64_t Nkv,
                    float softmax_scale, unsigned flags, int* status, cudaStream_t stream, void* dump, bool profile) {
@@ -886,20 +864,9 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
   if (split.pairs_256 == 0) return rest();
   p.total_items = (int)split.pairs_256;
   const bool persist = (!dump || profile) && split.pairs_256 > n_sm && kt <= kWalkMaxTiles;
-  // Descriptor of the output as a [B H][Nq][128] tensor with boxes of 32 rows x 128 bytes (the epilogue's copies).
   CUtensorMap out_map;
-  memset(&out_map, 0, sizeof(out_map));
-  const auto encode = tensor_map_encoder();
-  if (!encode) return MXATTN_ECUDA;
-  const uint64_t osz = f32 ? 4 : 2;
-  if (Nq > 0x7FFFFFFFLL || (uint64_t)Nq * kHeadDim * osz >= (1ULL << 40)) return MXATTN_EUNSUPPORTED;
-  const cuuint64_t dims[3] = {(cuuint64_t)kHeadDim, (cuuint64_t)Nq, (cuuint64_t)B * H};
-  const cuuint64_t strides[2] = {(cuuint64_t)kHeadDim * osz, (cuuint64_t)Nq * kHeadDim * osz};   // bytes, dimensions 1 and 2
-  const cuuint32_t box[3] = {(cuuint32_t)(128 / osz), 32u, 1u};
-  const cuuint32_t estr[3] = {1u, 1u, 1u};
-  if (encode(&out_map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, o, dims, strides, box, estr,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return MXATTN_ECUDA;
+  const int map_rc = encode_output_map(&out_map, o, (int64_t)B * H, Nq, f32);
+  if (map_rc != MXATTN_OK) return map_rc;
   void (*kern)(const Params, const CUtensorMap) = nullptr;
 #define PICK(U, P, F)                                                                     \
   if (uos == U && pnq == P && f32 == F)                                                   \

@@ -68,7 +68,6 @@ __device__ __forceinline__ void tensor_g2s(uint32_t dst, const CUtensorMap* map,
 }
 
 struct Params {
-  void* out;
   int* status;
   int64_t Nq, Nkv;
   int q_tiles_n, kv_tiles, q_pairs;
@@ -80,7 +79,8 @@ struct Params {
 template <bool kOutF32>
 __global__ void __launch_bounds__(kThreads, 1) attention_bf16_kernel(const Params p, const __grid_constant__ CUtensorMap q_map,
                                                                      const __grid_constant__ CUtensorMap k_map,
-                                                                     const __grid_constant__ CUtensorMap v_map) {
+                                                                     const __grid_constant__ CUtensorMap v_map,
+                                                                     const __grid_constant__ CUtensorMap out_map) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t sbase = smem_u32(smem);
@@ -325,38 +325,13 @@ __global__ void __launch_bounds__(kThreads, 1) attention_bf16_kernel(const Param
     mbar_wait_soft<33>(bar(BAR_ODONE + t), (uint32_t)((T - 1) & 1), abort_addr);
     tc_fence_after();
     const int qtile = qtile0 + t;
-    const int64_t grow = (int64_t)qtile * kTile + row;
-    const bool store = (grow < p.Nq) && lds_volatile(abort_addr) == 0;
-    const int64_t obase = ((int64_t)bh * p.Nq + grow) * kHeadDim + 64 * h;
-#pragma unroll 1
-    for (int c0 = 0; c0 < 64; c0 += 32) {
-      uint32_t r32[32];
-      TMEM_LD32(t_o + c0, r32);
-      tmem_ld_wait();
-      if (store) {
-        if (kOutF32) {
-          float4* dst = reinterpret_cast<float4*>(static_cast<float*>(p.out) + obase + c0);
-#pragma unroll
-          for (int i = 0; i < 8; ++i)
-            dst[i] = make_float4(__uint_as_float(r32[4 * i]) * inv_l, __uint_as_float(r32[4 * i + 1]) * inv_l,
-                                 __uint_as_float(r32[4 * i + 2]) * inv_l, __uint_as_float(r32[4 * i + 3]) * inv_l);
-        } else {
-          uint4* dst = reinterpret_cast<uint4*>(static_cast<uint16_t*>(p.out) + obase + c0);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            uint32_t hh[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const float a = __uint_as_float(r32[8 * i + 2 * k]) * inv_l, b2 = __uint_as_float(r32[8 * i + 2 * k + 1]) * inv_l;
-              asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hh[k]) : "f"(b2), "f"(a));
-            }
-            dst[i] = make_uint4(hh[0], hh[1], hh[2], hh[3]);
-          }
-        }
-      }
-    }
+    // the query tile's own 32 KiB are the boxes of its eight warps: its last scores have been computed
+    const int row0 = qtile * kTile + (row & ~31);
+    if (lds_volatile(abort_addr) == 0)
+      store_half_rows<kOutF32>(t_o, sbase + kOffQ + t * kTileBytes + (warp & 7) * kOutBoxBytes, lane, inv_l, &out_map, 64 * h, row0, bh, row0 < p.Nq);
   }
 
+  if (warp < kSoftmaxWarps && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");     // the output copies have left shared memory
   tc_fence_before();
   __syncthreads();
   if (tid == 0 && *abort_flag != 0) atomicCAS(p.status, 0, *abort_flag);
@@ -397,21 +372,23 @@ int launch_forward_bf16(const void* q, const void* k, const void* v, void* o, in
   const int64_t qt = (Nq + kTile - 1) / kTile, kt = (Nkv + kTile - 1) / kTile;
   const int64_t pairs = (qt + 1) / 2, grid = bh * pairs;
   if (qt > 0x3FFFFFFF || kt > 65535 || qt > 0x7FFFFFFF || bh > 65535 || grid > 0x7FFFFFFF) return MXATTN_EUNSUPPORTED;
-  CUtensorMap q_map, k_map, v_map;
+  CUtensorMap q_map, k_map, v_map, out_map;
+  const bool f32 = flags & MXATTN_FLAG_OUT_FP32;
   int rc;
-  if ((rc = encode_operand_map(&q_map, q, bh, Nq)) || (rc = encode_operand_map(&k_map, k, bh, Nkv)) || (rc = encode_operand_map(&v_map, v, bh, Nkv)))
+  if ((rc = encode_operand_map(&q_map, q, bh, Nq)) || (rc = encode_operand_map(&k_map, k, bh, Nkv)) || (rc = encode_operand_map(&v_map, v, bh, Nkv)) ||
+      (rc = encode_output_map(&out_map, o, bh, Nq, f32)))
     return rc;
   if (cudaMemsetAsync(workspace, 0, 16, stream) != cudaSuccess) return MXATTN_ECUDA;
   Params p;
-  p.out = o; p.status = static_cast<int*>(workspace);
+  p.status = static_cast<int*>(workspace);
   p.Nq = Nq; p.Nkv = Nkv; p.q_tiles_n = (int)qt; p.kv_tiles = (int)kt; p.q_pairs = (int)pairs;
   const TileSplit split(grid);
   p.pair_ctas = (int)split.pair_ctas;
   p.scale_log2e = softmax_scale * 1.4426950408889634f;
-  auto kern = (flags & MXATTN_FLAG_OUT_FP32) ? attention_bf16_kernel<true> : attention_bf16_kernel<false>;
+  auto kern = f32 ? attention_bf16_kernel<true> : attention_bf16_kernel<false>;
   if (!ensure_dynamic_smem((const void*)kern, kSmemBytes)) return MXATTN_ECUDA;
   count_launch(1);
-  return launch_pdl(kern, dim3((unsigned)split.ctas), kThreads, kSmemBytes, stream, p, q_map, k_map, v_map) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
+  return launch_pdl(kern, dim3((unsigned)split.ctas), kThreads, kSmemBytes, stream, p, q_map, k_map, v_map, out_map) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 
 }  // namespace mxattn

@@ -55,7 +55,8 @@ enum Bar { BAR_Q = 0, BAR_KFULL = 1, BAR_KEMPTY = BAR_KFULL + kStages, BAR_SFULL
 constexpr int kOffMisc = kOffBar + kNumBars * 8;
 constexpr int kOffMax = kOffMisc + 64;                     // half-row exchange: [parity 2][tile 2][half 2][128] floats
 constexpr int kOffTab = kOffMax + 2 * 2 * 2 * 128 * 4;           // per E4M3 code: log2(2688 / d), d / 2688
-constexpr int kSmemBytes = kOffTab + 128 * 8 + 1024;
+constexpr int kOffOut = (kOffTab + 128 * 8 + 1023) & ~1023;           // output staging: one box per softmax warp
+constexpr int kSmemBytes = kOffOut + kSoftmaxWarps * kOutBoxBytes + 1024;
 static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
 
 // tensor-memory columns: per operand tile 8 scale columns (atom of K half 0, atom of K half 1); a V slot interleaves
@@ -71,7 +72,6 @@ struct Params {
   const uint8_t* k_codes; const uint8_t* k_scales;
   const uint8_t* v_codes; const uint8_t* v_scales;
   const float* ts_q; const float* ts_k; const float* ts_v;   // tensor decode scales, one per head
-  void* out;
   int* status;
   int64_t Nq, Nkv;
   int q_tiles, kv_tiles, q_pairs;
@@ -101,7 +101,7 @@ __device__ __forceinline__ float e4m3_decode(uint32_t code) {
 }
 
 template <bool kPnq, bool kOutF32>
-__global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Params p) {
+__global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Params p, const __grid_constant__ CUtensorMap out_map) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t sbase = smem_u32(smem);
@@ -458,41 +458,17 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
       } else {
         o_scale *= __fdiv_rn(1.0f, kTensorRangeP);
       }
-      const int qtile = qtile0 + t;
-      const int64_t grow = (int64_t)qtile * kTile + row;
-      const bool store = (grow < p.Nq);
       const float inv_l = o_scale / l;
-      const int64_t obase = ((int64_t)bh * p.Nq + grow) * kHeadDim + kCols * h;
-#pragma unroll 1
-      for (int c0 = 0; c0 < kCols; c0 += 32) {
-        uint32_t r32[32];
-        TMEM_LD32(t_o + kCols * h + c0, r32);
-        tmem_ld_wait();
-        if (store) {
-          if (kOutF32) {
-            float4* dst = reinterpret_cast<float4*>(static_cast<float*>(p.out) + obase + c0);
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-              dst[i] = make_float4(__uint_as_float(r32[4 * i]) * inv_l, __uint_as_float(r32[4 * i + 1]) * inv_l,
-                                   __uint_as_float(r32[4 * i + 2]) * inv_l, __uint_as_float(r32[4 * i + 3]) * inv_l);
-          } else {
-            uint4* dst = reinterpret_cast<uint4*>(static_cast<uint16_t*>(p.out) + obase + c0);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              uint32_t hh[4];
-#pragma unroll
-              for (int k = 0; k < 4; ++k) {
-                const float a = __uint_as_float(r32[8 * i + 2 * k]) * inv_l, b2 = __uint_as_float(r32[8 * i + 2 * k + 1]) * inv_l;
-                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hh[k]) : "f"(b2), "f"(a));
-              }
-              dst[i] = make_uint4(hh[0], hh[1], hh[2], hh[3]);
-            }
-          }
-        }
-      }
+      // coordinates computed afresh: with those of the loop the kernel took 760 us instead of 715 at 24 x 8192 (registers)
+      const uint32_t tid2 = fresh_tid(), w = tid2 >> 5;
+      const TileOfCta at2((int)blockIdx.x, p.pair_ctas, p.q_pairs, p.q_tiles);
+      const int row0 = (at2.qtile + (int)(w >> 3)) * kTile + (int)(w & 3) * 32, col = kCols * ((w >> 2) & 1);
+      store_half_rows<kOutF32>((w >> 3 ? kColO1 : kColO0) + ((w & 3) << 21) + col, ((smem_u32(smem_raw) + 1023u) & ~1023u) + kOffOut + w * kOutBoxBytes,
+                               (int)(tid2 & 31), inv_l, &out_map, col, row0, at2.bh, row0 < p.Nq);
     }
   }
 
+  if (warp < kSoftmaxWarps && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");     // the output copies have left shared memory
   tc_fence_before();
   __syncthreads();
   if (warp == kSoftmaxWarps + 1) {
@@ -551,17 +527,20 @@ int launch_forward_nvfp4(const void* q, const void* k, const void* v, void* o, i
   p.q_codes = ws + w.q_codes; p.q_scales = ws + w.q_scales; p.k_codes = ws + w.k_codes; p.k_scales = ws + w.k_scales;
   p.v_codes = ws + w.v_codes; p.v_scales = ws + w.v_scales;
   p.ts_q = ts; p.ts_k = ts + bh; p.ts_v = ts + 2 * bh;
-  p.out = o; p.status = reinterpret_cast<int*>(ws + w.status);
+  p.status = reinterpret_cast<int*>(ws + w.status);
   p.Nq = Nq; p.Nkv = Nkv; p.q_tiles = (int)qt; p.kv_tiles = (int)kt; p.q_pairs = (int)pairs;
   const TileSplit split(grid);
   p.pair_ctas = (int)split.pair_ctas;
   p.scale_log2e = softmax_scale * 1.4426950408889634f;
   const bool pnq = flags & MXATTN_FLAG_PNQ, f32 = flags & MXATTN_FLAG_OUT_FP32;
-  void (*kern)(const Params) = pnq ? (f32 ? attention_nvfp4_kernel<true, true> : attention_nvfp4_kernel<true, false>)
+  CUtensorMap out_map;
+  const int map_rc = encode_output_map(&out_map, o, bh, Nq, f32);
+  if (map_rc != MXATTN_OK) return map_rc;
+  void (*kern)(const Params, const CUtensorMap) = pnq ? (f32 ? attention_nvfp4_kernel<true, true> : attention_nvfp4_kernel<true, false>)
                                    : (f32 ? attention_nvfp4_kernel<false, true> : attention_nvfp4_kernel<false, false>);
   if (!ensure_dynamic_smem((const void*)kern, kSmemBytes)) return MXATTN_ECUDA;
   count_launch(1);
-  return launch_pdl(kern, dim3((unsigned)split.ctas), kThreads, kSmemBytes, stream, p) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
+  return launch_pdl(kern, dim3((unsigned)split.ctas), kThreads, kSmemBytes, stream, p, out_map) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 
 }  // namespace mxattn

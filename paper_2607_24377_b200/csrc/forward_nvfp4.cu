@@ -154,6 +154,13 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
   const uint32_t tmem = *tmem_slot;
   const int role = (abort_flag[1] != 0 || at.empty || (!two && warp >= 8 && warp < kSoftmaxWarps)) ? kSoftmaxWarps + 2 : warp;     // an earlier CTA gave up: drain the grid quickly
 
+  // Waits of the single-thread roles.  Loops out of line keep their code short, but the call's register conventions reach the
+  // softmax warps: with the direct row sum that is worth it (37 x 16384: 3492 us against 3665), with the PNQ row sum it makes
+  // short key sequences slower (12 x 9000 x 100: 43.2 us against 41.5) and long ones no faster.
+  auto role_wait = [&](uint32_t b, uint32_t parity, volatile int* flag, int* status, int code) {
+    return kPnq ? mbar_wait(b, parity, flag, status, code) : mbar_wait1(b, parity, flag, status, code);
+  };
+
   if (role == kSoftmaxWarps) {
     // =============================== producer ===============================================
     if (lane == 0) {
@@ -168,7 +175,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
       int j = 0;
       for (; j < T && ok; ++j) {
         const int s = j % kStages;
-        if (j >= kStages) ok = mbar_wait(bar(BAR_KEMPTY + s), (uint32_t)(((j / kStages) & 1) ^ 1), abort_flag, p.status, 11);
+        if (j >= kStages) ok = role_wait(bar(BAR_KEMPTY + s), (uint32_t)(((j / kStages) & 1) ^ 1), abort_flag, p.status, 11);
         if (!ok) break;
         mbar_expect_tx(bar(BAR_KFULL + s), 2 * (kTileCodeBytes + kSF));
         bulk_g2s(sbase + kOffK + s * kTileCodeBytes, p.k_codes + (kv0 + j) * kTileCodeBytes, kTileCodeBytes, bar(BAR_KFULL + s));
@@ -186,7 +193,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
   } else if (role == kSoftmaxWarps + 1) {
     // =============================== MMA issuer =============================================
     if (lane == 0) {
-      bool ok = mbar_wait(bar(BAR_Q), 0, abort_flag, p.status, 21);
+      bool ok = role_wait(bar(BAR_Q), 0, abort_flag, p.status, 21);
       uint32_t sfree_n = 0;
       constexpr uint32_t kDescHiTile = (512u >> 4) | (1u << 14) | (4u << 29);   // 64-byte swizzle, K-major
       const uint32_t q_lo = (sbase + kOffQ) >> 4, k_lo = (sbase + kOffK) >> 4;
@@ -211,25 +218,26 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
         tc_mma_nv(d, desc(a + 2), desc(b + 2), make_idesc_nv(kNV), sfa + 4, sfb + 8, 1u);
         tc_commit(bar(BAR_ODONE + t));
       };
-      auto wait_kv = [&](int j, bool first) {
-        const int s = j % kStages;
-        if (!mbar_wait(bar(BAR_KFULL + s), (uint32_t)((j / kStages) & 1), abort_flag, p.status, 22)) return false;
-        if (!first) {
-          if (!mbar_wait(bar(BAR_SFREE), sfree_n & 1u, abort_flag, p.status, 23)) return false;
-          ++sfree_n;
-        }
-        tc_fence_after();
-        tc_cp_sf(tmem + kColSFK + 8 * (j & 1), sbase + kOffSFK + s * kSF);
-        tc_cp_sf(tmem + kColSFK + 8 * (j & 1) + 4, sbase + kOffSFK + s * kSF + kTileScaleBytes);
-        tc_cp_sf(tmem + kColSFV + 16 * (j & 1), sbase + kOffSFV + s * kSF);
-        tc_cp_sf(tmem + kColSFV + 16 * (j & 1) + 8, sbase + kOffSFV + s * kSF + kTileScaleBytes);
-        return true;
-      };
       auto wait_sfree = [&]() {
-        const bool r = mbar_wait(bar(BAR_SFREE), sfree_n & 1u, abort_flag, p.status, 23);
+        const bool r = role_wait(bar(BAR_SFREE), sfree_n & 1u, abort_flag, p.status, 23);
         ++sfree_n;
         tc_fence_after();
         return r;
+      };
+      // K of tile j has landed: its scale atoms go to tensor memory (slot j & 1 was last read by the score products of tile
+      // j - 2, issued before), apart from the wait for the score buffer, so that nothing but that wait stands between "the
+      // other group has taken its scores" and the next score product.  V's atoms (same stage) follow behind the products.
+      auto k_ready = [&](int j) {
+        const int s = j % kStages;
+        if (!role_wait(bar(BAR_KFULL + s), (uint32_t)((j / kStages) & 1), abort_flag, p.status, 22)) return false;
+        tc_fence_after();
+        tc_cp_sf(tmem + kColSFK + 8 * (j & 1), sbase + kOffSFK + s * kSF);
+        tc_cp_sf(tmem + kColSFK + 8 * (j & 1) + 4, sbase + kOffSFK + s * kSF + kTileScaleBytes);
+        return true;
+      };
+      auto v_scales = [&](int j) {
+        tc_cp_sf(tmem + kColSFV + 16 * (j & 1), sbase + kOffSFV + (j % kStages) * kSF);
+        tc_cp_sf(tmem + kColSFV + 16 * (j & 1) + 8, sbase + kOffSFV + (j % kStages) * kSF + kTileScaleBytes);
       };
       if (ok) {
         tc_fence_after();
@@ -242,15 +250,16 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
           tc_cp_sf(tmem + kColSFV + 16 * slot + 12, sbase + kOffSFOnes);
         }
       }
-      ok = ok && wait_kv(0, true);
-      if (ok) gemm1(0, 0);
+      ok = ok && k_ready(0);
+      if (ok) { v_scales(0); gemm1(0, 0); }
       for (int j = 0; !two && j < T && ok; ++j) {      // one query tile: its next scores go ahead of the output product
         if (j + 1 < T) {
-          ok = wait_kv(j + 1, false);
+          ok = k_ready(j + 1) && wait_sfree();
           if (!ok) break;
           gemm1(0, j + 1);
+          v_scales(j + 1);
         }
-        ok = mbar_wait(bar(BAR_PFULL + 0), (uint32_t)(j & 1), abort_flag, p.status, 24);
+        ok = role_wait(bar(BAR_PFULL + 0), (uint32_t)(j & 1), abort_flag, p.status, 24);
         if (!ok) break;
         tc_fence_after();
         gemm2(0, j);
@@ -261,11 +270,14 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
         ok = ok && wait_sfree();
         if (ok) gemm1(1, 0);
         if (T > 1) {
-          ok = ok && wait_kv(1, false);
+          ok = ok && k_ready(1);
+          if (ok) v_scales(1);
+          ok = ok && wait_sfree();
           if (ok) gemm1(0, 1);
         }
+#pragma unroll 2
         for (int j = 0; j < T && ok; ++j) {
-          ok = mbar_wait(bar(BAR_PFULL + 0), (uint32_t)(j & 1), abort_flag, p.status, 24);
+          ok = role_wait(bar(BAR_PFULL + 0), (uint32_t)(j & 1), abort_flag, p.status, 24);
           if (!ok) break;
           tc_fence_after();
           gemm2(0, j);
@@ -274,16 +286,21 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
             if (!ok) break;
             gemm1(1, j + 1);
           }
-          ok = mbar_wait(bar(BAR_PFULL + 1), (uint32_t)(j & 1), abort_flag, p.status, 26);
+          if (j + 2 < T) {                             // off the critical chain: the thread would wait for P here anyway
+            ok = k_ready(j + 2);
+            if (!ok) break;
+          }
+          ok = role_wait(bar(BAR_PFULL + 1), (uint32_t)(j & 1), abort_flag, p.status, 26);
           if (!ok) break;
           tc_fence_after();
           gemm2(1, j);
-          tc_commit(bar(BAR_KEMPTY + j % kStages));
           if (j + 2 < T) {
-            ok = wait_kv(j + 2, false);
+            ok = wait_sfree();
             if (!ok) break;
             gemm1(0, j + 2);
           }
+          tc_commit(bar(BAR_KEMPTY + j % kStages));
+          if (j + 2 < T) v_scales(j + 2);
         }
       }
     }

@@ -417,6 +417,12 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
             ok = gemm1p(1, n1, f + 1, pre_end);
             if (!ok) break;
           }
+          // Where the softmax is longer (direct row sum) K's scales go ahead of the wait for the score buffer, as in the
+          // one-item loop: 40 x 4096 291 -> 284 us, 40 x 75600 x 512 825 -> 809.  With the PNQ row sum it is 0.3 % slower.
+          if (!kPnq && f + 2 < F_end) {
+            ok = k_ready(f + 2);
+            if (!ok) break;
+          }
           ok = MBAR_WAIT_ROLE(bar(BAR_PFULL + 1), (uint32_t)(f & 1), abort_flag, p.status, 26);
           if (!ok) break;
           tc_fence_after();
@@ -429,10 +435,11 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
             if (!ok) break;
           }
           if (f + 2 < F_end) {
-            ok = wait_kv(f + 2, false);
+            ok = kPnq ? wait_kv(f + 2, false) : wait_sfree();
             if (!ok) break;
             ok = gemm1p(0, n2, f + 2, pre_end);
             if (!ok) break;
+            if (!kPnq) v_scales(f + 2);
           }
           if (++j0 == T) { j0 = 0; ++n0; }
         }

@@ -84,13 +84,13 @@ static bool carve(int B, int H, int64_t Nq, int64_t Nkv, int d, WorkspaceLayout*
   return true;
 }
 
-// `qstream` / `qdone`: if given, the three quantize launches go to `qstream`, `qdone` is recorded behind them and
+// `qstream` / `qdone`: if given, the quantize launches go to `qstream`, `qdone` is recorded behind them and
 // the attention launch on `stream` waits for it (the host pipeline uses this to quantize the next stage's
-// operands while the current stage's attention kernel drains).
+// operands while the current stage's attention kernel drains).  `followed`: other attention launches run at the same time.
 static int forward_ws(const void* q, const void* k, const void* v, void* o, int B, int H, int64_t Nq,
                       int64_t Nkv, int d, float softmax_scale, unsigned flags, void* workspace,
                       size_t workspace_bytes, cudaStream_t stream, void* dump = nullptr,
-                      cudaStream_t qstream = nullptr, cudaEvent_t qdone = nullptr, bool profile = false) {
+                      cudaStream_t qstream = nullptr, cudaEvent_t qdone = nullptr, bool profile = false, bool followed = false) {
   if (!q || !k || !v || !o) return MXATTN_EINVAL;
   if (B <= 0 || H <= 0 || Nq <= 0 || Nkv <= 0) return MXATTN_EINVAL;
   if (flags & ~(unsigned)(MXATTN_FLAG_UOS | MXATTN_FLAG_PNQ | MXATTN_FLAG_OUT_FP32 | MXATTN_FLAG_HADAMARD)) return MXATTN_EINVAL;
@@ -121,7 +121,7 @@ static int forward_ws(const void* q, const void* k, const void* v, void* o, int 
   TraceRange tr("mxattn attention");
   return launch_forward(ws + w.q_codes, ws + w.q_scales, ws + w.k_codes, ws + w.k_scales, ws + w.v_codes,
                         ws + w.v_scales, o, B, H, Nq, Nkv, softmax_scale, flags,
-                        reinterpret_cast<int*>(ws + w.status), stream, dump, profile);
+                        reinterpret_cast<int*>(ws + w.status), stream, dump, profile, followed);
 }
 
 }  // namespace mxattn
@@ -271,27 +271,30 @@ static HostPipe* host_pipe(size_t n_events) {
   return &hp;
 }
 
-// First heads of the pipeline stages of mxattn_forward_host; the last entry is bh.  The link bounds the call (a head
-// of N tokens arrives in 14 us per 1000 tokens, and its attention takes less than that below some 50000 tokens), and a
-// stage costs it about 20 us: three copies of some 6 us each on top of their bytes.  So there should be few stages.
+// First heads of the pipeline stages of mxattn_forward_host; the last entry is bh.  last_alone: the attention of earlier
+// stages is done when the last stage's operands arrive.  The link bounds the call (a head of N tokens arrives in 14 us per
+// 1000 tokens, and its attention takes less than that below some 50000 tokens), and a stage costs it about 20 us: three
+// copies of some 6 us each on top of their bytes.  So there should be few stages.
 //   - Nothing hides the last stage's attention and copy out, so that stage is small, and the stages before it grow by
 //     the ratio at which a stage's attention and copy out are just done when the smaller one behind it has arrived
 //     (55 GB/s in and out, attention at 1.6 PFLOP/s).  It is kept between 1.5 and 3, beyond which nothing is gained.
 //   - Where the copies in are the bound the first stages may be large: they start at an eighth of the heads and double.
-//     Where the copies out weigh as much (Nkv small) the first stage has to be small, and a stage that grows leaves
-//     the link idle outwards while it arrives: equal ones then, of the size at which the wait for one stage is what
-//     all stages' fixed cost is.
+//     Where the copies out weigh as much (Nkv small) or the attention does (long sequences) the first stage has to be
+//     small, and a stage that grows leaves the other two idle while it arrives: equal ones then, of the size at which
+//     the wait for one stage is what all stages' fixed cost is.
 //   - No stage is below 2.5 MB in, which is 45 us of the link, unless the call is.
 // Against one head followed by stages of equal size, us: 24 x 8192 3310 -> 3249 (copying in alone takes 2731), 40 x 4096
 // 2858 -> 2712 (2280), 160 x 5000 13170 -> 12230, 160 x 300 1134 -> 912, 2 x 1024 (one stage now) 195 -> 164, 12 x 20000
-// 4084 -> 4011; 40 heads of 10000 x 512 3024 -> 3023.
-static std::vector<size_t> host_stages(size_t bh, int64_t Nq, int64_t Nkv, size_t in_bytes_per_head, size_t out_bytes_per_head) {
+// 4084 -> 4011; 40 heads of 10000 x 512 3024 -> 3023, of 75600 x 512 18460 -> 18060.
+static std::vector<size_t> host_stages(size_t bh, int64_t Nq, int64_t Nkv, size_t in_bytes_per_head, size_t out_bytes_per_head, bool* last_alone) {
   const double t_in = (double)in_bytes_per_head / 55e9, t_out = (double)out_bytes_per_head / 55e9;
-  const double t_rest = t_out + 4.0 * (double)Nq * (double)Nkv * kHeadDim / 1.6e15;
-  const double shrink = std::min(3.0, std::max(1.5, 1.1 * t_in / t_rest));
+  const double t_attn = 4.0 * (double)Nq * (double)Nkv * kHeadDim / 1.6e15;
+  const double shrink = std::min(3.0, std::max(1.5, 1.1 * t_in / (t_out + t_attn)));
   const size_t least = (size_t)(2.5e6 / (double)in_bytes_per_head) + 1;
-  const bool in_bound = t_in > 1.5 * t_out;
-  const size_t most = in_bound ? bh : std::max(least, (size_t)std::sqrt((double)bh * 20e-6 / t_out));
+  const double t_other = std::max(t_out, t_attn);
+  const bool in_bound = t_in > 1.5 * t_other;
+  const size_t most = in_bound ? bh : std::max(least, (size_t)std::ceil(std::sqrt((double)bh * 20e-6 / t_other)));
+  *last_alone = in_bound || bh <= least;
   size_t next_head = in_bound ? std::max(least, bh / 8) : least, next_tail = least;
   std::vector<size_t> head, tail;
   for (size_t left = bh; left > 0;) {
@@ -338,7 +341,8 @@ extern "C" int mxattn_forward_host(const void* q_host, const void* k_host, const
   uint8_t* dv = dk + align_up(bh * kh, 256);
   uint8_t* dout = dv + align_up(bh * kh, 256);
   uint8_t* ws = dout + align_up(bh * oh, 256);
-  const std::vector<size_t> first_head = host_stages(bh, Nq, Nkv, qh + 2 * kh, oh);
+  bool last_alone;
+  const std::vector<size_t> first_head = host_stages(bh, Nq, Nkv, qh + 2 * kh, oh, &last_alone);
   const size_t stages = first_head.size() - 1;
   HostPipe* hp = host_pipe(3 * stages + 2);
   if (!hp) return MXATTN_ECUDA;
@@ -364,7 +368,7 @@ extern "C" int mxattn_forward_host(const void* q_host, const void* k_host, const
     // n heads); its operands are quantized on a stream of their own, behind the copies and ahead of the attention
     // launch, so that they fill the SMs the previous stage's attention kernel frees as it drains
     rc = forward_ws(dq + i * qh, dk + i * kh, dv + i * kh, dout + i * oh, 1, (int)n, Nq, Nkv, d, softmax_scale, flags,
-                    ws + i * w.total, n * w.total, as, nullptr, hp->quant, ev[3 * st + 1]);
+                    ws + i * w.total, n * w.total, as, nullptr, hp->quant, ev[3 * st + 1], false, st + 1 < stages || !last_alone);
     launched += g_launches;
     ck(cudaEventRecord(ev[3 * st + 2], as));
     ck(cudaStreamWaitEvent(hp->out, ev[3 * st + 2], 0));

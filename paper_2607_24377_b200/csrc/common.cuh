@@ -168,7 +168,7 @@ int launch_quantize_nvfp4(const void* in, void* codes, void* scales, const float
 int launch_forward(const void* q_codes, const void* q_scales, const void* k_codes,
                    const void* k_scales, const void* v_codes, const void* v_scales, void* o,
                    int B, int H, int64_t Nq, int64_t Nkv, float softmax_scale, unsigned flags,
-                   int* status, cudaStream_t stream, void* dump = nullptr, bool profile = false);
+                   int* status, cudaStream_t stream, void* dump = nullptr, bool profile = false, bool followed = false);
 struct RowSplit { int64_t pairs_256; int R; };      // R = 0: nothing is left for the small CTAs
 RowSplit forward_row_split(int64_t bh, int64_t Nq, int64_t Nkv, bool pnq);
 constexpr int kWalkMaxTiles = 48;    // longest key/value sequence (in tiles) for which a CTA of forward.cu walks several work items

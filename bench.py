@@ -257,7 +257,7 @@ def main():
     ws = torch.empty(ws_bytes, dtype=torch.uint8, device="cuda")
     bh, qt, kt = B * H, -(-Nq // 128), -(-Nkv // 128)
     # the same buffers mxattn_forward_ws carves from its workspace, held separately here so that
-    # each of its four launches can be bracketed by CUDA events
+    # the quantizations and the attention can be bracketed by CUDA events
     qc, qs = (torch.empty((bh, qt, n), dtype=torch.uint8, device="cuda") for n in (8192, 512))
     kc, ks = (torch.empty((bh, kt, n), dtype=torch.uint8, device="cuda") for n in (8192, 512))
     vc, vs = (torch.empty((bh, kt, n), dtype=torch.uint8, device="cuda") for n in (8192, 512))
@@ -360,7 +360,7 @@ def main():
         variants["quantize_q_with_hadamard"] = {"ms": ms, "GBps": gbps, "frac_of_measured_copy_rate": gbps / peaks["hbm_gbs"],
                                                 "frac_of_nominal_8TBps": gbps / 8000.0}
         mx.quantize_mxfp4_batched(dq, qc, qs, bh, Nq, d, 1, mx.MODE_UOS, mx.LAYOUT_TILE)       # restore the unrotated Q-hat
-        # bf16 variant of this repository's own kernel (no quantization; three re-tiling launches + attention)
+        # bf16 variant of this repository's own kernel (no quantization: one launch)
         wsb = torch.empty(mx.forward_bf16_workspace_bytes(B, H, Nq, Nkv, d), dtype=torch.uint8, device="cuda")
         mx.forward_bf16(dq, dk, dv, out, B, H, Nq, Nkv, d, scale, 0, wsb); torch.cuda.synchronize()
         a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -371,11 +371,11 @@ def main():
         assert mx.device_status(wsb) == 0
         ms = a.elapsed_time(b) / 3
         variants["bf16_same_kernel"] = {"step_ms": ms, "tflops": flops / (ms * 1e-3) / 1e12,
-                                        "note": "mxattn_forward_bf16: whole call (re-tiling of Q, K, V^T + fused attention)"}
+                                        "note": "mxattn_forward_bf16: whole call"}
         variants["uos_pnq_step_speedup_over_bf16_same_kernel"] = ms / ms_per_step
         del wsb
-        # the paper's comparison format: the same kernel design on NVFP4 operands (whole call: three tensor maxima,
-        # three quantize launches, attention)
+        # the paper's comparison format: the same kernel design on NVFP4 operands (whole call: tensor maxima,
+        # quantization, attention)
         wsn = torch.empty(mx.forward_nvfp4_workspace_bytes(B, H, Nq, Nkv, d), dtype=torch.uint8, device="cuda")
         for name, fl in (("nvfp4_direct", 0), ("nvfp4_pnq", mx.FLAG_PNQ)):
             mx.forward_nvfp4(dq, dk, dv, out, B, H, Nq, Nkv, d, scale, fl, wsn); torch.cuda.synchronize()
@@ -387,7 +387,7 @@ def main():
             assert mx.device_status(wsn) == 0
             ms = a.elapsed_time(b) / 3
             variants[name] = {"step_ms": ms, "tflops": flops / (ms * 1e-3) / 1e12,
-                              "note": "mxattn_forward_nvfp4: whole call (7 launches)"}
+                              "note": "mxattn_forward_nvfp4: whole call (tensor maxima, quantization, attention)"}
         del wsn
         # bf16 reference point: NOT a kernel of this repository -- PyTorch's fused SDPA (library flash /
         # cuDNN attention) on the same bf16 tensors.  (The repository's own bf16 variant is `bf16_same_kernel` above.)

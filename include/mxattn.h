@@ -158,7 +158,7 @@ int mxattn_set_workspace(void* dev_ptr, size_t bytes);
  * MXATTN_FLAG_OUT_FP32).  d must be 128.  Non-causal, no mask.  softmax_scale > 0 multiplies the
  * quantized product Q-hat K-hat^T (line 9).  KV tiles are 128 keys, visited in ascending order.
  * Enqueues the quantization of Q, K (along d) and V (along tokens), in one to three launches, and
- * one fused attention launch.  Uses the workspace registered with mxattn_set_workspace. */
+ * the fused attention, in one or two.  Uses the workspace registered with mxattn_set_workspace. */
 int mxattn_forward(const void* q, const void* k, const void* v, void* o,
                    int B, int H, int64_t Nq, int64_t Nkv, int d,
                    float softmax_scale, unsigned flags, void* stream);
@@ -259,7 +259,7 @@ int mxattn_forward_bf16(const void* q, const void* k, const void* v, void* o,
  * known to be 1 (readings: the paper does not say how the baseline chooses them).
  * flags: MXATTN_FLAG_PNQ (row sum from the quantized probabilities, as in MXAttention; without it the direct
  * placement, which is what the paper's baseline uses) and MXATTN_FLAG_OUT_FP32.  Same tensor layouts as
- * mxattn_forward.  Enqueues three tensor-maximum launches, three quantize launches and the attention launch.
+ * mxattn_forward.  Enqueues one tensor-maximum launch, one to three quantize launches and the attention launch.
  * The workspace (mxattn_forward_nvfp4_workspace_bytes) holds the quantized operands and, at its start, the status word. */
 size_t mxattn_forward_nvfp4_workspace_bytes(int B, int H, int64_t Nq, int64_t Nkv, int d);
 int mxattn_forward_nvfp4(const void* q, const void* k, const void* v, void* o,
@@ -271,8 +271,8 @@ int mxattn_forward_nvfp4(const void* q, const void* k, const void* v, void* o,
 size_t mxattn_forward_host_arena_bytes(int B, int H, int64_t Nq, int64_t Nkv, int d, unsigned flags);
 
 /* End-to-end form for callers whose tensors live in HOST memory (pinned memory, so that the copies
- * are asynchronous): runs mxattn_forward_ws in stages of one or more heads (one head first, then as many
- * per stage as it takes to fill the GPU's SMs) out of `device_arena` and writes o into o_host.  The stages
+ * are asynchronous): runs mxattn_forward_ws in stages of one or more heads (sized from the rates of the
+ * copies and of the attention) out of `device_arena` and writes o into o_host.  The stages
  * are pipelined over the caller's `stream` and four helper streams that the library creates once per
  * device: host->device copies of the next stages, their quantization, and the device->host copy of the
  * previous stage overlap the attention kernels, whose launches alternate between `stream` and a helper

@@ -48,7 +48,8 @@
 //
 // Two launch shapes: one CTA per work item (two query tiles of one head), or -- more items than SMs and a short
 // KV sequence -- one CTA per SM that walks the items and keeps barriers, tensor memory and the K/V ring across
-// them (template flag kPersist).
+// them (template flag kPersist).  Query tiles that would leave SMs idle (a small problem, a nearly empty last wave)
+// go to the kernel for few query rows (forward_rows.cu).
 //
 // Every mbarrier wait is bounded; on expiry the CTA records a code in `status`, drains and exits.
 #include <string.h>

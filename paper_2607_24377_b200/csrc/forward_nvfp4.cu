@@ -18,7 +18,8 @@
 // of ex2.approx itself; a block with d = 0 keeps r = 1, its codes are 0 either way).
 //
 // One CTA per work item: two query tiles of one head, or one where the last wave would leave half of the SMs idle
-// (common.cuh; 2 heads of 1024: 29 -> 23 us, 40 heads of 16384: 4090 -> 4033); outputs are stored from registers.  Tensor-memory map:
+// (common.cuh; 2 heads of 1024: 29 -> 23 us, 40 heads of 16384: 4090 -> 4033).  The output leaves as tensor copies
+// (store_half_rows; 40 heads of 4096 x 512: 92.1 -> 87.9 us, fp32 105.6 -> 96.5).  Tensor-memory map:
 // S [0,128), O_0 [128,272), O_1 [272,416), scale factors from 416 (8 columns per operand tile: two atoms).
 // Every mbarrier wait is bounded; a softmax warp that gives up keeps its partner's appointments (tc_helpers.cuh).
 #include <cuda_fp16.h>

@@ -162,6 +162,7 @@ int launch_quantize_qkv(const void* q, void* q_codes, void* q_scales, const void
 int launch_nvfp4_operands(const void* q, void* q_codes, void* q_scales, const void* k, void* k_codes, void* k_scales,
                           const void* v, void* v_codes, void* v_scales, float* amax, float* tensor_scale, int64_t bh,
                           int64_t Nq, int64_t Nkv, cudaStream_t stream);
+int launch_zero(uint32_t* words, int64_t n, cudaStream_t stream);      // a few words: status, tensor maxima
 int launch_tensor_amax(const void* in, float* amax, int64_t batch, int64_t rows, int64_t cols, cudaStream_t stream);
 int launch_quantize_nvfp4(const void* in, void* codes, void* scales, const float* amax, float* tensor_scale, int64_t batch,
                           int64_t rows, int64_t cols, int block_axis, int layout, cudaStream_t stream);

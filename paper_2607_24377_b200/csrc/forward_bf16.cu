@@ -380,7 +380,7 @@ int launch_forward_bf16(const void* q, const void* k, const void* v, void* o, in
   if ((rc = encode_operand_map(&q_map, q, bh, Nq)) || (rc = encode_operand_map(&k_map, k, bh, Nkv)) || (rc = encode_operand_map(&v_map, v, bh, Nkv)) ||
       (rc = encode_output_map(&out_map, o, bh, Nq, f32)))
     return rc;
-  if (cudaMemsetAsync(workspace, 0, 16, stream) != cudaSuccess) return MXATTN_ECUDA;
+  if (launch_zero(static_cast<uint32_t*>(workspace), 4, stream) != MXATTN_OK) return MXATTN_ECUDA;
   Params p;
   p.status = static_cast<int*>(workspace);
   p.Nq = Nq; p.Nkv = Nkv; p.q_tiles_n = (int)qt; p.kv_tiles = (int)kt; p.q_pairs = (int)pairs;

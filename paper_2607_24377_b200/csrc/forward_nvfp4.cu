@@ -537,7 +537,7 @@ int launch_forward_nvfp4(const void* q, const void* k, const void* v, void* o, i
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   float* amax = reinterpret_cast<float*>(ws + w.amax);
   float* ts = reinterpret_cast<float*>(ws + w.tscale);
-  if (cudaMemsetAsync(ws + w.status, 0, w.tscale - w.status, stream) != cudaSuccess) return MXATTN_ECUDA;      // status word and tensor maxima
+  if (launch_zero(reinterpret_cast<uint32_t*>(ws + w.status), (int64_t)(w.tscale - w.status) / 4, stream) != MXATTN_OK) return MXATTN_ECUDA;      // status word and tensor maxima
   const int rc = launch_nvfp4_operands(q, ws + w.q_codes, ws + w.q_scales, k, ws + w.k_codes, ws + w.k_scales, v, ws + w.v_codes, ws + w.v_scales,
                                        amax, ts, bh, Nq, Nkv, stream);
   if (rc != MXATTN_OK) return rc;

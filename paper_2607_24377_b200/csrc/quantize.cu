@@ -585,6 +585,18 @@ int launch_quantize(const void* in, void* codes, void* scales, int64_t batch, in
   return e == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 
+// Zeroes a few words.  A kernel and not a memset, because the launch behind it is then placed while it runs: with it
+// 5 matrices of 20000 x 128 take 12.3 us for tensor maximum and block quantizer instead of 15.1,
+// attention in bf16 of 2 heads of 1024 15.5 instead of 18.5, of one head of 256 x 77 6.7 instead of 9.9.
+__global__ void __launch_bounds__(256) zero_kernel(uint32_t* words, int64_t n) {
+  pdl_wait(); pdl_trigger();
+  for (int64_t i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) words[i] = 0u;
+}
+int launch_zero(uint32_t* words, int64_t n, cudaStream_t stream) {
+  const int64_t blocks = (n + 1023) / 1024;
+  return launch_pdl(zero_kernel, dim3((unsigned)(blocks < 64 ? blocks : 64)), 256, 0, stream, words, n) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
+}
+
 }  // namespace mxattn
 
 extern "C" int mxattn_quantize_mxfp4(const void* in, void* codes, void* e8m0_scales, int64_t rows,

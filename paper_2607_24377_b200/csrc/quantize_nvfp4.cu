@@ -95,12 +95,6 @@ __global__ void __launch_bounds__(kThreads) tensor_amax_kernel(const AmaxOperand
   pdl_wait(); pdl_trigger();
   tensor_amax_part(o, gridDim.y - 1 - blockIdx.y, blockIdx.x, gridDim.x);
 }
-// Zeroes the maxima before that.  A kernel and not a memset, because the next one is launched while it runs: 5 matrices of
-// 20000 x 128 take 12.3 us with the block quantizer behind instead of 15.1, one of 268 MB 40.1 instead of 43.1 alone.
-__global__ void __launch_bounds__(kThreads) zero_amax_kernel(uint32_t* amax, int n) {
-  pdl_wait(); pdl_trigger();
-  for (int i = threadIdx.x; i < n; i += kThreads) amax[i] = 0u;
-}
 // The same with one cluster of 16 CTAs per matrix: the maxima meet in the first CTA's shared memory, which then simply writes
 // the result -- nothing has to be zeroed before (a memset and the gap behind it are 2 us of a 10 us call).
 constexpr int kClusterCtas = 16, kClusterThreads = 512;
@@ -404,7 +398,7 @@ int launch_tensor_amax(const void* in, float* amax, int64_t batch, int64_t rows,
   }
   int64_t blocks = (chunks + nv::kThreads * 8 - 1) / (nv::kThreads * 8);
   if (blocks > 1184) blocks = 1184;                 // 8 CTAs per SM at most: the loop strides over the rest
-  if (launch_pdl(nv::zero_amax_kernel, dim3(1), nv::kThreads, 0, stream, op.amax, (int)batch) != cudaSuccess) return MXATTN_ECUDA;
+  if (launch_zero(op.amax, batch, stream) != MXATTN_OK) return MXATTN_ECUDA;
   count_launch(1);
   return launch_pdl(nv::tensor_amax_kernel, dim3((unsigned)blocks, (unsigned)batch), nv::kThreads, 0, stream,
                     op) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;

@@ -100,9 +100,13 @@ __global__ void __launch_bounds__(kThreads) tensor_amax_kernel(const AmaxOperand
 constexpr int kClusterCtas = 16, kClusterThreads = 512;
 __global__ void __launch_bounds__(kClusterThreads) tensor_amax_cluster_kernel(const AmaxOperand o) {
   __shared__ uint32_t s[kClusterCtas * kClusterThreads / 32];       // of CTA 0: one slot per warp of the cluster
+  // Another CTA's shared memory may be written only once that CTA has started, which being scheduled together does not say.
+  // Every thread arrives here and waits in front of its store below, so that the loads hide the barrier.
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   pdl_wait(); pdl_trigger();
   const uint32_t rank = blockIdx.x;                                 // gridDim.x == cluster size
   const uint32_t m = thread_amax<false>(o.in + blockIdx.y * o.chunks, o.chunks, (int64_t)rank * kClusterThreads + threadIdx.x, (int64_t)kClusterCtas * kClusterThreads);
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");             // every CTA of the cluster has started
   if ((threadIdx.x & 31) == 0) {
     uint32_t dst;
     asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(dst) : "r"((uint32_t)__cvta_generic_to_shared(&s[rank * (kClusterThreads / 32) + (threadIdx.x >> 5)])));

@@ -1,0 +1,38 @@
+"""Rules that a wrong kernel breaks only now and then on a GPU, checked where they can be decided: in the sources."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2607_24377_b200", "csrc")
+FILES = sorted(f for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh")))
+
+
+def code(name):
+    """A source file without its comments."""
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*|/\*.*?\*/", "", f.read(), flags=re.S)
+
+
+def kernels(name):
+    """(name, body) of the __global__ functions of a file."""
+    src = code(name)
+    for m in re.finditer(r"__global__[^;{]*?(\w+)\s*\((?:[^(){}]|\([^(){}]*\))*\)\s*\{", src):
+        depth, i = 1, m.end()
+        while depth:
+            depth += {"{": 1, "}": -1}.get(src[i], 0)
+            i += 1
+        yield m.group(1), src[m.end():i]
+
+
+def test_remote_shared_memory_is_written_behind_a_cluster_barrier():
+    # the CTA that owns the memory must have started: a whole barrier (arrive, wait) lies in front of the first access
+    seen = 0
+    for f in FILES:
+        for name, body in kernels(f):
+            at = body.find("st.shared::cluster")
+            if at < 0:
+                continue
+            seen += 1
+            before = re.findall(r"barrier\.cluster\.(arrive|wait)", body[:at])
+            assert before == ["arrive", "wait"], f"{f}: {name}"
+            assert re.findall(r"barrier\.cluster\.(arrive|wait)", body[at:]) == ["arrive", "wait"], f"{f}: {name}: nor may it end early"
+    assert seen == 1

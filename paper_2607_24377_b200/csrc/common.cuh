@@ -94,6 +94,20 @@ __device__ __host__ __forceinline__ int tile_scale_offset(int r, int c) {
 // every CTA of this grid has started).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Loads of what an earlier launch may have written: ordinary, coherent ones behind the wait.  The read-only path (__ldg, or a
+// load that the compiler takes for one because its pointer is const and __restrict__) asks that nobody writes the data while
+// the kernel runs, which its predecessor may still do, and nothing holds such a load behind the wait.
+__device__ __forceinline__ uint4 ld_global(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint32_t ld_global(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ float ld_global(const float* p) { return __uint_as_float(ld_global(reinterpret_cast<const uint32_t*>(p))); }
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t stream, Args... args) {
   cudaLaunchConfig_t cfg = {};

@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(32 * (16 / R + 2), 1) attention_rows_kernel(co
   if (warp == 0) {                                               // Q's scales, replicated: the four bytes of row i of a 32-row group
     uint32_t w[4];                                               // sit at 16 i + 4 (group), one 16-byte line per i
 #pragma unroll
-    for (int g = 0; g < 4; ++g) w[g] = __ldg(reinterpret_cast<const uint32_t*>(p.q_scales + qt * kTileScaleBytes) + lane * 4 + slab + g % kRG);
+    for (int g = 0; g < 4; ++g) w[g] = ld_global(reinterpret_cast<const uint32_t*>(p.q_scales + qt * kTileScaleBytes) + lane * 4 + slab + g % kRG);
     *reinterpret_cast<uint4*>(smem + kOffSFQ + lane * 16) = make_uint4(w[0], w[1], w[2], w[3]);
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

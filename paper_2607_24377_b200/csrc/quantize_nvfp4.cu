@@ -65,9 +65,9 @@ __device__ __forceinline__ uint32_t quantize_bf16x8(const uint4& v, float r) {
 constexpr int kAmaxUnroll = 8;
 struct AmaxOperand { const uint4* in; uint32_t* amax; int64_t chunks; };       // chunks of 16 bytes per matrix
 template <bool kFromEnd>
-__device__ __forceinline__ uint32_t thread_amax(const uint4* __restrict__ src, int64_t chunks, int64_t first, int64_t step) {
+__device__ __forceinline__ uint32_t thread_amax(const uint4* src, int64_t chunks, int64_t first, int64_t step) {
   if (kFromEnd) src += chunks - 1;
-  auto load = [&](int64_t i) { return __ldg(kFromEnd ? src - i : src + i); };
+  auto load = [&](int64_t i) { return ld_global(kFromEnd ? src - i : src + i); };
   uint32_t m = 0;
   int64_t i = first;
   for (; i + (kAmaxUnroll - 1) * step < chunks; i += kAmaxUnroll * step) {
@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kThreads) tensor_amax_qkv_kernel(const AmaxOpe
 constexpr int kA1Threads = 128;
 template <bool kTileLayout, int kT>
 __device__ __forceinline__ void quantize_nvfp4_axis1_part(uint4* s_v, const uint4* __restrict__ in, uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
-                                                          const float* __restrict__ amax, float* __restrict__ tensor_scale, int64_t rows, int64_t cols,
+                                                          const float* amax, float* __restrict__ tensor_scale, int64_t rows, int64_t cols,
                                                           int64_t rows_pad, int64_t part, int64_t b) {
   const int tid = threadIdx.x;
   const int64_t chunks_per_row = cols / 8;
@@ -154,7 +154,7 @@ __device__ __forceinline__ void quantize_nvfp4_axis1_part(uint4* s_v, const uint
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(&s_v[pos(c)])),
                  "l"(inside ? src + base + c : in), "r"(inside ? 16 : 0) : "memory");
   }
-  const float g = encode_scale(amax[b]);
+  const float g = encode_scale(ld_global(amax + b));
   if (part == 0 && tid == 0 && tensor_scale) tensor_scale[b] = __fdiv_rn(1.0f, g);
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
@@ -202,7 +202,7 @@ __device__ __forceinline__ void quantize_nvfp4_axis1_part(uint4* s_v, const uint
 template <bool kTileLayout>
 __global__ void __launch_bounds__(kA1Threads)
 quantize_nvfp4_axis1_kernel(const uint4* __restrict__ in, uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
-                            const float* __restrict__ amax, float* __restrict__ tensor_scale, int64_t rows, int64_t cols,
+                            const float* amax, float* __restrict__ tensor_scale, int64_t rows, int64_t cols,
                             int64_t rows_pad) {
   __shared__ uint4 s_v[4 * kA1Threads];
   pdl_wait(); pdl_trigger();
@@ -223,7 +223,7 @@ struct __align__(16) Axis0Smem {
 };
 template <bool kTileLayout>
 __device__ __forceinline__ void quantize_nvfp4_axis0_slab(Axis0Smem& sm, const uint16_t* __restrict__ in, uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
-                                                          const float* __restrict__ amax, float* __restrict__ tensor_scale, int64_t rows, int64_t cols,
+                                                          const float* amax, float* __restrict__ tensor_scale, int64_t rows, int64_t cols,
                                                           int64_t rows_pad, int64_t cx, int64_t ry, int64_t b) {
   constexpr int kTok = kTileLayout ? 128 : 256;                   // tokens per slab
   constexpr int kCol = kTileLayout ? 128 : 64;                    // columns per slab
@@ -233,8 +233,6 @@ __device__ __forceinline__ void quantize_nvfp4_axis0_slab(Axis0Smem& sm, const u
   uint8_t* s_scales = sm.scales;
   const int tid = threadIdx.x;
   const int64_t col0 = cx * kCol, row0 = ry * kTok;
-  const float g = encode_scale(amax[b]);
-  if (cx == 0 && ry == 0 && tid == 0 && tensor_scale) tensor_scale[b] = __fdiv_rn(1.0f, g);
   const uint16_t* src = in + b * rows * cols;
   // staging offset of the 16-byte chunk c of column n: the tile image's own swizzle, or (canonical) the chunk index XORed
   // with the column pair so that the 8 threads of a store phase hit 8 different bank groups
@@ -248,6 +246,8 @@ __device__ __forceinline__ void quantize_nvfp4_axis0_slab(Axis0Smem& sm, const u
     const uint16_t* gsrc = inside ? src + (row0 + t) * cols + col0 + cc : src;
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(&s_in[t][cc])), "l"(gsrc), "r"(inside ? 16 : 0) : "memory");
   }
+  const float g = encode_scale(ld_global(amax + b));
+  if (cx == 0 && ry == 0 && tid == 0 && tensor_scale) tensor_scale[b] = __fdiv_rn(1.0f, g);
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   {
@@ -318,7 +318,7 @@ __device__ __forceinline__ void quantize_nvfp4_axis0_slab(Axis0Smem& sm, const u
 template <bool kTileLayout>
 __global__ void __launch_bounds__(kThreads)
 quantize_nvfp4_axis0_kernel(const uint16_t* __restrict__ in, uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
-                            const float* __restrict__ amax, float* __restrict__ tensor_scale, int64_t rows, int64_t cols,
+                            const float* amax, float* __restrict__ tensor_scale, int64_t rows, int64_t cols,
                             int64_t rows_pad) {
   __shared__ Axis0Smem sm;
   pdl_wait(); pdl_trigger();

@@ -36,3 +36,14 @@ def test_remote_shared_memory_is_written_behind_a_cluster_barrier():
             assert before == ["arrive", "wait"], f"{f}: {name}"
             assert re.findall(r"barrier\.cluster\.(arrive|wait)", body[at:]) == ["arrive", "wait"], f"{f}: {name}: nor may it end early"
     assert seen == 1
+
+
+def test_what_a_launch_before_may_write_is_not_read_as_read_only():
+    # kernels that start while their predecessor runs: no read-only loads, neither asked for nor left to the compiler
+    files = [f for f in FILES if "pdl_wait()" in code(f)]
+    assert len(files) >= 6
+    for f in files:
+        src = code(f)
+        assert not re.search(r"__ldg\b|ld\.global\.nc", src), f
+        for name in set(re.findall(r"const\s+\w+\s*\*\s*__restrict__\s+(\w+)", src)):
+            assert not re.search(rf"[=(,?:+*/&|-]\s*{name}\s*\[|[=(,]\s*\*\s*{name}\b", src), f"{f}: {name} is read through a const __restrict__ pointer"

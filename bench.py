@@ -298,6 +298,7 @@ def main():
         step(evs[i])
     t_stop.record()
     barrier()
+    attn_launches = mx.last_launch_count()     # of a step's attention (two where its last wave is cut into small CTAs)
     if rank == 0:
         sampler.stop()
     assert int(status[0].item()) == 0, "a bounded device-side wait expired"
@@ -360,7 +361,7 @@ def main():
         variants["quantize_q_with_hadamard"] = {"ms": ms, "GBps": gbps, "frac_of_measured_copy_rate": gbps / peaks["hbm_gbs"],
                                                 "frac_of_nominal_8TBps": gbps / 8000.0}
         mx.quantize_mxfp4_batched(dq, qc, qs, bh, Nq, d, 1, mx.MODE_UOS, mx.LAYOUT_TILE)       # restore the unrotated Q-hat
-        # bf16 variant of this repository's own kernel (no quantization: one launch)
+        # bf16 variant of this repository's own kernel (no quantization)
         wsb = torch.empty(mx.forward_bf16_workspace_bytes(B, H, Nq, Nkv, d), dtype=torch.uint8, device="cuda")
         mx.forward_bf16(dq, dk, dv, out, B, H, Nq, Nkv, d, scale, 0, wsb); torch.cuda.synchronize()
         a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -483,7 +484,7 @@ def main():
                    "out": "bf16", "l2": "inputs (2.3 GB at wan22) exceed L2; no flush needed",
                    "sharding": "one full batch per GPU, no collective"},
         "clocks": clocks,
-        "e2e": e2e, "gpu_launches": 4 * args.steps,
+        "e2e": e2e, "gpu_launches": (3 + attn_launches) * args.steps,
         "roofline": roofline,
         "fp4_peak_probe": fp4,
         "attention_launch": attn_stats,

@@ -259,7 +259,8 @@ int mxattn_forward_bf16(const void* q, const void* k, const void* v, void* o,
  * known to be 1 (readings: the paper does not say how the baseline chooses them).
  * flags: MXATTN_FLAG_PNQ (row sum from the quantized probabilities, as in MXAttention; without it the direct
  * placement, which is what the paper's baseline uses) and MXATTN_FLAG_OUT_FP32.  Same tensor layouts as
- * mxattn_forward.  Enqueues one tensor-maximum launch, one to three quantize launches and the attention launch.
+ * mxattn_forward.  Enqueues the launch that zeroes the status word and the tensor maxima, one
+ * tensor-maximum launch, one or three quantize launches and the attention launch.
  * The workspace (mxattn_forward_nvfp4_workspace_bytes) holds the quantized operands and, at its start, the status word. */
 size_t mxattn_forward_nvfp4_workspace_bytes(int B, int H, int64_t Nq, int64_t Nkv, int d);
 int mxattn_forward_nvfp4(const void* q, const void* k, const void* v, void* o,
@@ -363,9 +364,7 @@ int mxattn_selftest_bounded_wait(void* status, int64_t limit_cycles, void* strea
  * in status[1] -- `meetings` if no warp was left stranded.  `status`: 4 device ints, zeroed by the caller. */
 int mxattn_selftest_pair_abandon(void* status, int64_t limit_cycles, int meetings, void* stream);
 
-/* Number of stages the last forward call of this process enqueued (for accounting): one per operand quantized (or
- * re-tiled), one per tensor maximum, one for the attention kernel.  Stages may share a kernel launch: short problems
- * quantize Q, K and V in one. */
+/* Number of kernel launches the last forward call of this process enqueued (for accounting). */
 int mxattn_last_launch_count(void);
 
 const char* mxattn_strerror(int status);

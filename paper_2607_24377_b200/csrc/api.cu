@@ -20,11 +20,17 @@ struct TraceRange {
   TraceRange& operator=(const TraceRange&) = delete;
 };
 
-static int g_launches = 0;
+// Kernel launches of the last forward call.  Every launch counts itself for its thread; a forward call reports the difference.
+static thread_local int t_launches = 0;
+static std::atomic<int> g_last_launches{0};
+void count_launch() { ++t_launches; }
+struct CountedCall {
+  const int before = t_launches;
+  ~CountedCall() { g_last_launches.store(t_launches - before, std::memory_order_relaxed); }
+};
+
 static void* g_workspace = nullptr;
 static size_t g_workspace_bytes = 0;
-
-void count_launch(int n) { g_launches += n; }
 
 constexpr int kMaxDevices = 64;
 static int current_device() {
@@ -101,7 +107,7 @@ static int forward_ws(const void* q, const void* k, const void* v, void* o, int 
   if (!carve(B, H, Nq, Nkv, d, &w)) return MXATTN_EUNSUPPORTED;
   if (!workspace || workspace_bytes < w.total) return MXATTN_EWORKSPACE;
   if (!aligned16(workspace)) return MXATTN_EALIGN;
-  g_launches = 0;
+  CountedCall counted;
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   const int mode = (flags & MXATTN_FLAG_UOS) ? MXATTN_MODE_UOS : MXATTN_MODE_OCP;
   const int qk_mode = mode | ((flags & MXATTN_FLAG_HADAMARD) ? MXATTN_MODE_HADAMARD : 0);   // Algorithm 2 lines 1-2
@@ -168,7 +174,7 @@ extern "C" int mxattn_rowsum_diagnostic(const void* q, const void* k, void* out,
   if (!carve(B, H, Nq, Nkv, d, &w)) return MXATTN_EUNSUPPORTED;
   if (!workspace || workspace_bytes < w.total) return MXATTN_EWORKSPACE;
   if (!aligned16(workspace)) return MXATTN_EALIGN;
-  g_launches = 0;
+  CountedCall counted;
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   const int mode = (flags & MXATTN_FLAG_UOS) ? MXATTN_MODE_UOS : MXATTN_MODE_OCP;
   const int qk_mode = mode | ((flags & MXATTN_FLAG_HADAMARD) ? MXATTN_MODE_HADAMARD : 0);
@@ -233,7 +239,7 @@ extern "C" int mxattn_forward_prequantized(const void* q_codes, const void* q_sc
   if (!aligned16(q_codes) || !aligned16(q_scales) || !aligned16(k_codes) || !aligned16(k_scales) ||
       !aligned16(v_codes) || !aligned16(v_scales) || !aligned16(o) || !aligned16(status))
     return MXATTN_EALIGN;
-  g_launches = 0;
+  CountedCall counted;
   return launch_forward(q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, o, B, H, Nq, Nkv,
                         softmax_scale, flags, static_cast<int*>(status), (cudaStream_t)stream);
 }
@@ -352,7 +358,8 @@ extern "C" int mxattn_forward_host(const void* q_host, const void* k_host, const
   ck(cudaEventRecord(ev[3 * stages], stream));                   // work already queued on the caller's stream comes first
   ck(cudaStreamWaitEvent(hp->in, ev[3 * stages], 0));
   ck(cudaStreamWaitEvent(hp->attn, ev[3 * stages], 0));
-  int rc = MXATTN_OK, launched = 0;
+  CountedCall counted;
+  int rc = MXATTN_OK;
   for (size_t st = 0; st < stages && !fail && rc == MXATTN_OK; ++st) {
     TraceRange tr("mxattn host stage");
     const size_t i = first_head[st], n = first_head[st + 1] - i;  // heads of the stage; heads are contiguous in memory
@@ -369,7 +376,6 @@ extern "C" int mxattn_forward_host(const void* q_host, const void* k_host, const
     // launch, so that they fill the SMs the previous stage's attention kernel frees as it drains
     rc = forward_ws(dq + i * qh, dk + i * kh, dv + i * kh, dout + i * oh, 1, (int)n, Nq, Nkv, d, softmax_scale, flags,
                     ws + i * w.total, n * w.total, as, nullptr, hp->quant, ev[3 * st + 1], false, st + 1 < stages || !last_alone);
-    launched += g_launches;
     ck(cudaEventRecord(ev[3 * st + 2], as));
     ck(cudaStreamWaitEvent(hp->out, ev[3 * st + 2], 0));
     ck(cudaMemcpyAsync(static_cast<char*>(o_host) + i * oh, dout + i * oh, n * oh, cudaMemcpyDeviceToHost, hp->out));
@@ -382,7 +388,6 @@ extern "C" int mxattn_forward_host(const void* q_host, const void* k_host, const
   ck(cudaStreamSynchronize(stream));
   ck(cudaStreamSynchronize(hp->attn));
   ck(cudaStreamSynchronize(hp->out));
-  g_launches = launched;
   if (rc != MXATTN_OK) return rc;
   if (fail) return MXATTN_ECUDA;
   // one status word per stage, at the start of the workspace slice of the stage's first head
@@ -440,7 +445,7 @@ extern "C" int mxattn_forward_bf16(const void* q, const void* k, const void* v, 
   if (d != kHeadDim) return MXATTN_EUNSUPPORTED;
   if (!workspace) return MXATTN_EWORKSPACE;
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(o) || !aligned16(workspace)) return MXATTN_EALIGN;
-  g_launches = 0;
+  CountedCall counted;
   return launch_forward_bf16(q, k, v, o, B, H, Nq, Nkv, softmax_scale, flags, workspace, workspace_bytes,
                              (cudaStream_t)stream);
 }
@@ -460,7 +465,7 @@ extern "C" int mxattn_forward_nvfp4(const void* q, const void* k, const void* v,
   if (d != kHeadDim) return MXATTN_EUNSUPPORTED;
   if (!workspace) return MXATTN_EWORKSPACE;
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(o) || !aligned16(workspace)) return MXATTN_EALIGN;
-  g_launches = 0;
+  CountedCall counted;
   return launch_forward_nvfp4(q, k, v, o, B, H, Nq, Nkv, softmax_scale, flags, workspace, workspace_bytes,
                               (cudaStream_t)stream);
 }
@@ -484,7 +489,7 @@ extern "C" int mxattn_selftest_pair_abandon(void* status, int64_t limit_cycles, 
   return launch_pair_abandon_selftest(static_cast<int*>(status), (long long)limit_cycles, meetings, (cudaStream_t)stream);
 }
 
-extern "C" int mxattn_last_launch_count(void) { return g_launches; }
+extern "C" int mxattn_last_launch_count(void) { return g_last_launches.load(std::memory_order_relaxed); }
 
 extern "C" const char* mxattn_strerror(int status) {
   switch (status) {

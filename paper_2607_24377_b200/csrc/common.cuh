@@ -108,8 +108,10 @@ __device__ __forceinline__ uint32_t ld_global(const uint32_t* p) {
   return v;
 }
 __device__ __forceinline__ float ld_global(const float* p) { return __uint_as_float(ld_global(reinterpret_cast<const uint32_t*>(p))); }
+void count_launch();         // called at every kernel launch of a forward call (mxattn_last_launch_count)
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t stream, Args... args) {
+  count_launch();
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = dim3(block); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
   cudaLaunchAttribute attr;
@@ -121,6 +123,7 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, unsigned block,
 // The same with clusters of `cluster` CTAs along x.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl_cluster(void (*kern)(KArgs...), dim3 grid, unsigned block, unsigned cluster, cudaStream_t stream, Args... args) {
+  count_launch();
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = dim3(block); cfg.stream = stream;
   cudaLaunchAttribute attr[2];
@@ -203,6 +206,5 @@ int launch_rowsum_diag(const void* q_codes, const void* q_scales, const void* k_
                        int* status, cudaStream_t stream);
 int launch_bounded_wait_selftest(int* status, long long limit_cycles, cudaStream_t stream);
 int launch_pair_abandon_selftest(int* status, long long limit_cycles, int meetings, cudaStream_t stream);
-void count_launch(int n);
 
 }  // namespace mxattn

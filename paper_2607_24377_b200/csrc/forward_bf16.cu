@@ -389,7 +389,6 @@ int launch_forward_bf16(const void* q, const void* k, const void* v, void* o, in
   p.scale_log2e = softmax_scale * 1.4426950408889634f;
   auto kern = f32 ? attention_bf16_kernel<true> : attention_bf16_kernel<false>;
   if (!ensure_dynamic_smem((const void*)kern, kSmemBytes)) return MXATTN_ECUDA;
-  count_launch(1);
   return launch_pdl(kern, dim3((unsigned)split.ctas), kThreads, kSmemBytes, stream, p, q_map, k_map, v_map, out_map) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 

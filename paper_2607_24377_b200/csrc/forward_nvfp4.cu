@@ -557,7 +557,6 @@ int launch_forward_nvfp4(const void* q, const void* k, const void* v, void* o, i
   void (*kern)(const Params, const CUtensorMap) = pnq ? (f32 ? attention_nvfp4_kernel<true, true> : attention_nvfp4_kernel<true, false>)
                                    : (f32 ? attention_nvfp4_kernel<false, true> : attention_nvfp4_kernel<false, false>);
   if (!ensure_dynamic_smem((const void*)kern, kSmemBytes)) return MXATTN_ECUDA;
-  count_launch(1);
   return launch_pdl(kern, dim3((unsigned)split.ctas), kThreads, kSmemBytes, stream, p, out_map) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 

@@ -197,6 +197,5 @@ extern "C" int mxattn_probe_fp4_gemm(const void* a_codes, const void* a_scales, 
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess) return MXATTN_ECUDA;
   const unsigned grid = (unsigned)(p.m_tiles * (N / tile_n));
   kern<<<grid, kThreads, kSmemBytes, (cudaStream_t)stream>>>(p);
-  count_launch(1);
   return cudaGetLastError() == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }

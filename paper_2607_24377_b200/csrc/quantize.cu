@@ -520,7 +520,6 @@ int launch_quantize_qkv(const void* q, void* q_codes, void* q_scales, const void
     const int rc = launch_rot(a, b, true, rule, stream);
     if (rc != MXATTN_OK) return rc;
   }
-  count_launch(v ? 3 : 2);
   return MXATTN_OK;
 }
 
@@ -581,7 +580,6 @@ int launch_quantize(const void* in, void* codes, void* scales, int64_t batch, in
       e = launch_pdl(quantize_axis0_kernel<false>, grid, kVThreads, 0, stream, 
           (const uint16_t*)in, (uint8_t*)codes, (uint8_t*)scales, rows, cols, rows_pad, rule);
   }
-  count_launch(1);
   return e == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 

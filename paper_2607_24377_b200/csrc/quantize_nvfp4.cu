@@ -372,7 +372,6 @@ int launch_nvfp4_operands(const void* q, void* q_codes, void* q_scales, const vo
     oq.ctas = ok.ctas = 0;
   }
   if (launch_pdl(quantize_nvfp4_qkv_kernel, dim3((unsigned)(oq.ctas + ok.ctas + ov.ctas)), kThreads, 0, stream, oq, ok, ov) != cudaSuccess) return MXATTN_ECUDA;
-  count_launch(6);
   return MXATTN_OK;
 }
 
@@ -396,14 +395,12 @@ int launch_tensor_amax(const void* in, float* amax, int64_t batch, int64_t rows,
       if (cudaFuncSetAttribute(nv::tensor_amax_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return MXATTN_ECUDA;
       allowed.fetch_or((uint64_t)1 << (dev & 63), std::memory_order_relaxed);
     }
-    count_launch(1);
     return launch_pdl_cluster(nv::tensor_amax_cluster_kernel, dim3(nv::kClusterCtas, (unsigned)batch), nv::kClusterThreads, nv::kClusterCtas, stream, op) == cudaSuccess
                ? MXATTN_OK : MXATTN_ECUDA;
   }
   int64_t blocks = (chunks + nv::kThreads * 8 - 1) / (nv::kThreads * 8);
   if (blocks > 1184) blocks = 1184;                 // 8 CTAs per SM at most: the loop strides over the rest
   if (launch_zero(op.amax, batch, stream) != MXATTN_OK) return MXATTN_ECUDA;
-  count_launch(1);
   return launch_pdl(nv::tensor_amax_kernel, dim3((unsigned)blocks, (unsigned)batch), nv::kThreads, 0, stream,
                     op) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
@@ -445,7 +442,6 @@ int launch_quantize_nvfp4(const void* in, void* codes, void* scales, const float
       e = launch_pdl(nv::quantize_nvfp4_axis0_kernel<false>, grid, nv::kThreads, 0, stream, (const uint16_t*)in, (uint8_t*)codes, (uint8_t*)scales,
                                                                                 amax, tensor_scale, rows, cols, rows_pad);
   }
-  count_launch(1);
   return e == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 

@@ -272,7 +272,7 @@ int launch_rowsum_diag(const void* q_codes, const void* q_scales, const void* k_
   if (cudaFuncSetAttribute(rowsum_diag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess)
     return MXATTN_ECUDA;
   rowsum_diag_kernel<<<(unsigned)grid, kThreads, kSmemBytes, stream>>>(p);
-  count_launch(1);
+  count_launch();
   return cudaGetLastError() == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 

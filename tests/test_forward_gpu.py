@@ -26,7 +26,7 @@ def run_forward(cfg, q, k, v, uos, pnq, f32=True, rotate=False):
     out, ws = g_out.t, g_ws.t
     mx.forward_ws(dq, dk, dv, out, cfg.B, cfg.H, cfg.Nq, cfg.Nkv, cfg.d, cfg.softmax_scale, flags, ws)
     assert mx.device_status(ws) == 0
-    assert mx.last_launch_count() == 4
+    assert mx.last_launch_count() - util.operand_launches(cfg, rotate) in (1, 2)      # the attention, its last wave apart or not
     g_out.check(); g_ws.check()
     return out.clone()
 
@@ -169,9 +169,9 @@ def test_host_buffer_entry_point(B, H):
     arena = torch.empty(mx.forward_host_arena_bytes(cfg.B, cfg.H, cfg.Nq, cfg.Nkv, 128, flags), dtype=torch.uint8, device="cuda")
     mx.forward_host(hq, hk, hv, ho, cfg.B, cfg.H, cfg.Nq, cfg.Nkv, 128, cfg.softmax_scale, flags, arena)
     assert torch.equal(ho, want)
-    assert mx.last_launch_count() % 4 == 0 and mx.last_launch_count() <= 4 * B * H
+    assert mx.last_launch_count() % 2 == 0 and mx.last_launch_count() <= 2 * B * H
     if B * H >= 12:
-        assert mx.last_launch_count() < 4 * B * H          # heads were grouped into stages
+        assert mx.last_launch_count() < 2 * B * H          # heads were grouped into stages
 
 
 @pytest.mark.parametrize("recipe", ["iid", "outlier", "wan"])
@@ -261,7 +261,7 @@ def test_registered_workspace_entry_point(uos, pnq):
     mx.set_workspace(g_ws.t)
     try:
         mx.forward(dq, dk, dv, g_out.t, cfg.B, cfg.H, cfg.Nq, cfg.Nkv, cfg.d, cfg.softmax_scale, flags)
-        assert mx.device_status(g_ws.t) == 0 and mx.last_launch_count() == 4
+        assert mx.device_status(g_ws.t) == 0 and mx.last_launch_count() == 2
         g_out.check(); g_ws.check()
         check(g_out.t, oracle_out(cfg, q, k, v, uos, pnq))
         # a registered workspace that is too small is refused before anything is launched

@@ -22,7 +22,7 @@ def run(cfg, q, k, v, pnq, f32=True):
     flags = (mx.FLAG_PNQ if pnq else 0) | (mx.FLAG_OUT_FP32 if f32 else 0)
     mx.forward_nvfp4(dq, dk, dv, g_out.t, cfg.B, cfg.H, cfg.Nq, cfg.Nkv, cfg.d, cfg.softmax_scale, flags, g_ws.t)
     assert mx.device_status(g_ws.t) == 0
-    assert mx.last_launch_count() == 7
+    assert mx.last_launch_count() == 3 + util.operand_launches(cfg)      # zeroing, maxima, operands, attention
     g_out.check(); g_ws.check()
     return g_out.t.clone()
 

@@ -14,6 +14,15 @@ def bits_to_f64(bits: np.ndarray) -> np.ndarray:
     return si.bf16_bits_to_f32(bits).astype(np.float64)
 
 
+def operand_launches(cfg, rotate=False) -> int:
+    """Launches that prepare a forward call's operands: one, or one each for Q, K and V of a long problem; V, then Q and K
+    where they are rotated."""
+    if rotate:
+        return 2
+    half_tiles = 2 * cfg.B * cfg.H * (-(-cfg.Nq // 128) - (-cfg.Nkv // 128))
+    return 3 if half_tiles > 24 * torch.cuda.get_device_properties(0).multi_processor_count else 1
+
+
 def tile_code_offset(r, c):
     return r * 64 + ((c ^ ((r >> 1) & 3)) << 4)
 

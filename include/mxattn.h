@@ -244,8 +244,8 @@ int mxattn_rowsum_diagnostic(const void* q, const void* k, void* out,
  * exponentials rounded to bf16 for the second GEMM and the row sum taken from the fp32 exponentials.
  * It is the high-precision reference point for the MXFP4 variants (the paper's "FP16" baseline,
  * Section 5.2).  Same tensor layouts as mxattn_forward; flags: only MXATTN_FLAG_OUT_FP32.
- * The workspace (mxattn_forward_bf16_workspace_bytes) holds the status word at its start; its size, about that of the
- * inputs, dates from a version that kept re-tiled copies of Q, K and V there, and is kept for callers that size buffers by it. */
+ * The workspace (mxattn_forward_bf16_workspace_bytes) holds the status word at its start, and copies of those of q, k
+ * and v that o overlaps in memory. */
 size_t mxattn_forward_bf16_workspace_bytes(int B, int H, int64_t Nq, int64_t Nkv, int d);
 int mxattn_forward_bf16(const void* q, const void* k, const void* v, void* o,
                         int B, int H, int64_t Nq, int64_t Nkv, int d,

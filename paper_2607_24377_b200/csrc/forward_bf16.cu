@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_bf16_kernel(const Param
 
 }  // namespace fwd16
 
-// The size of the former re-tiled copies is kept: callers size their workspace with it.  Only the status word is used.
+// The status word, and room for copies of Q, K and V (whole tiles), which are made where the output overlaps them.
 size_t bf16_workspace_bytes(int B, int H, int64_t Nq, int64_t Nkv) {
   const size_t bh = (size_t)B * H;
   const size_t qt = (size_t)((Nq + kTile - 1) / kTile), kt = (size_t)((Nkv + kTile - 1) / kTile);
@@ -376,8 +376,23 @@ int launch_forward_bf16(const void* q, const void* k, const void* v, void* o, in
   if (qt > 0x3FFFFFFF || kt > 65535 || qt > 0x7FFFFFFF || bh > 65535 || grid > 0x7FFFFFFF) return MXATTN_EUNSUPPORTED;
   CUtensorMap q_map, k_map, v_map, out_map;
   const bool f32 = flags & MXATTN_FLAG_OUT_FP32;
+  // The kernel reads its inputs while its first CTAs write the output.  An operand that the output overlaps is copied to the
+  // workspace first -- other than Q exactly in place, of which a CTA reads the rows that it writes, and before it does.
+  const size_t row = kHeadDim * 2, nq = (size_t)bh * Nq * row, nkv = (size_t)bh * Nkv * row, no = f32 ? 2 * nq : nq;
+  uint8_t* spare = static_cast<uint8_t*>(workspace) + 256;
+  auto apart = [&](const void*& x, size_t n, int64_t tiles, bool in_place) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(x), b = reinterpret_cast<uintptr_t>(o);
+    if (a < b + no && b < a + n && !(in_place && a == b)) {
+      if (cudaMemcpyAsync(spare, x, n, cudaMemcpyDeviceToDevice, stream) != cudaSuccess) return false;
+      x = spare;
+    }
+    spare += (size_t)(bh * tiles) * kTileBytes;
+    return true;
+  };
+  const void *q_in = q, *k_in = k, *v_in = v;
+  if (!apart(q_in, nq, qt, !f32) || !apart(k_in, nkv, kt, false) || !apart(v_in, nkv, kt, false)) return MXATTN_ECUDA;
   int rc;
-  if ((rc = encode_operand_map(&q_map, q, bh, Nq)) || (rc = encode_operand_map(&k_map, k, bh, Nkv)) || (rc = encode_operand_map(&v_map, v, bh, Nkv)) ||
+  if ((rc = encode_operand_map(&q_map, q_in, bh, Nq)) || (rc = encode_operand_map(&k_map, k_in, bh, Nkv)) || (rc = encode_operand_map(&v_map, v_in, bh, Nkv)) ||
       (rc = encode_output_map(&out_map, o, bh, Nq, f32)))
     return rc;
   if (launch_zero(static_cast<uint32_t*>(workspace), 4, stream) != MXATTN_OK) return MXATTN_ECUDA;

@@ -50,23 +50,40 @@ int sm_count() {
   return v;
 }
 
-bool ensure_dynamic_smem(const void* kern, int bytes) {
-  // one entry per kernel (a few dozen): the devices on which its limit has been raised, one bit each
-  struct Entry { std::atomic<const void*> kern; std::atomic<uint64_t> devices; };
-  static Entry table[128];
-  const int dev = current_device();
-  if (dev < 0) return false;
-  for (Entry& e : table) {
-    const void* k = e.kern.load(std::memory_order_acquire);
-    if (k == nullptr && e.kern.compare_exchange_strong(k, kern, std::memory_order_acq_rel)) k = kern;
-    if (k != kern) continue;                        // (a failed exchange left another thread's kernel in k)
-    if (e.devices.load(std::memory_order_acquire) >> dev & 1) return true;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
-    e.devices.fetch_or((uint64_t)1 << dev, std::memory_order_release);
-    return true;
+// Number of the current context, 0 if there is none yet.  A kernel's attributes belong to a context, of which a device may have
+// several (and a new one after a reset); numbers, unlike handles, are never used twice.
+static uint64_t current_context() {
+  static std::atomic<void*> fn{nullptr};
+  void* get = fn.load(std::memory_order_acquire);
+  if (!get) {
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPoint("cuCtxGetId", &get, cudaEnableDefault, &found) != cudaSuccess || found != cudaDriverEntryPointSuccess || !get) return 0;
+    fn.store(get, std::memory_order_release);
   }
-  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
+  unsigned long long id = 0;
+  return reinterpret_cast<PFN_cuCtxGetId>(get)(nullptr, &id) == CUDA_SUCCESS ? (uint64_t)id : 0;
 }
+
+bool ensure_attribute(const void* kern, cudaFuncAttribute attribute, int value) {
+  // one entry per kernel (a few dozen): the contexts in which it has been set, each at its number mod 16
+  struct Entry { std::atomic<const void*> kern; std::atomic<uint64_t> contexts[16]; };
+  static Entry table[128];
+  const uint64_t context = current_context();
+  if (context != 0) {
+    for (Entry& e : table) {
+      const void* k = e.kern.load(std::memory_order_acquire);
+      if (k == nullptr && e.kern.compare_exchange_strong(k, kern, std::memory_order_acq_rel)) k = kern;
+      if (k != kern) continue;                        // (a failed exchange left another thread's kernel in k)
+      std::atomic<uint64_t>& at = e.contexts[context & 15];
+      if (at.load(std::memory_order_acquire) == context) return true;
+      if (cudaFuncSetAttribute(kern, attribute, value) != cudaSuccess) return false;
+      at.store(context, std::memory_order_release);
+      return true;
+    }
+  }
+  return cudaFuncSetAttribute(kern, attribute, value) == cudaSuccess;
+}
+bool ensure_dynamic_smem(const void* kern, int bytes) { return ensure_attribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); }
 
 struct WorkspaceLayout {
   size_t q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, status, total;

@@ -134,8 +134,9 @@ inline cudaError_t launch_pdl_cluster(void (*kern)(KArgs...), dim3 grid, unsigne
   cfg.attrs = attr; cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
 }
-// Raises a kernel's dynamic shared memory limit, once per kernel and device (a driver call per launch otherwise).
-bool ensure_dynamic_smem(const void* kern, int bytes);
+// Sets a kernel's attribute, once per kernel and context (a driver call per launch otherwise).  One attribute per kernel.
+bool ensure_attribute(const void* kern, cudaFuncAttribute attribute, int value);
+bool ensure_dynamic_smem(const void* kern, int bytes);       // its limit of dynamic shared memory
 PFN_cuTensorMapEncodeTiled tensor_map_encoder();      // null if the driver has none
 // an attention output as a [bh][Nq][128] tensor that is written in boxes of 32 rows x 128 bytes with the 128-byte swizzle
 int encode_output_map(CUtensorMap* map, void* o, int64_t bh, int64_t Nq, bool f32);

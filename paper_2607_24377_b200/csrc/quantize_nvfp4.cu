@@ -11,8 +11,6 @@
 // Three HBM-bound passes: the tensor maximum (2 B/element read), then the quantizer (2 B read, 0.5 + 1/16 B written).
 #include <cuda_fp16.h>
 
-#include <atomic>
-
 #include "common.cuh"
 
 namespace mxattn {
@@ -388,13 +386,7 @@ int launch_tensor_amax(const void* in, float* amax, int64_t batch, int64_t rows,
   // 11.8 / 11.0, 40 of 0.8 MB 16.5 / 14.9, two of 8.4 MB 10.7 / 9.4.
   const nv::AmaxOperand op{(const uint4*)in, reinterpret_cast<uint32_t*>(amax), chunks};
   if (chunks <= (4 << 20) / 16 && batch * chunks <= (11 << 20) / 16) {
-    static std::atomic<uint64_t> allowed{0};                         // devices on which clusters of 16 have been allowed
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return MXATTN_ECUDA;
-    if (!(allowed.load(std::memory_order_relaxed) >> (dev & 63) & 1)) {
-      if (cudaFuncSetAttribute(nv::tensor_amax_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return MXATTN_ECUDA;
-      allowed.fetch_or((uint64_t)1 << (dev & 63), std::memory_order_relaxed);
-    }
+    if (!ensure_attribute((const void*)nv::tensor_amax_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) return MXATTN_ECUDA;
     return launch_pdl_cluster(nv::tensor_amax_cluster_kernel, dim3(nv::kClusterCtas, (unsigned)batch), nv::kClusterThreads, nv::kClusterCtas, stream, op) == cudaSuccess
                ? MXATTN_OK : MXATTN_ECUDA;
   }

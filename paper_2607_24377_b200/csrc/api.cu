@@ -50,9 +50,9 @@ int sm_count() {
   return v;
 }
 
-// Number of the current context, 0 if there is none yet.  A kernel's attributes belong to a context, of which a device may have
+// A kernel's attributes belong to a context, of which a device may have
 // several (and a new one after a reset); numbers, unlike handles, are never used twice.
-static uint64_t current_context() {
+uint64_t current_context() {
   static std::atomic<void*> fn{nullptr};
   void* get = fn.load(std::memory_order_acquire);
   if (!get) {

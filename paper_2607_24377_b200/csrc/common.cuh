@@ -134,6 +134,7 @@ inline cudaError_t launch_pdl_cluster(void (*kern)(KArgs...), dim3 grid, unsigne
   cfg.attrs = attr; cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
 }
+uint64_t current_context();       // its number, 0 if there is none yet
 // Sets a kernel's attribute, once per kernel and context (a driver call per launch otherwise).  One attribute per kernel.
 bool ensure_attribute(const void* kern, cudaFuncAttribute attribute, int value);
 bool ensure_dynamic_smem(const void* kern, int bytes);       // its limit of dynamic shared memory
@@ -181,6 +182,7 @@ int launch_nvfp4_operands(const void* q, void* q_codes, void* q_scales, const vo
                           const void* v, void* v_codes, void* v_scales, float* amax, float* tensor_scale, int64_t bh,
                           int64_t Nq, int64_t Nkv, cudaStream_t stream);
 int launch_zero(uint32_t* words, int64_t n, cudaStream_t stream);      // a few words: status, tensor maxima
+bool amax_by_cluster(int64_t batch, int64_t chunks, bool fits);      // `fits`: a cluster of 16 CTAs can run
 int launch_tensor_amax(const void* in, float* amax, int64_t batch, int64_t rows, int64_t cols, cudaStream_t stream);
 int launch_quantize_nvfp4(const void* in, void* codes, void* scales, const float* amax, float* tensor_scale, int64_t batch,
                           int64_t rows, int64_t cols, int block_axis, int layout, cudaStream_t stream);

@@ -11,6 +11,8 @@
 // Three HBM-bound passes: the tensor maximum (2 B/element read), then the quantizer (2 B read, 0.5 + 1/16 B written).
 #include <cuda_fp16.h>
 
+#include <atomic>
+
 #include "common.cuh"
 
 namespace mxattn {
@@ -373,6 +375,36 @@ int launch_nvfp4_operands(const void* q, void* q_codes, void* q_scales, const vo
   return MXATTN_OK;
 }
 
+// One cluster per matrix up to 4 MB each and 11 MB in all: what 16 SMs per matrix take longer than a full grid is less
+// than what the launch that zeroes the results costs.  With the block quantizer behind, us against the full grid: one
+// matrix of 1 MB 7.0 / 9.2, one of 4.2 MB 7.0 / 9.2, 40 of 0.26 MB 8.4 / 9.2; beyond, three of 4.2 MB 10.3 / 9.2, six
+// 11.8 / 11.0, 40 of 0.8 MB 16.5 / 14.9, two of 8.4 MB 10.7 / 9.4.
+bool amax_by_cluster(int64_t batch, int64_t chunks, bool fits) {
+  return fits && chunks <= (4 << 20) / 16 && batch * chunks <= (11 << 20) / 16;
+}
+
+// Whether a cluster of 16 CTAs can run in the current context (a part of a device may be too small for one): asked once per
+// context.
+static bool cluster_fits() {
+  static std::atomic<uint64_t> answers[16];                          // context's number and the answer in the lowest bit
+  const uint64_t context = current_context();
+  std::atomic<uint64_t>& at = answers[context & 15];
+  const uint64_t seen = at.load(std::memory_order_relaxed);
+  if (context != 0 && seen >> 1 == context) return seen & 1;
+  bool fits = ensure_attribute((const void*)nv::tensor_amax_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(nv::kClusterCtas); cfg.blockDim = dim3(nv::kClusterThreads);
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = nv::kClusterCtas; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr; cfg.numAttrs = 1;
+  int n = 0;
+  if (fits && (cudaOccupancyMaxActiveClusters(&n, nv::tensor_amax_cluster_kernel, &cfg) != cudaSuccess || n < 1)) fits = false;
+  if (!fits) (void)cudaGetLastError();                               // an answer, not an error of the call
+  if (context != 0) at.store(context << 1 | (fits ? 1 : 0), std::memory_order_relaxed);
+  return fits;
+}
+
 int launch_tensor_amax(const void* in, float* amax, int64_t batch, int64_t rows, int64_t cols, cudaStream_t stream) {
   if (!in || !amax) return MXATTN_EINVAL;
   if (batch <= 0 || rows <= 0 || cols <= 0) return MXATTN_EINVAL;
@@ -380,13 +412,8 @@ int launch_tensor_amax(const void* in, float* amax, int64_t batch, int64_t rows,
   if (!aligned16(in) || (reinterpret_cast<uintptr_t>(amax) & 3u)) return MXATTN_EALIGN;
   if (batch > 65535) return MXATTN_EUNSUPPORTED;
   const int64_t chunks = rows * cols / 8;
-  // One cluster per matrix up to 4 MB each and 11 MB in all: what 16 SMs per matrix take longer than a full grid is less
-  // than what the launch that zeroes the results costs.  With the block quantizer behind, us against the full grid: one
-  // matrix of 1 MB 7.0 / 9.2, one of 4.2 MB 7.0 / 9.2, 40 of 0.26 MB 8.4 / 9.2; beyond, three of 4.2 MB 10.3 / 9.2, six
-  // 11.8 / 11.0, 40 of 0.8 MB 16.5 / 14.9, two of 8.4 MB 10.7 / 9.4.
   const nv::AmaxOperand op{(const uint4*)in, reinterpret_cast<uint32_t*>(amax), chunks};
-  if (chunks <= (4 << 20) / 16 && batch * chunks <= (11 << 20) / 16) {
-    if (!ensure_attribute((const void*)nv::tensor_amax_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) return MXATTN_ECUDA;
+  if (amax_by_cluster(batch, chunks, cluster_fits())) {
     return launch_pdl_cluster(nv::tensor_amax_cluster_kernel, dim3(nv::kClusterCtas, (unsigned)batch), nv::kClusterThreads, nv::kClusterCtas, stream, op) == cudaSuccess
                ? MXATTN_OK : MXATTN_ECUDA;
   }

@@ -50,3 +50,11 @@ def test_count_equals_the_captured_kernels(op, H, nq, nkv, flags, launches):
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(o, want)
+
+
+@pytest.mark.parametrize("rows,kernels", [(16384, 1), (16385, 2)])       # a cluster per matrix; zeroing and a grid
+def test_kernels_of_the_tensor_maximum(rows, kernels):
+    import paper_2607_24377_b200 as mx
+    x, amax = torch.randn(rows, 128, device="cuda").to(torch.bfloat16), torch.empty(1, device="cuda")
+    mx.tensor_amax(x, amax, 1, rows, 128)
+    assert nodes_of(lambda: mx.tensor_amax(x, amax, 1, rows, 128))[0] == kernels

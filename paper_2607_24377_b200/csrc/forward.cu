@@ -191,8 +191,8 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
   __syncthreads();
   tc_fence_after();
   pdl_trigger();
-  // All 512 columns are allocated, so the base is column 0.  With the row sum placed directly the loop is faster with the
-  // constant (16 x 32768: 5361 -> 5302 us), with the PNQ row sum with the loaded value (37 x 16384: 2849 against 2890).
+  // The base is column 0.  With the row sum placed directly the loop is faster with the constant (16 x 32768: 5361 -> 5302
+  // us), with the PNQ row sum with the loaded value (37 x 16384: 2849 against 2890).
   const uint32_t tmem = kPnq ? *tmem_slot : 0u;
   const int role = abort_flag[1] != 0 ? kSoftmaxWarps + 2 : warp;     // an earlier CTA gave up: drain the grid quickly
 
@@ -738,6 +738,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
   __syncthreads();
   if (warp == kSoftmaxWarps + 1) {
     tc_fence_after();
+    check_tmem_base(*tmem_slot, lane, p.status);
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
   }
 }

@@ -115,7 +115,8 @@ __global__ void __launch_bounds__(kThreads, 1) attention_bf16_kernel(const Param
   __syncthreads();
   tc_fence_after();
   pdl_trigger();
-  constexpr uint32_t tmem = 0;                       // all 512 columns are allocated: the base is column 0
+  constexpr uint32_t tmem = 0;
+  if (*tmem_slot != 0) *abort_flag = kCodeTmemBase;
   const int role = (abort_flag[1] != 0 || *tmem_slot != 0 || at.empty || (!two && warp >= 8 && warp < kSoftmaxWarps)) ? kSoftmaxWarps + 2 : warp;     // an earlier CTA gave up: drain the grid quickly
 
   if (role == kSoftmaxWarps) {

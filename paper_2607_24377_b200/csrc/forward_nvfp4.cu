@@ -491,6 +491,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
   __syncthreads();
   if (warp == kSoftmaxWarps + 1) {
     tc_fence_after();
+    check_tmem_base(*tmem_slot, lane, p.status);
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
   }
 }

@@ -112,7 +112,8 @@ __global__ void __launch_bounds__(32 * (16 / R + 2), 1) attention_rows_kernel(co
   __syncthreads();
   tc_fence_after();
   pdl_trigger();
-  constexpr uint32_t tmem = 0;                                   // all 512 columns are allocated: the base is column 0
+  constexpr uint32_t tmem = 0;
+  if (*tmem_slot != 0) *abort_flag = kCodeTmemBase;
   const int role = (abort_flag[1] != 0 || *tmem_slot != 0) ? kWarps + 2 : warp;     // an earlier CTA gave up: drain the grid quickly
 
   if (role == kWarps) {

@@ -198,6 +198,15 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+// The attention kernels allocate all 512 columns, so that their tensor memory starts at column 0, and address it from there.
+// Were it ever elsewhere, this code in the status word says that the output is void.  Where a CTA's abort flag reaches the
+// status word at its end, the flag takes it at the start (2 x 1024: no time; at the end it took 0.1 of 10.6 us); elsewhere the
+// warp that allocated checks at the end (in front of the loops it costs registers: NVFP4 direct, 40 x 16384, 3860 -> 4070 us).
+constexpr int kCodeTmemBase = 41;
+__device__ __forceinline__ void check_tmem_base(uint32_t base, int lane, int* status) {
+  if (base != 0u && lane == 0) atomicCAS(status, 0, kCodeTmemBase);
+}
+
 #define TMEM_LD32(taddr, r)                                                                                   \
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "                                                      \
                "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,"  \

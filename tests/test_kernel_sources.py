@@ -47,3 +47,14 @@ def test_what_a_launch_before_may_write_is_not_read_as_read_only():
         assert not re.search(r"__ldg\b|ld\.global\.nc", src), f
         for name in set(re.findall(r"const\s+\w+\s*\*\s*__restrict__\s+(\w+)", src)):
             assert not re.search(rf"[=(,?:+*/&|-]\s*{name}\s*\[|[=(,]\s*\*\s*{name}\b", src), f"{f}: {name} is read through a const __restrict__ pointer"
+
+
+def test_attention_kernels_check_where_their_tensor_memory_starts():
+    # they address it from column 0: were it elsewhere, a void output would have to show in the status word
+    for f in ("forward.cu", "forward_rows.cu", "forward_bf16.cu", "forward_nvfp4.cu"):
+        bodies = [body for _, body in kernels(f) if "tcgen05.alloc" in body]
+        assert len(bodies) == 1, f
+        at_end = re.search(r"check_tmem_base\(\*tmem_slot, lane, p\.status\);\s*asm volatile\(\"tcgen05\.dealloc", bodies[0])
+        at_start = re.search(r"if \(\*tmem_slot != 0\) \*abort_flag = kCodeTmemBase;\s*const int role", bodies[0])
+        reported = re.search(r"if \(tid == 0 && \*abort_flag != 0\) atomicCAS\(p\.status, 0, \*abort_flag\);", bodies[0])
+        assert at_end or (at_start and reported), f

@@ -147,8 +147,8 @@ int sm_count();              // of the current device (0 on error)
 // of pairs fills at most half of the SMs, each of its tiles gets a CTA of its own, which takes less time than a pair.
 struct TileSplit {
   int64_t pair_ctas, ctas;
-  explicit TileSplit(int64_t pairs) {
-    const int64_t n_sm = sm_count(), rest = n_sm > 0 ? pairs % n_sm : 0;
+  TileSplit(int64_t pairs, int64_t n_sm) {
+    const int64_t rest = pairs % n_sm;
     pair_ctas = 2 * rest <= n_sm ? pairs - rest : pairs;
     ctas = pair_ctas + 2 * (pairs - pair_ctas);
   }
@@ -191,7 +191,7 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
                    int B, int H, int64_t Nq, int64_t Nkv, float softmax_scale, unsigned flags,
                    int* status, cudaStream_t stream, void* dump = nullptr, bool profile = false, bool followed = false);
 struct RowSplit { int64_t pairs_256; int R; };      // R = 0: nothing is left for the small CTAs
-RowSplit forward_row_split(int64_t bh, int64_t Nq, int64_t Nkv, bool pnq);
+RowSplit forward_row_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq);
 constexpr int kWalkMaxTiles = 48;    // longest key/value sequence (in tiles) for which a CTA of forward.cu walks several work items
 int launch_forward_rows(int R, int64_t first_pair, const void* q_codes, const void* q_scales, const void* k_codes, const void* k_scales,
                         const void* v_codes, const void* v_scales, void* o, int B, int H, int64_t Nq, int64_t Nkv,

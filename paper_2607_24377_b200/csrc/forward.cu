@@ -864,7 +864,7 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
   // query tiles that would leave SMs idle (a problem smaller than the GPU, or a last wave that is nearly empty) go to the
   // kernel for few query rows
   // (not where other attention launches run beside: their CTAs fill those SMs; 24 x 119056 in stages of one head 99.0 -> 93.1 ms)
-  const RowSplit split = dump || followed ? RowSplit{grid, 0} : forward_row_split((int64_t)B * H, Nq, Nkv, pnq);
+  const RowSplit split = dump || followed ? RowSplit{grid, 0} : forward_row_split(n_sm, (int64_t)B * H, Nq, Nkv, pnq);
   auto rest = [&]() {
     return split.R == 0 ? (int)MXATTN_OK
                         : launch_forward_rows(split.R, split.pairs_256, q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, o, B, H, Nq, Nkv,

@@ -375,6 +375,8 @@ int launch_forward_bf16(const void* q, const void* k, const void* v, void* o, in
   const int64_t qt = (Nq + kTile - 1) / kTile, kt = (Nkv + kTile - 1) / kTile;
   const int64_t pairs = (qt + 1) / 2, grid = bh * pairs;
   if (qt > 0x3FFFFFFF || kt > 65535 || qt > 0x7FFFFFFF || bh > 65535 || grid > 0x7FFFFFFF) return MXATTN_EUNSUPPORTED;
+  const int n_sm = sm_count();
+  if (n_sm == 0) return MXATTN_ECUDA;
   CUtensorMap q_map, k_map, v_map, out_map;
   const bool f32 = flags & MXATTN_FLAG_OUT_FP32;
   // The kernel reads its inputs while its first CTAs write the output.  An operand that the output overlaps is copied to the
@@ -400,7 +402,7 @@ int launch_forward_bf16(const void* q, const void* k, const void* v, void* o, in
   Params p;
   p.status = static_cast<int*>(workspace);
   p.Nq = Nq; p.Nkv = Nkv; p.q_tiles_n = (int)qt; p.kv_tiles = (int)kt; p.q_pairs = (int)pairs;
-  const TileSplit split(grid);
+  const TileSplit split(grid, n_sm);
   p.pair_ctas = (int)split.pair_ctas;
   p.scale_log2e = softmax_scale * 1.4426950408889634f;
   auto kern = f32 ? attention_bf16_kernel<true> : attention_bf16_kernel<false>;

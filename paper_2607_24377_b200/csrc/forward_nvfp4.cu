@@ -535,6 +535,8 @@ int launch_forward_nvfp4(const void* q, const void* k, const void* v, void* o, i
   const int64_t qt = (Nq + kTile - 1) / kTile, kt = (Nkv + kTile - 1) / kTile;
   const int64_t pairs = (qt + 1) / 2, grid = bh * pairs;
   if (qt > 0x3FFFFFFF || kt > 0x3FFFFFFF || grid > 0x7FFFFFFF) return MXATTN_EUNSUPPORTED;
+  const int n_sm = sm_count();
+  if (n_sm == 0) return MXATTN_ECUDA;
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   float* amax = reinterpret_cast<float*>(ws + w.amax);
   float* ts = reinterpret_cast<float*>(ws + w.tscale);
@@ -548,7 +550,7 @@ int launch_forward_nvfp4(const void* q, const void* k, const void* v, void* o, i
   p.ts_q = ts; p.ts_k = ts + bh; p.ts_v = ts + 2 * bh;
   p.status = reinterpret_cast<int*>(ws + w.status);
   p.Nq = Nq; p.Nkv = Nkv; p.q_tiles = (int)qt; p.kv_tiles = (int)kt; p.q_pairs = (int)pairs;
-  const TileSplit split(grid);
+  const TileSplit split(grid, n_sm);
   p.pair_ctas = (int)split.pair_ctas;
   p.scale_log2e = softmax_scale * 1.4426950408889634f;
   const bool pnq = flags & MXATTN_FLAG_PNQ, f32 = flags & MXATTN_FLAG_OUT_FP32;

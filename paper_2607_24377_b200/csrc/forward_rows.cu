@@ -355,8 +355,8 @@ __global__ void __launch_bounds__(32 * (16 / R + 2), 1) attention_rows_kernel(co
 // small CTAs; and where the last wave of 256-row CTAs would be nearly empty, its items are cut into small CTAs instead:
 // 24 heads of 8192 queries are 5.19 waves (direct row sum 647 -> 603 us).  That second launch waits for the last of the full
 // waves, which costs a few us, and more where the CTAs of forward.cu do not walk their items in step.
-RowSplit forward_row_split(int64_t bh, int64_t Nq, int64_t Nkv, bool pnq) {
-  const int64_t n_sm = sm_count() > 0 ? sm_count() : 148, T = (Nkv + kTile - 1) / kTile, tiles = (Nq + kTile - 1) / kTile;
+RowSplit forward_row_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq) {
+  const int64_t T = (Nkv + kTile - 1) / kTile, tiles = (Nq + kTile - 1) / kTile;
   const int64_t pairs = (tiles + 1) / 2, total = bh * pairs, full = total / n_sm;
   const int64_t c256 = T * (pnq ? 2700 : 3050) + 4400;
   RowSplit best{total, 0};

@@ -486,7 +486,8 @@ static int launch_rot(const rot::Operand& a, const rot::Operand& b, bool tile, u
                     : rule == kRuleUos ? rot::quantize_axis1_rot_tc_kernel<false, 1> : rot::quantize_axis1_rot_tc_kernel<false, 2>);
   if (!ensure_dynamic_smem((const void*)kern, rot::kSmemBytes)) return MXATTN_ECUDA;
   const int64_t n = (int64_t)a.n_tiles + b.n_tiles, most = 2 * (int64_t)sm_count();
-  return launch_pdl(kern, dim3((unsigned)min(most > 0 ? most : (int64_t)296, n)), rot::kThreads, rot::kSmemBytes, stream, a, b, rule) == cudaSuccess
+  if (most == 0) return MXATTN_ECUDA;
+  return launch_pdl(kern, dim3((unsigned)min(most, n)), rot::kThreads, rot::kSmemBytes, stream, a, b, rule) == cudaSuccess
              ? MXATTN_OK : MXATTN_ECUDA;
 }
 

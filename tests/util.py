@@ -1,4 +1,6 @@
 """Helpers shared by the GPU parity tests (host-side marshalling only)."""
+import ctypes
+
 import numpy as np
 import torch
 
@@ -21,6 +23,19 @@ def operand_launches(cfg, rotate=False) -> int:
         return 2
     half_tiles = 2 * cfg.B * cfg.H * (-(-cfg.Nq // 128) - (-cfg.Nkv // 128))
     return 3 if half_tiles > 24 * torch.cuda.get_device_properties(0).multi_processor_count else 1
+
+
+class _RowSplit(ctypes.Structure):
+    _fields_ = [("pairs_256", ctypes.c_int64), ("R", ctypes.c_int)]
+
+
+def row_split(n_sm, heads, nq, nkv, pnq):
+    """What the MXFP4 forward gives to CTAs of 256 query rows (pairs of query tiles) and, if R > 0, to CTAs of 128/R rows."""
+    import paper_2607_24377_b200 as mx
+    f = mx.lib()._ZN6mxattn17forward_row_splitEllllb
+    f.argtypes, f.restype = [ctypes.c_int64] * 4 + [ctypes.c_bool], _RowSplit
+    s = f(n_sm, heads, nq, nkv, pnq)
+    return s.pairs_256, s.R
 
 
 def tile_code_offset(r, c):

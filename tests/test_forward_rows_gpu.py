@@ -1,5 +1,6 @@
-"""The attention kernel for few query rows (32 or 64 rows per CTA, replicated down the operand tile): against the oracle at
-its edges, and bit for bit against the 256-row kernel, which the same heads reach when many copies of them fill the GPU."""
+"""The attention kernel for few query rows (128/R rows per CTA, R = 4, 2 or 1, replicated R times down the operand tile):
+against the oracle at its edges, and bit for bit against the 256-row kernel, which the same heads reach when many copies of
+them fill the GPU."""
 import numpy as np
 import pytest
 import torch
@@ -22,7 +23,12 @@ def run(cfg, q, k, v, flags):
     return out.t.clone()
 
 
-# rows per CTA 32 (few heads) or 64 (the last three); query counts around the row groups, key counts around blocks and tiles
+def rows_per_cta(heads, nq, nkv, pnq):
+    """(pairs of query tiles in 256-row CTAs, R of the rest) on this device"""
+    return util.row_split(torch.cuda.get_device_properties(0).multi_processor_count, heads, nq, nkv, pnq)
+
+
+# R = 4 (few heads), 2 (50 and 70 heads) or 1 (20 heads); query counts around the row groups, key counts around blocks and tiles
 @pytest.mark.parametrize("H,nq,nkv", [(1, 1, 1), (2, 31, 33), (2, 33, 128), (1, 97, 129), (3, 64, 640), (1, 160, 1100),
                                       (50, 127, 300), (70, 65, 31), (20, 449, 257)])
 @pytest.mark.parametrize("uos,pnq", [(True, True), (False, False)])
@@ -43,7 +49,8 @@ def test_bit_identical_to_the_256_row_kernel(heads, f32):
     flags = mx.FLAG_UOS | mx.FLAG_PNQ | (mx.FLAG_OUT_FP32 if f32 else 0)
     one = si.custom_config("rb", 1, heads, 300, 700, 5)
     q, k, v = si.make_all(one)
-    want = run(one, q, k, v, flags)                                    # 32 (2 heads) or 64 rows (40 heads) per CTA
+    assert rows_per_cta(heads, 300, 700, True) == (0, 4 if heads == 2 else 1)
+    want = run(one, q, k, v, flags)
     many = si.custom_config("rm", 640 // heads, heads, 300, 700, 5)    # 1280 pairs of query tiles
     rep = lambda x: np.ascontiguousarray(np.broadcast_to(x, (many.B,) + x.shape[1:]))
     got = run(many, rep(q), rep(k), rep(v), flags)
@@ -61,6 +68,24 @@ def test_last_wave_cut_into_small_ctas(heads, nq, nkv, pnq):
     one = si.custom_config("lw", 1, 1, nq, nkv, 6)
     q, k, v = si.make_all(one)
     want = run(one, q, k, v, flags)
+    assert rows_per_cta(1, nq, nkv, pnq) == (0, 4) and rows_per_cta(heads, nq, nkv, pnq) == (148, 4)
     many = si.custom_config("lm", 1, heads, nq, nkv, 6)
     rep = lambda x: np.ascontiguousarray(np.broadcast_to(x, (1, heads) + x.shape[2:]))
     assert torch.equal(run(many, rep(q), rep(k), rep(v), flags), want.expand(1, heads, nq, 128))
+
+
+# 64 rows per CTA, alone and behind a full wave (44 and 45 heads), and 128 rows behind one (50 heads): every head must come out as
+# it does from the 256-row kernel, which 148 heads, whole waves, keep to
+@pytest.mark.parametrize("heads,nq,nkv,split", [(49, 127, 300, (0, 2)), (70, 65, 1100, (0, 2)), (49, 128, 640, (0, 2)),
+                                                (44, 1000, 700, (148, 2)), (45, 897, 1300, (148, 2)), (50, 1000, 700, (148, 1))])
+@pytest.mark.parametrize("pnq", [True, False])
+def test_64_and_128_rows_per_cta_equal_the_256_row_kernel(heads, nq, nkv, split, pnq):
+    import paper_2607_24377_b200 as mx
+    flags = mx.FLAG_UOS | (mx.FLAG_PNQ if pnq else 0)
+    assert rows_per_cta(heads, nq, nkv, pnq) == split and rows_per_cta(148, nq, nkv, pnq)[1] == 0
+    few = si.custom_config("h64", 1, heads, nq, nkv, 8)
+    q, k, v = si.make_all(few)
+    got = run(few, q, k, v, flags)
+    many = si.custom_config("h64m", 1, 148, nq, nkv, 8)
+    rep = lambda x: np.ascontiguousarray(x[:, np.arange(148) % heads])
+    assert torch.equal(run(many, rep(q), rep(k), rep(v), flags)[:, :heads], got)

@@ -294,6 +294,7 @@ static HostPipe* host_pipe(size_t n_events) {
   return &hp;
 }
 
+namespace mxattn {
 // First heads of the pipeline stages of mxattn_forward_host; the last entry is bh.  last_alone: the attention of earlier
 // stages is done when the last stage's operands arrive.  The link bounds the call (a head of N tokens arrives in 14 us per
 // 1000 tokens, and its attention takes less than that below some 50000 tokens), and a stage costs it about 20 us: three
@@ -309,31 +310,46 @@ static HostPipe* host_pipe(size_t n_events) {
 // Against one head followed by stages of equal size, us: 24 x 8192 3310 -> 3249 (copying in alone takes 2731), 40 x 4096
 // 2858 -> 2712 (2280), 160 x 5000 13170 -> 12230, 160 x 300 1134 -> 912, 2 x 1024 (one stage now) 195 -> 164, 12 x 20000
 // 4084 -> 4011; 40 heads of 10000 x 512 3024 -> 3023, of 75600 x 512 18460 -> 18060.
-static std::vector<size_t> host_stages(size_t bh, int64_t Nq, int64_t Nkv, size_t in_bytes_per_head, size_t out_bytes_per_head, bool* last_alone) {
+//   - Up to eight heads of which one fits the SMs and two do not (256 query rows per CTA): a stage of two leaves a second
+//     wave, which is late when the last stage follows right behind.  There the sizes grow by the ratio itself, kept above
+//     1.25, and not by what it rounds to, and the larger stages come first (2, 1, 1 instead of 1, 2, 1).  Direct row sum /
+//     PNQ, 21070 x 21070: 4 heads 1811 / 1735 -> 1653 / 1651, 6 heads 2447 / 2390 -> 2286 / 2321, 8 heads 3159 / 3076 -> 2998 / 3037;
+//     28000 x 28000, 4 heads 2420 / 2287 -> 2149 / 2134.  Where two heads fit (18000 x 18000) it is 3 to 8 % slower, from
+//     twelve heads on as fast.
+// first[0 .. stages] receives the first heads (room for bh + 1); the number of stages is returned.
+size_t host_stages(size_t bh, int64_t Nq, int64_t Nkv, size_t in_bytes_per_head, size_t out_bytes_per_head, int n_sm, size_t* first, bool* last_alone) {
   const double t_in = (double)in_bytes_per_head / 55e9, t_out = (double)out_bytes_per_head / 55e9;
   const double t_attn = 4.0 * (double)Nq * (double)Nkv * kHeadDim / 1.6e15;
-  const double shrink = std::min(3.0, std::max(1.5, 1.1 * t_in / (t_out + t_attn)));
+  const double ratio = 1.1 * t_in / (t_out + t_attn);
   const size_t least = (size_t)(2.5e6 / (double)in_bytes_per_head) + 1;
   const double t_other = std::max(t_out, t_attn);
   const bool in_bound = t_in > 1.5 * t_other;
+  const int64_t ctas = (Nq + 2 * kTile - 1) / (2 * kTile);       // of a head
+  const bool late = in_bound && ratio < 1.5 && bh <= 8 && ctas <= n_sm && 2 * ctas > n_sm;
+  const double shrink = std::min(3.0, std::max(late ? 1.25 : 1.5, ratio));
   const size_t most = in_bound ? bh : std::max(least, (size_t)std::ceil(std::sqrt((double)bh * 20e-6 / t_other)));
   *last_alone = in_bound || bh <= least;
   size_t next_head = in_bound ? std::max(least, bh / 8) : least, next_tail = least;
+  double size_tail = (double)least;
   std::vector<size_t> head, tail;
   for (size_t left = bh; left > 0;) {
-    const bool at_head = next_head < next_tail;
+    const bool at_head = next_head < next_tail && !(late && left <= next_tail);
     size_t& next = at_head ? next_head : next_tail;
     // what would be left over and too small for a stage of its own joins this one
     const size_t n = 4 * left < 5 * next || left < next + least ? left : next;
     (at_head ? head : tail).push_back(n);
-    next = std::min(most, at_head ? 2 * n : (size_t)std::lround(shrink * (double)n));
+    if (!at_head) size_tail = shrink * (late ? size_tail : (double)n);
+    next = std::min(most, at_head ? 2 * n : (size_t)std::lround(size_tail));
     left -= n;
   }
-  std::vector<size_t> first(1, 0);
-  for (size_t n : head) first.push_back(first.back() + n);
-  for (size_t k = tail.size(); k-- > 0;) first.push_back(first.back() + tail[k]);
-  return first;
+  size_t stages = 0;
+  first[0] = 0;
+  auto add = [&](size_t n) { first[stages + 1] = first[stages] + n; ++stages; };
+  for (size_t n : head) add(n);
+  for (size_t k = tail.size(); k-- > 0;) add(tail[k]);
+  return stages;
 }
+}  // namespace mxattn
 
 extern "C" size_t mxattn_forward_host_arena_bytes(int B, int H, int64_t Nq, int64_t Nkv, int d, unsigned flags) {
   WorkspaceLayout w;
@@ -365,8 +381,8 @@ extern "C" int mxattn_forward_host(const void* q_host, const void* k_host, const
   uint8_t* dout = dv + align_up(bh * kh, 256);
   uint8_t* ws = dout + align_up(bh * oh, 256);
   bool last_alone;
-  const std::vector<size_t> first_head = host_stages(bh, Nq, Nkv, qh + 2 * kh, oh, &last_alone);
-  const size_t stages = first_head.size() - 1;
+  std::vector<size_t> first_head(bh + 1);
+  const size_t stages = host_stages(bh, Nq, Nkv, qh + 2 * kh, oh, sm_count(), first_head.data(), &last_alone);
   HostPipe* hp = host_pipe(3 * stages + 2);
   if (!hp) return MXATTN_ECUDA;
   cudaEvent_t* ev = hp->ev.data();

@@ -30,3 +30,23 @@ def test_last_wave_is_divided_for_the_sms_that_there_are(n_sm, pnq):
         assert pairs == (total if r == 0 else total // n_sm * n_sm)          # whole waves, or everything
     assert util.row_split(n_sm, n_sm, 256, 1024, pnq) == (n_sm, 0)            # exactly a wave
     assert util.row_split(n_sm, 1, 32, 1024, pnq) == (0, 4)                   # a single group of rows
+
+
+def stages(heads, nq, nkv, n_sm=148):
+    f = rule("_ZN6mxattn11host_stagesEmllmmiPmPb", ctypes.c_size_t, ctypes.c_int64, ctypes.c_int64, ctypes.c_size_t, ctypes.c_size_t, ctypes.c_int,
+             ctypes.POINTER(ctypes.c_size_t), ctypes.POINTER(ctypes.c_bool), restype=ctypes.c_size_t)
+    first, alone = (ctypes.c_size_t * (heads + 1))(), ctypes.c_bool()
+    n = f(heads, nq, nkv, 256 * (nq + 2 * nkv), 256 * nq, n_sm, first, ctypes.byref(alone))
+    assert first[0] == 0 and first[n] == heads
+    return [first[i + 1] - first[i] for i in range(n)]
+
+
+def test_stages_of_the_host_form():
+    for heads in (*range(1, 20), 40, 160):                    # every head once, no empty stage, whatever the sizes
+        for nq, nkv in ((1, 1), (300, 300), (8192, 8192), (18000, 18000), (21070, 21070), (28000, 28000), (75600, 512), (130, 9000), (75600, 75600)):
+            s = stages(heads, nq, nkv)
+            assert min(s) >= 1 and sum(s) == heads
+    # two heads fit the SMs: sizes double or halve towards the end; they do not, and heads are few: two single ones at the end
+    assert stages(4, 18000, 18000) == [1, 2, 1] and stages(24, 8192, 8192) == [3, 6, 8, 4, 2, 1]
+    assert stages(4, 21070, 21070) == [2, 1, 1] and stages(5, 28000, 28000) == [1, 2, 1, 1] and stages(6, 24000, 24000) == [1, 1, 2, 1, 1]
+    assert stages(4, 21070, 21070, n_sm=300) == [1, 2, 1] and stages(12, 21070, 21070)[-2:] == [2, 1]

@@ -16,6 +16,7 @@ pytestmark = pytest.mark.gpu
     (23, 2200, 2200),     # copies in are the bound: growing, then shrinking stages
     (13, 6000, 100),      # copies out weigh as much: equal stages
     (9, 130, 9000),       # Q and the output are small
+    (4, 19500, 19500),    # two heads are more than a wave: the larger stages first
 ])
 def test_host_stages_equal_the_device_path(H, Nq, Nkv):
     import paper_2607_24377_b200 as mx

@@ -1,5 +1,5 @@
-// C-ABI entry points that orchestrate the kernels: workspace carving, the three quantize
-// launches plus the fused attention launch (paper Algorithm 2, lines 3-19), and the host-buffer
+// C-ABI entry points that orchestrate the kernels: workspace carving, the operand launches (one to
+// three) and the fused attention (one or two; paper Algorithm 2, lines 3-19), and the host-buffer
 // end-to-end form.
 #include <algorithm>
 #include <atomic>

@@ -23,7 +23,8 @@
 // The output leaves as tensor copies (store_half_rows) from the query tiles' own shared memory: 69.8 -> 65.6 us at
 // H=40, 4096 x 512 (fp32 84.3 -> 71.9), 123 -> 115 at H=24, 8192 x 1024.
 // A last wave that would leave half of the SMs idle runs with one query tile per CTA (common.cuh): 755 -> 646 us at
-// H=24, N=8192 (5.19 waves), 25 -> 19 us at 2 heads of 1024.
+// H=24, N=8192 (5.19 waves), 25 -> 19 us at 2 heads of 1024.  (All figures in series of a few calls at full clock; under the power
+// limit the same 24 x 8192 takes 674 us in the mean of 20 calls back to back, 706 to 721 of some hundred, 787 of 2000.)
 #include <string.h>
 
 #include <type_traits>

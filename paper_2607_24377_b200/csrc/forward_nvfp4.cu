@@ -14,8 +14,9 @@
 //   per block: M = its largest p = exp2(s_max * c - m_new * c), d = E4M3(fl32(fl32(M * 2688) * fl32(1/6))), scale byte = d
 //   per element: codes = E2M1(exp2(s_i * c - m_new * c + log2(2688 / d)))      half a packed fma + one ex2
 // which is the library's NVFP4 recipe (include/mxattn.h) with the tensor maximum 1, the element multiplier
-// r = 2688 / d folded into the exponent (the recipe's fl32(p_i * r) differs from this by about 2e-7 relative, the order
-// of ex2.approx itself; a block with d = 0 keeps r = 1, its codes are 0 either way).
+// r = 2688 / d folded into the exponent (the recipe's fl32(p_i * r) differs from this by about 2e-7 relative for the blocks
+// that carry a row, d > 168, the order of ex2.approx itself, and by up to 1.5e-6 for the smallest scales, whose logarithm
+// is a larger number; a block with d = 0 keeps r = 1, its codes are 0 either way).
 //
 // One CTA per work item: two query tiles of one head, or one where the last wave would leave half of the SMs idle
 // (common.cuh; 2 heads of 1024: 29 -> 23 us, 40 heads of 16384: 4090 -> 4033).  The output leaves as tensor copies
@@ -89,11 +90,6 @@ __device__ __forceinline__ void tc_mma_nv(uint32_t d_tmem, uint64_t a_desc, uint
   asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
                "tcgen05.mma.cta_group::1.kind::mxf4nvf4.block_scale.block16 [%0], %1, %2, %3, [%5], [%6], p;\n\t}"
                ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(sfa), "r"(sfb) : "memory");
-}
-__device__ __forceinline__ uint32_t e4m3_encode(float y) {
-  uint16_t r;
-  asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(0.0f), "f"(y));
-  return (uint32_t)(r & 0xFFu);
 }
 __device__ __forceinline__ float e4m3_decode(uint32_t code) {
   uint32_t h2;
@@ -376,8 +372,8 @@ __global__ void __launch_bounds__(kThreads, 1) attention_nvfp4_kernel(const Para
       float alpha = 1.0f;
       // Block scales: the block's largest probability by the elements' own expression, then the two-level recipe, two blocks
       // per conversion.  The element multiplier 2688 / d_b is folded into the exponent as its logarithm, which (like
-      // d_b / 2688) comes from a table of the 127 codes, correctly rounded: relative difference about 2e-7, the order of
-      // ex2.approx itself.  (Computed per block -- decode, lg2.approx on the mantissa, two additions and the selections for
+      // d_b / 2688) comes from a table of the 127 codes: log2f of the rounded quotient, within a unit in the last place of the
+      // logarithm plus the quotient's 9e-8.  (Computed per block -- decode, lg2.approx on the mantissa, two additions and the selections for
       // subnormal and zero codes -- it was 22 instructions per block instead of 8.)  A block whose scale rounds to zero
       // keeps multiplier 1: its probabilities are below 2.2e-6 and round to code 0 either way, and the direct placement
       // still sums them.

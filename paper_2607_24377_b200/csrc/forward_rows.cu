@@ -354,7 +354,10 @@ __global__ void __launch_bounds__(32 * (16 / R + 2), 1) attention_rows_kernel(co
 // cycles per row, so a problem that fills whole waves of 256-row CTAs stays there; a problem smaller than a wave goes to
 // small CTAs; and where the last wave of 256-row CTAs would be nearly empty, its items are cut into small CTAs instead:
 // 24 heads of 8192 queries are 5.19 waves (direct row sum 647 -> 603 us).  That second launch waits for the last of the full
-// waves, which costs a few us, and more where the CTAs of forward.cu do not walk their items in step.
+// waves.  With PNQ it adds what the same rows take by themselves, within 2 us (28 pairs behind 1, 5 and 20 waves: 41.8, 41.2,
+// 40.9 us for 41.6 at 48 tiles; 102.2, 101.7, 102.4 for 100.4 at 128), with the direct row sum up to 12 us more (5 waves of
+// 128 tiles: 116.3 for 104.7; 46 us more in one series of ten, 20 waves of 48 tiles), as CTAs drift apart.  The estimate charges
+// 4000 cycles, and a tenth of a wave where CTAs do not walk their items, so that a close call keeps to one launch.
 RowSplit forward_row_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq) {
   const int64_t T = (Nkv + kTile - 1) / kTile, tiles = (Nq + kTile - 1) / kTile;
   const int64_t pairs = (tiles + 1) / 2, total = bh * pairs, full = total / n_sm;

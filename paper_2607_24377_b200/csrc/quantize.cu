@@ -502,8 +502,9 @@ int launch_quantize_qkv(const void* q, void* q_codes, void* q_scales, const void
   QkvOperand ok{k, (uint8_t*)k_codes, (uint8_t*)k_scales, Nkv, kt, rotate ? 0 : 2 * bh * kt};
   QkvOperand ov{v, (uint8_t*)v_codes, (uint8_t*)v_scales, Nkv, kt, v ? bh * kt : 0};
   // Long problems are bound by bandwidth: Q and K then run in the kernel of their own, which has six CTAs per SM where the
-  // shared one has four (its registers and shared memory are sized for V) -- 774 MB of Q: 0.12 against 0.14 ms.  From 24
-  // CTAs per SM on that outweighs the two further launches.
+  // shared one has four (its registers and shared memory are sized for V) -- 774 MB of Q: 0.12 against 0.14 ms.  That
+  // outweighs the two further launches somewhere between 18 and 35 CTAs per SM: whole call of 40 heads against 128 keys, us,
+  // one launch / apart: 1280 queries (6 per SM) 15.8 / 20.5, 4096 (18) 32.8 / 34.0, 8192 (35) 57.9 / 56.6, 16384 (70) 104.2 / 98.8.
   const int n_sm = sm_count();
   if (n_sm == 0) return MXATTN_ECUDA;
   if (!rotate && oq.ctas + ok.ctas > 24 * (int64_t)n_sm && bh <= 65535) {

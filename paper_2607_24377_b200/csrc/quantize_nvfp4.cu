@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(kThreads) tensor_amax_qkv_kernel(const AmaxOpe
 // Canonical layout: chunks = rows * cols / 8 per matrix; tile layout (cols == 128): chunks = rows_pad * 16, rows beyond
 // `rows` read as zero.  As a kernel of its own it runs in CTAs of 128 threads (grid = (ceil(chunks / 512), batch)): a CTA
 // alternates between loading and computing, and sixteen small ones per SM keep the loads flowing better than eight of
-// 256 threads (16M / 34M / 134M elements, 128 columns: 9.2 -> 8.7, 15.9 -> 15.1, 59.5 -> 57.1 us).
+// 256 threads (quantizer alone, 8 matrices of 128 columns, 2^24 / 2^25 / 2^27 elements: 8.7 -> 8.0, 15.0 -> 14.2, 55.9 -> 53.7 us).
 constexpr int kA1Threads = 128;
 template <bool kTileLayout, int kT>
 __device__ __forceinline__ void quantize_nvfp4_axis1_part(uint4* s_v, const uint4* __restrict__ in, uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
@@ -365,7 +365,10 @@ int launch_nvfp4_operands(const void* q, void* q_codes, void* q_scales, const vo
   QkvOperand oq{q, (uint8_t*)q_codes, (uint8_t*)q_scales, amax, tensor_scale, Nq, qt, 2 * bh * qt};
   QkvOperand ok{k, (uint8_t*)k_codes, (uint8_t*)k_scales, amax + bh, tensor_scale + bh, Nkv, kt, 2 * bh * kt};
   QkvOperand ov{v, (uint8_t*)v_codes, (uint8_t*)v_scales, amax + 2 * bh, tensor_scale + 2 * bh, Nkv, kt, bh * kt};
-  if (oq.ctas + ok.ctas > 24 * (int64_t)n_sm) {    // long problems: a kernel of their own for Q and K (quantize.cu has the reason)
+  // Long problems: a kernel of their own for Q and K (quantize.cu has the reason).  The sides cross later than there, but
+  // within 1 % of one another: 40 heads against 128 keys, us, one launch / apart: 1280 queries (6 per SM) 22.7 / 26.7, 8192
+  // (35) 110.1 / 111.2, 16384 (70) 208.7 / 206.8; 24 x 8192 (42) 720.0 / 719.4.
+  if (oq.ctas + ok.ctas > 24 * (int64_t)n_sm) {
     for (const QkvOperand* o : {&oq, &ok})
       if (launch_pdl(quantize_nvfp4_axis1_kernel<true>, dim3((unsigned)(kTile * kHeadDim / 32 / kA1Threads * o->tiles), (unsigned)bh), kA1Threads, 0, stream, (const uint4*)o->in, o->codes, o->scales,
                      o->amax, o->tensor_scale, o->rows, (int64_t)kHeadDim, o->tiles * kTile) != cudaSuccess) return MXATTN_ECUDA;

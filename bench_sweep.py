@@ -11,7 +11,7 @@
 * row-sum diagnostic (Section 5.3): mean row sum of the quantized materialized probabilities and its split
   by quantization outcome, OCP / UOS / UOS+Hadamard, on three synthetic recipes at N=4096;
 * short key/value sequences (cross-attention shapes): H=37, Nq=16384, 1 .. 96 KV tiles of 128 keys, attention launch
-  only on pre-quantized operands: time and TFLOP/s (up to 48 tiles the launch uses the item-walking variant);
+  only on pre-quantized operands: time and TFLOP/s (the launch walks items of one query tile);
 * Q_max study (paper Section 5.4.1 and its table of per-block optima): the ceiling-family boundary swept from 6.00 to
   8.00 in steps of 0.05 with mxattn_quantize_mxfp4_qmax on synthetic Q, K, V of 40 heads per recipe (the heads stand in
   for the paper's 40 attention blocks): tensor MSE per point, and the histogram of the per-head optimum;
@@ -65,7 +65,7 @@ def cycle_profile(mx, torch, cfg, dev):
     ms_prof = timed(lambda: mx.forward_cycle_profile(dq, dk, dv, out, B, H, Nq, Nkv, d, cfg.softmax_scale, flags, ws, prof))
     assert mx.device_status(ws) == 0 and torch.equal(out, ref)
     p = prof.view(-1, 18, 16).cpu().numpy().astype(np.float64)
-    p = p[p[:, 17, 9] > 0]                                    # CTAs that ran (one per SM in the item-walking variant)
+    p = p[p[:, 17, 9] > 0]                                    # CTAs that ran
     tiles = p[:, 17, 9][:, None]
     kv_tiles = -(-Nkv // 128)
     sm = p[:, :16, :]

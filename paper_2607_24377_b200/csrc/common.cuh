@@ -192,11 +192,12 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
                    int* status, cudaStream_t stream, void* dump = nullptr, bool profile = false, bool followed = false);
 struct RowSplit { int64_t pairs_256; int R; };      // R = 0: nothing is left for the small CTAs
 RowSplit forward_row_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq);
-// Longest key/value sequence (in tiles) for which a CTA of forward.cu walks several work items.  40 heads of 8192 queries,
-// us, walking / one item per CTA, at 16, 32, 48, 56, 64, 96 tiles: PNQ 261 / 283, 473 / 485, 681 / 684, 784 / 782, 886 / 880,
-// 1291 / 1269.  With the direct row sum walking stays ahead: 290 / 317, 527 / 550, 758 / 777, 872 / 890, 985 / 1002, 1433 / 1441.
-constexpr int kWalkMaxTiles = 48;
+struct WalkSplit { bool walk; int64_t pairs; };     // whether forward_walk.cu takes the first `pairs` pairs (the rest: small CTAs)
+WalkSplit forward_walk_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq, bool followed, const RowSplit& split);     // `followed`: other attention launches run beside
 int launch_forward_rows(int R, int64_t first_pair, const void* q_codes, const void* q_scales, const void* k_codes, const void* k_scales,
+                        const void* v_codes, const void* v_scales, void* o, int B, int H, int64_t Nq, int64_t Nkv,
+                        float softmax_scale, unsigned flags, int* status, cudaStream_t stream);
+int launch_forward_walk(int64_t n_sm, int64_t pairs, const void* q_codes, const void* q_scales, const void* k_codes, const void* k_scales,
                         const void* v_codes, const void* v_scales, void* o, int B, int H, int64_t Nq, int64_t Nkv,
                         float softmax_scale, unsigned flags, int* status, cudaStream_t stream);
 size_t forward_dump_bytes(int B, int H, int64_t Nq, int64_t Nkv);

@@ -46,10 +46,9 @@
 // swizzle) and leaves as one tensor copy per warp (fp32: two) through a tensor map of the output, so that whole
 // lines are written and the stores do not queue in front of the next tile's shared-memory traffic.
 //
-// Two launch shapes: one CTA per work item (two query tiles of one head), or -- more items than SMs and a short
-// KV sequence -- one CTA per SM that walks the items and keeps barriers, tensor memory and the K/V ring across
-// them (template flag kPersist).  Query tiles that would leave SMs idle (a small problem, a nearly empty last wave)
-// go to the kernel for few query rows (forward_rows.cu).
+// One CTA per work item (two query tiles of one head).  launch_forward gives this kernel the long key/value sequences;
+// forward_walk.cu takes the others, and query tiles that would leave SMs idle go to the kernel for few query rows
+// (forward_rows.cu).
 //
 // Every mbarrier wait is bounded; on expiry the CTA records a code in `status`, drains and exits.
 #include <string.h>
@@ -75,17 +74,17 @@ constexpr int kVStageBytes = kNV * 64;           // 9216
 constexpr int kDumpTileBytes = kTileCodeBytes + kTileScaleBytes + kTile * 4;   // debug dump: codes, scale atom, m per row
 
 // shared memory map (byte offsets from a 1024-aligned base)
-constexpr int kOffQ = 0;                                   // 2 buffers x 2 tiles x 8192 (the second buffer: persistent variant)
-constexpr int kOffK = kOffQ + 4 * kTileCodeBytes;          // 4 x 8192
+constexpr int kOffQ = 0;                                   // 2 tiles x 8192
+constexpr int kOffK = kOffQ + 2 * kTileCodeBytes;          // 4 x 8192
 constexpr int kOffV = kOffK + kStages * kTileCodeBytes;    // 4 x 9216
 constexpr int kOffP = kOffV + kStages * kVStageBytes;      // 2 x 8192
-constexpr int kOffSFQ = kOffP + 2 * kTileCodeBytes;        // 2 buffers x 2 x 512
-constexpr int kOffSFK = kOffSFQ + 4 * kTileScaleBytes;     // 4 x 512
+constexpr int kOffSFQ = kOffP + 2 * kTileCodeBytes;        // 2 x 512
+constexpr int kOffSFK = kOffSFQ + 2 * kTileScaleBytes;     // 4 x 512
 constexpr int kOffSFV = kOffSFK + kStages * kTileScaleBytes;   // 4 x 512
 constexpr int kOffSFOnes = kOffSFV + kStages * kTileScaleBytes; // 512
 constexpr int kOffSFP = kOffSFOnes + kTileScaleBytes;      // 2 x 512
 constexpr int kOffBar = kOffSFP + 2 * kTileScaleBytes;     // barriers
-constexpr int kNumBars = 4 + 2 * kStages + 2 + 1 + 2 + 2;  // Q full/empty[2], K/V stage full+empty, S_full[2], S_free, P_full[2], O_done[2]
+constexpr int kNumBars = 1 + 2 * kStages + 2 + 1 + 2 + 2;  // Q, K/V stage full+empty, S_full[2], S_free, P_full[2], O_done[2]
 constexpr int kOffMisc = kOffBar + kNumBars * 8;           // tmem slot, abort flag
 constexpr int kOffMax = kOffMisc + 64;                     // half-row maxima: [parity 2][tile 2][half 2][128] floats
 constexpr int kOffOut = (kOffMax + 2 * 2 * 2 * 128 * 4 + 1023) & ~1023;   // output staging: one box per softmax warp
@@ -93,7 +92,7 @@ constexpr int kSmemBytes = kOffOut + kSoftmaxWarps * kOutBoxBytes + 1024;   // +
 static_assert(kOffOut % 1024 == 0 && kOutBoxBytes % 1024 == 0, "swizzled boxes start on the swizzle pattern's period");
 static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
 
-enum Bar { BAR_Q = 0, BAR_QEMPTY = 2, BAR_KFULL = 4, BAR_KEMPTY = BAR_KFULL + kStages,     // one full / empty pair per K/V stage
+enum Bar { BAR_Q = 0, BAR_KFULL = 1, BAR_KEMPTY = BAR_KFULL + kStages,     // one full / empty pair per K/V stage
            BAR_SFULL = BAR_KEMPTY + kStages, BAR_SFREE = BAR_SFULL + 2,
            BAR_PFULL = BAR_SFREE + 1, BAR_ODONE = BAR_PFULL + 2 };
 
@@ -115,24 +114,15 @@ struct Params {
 };
 
 // ---------------------------------------------------------------------------------------------
-// kPersist: the CTA walks several work items (blockIdx.x, blockIdx.x + gridDim.x, ...) and keeps its barriers,
-// tensor memory and pipelines across them: the next item's Q tiles and first K/V tiles are fetched and its first
-// scores computed while the current item drains.  Used for short KV sequences, where the per-CTA set-up, the
-// latency of the first loads and the launch gap between CTAs are a large share of an item's time.
-// Waits of the single-thread roles.  In the item-walking variant their loops carry the item bookkeeping as well, and
-// keeping the waits' slow path out of line there shortens the time per tile by 6 %; in the one-item variant the same
-// change measured 3 % slower, so that one keeps the inline form.
 // kProf (cycle profile, never in a timed build): every role accumulates SM cycles per phase of its loop and writes them
 // to p.dump as [CTA][warp 0..17][16] int64 (softmax warps: slots 0-8 = S-full wait, score load, maxima, pair
 // exchange, O-done wait, block exponents, exponentials + pack, hand-over, epilogue; slot 9 = tiles; producer and
 // issuer: slots 0-7 = cycles inside the wait with code c at slot c mod 8, slot 8 = cycles of the whole loop, slot 9 = tiles).
-#define MBAR_WAIT_ROLE(...) (kProf ? prof_wait(__VA_ARGS__) : (kPersist ? mbar_wait1(__VA_ARGS__) : mbar_wait(__VA_ARGS__)))
+#define MBAR_WAIT_ROLE(...) (kProf ? prof_wait(__VA_ARGS__) : mbar_wait(__VA_ARGS__))
 #define PROF_MARK(i) do { if (kProf) { const long long prof_now = clock64(); prof_t[i] += prof_now - prof_prev; prof_prev = prof_now; } } while (0)
 constexpr int kProfSlots = 16;
-template <bool kUos, bool kPnq, bool kOutF32, bool kDump, bool kPersist, bool kProf = false>
+template <bool kUos, bool kPnq, bool kOutF32, bool kDump, bool kProf = false>
 __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, const __grid_constant__ CUtensorMap out_map) {
-  static_assert(!(kDump && kPersist), "the tile dump is written by the one-item-per-CTA variant only");
-  constexpr int kOutSize = kOutF32 ? 4 : 2, kBoxCols = 128 / kOutSize;
   static_assert(!(kDump && kProf), "the dump buffer holds either the tile dump or the cycle profile");
   long long prof_t[kProfSlots];
   long long prof_prev = 0;
@@ -156,12 +146,11 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int T = p.kv_tiles;
-  const int bh0 = blockIdx.x / p.q_pairs, pair0 = blockIdx.x - bh0 * p.q_pairs;
+  const int bh = blockIdx.x / p.q_pairs, pair = blockIdx.x - bh * p.q_pairs;
 
   // ---- setup -------------------------------------------------------------------------------
   if (tid == 0) {
-    mbar_init(bar(BAR_Q + 0), 1); mbar_init(bar(BAR_Q + 1), 1);
-    mbar_init(bar(BAR_QEMPTY + 0), 1); mbar_init(bar(BAR_QEMPTY + 1), 1);
+    mbar_init(bar(BAR_Q), 1);
     for (int s = 0; s < kStages; ++s) {
       mbar_init(bar(BAR_KFULL + s), 1); mbar_init(bar(BAR_KEMPTY + s), 1);
     }
@@ -199,50 +188,36 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
   if (role == kSoftmaxWarps) {
     // =============================== producer ===============================================
     if (lane == 0) {
-      int F = 0;                                   // tiles issued so far, over all items of this CTA
-      int q_issued = 0;                            // items whose Q tiles were issued
       bool ok = true;
       if (kProf) prof_prev = clock64();
-      for (int n = 0, item = blockIdx.x; (kPersist ? item < p.total_items : n < 1) && ok; ++n, item += gridDim.x) {
-        const int bh = item / p.q_pairs, pair = item - bh * p.q_pairs;
-        const int qb = kPersist ? (n & 1) : 0;     // Q buffer
-        // the Q buffer of item n - 2 is free once every GEMM 1 of that item has completed
-        if (kPersist && n >= 2) ok = MBAR_WAIT_ROLE(bar(BAR_QEMPTY + qb), (uint32_t)(((n - 2) >> 1) & 1), abort_flag, p.status, 13);
+      const int64_t qt0 = (int64_t)bh * p.q_tiles + 2 * pair;
+      const int64_t qt1 = (2 * pair + 1 < p.q_tiles) ? qt0 + 1 : qt0;     // odd tail: reuse tile 0 (result unused)
+      mbar_expect_tx(bar(BAR_Q), 2 * (kTileCodeBytes + kTileScaleBytes));
+      bulk_g2s(sbase + kOffQ, p.q_codes + qt0 * kTileCodeBytes, kTileCodeBytes, bar(BAR_Q));
+      bulk_g2s(sbase + kOffQ + kTileCodeBytes, p.q_codes + qt1 * kTileCodeBytes, kTileCodeBytes, bar(BAR_Q));
+      bulk_g2s(sbase + kOffSFQ, p.q_scales + qt0 * kTileScaleBytes, kTileScaleBytes, bar(BAR_Q));
+      bulk_g2s(sbase + kOffSFQ + kTileScaleBytes, p.q_scales + qt1 * kTileScaleBytes, kTileScaleBytes, bar(BAR_Q));
+      const int64_t kv0 = (int64_t)bh * T;
+      int j = 0;
+      for (; j < T; ++j) {
+        const int s = j % kStages;
+        if (j >= kStages) ok = MBAR_WAIT_ROLE(bar(BAR_KEMPTY + s), (uint32_t)((j / kStages) & 1) ^ 1u, abort_flag, p.status, 11);
         if (!ok) break;
-        const int64_t qt0 = (int64_t)bh * p.q_tiles + 2 * pair;
-        const int64_t qt1 = (2 * pair + 1 < p.q_tiles) ? qt0 + 1 : qt0;     // odd tail: reuse tile 0 (result unused)
-        const uint32_t sq = sbase + kOffQ + qb * 2 * kTileCodeBytes, ssf = sbase + kOffSFQ + qb * 2 * kTileScaleBytes;
-        mbar_expect_tx(bar(BAR_Q + qb), 2 * (kTileCodeBytes + kTileScaleBytes));
-        bulk_g2s(sq, p.q_codes + qt0 * kTileCodeBytes, kTileCodeBytes, bar(BAR_Q + qb));
-        bulk_g2s(sq + kTileCodeBytes, p.q_codes + qt1 * kTileCodeBytes, kTileCodeBytes, bar(BAR_Q + qb));
-        bulk_g2s(ssf, p.q_scales + qt0 * kTileScaleBytes, kTileScaleBytes, bar(BAR_Q + qb));
-        bulk_g2s(ssf + kTileScaleBytes, p.q_scales + qt1 * kTileScaleBytes, kTileScaleBytes, bar(BAR_Q + qb));
-        q_issued = n + 1;
-        const int64_t kv0 = (int64_t)bh * T;
-        for (int j = 0; j < T && ok; ++j, ++F) {
-          const int s = F % kStages;
-          const uint32_t ph = (uint32_t)((F / kStages) & 1);
-          if (F >= kStages) ok = MBAR_WAIT_ROLE(bar(BAR_KEMPTY + s), ph ^ 1u, abort_flag, p.status, 11);
-          if (!ok) break;
-          // K-hat_j and V-hat_j travel together: one full / one empty barrier per stage (the issuer thread's time
-          // per tile is what bounds the kernel, and every wait or commit it does not need shortens it)
-          mbar_expect_tx(bar(BAR_KFULL + s), 2 * (kTileCodeBytes + kTileScaleBytes));
-          bulk_g2s(sbase + kOffK + s * kTileCodeBytes, p.k_codes + (kv0 + j) * kTileCodeBytes, kTileCodeBytes, bar(BAR_KFULL + s));
-          bulk_g2s(sbase + kOffSFK + s * kTileScaleBytes, p.k_scales + (kv0 + j) * kTileScaleBytes, kTileScaleBytes, bar(BAR_KFULL + s));
-          bulk_g2s(sbase + kOffV + s * kVStageBytes, p.v_codes + (kv0 + j) * kTileCodeBytes, kTileCodeBytes, bar(BAR_KFULL + s));
-          bulk_g2s(sbase + kOffSFV + s * kTileScaleBytes, p.v_scales + (kv0 + j) * kTileScaleBytes, kTileScaleBytes, bar(BAR_KFULL + s));
-        }
+        // K-hat_j and V-hat_j travel together: one full / one empty barrier per stage (the issuer thread's time
+        // per tile is what bounds the kernel, and every wait or commit it does not need shortens it)
+        mbar_expect_tx(bar(BAR_KFULL + s), 2 * (kTileCodeBytes + kTileScaleBytes));
+        bulk_g2s(sbase + kOffK + s * kTileCodeBytes, p.k_codes + (kv0 + j) * kTileCodeBytes, kTileCodeBytes, bar(BAR_KFULL + s));
+        bulk_g2s(sbase + kOffSFK + s * kTileScaleBytes, p.k_scales + (kv0 + j) * kTileScaleBytes, kTileScaleBytes, bar(BAR_KFULL + s));
+        bulk_g2s(sbase + kOffV + s * kVStageBytes, p.v_codes + (kv0 + j) * kTileCodeBytes, kTileCodeBytes, bar(BAR_KFULL + s));
+        bulk_g2s(sbase + kOffSFV + s * kTileScaleBytes, p.v_scales + (kv0 + j) * kTileScaleBytes, kTileScaleBytes, bar(BAR_KFULL + s));
       }
-      if (kProf) { prof_t[8] = clock64() - prof_prev; prof_t[9] = F; }
+      if (kProf) { prof_t[8] = clock64() - prof_prev; prof_t[9] = j; }
       if (!ok || *abort_flag) {
         // gave up: let copies already in flight land before the CTA's shared memory is released
         const long long t0 = clock64();
-        for (int f = (F > kStages ? F - kStages : 0); f < F; ++f)
+        for (int f = (j > kStages ? j - kStages : 0); f < j; ++f)
           while (!mbar_try(bar(BAR_KFULL + f % kStages), (uint32_t)((f / kStages) & 1)) && clock64() - t0 < 200000000LL) {}
-        for (int n = (q_issued > 2 ? q_issued - 2 : 0); n < q_issued; ++n) {
-          const int qb = kPersist ? (n & 1) : 0;
-          while (!mbar_try(bar(BAR_Q + qb), (uint32_t)((kPersist ? (n >> 1) : 0) & 1)) && clock64() - t0 < 200000000LL) {}
-        }
+        while (!mbar_try(bar(BAR_Q), 0u) && clock64() - t0 < 200000000LL) {}
       }
     }
   } else if (role == kSoftmaxWarps + 1) {
@@ -258,42 +233,23 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
       const uint32_t q_lo = (sbase + kOffQ) >> 4, k_lo = (sbase + kOffK) >> 4;
       const uint32_t v_lo = (sbase + kOffV) >> 4, p_lo = (sbase + kOffP) >> 4;
       auto desc = [](uint32_t lo) { return ((uint64_t)kDescHiTile << 32) | lo; };
-      // A tile is named by its item n (0, 1, ... of this CTA), its index j inside the item and its index f among
-      // all tiles of the CTA (f = n T + j; f = j without kPersist).  Stages, slots and barrier parities follow f.
-      auto gemm1 = [&](int t, int n, int j, int f) {      // S = Q_t K_j^T
+      auto gemm1 = [&](int t, int j) {      // S = Q_t K_j^T
         const uint32_t a = q_lo + (uint32_t)t * (kTileCodeBytes >> 4);
-        const uint32_t b = k_lo + (uint32_t)(f % kStages) * (kTileCodeBytes >> 4);
-        const uint32_t sfa = tmem + kColSFQ + 4 * t, sfb = tmem + kColSFK + 4 * (f & 1);
+        const uint32_t b = k_lo + (uint32_t)(j % kStages) * (kTileCodeBytes >> 4);
+        const uint32_t sfa = tmem + kColSFQ + 4 * t, sfb = tmem + kColSFK + 4 * (j & 1);
         tc_mma(tmem + kColS, desc(a), desc(b), make_idesc(128, 0), sfa, sfb, 0u);
         tc_mma(tmem + kColS, desc(a + 2), desc(b + 2), make_idesc(128, 1), sfa, sfb, 1u);   // K 64..127: +32 bytes
         tc_commit(bar(BAR_SFULL + t));
-        return true;
       };
-      auto gemm2 = [&](int t, int n, int j, int f) {      // O_t += P_t [V_j | 1]
+      auto gemm2 = [&](int t, int j) {      // O_t += P_t [V_j | 1]
         tc_cp_sf(tmem + kColSFP + 4 * t, sbase + kOffSFP + t * kTileScaleBytes);
         const uint32_t a = p_lo + (uint32_t)t * (kTileCodeBytes >> 4);
-        const uint32_t b = v_lo + (uint32_t)(f % kStages) * (kVStageBytes >> 4);
+        const uint32_t b = v_lo + (uint32_t)(j % kStages) * (kVStageBytes >> 4);
         const uint32_t d = tmem + (t ? kColO1 : kColO0);
-        const uint32_t sfa = tmem + kColSFP + 4 * t, sfb = tmem + kColSFV + 8 * (f & 1);
+        const uint32_t sfa = tmem + kColSFP + 4 * t, sfb = tmem + kColSFV + 8 * (j & 1);
         tc_mma(d, desc(a), desc(b), make_idesc(kNV, 0), sfa, sfb, j > 0 ? 1u : 0u);
         tc_mma(d, desc(a + 2), desc(b + 2), make_idesc(kNV, 1), sfa, sfb, 1u);
         tc_commit(bar(BAR_ODONE + t));
-        return true;
-      };
-      // K-hat and V-hat of tile f have landed (and, unless `first`, the score buffer is free): one fence, then the
-      // scale atoms of both go to tensor memory -- V's two tiles ahead of its GEMM, which keeps that copy out of the
-      // path from "P is ready" to "GEMM 2 issued" (slot f & 1 was last read by the GEMMs of tile f - 2, issued before)
-      auto wait_kv = [&](int f, bool first) {
-        const int s = f % kStages;
-        if (!MBAR_WAIT_ROLE(bar(BAR_KFULL + s), (uint32_t)((f / kStages) & 1), abort_flag, p.status, 22)) return false;
-        if (!first) {
-          if (!MBAR_WAIT_ROLE(bar(BAR_SFREE), sfree_n & 1u, abort_flag, p.status, 23)) return false;
-          ++sfree_n;
-        }
-        tc_fence_after();
-        tc_cp_sf(tmem + kColSFK + 4 * (f & 1), sbase + kOffSFK + s * kTileScaleBytes);
-        tc_cp_sf(tmem + kColSFV + 8 * (f & 1), sbase + kOffSFV + s * kTileScaleBytes);
-        return true;
       };
       auto wait_sfree = [&]() {
         const bool r = MBAR_WAIT_ROLE(bar(BAR_SFREE), sfree_n & 1u, abort_flag, p.status, 23);
@@ -321,133 +277,50 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
       // V-hat's scale atom of tile f (its stage has landed together with K-hat's; slot f & 1 was last read by the output
       // products of tile f - 2)
       auto v_scales = [&](int f) { tc_cp_sf(tmem + kColSFV + 8 * (f & 1), sbase + kOffSFV + (f % kStages) * kTileScaleBytes); };
-      if (!kPersist) {
-        // prologue: S(0,0), S(1,0), S(0,1)
-        ok = ok && k_ready(0);
-        if (ok) { v_scales(0); gemm1(0, 0, 0, 0); }
+      // prologue: S(0,0), S(1,0), S(0,1)
+      ok = ok && k_ready(0);
+      if (ok) { v_scales(0); gemm1(0, 0); }
+      ok = ok && wait_sfree();
+      if (ok) gemm1(1, 0);
+      if (T > 1) {
+        ok = ok && k_ready(1);
+        if (ok) v_scales(1);
         ok = ok && wait_sfree();
-        if (ok) gemm1(1, 0, 0, 0);
-        if (T > 1) {
-          ok = ok && k_ready(1);
-          if (ok) v_scales(1);
-          ok = ok && wait_sfree();
-          if (ok) gemm1(0, 0, 1, 1);
-        }
-        // unrolled by the number of stages: stage indices, parities and descriptor offsets become constants, and the
-        // thread's scalar instructions between its tcgen05 instructions are part of the kernel's critical path
+        if (ok) gemm1(0, 1);
+      }
+      // unrolled by the number of stages: stage indices, parities and descriptor offsets become constants, and the
+      // thread's scalar instructions between its tcgen05 instructions are part of the kernel's critical path
 #pragma unroll 4
-        for (int j = 0; j < T && ok; ++j) {
-          const int s = j % kStages;
-          ok = MBAR_WAIT_ROLE(bar(BAR_PFULL + 0), (uint32_t)(j & 1), abort_flag, p.status, 24);     // V_j arrived with K_j
+      for (int j = 0; j < T && ok; ++j) {
+        const int s = j % kStages;
+        ok = MBAR_WAIT_ROLE(bar(BAR_PFULL + 0), (uint32_t)(j & 1), abort_flag, p.status, 24);     // V_j arrived with K_j
+        if (!ok) break;
+        tc_fence_after();
+        gemm2(0, j);
+        if (j + 1 < T) {
+          ok = wait_sfree();
           if (!ok) break;
-          tc_fence_after();
-          gemm2(0, 0, j, j);
-          if (j + 1 < T) {
-            ok = wait_sfree();
-            if (!ok) break;
-            gemm1(1, 0, j + 1, j + 1);
-          }
-          if (j + 2 < T) {                           // off the critical chain: the thread would wait for P-hat here anyway
-            ok = k_ready(j + 2);
-            if (!ok) break;
-          }
-          ok = MBAR_WAIT_ROLE(bar(BAR_PFULL + 1), (uint32_t)(j & 1), abort_flag, p.status, 26);
-          if (!ok) break;
-          tc_fence_after();
-          gemm2(1, 0, j, j);
-          if (j + 2 < T) {
-            ok = wait_sfree();
-            if (!ok) break;
-            gemm1(0, 0, j + 2, j + 2);
-          }
-          tc_commit(bar(BAR_KEMPTY + s));            // K_j and V_j may be overwritten once everything issued so far has completed
-          if (j + 2 < T) v_scales(j + 2);
+          gemm1(1, j + 1);
         }
-      } else {
-        // The same instruction stream over all tiles of all items of this CTA, f = 0 .. F_end - 1: the scores of
-        // the next item's first tiles are issued while the current item's last tiles are still in the softmax warps.
-        // Per tile the thread keeps one cursor (item n0, tile j0 of tile f) and derives two flags from it; what an
-        // item boundary adds is then one branch per GEMM 1.  `edge` of a GEMM 1 means: for query tile 0, the first
-        // tile of an item other than the CTA's first (wait for its Q tiles, copy their scales: every GEMM 1 of the
-        // previous item has been issued by then); for query tile 1, the last tile of its item (release the Q buffer).
-        // No barrier guards the accumulators across items: GEMM 2 of an item's first tile waits for that tile's
-        // P-hat, which the group's warps publish after their epilogue has read the previous item's accumulator.
-        const int n_items = (p.total_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-        const int F_end = n_items * T;
-        auto gemm1p = [&](int t, int n, int f, bool edge) {      // n: the item of tile f
-          const int qb = n & 1;
-          if (t == 0 && edge) {
-            if (!MBAR_WAIT_ROLE(bar(BAR_Q + qb), (uint32_t)((n >> 1) & 1), abort_flag, p.status, 21)) return false;
-            tc_fence_after();
-            tc_cp_sf(tmem + kColSFQ + 0, sbase + kOffSFQ + qb * 2 * kTileScaleBytes);
-            tc_cp_sf(tmem + kColSFQ + 4, sbase + kOffSFQ + (qb * 2 + 1) * kTileScaleBytes);
-          }
-          const uint32_t a = q_lo + (uint32_t)(qb * 2 + t) * (kTileCodeBytes >> 4);
-          const uint32_t b = k_lo + (uint32_t)(f % kStages) * (kTileCodeBytes >> 4);
-          const uint32_t sfa = tmem + kColSFQ + 4 * t, sfb = tmem + kColSFK + 4 * (f & 1);
-          tc_mma(tmem + kColS, desc(a), desc(b), make_idesc(128, 0), sfa, sfb, 0u);
-          tc_mma(tmem + kColS, desc(a + 2), desc(b + 2), make_idesc(128, 1), sfa, sfb, 1u);
-          tc_commit(bar(BAR_SFULL + t));
-          if (t == 1 && edge) tc_commit(bar(BAR_QEMPTY + qb));
-          return true;
-        };
-        const bool one = (T == 1);
-        int n0 = 0, j0 = 0;                          // tile f
-        ok = ok && wait_kv(0, true);
-        if (ok) ok = gemm1p(0, 0, 0, false);
-        ok = ok && wait_sfree();
-        if (ok) ok = gemm1p(1, 0, 0, one);
-        if (F_end > 1) {
-          ok = ok && wait_kv(1, false);
-          if (ok) ok = gemm1p(0, one ? 1 : 0, 1, one);
-        }
-#pragma unroll 4
-        for (int f = 0; f < F_end && ok; ++f) {
-          const bool item_end = (j0 == T - 1);       // tile f + 1 starts an item
-          const bool pre_end = one || (j0 == T - 2); // tile f + 1 ends an item, tile f + 2 starts one
-          const int n1 = n0 + (item_end ? 1 : 0), n2 = n1 + (pre_end ? 1 : 0);
-          ok = MBAR_WAIT_ROLE(bar(BAR_PFULL + 0), (uint32_t)(f & 1), abort_flag, p.status, 24);
+        if (j + 2 < T) {                           // off the critical chain: the thread would wait for P-hat here anyway
+          ok = k_ready(j + 2);
           if (!ok) break;
-          tc_fence_after();
-          gemm2(0, 0, j0, f);
-          // On the last tile of an item the score buffer is released only after the first group's epilogue, so
-          // the second group's GEMM 2 (and with it that group's epilogue) goes first there.
-          if (!item_end && f + 1 < F_end) {
-            ok = wait_sfree();
-            if (!ok) break;
-            ok = gemm1p(1, n1, f + 1, pre_end);
-            if (!ok) break;
-          }
-          // Where the softmax is longer (direct row sum) K's scales go ahead of the wait for the score buffer, as in the
-          // one-item loop: 40 x 4096 291 -> 284 us, 40 x 75600 x 512 825 -> 809.  With the PNQ row sum it is 0.3 % slower.
-          if (!kPnq && f + 2 < F_end) {
-            ok = k_ready(f + 2);
-            if (!ok) break;
-          }
-          ok = MBAR_WAIT_ROLE(bar(BAR_PFULL + 1), (uint32_t)(f & 1), abort_flag, p.status, 26);
-          if (!ok) break;
-          tc_fence_after();
-          gemm2(1, 0, j0, f);
-          tc_commit(bar(BAR_KEMPTY + f % kStages));
-          if (item_end && f + 1 < F_end) {
-            ok = wait_sfree();
-            if (!ok) break;
-            ok = gemm1p(1, n1, f + 1, pre_end);
-            if (!ok) break;
-          }
-          if (f + 2 < F_end) {
-            ok = kPnq ? wait_kv(f + 2, false) : wait_sfree();
-            if (!ok) break;
-            ok = gemm1p(0, n2, f + 2, pre_end);
-            if (!ok) break;
-            if (!kPnq) v_scales(f + 2);
-          }
-          if (++j0 == T) { j0 = 0; ++n0; }
         }
+        ok = MBAR_WAIT_ROLE(bar(BAR_PFULL + 1), (uint32_t)(j & 1), abort_flag, p.status, 26);
+        if (!ok) break;
+        tc_fence_after();
+        gemm2(1, j);
+        if (j + 2 < T) {
+          ok = wait_sfree();
+          if (!ok) break;
+          gemm1(0, j + 2);
+        }
+        tc_commit(bar(BAR_KEMPTY + s));            // K_j and V_j may be overwritten once everything issued so far has completed
+        if (j + 2 < T) v_scales(j + 2);
       }
       if (kProf) {
         prof_t[8] = clock64() - prof_prev;
-        prof_t[9] = kPersist ? (long long)((p.total_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x) * T : T;
+        prof_t[9] = T;
       }
     }
   } else if (role < kSoftmaxWarps) {
@@ -459,7 +332,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
     const uint32_t t_s = tmem + kColS + lane_addr + kCols * h;
     const uint32_t t_o = tmem + (t ? kColO1 : kColO0) + lane_addr;     // column 0 of this row's accumulator
     const float c = p.scale_log2e;
-    float m_run, l_run;                            // l_run: direct placement only (this thread's 64 columns)
+    float m_run = -INFINITY, l_run = 0.0f;         // l_run: direct placement only (this thread's 64 columns)
     // shared-space byte addresses of this thread's slots: its two 16-byte code chunks, its two scale
     // bytes, and the half-row maximum exchange (own slot / partner's slot; + 2048 on odd tiles)
     const uint32_t aP0 = sbase + kOffP + t * kTileCodeBytes + tile_code_offset(row, 2 * h);
@@ -470,25 +343,16 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
     const int pair_bar = 1 + (warp & 3) + 4 * t;   // named barrier shared with the partner warp (w, w^4)
     // The two warps of a pair meet at a named barrier in every tile (and once more per item under direct placement).
     // A warp whose bounded wait has run out therefore does not leave: it stops computing and waiting, but keeps every
-    // remaining appointment with its partner (keep_company below), for this item and all later ones, so that the
+    // remaining appointment with its partner (pair_keep_company below), so that the
     // partner -- which may have found the same mbarrier complete a moment earlier -- is never left alone at the
     // barrier.  The hot path carries no check for this.  Their waits watch a flag that nothing sets (they give up on
     // their own cycle limit only) and raise the CTA's flag on expiry.
     volatile int* const own_limit_only = abort_flag + 1;
     bool ok = true;
-    // Work items of this CTA (exactly one without kPersist).  F0 = tiles of the earlier items: the parities of the
-    // barriers that complete once per tile follow F0 + j.  X0 counts the earlier exchanges through the half-row
-    // slots (one per tile, plus the row-sum exchange of direct placement), which alternate between two buffers.
-    int item = blockIdx.x, F0 = 0, X0 = 0;
-    do {
-    int bh = bh0, pair = pair0;                     // with kPersist: set in the epilogue, the only place that needs them
-    m_run = -INFINITY;
-    l_run = 0.0f;
-
     int j = 0;                                      // after the loop: the first tile whose meeting has not been kept yet
-    if (kProf && F0 == 0) prof_prev = clock64();
-    if (ok) for (; j < T; ++j) {
-      ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar(BAR_SFULL + t), (uint32_t)((F0 + j) & 1), own_limit_only, p.status, 31, kWaitLimitCycles, abort_flag));
+    if (kProf) prof_prev = clock64();
+    for (; j < T; ++j) {
+      ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar(BAR_SFULL + t), (uint32_t)(j & 1), own_limit_only, p.status, 31, kWaitLimitCycles, abort_flag));
       if (!ok) break;
       PROF_MARK(0);
       tc_fence_after();
@@ -524,7 +388,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
 #pragma unroll
       for (int b = 1; b < kBlocksPerThread; ++b) own_max = fmaxf(own_max, bmax[b]);
       // half-row maximum -> partner thread (same row, other 64 columns), double-buffered by tile parity
-      const uint32_t par = (uint32_t)((X0 + j) & 1) * 2048u;
+      const uint32_t par = (uint32_t)(j & 1) * 2048u;
       PROF_MARK(2);
       sts32f(aMaxOwn + par, own_max);
       asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");      // only the two warps that share these rows
@@ -532,14 +396,14 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
       PROF_MARK(3);
       // GEMM 2 of the previous tile must have read P_t and updated O_t before this tile writes P_t or rescales
       // O_t; the probe of that barrier is issued while the partner's maximum is on its way
-      const bool o_ready = (j == 0) || mbar_test(bar(BAR_ODONE + t), (uint32_t)((F0 + j - 1) & 1));
+      const bool o_ready = (j == 0) || mbar_test(bar(BAR_ODONE + t), (uint32_t)((j - 1) & 1));
       const float m_new = max3(m_run, own_max, partner_max);   // line 10
       const bool moved = (m_new != m_run) && (j > 0);
       const float m_old = m_run;
       m_run = m_new;
       const float nmc = -(m_new * c);
       if (!__all_sync(0xFFFFFFFFu, o_ready)) {
-        ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar(BAR_ODONE + t), (uint32_t)((F0 + j - 1) & 1), own_limit_only, p.status, 32, kWaitLimitCycles, abort_flag));
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar(BAR_ODONE + t), (uint32_t)((j - 1) & 1), own_limit_only, p.status, 32, kWaitLimitCycles, abort_flag));
         if (!ok) { ++j; break; }                   // this tile's meeting has been kept
       }
       tc_fence_after();
@@ -642,66 +506,20 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
       if (kProf) prof_t[9] += 1;
     }
 
-    if (!ok) pair_keep_company(pair_bar, T - j);    // gave up (now or in an earlier item): only the meetings are kept
+    if (!ok) pair_keep_company(pair_bar, T - j);    // gave up: only the meetings are kept
 
     // ---- epilogue: O = O~ / l (line 18) ----
-    if (kPersist) {                                // the previous item's output copy has read this warp's box
-      if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-      __syncwarp();
-    }
-    if (ok) ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar(BAR_ODONE + t), (uint32_t)((F0 + T - 1) & 1), own_limit_only, p.status, 33, kWaitLimitCycles, abort_flag));
+    if (ok) ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar(BAR_ODONE + t), (uint32_t)((T - 1) & 1), own_limit_only, p.status, 33, kWaitLimitCycles, abort_flag));
     float l = l_run;
     if (!kPnq) {                                   // add the partner's half of the row sum (a meeting that is always kept)
-      const uint32_t par = (uint32_t)((X0 + T) & 1) * 2048u;
+      const uint32_t par = (uint32_t)(T & 1) * 2048u;
       sts32f(aMaxOwn + par, l_run);
       asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
       l = l_run + lds32f(aMaxPartner + par);
     }
     if (ok) {
       tc_fence_after();
-      if (kPersist) { bh = item / p.q_pairs; pair = item - bh * p.q_pairs; }
       const int qtile = 2 * pair + t;
-      if (kPersist) {
-        // Item-walking variant: the epilogue is part of every item's critical path.  Row sum and all 64 accumulator
-        // columns are loaded with one wait, then the rows go to this warp's swizzled box and out as a tensor
-        // copy (store_half_rows has the reasons).
-        uint32_t lr = 0, r64[kCols];
-        if (kPnq) asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(lr) : "r"(t_o + 128) : "memory");
-        TMEM_LD64(t_o + kCols * h, r64);
-        tmem_ld_wait();
-        if (kPnq) l = __uint_as_float(lr);
-        const float inv_l = 1.0f / l;
-        const uint32_t aBox = sbase + kOffOut + (t * 8 + h * 4 + (row >> 5)) * kOutBoxBytes;
-        const uint32_t aRow = aBox + (row & 31) * (kBoxCols * kOutSize);
-#pragma unroll
-        for (int b = 0; b < kCols / kBoxCols; ++b) {
-          if (b > 0) {                               // fp32: the first half has left the box
-            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-            __syncwarp();
-          }
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            uint32_t hh[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              if (kOutF32) {
-                hh[k] = __float_as_uint(__uint_as_float(r64[kBoxCols * b + 4 * i + k]) * inv_l);
-              } else {
-                const float a = __uint_as_float(r64[8 * i + 2 * k]) * inv_l, b2 = __uint_as_float(r64[8 * i + 2 * k + 1]) * inv_l;
-                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hh[k]) : "f"(b2), "f"(a));
-              }
-            }
-            sts128(aRow + ((i ^ (row & 7)) << 4), make_uint4(hh[0], hh[1], hh[2], hh[3]));
-          }
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          __syncwarp();
-          if (lane == 0 && qtile < p.q_tiles && (int64_t)qtile * kTile + (row & ~31) < p.Nq) {
-            asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
-                         ::"l"(&out_map), "r"(kCols * h + kBoxCols * b), "r"(qtile * kTile + (row & ~31)), "r"(bh), "r"(aBox) : "memory");
-            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-          }
-        }
-      } else {
       if (kPnq) {
         uint32_t lr;
         asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(lr) : "r"(t_o + 128) : "memory");
@@ -718,12 +536,8 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
       const int64_t row0 = (int64_t)qtile2 * kTile + (w & 3) * 32;
       store_half_rows<kOutF32>((w >> 3 ? kColO1 : kColO0) + ((w & 3) << 21) + col, ((smem_u32(smem_raw) + 1023u) & ~1023u) + kOffOut + w * kOutBoxBytes,
                                (int)(tid2 & 31), inv_l, &out_map, col, (int)row0, bh2, qtile2 < p.q_tiles && row0 < p.Nq);
-      }
     }
     PROF_MARK(8);
-    F0 += T;
-    X0 += T + (kPnq ? 0 : 1);
-    } while (kPersist && (item += (int)gridDim.x) < p.total_items);     // also after giving up: the meetings go on
   }
 
   if (kProf && lane == 0) {
@@ -856,15 +670,22 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
   p.softmax_scale = softmax_scale;
 
   const bool uos = flags & MXATTN_FLAG_UOS, pnq = flags & MXATTN_FLAG_PNQ, f32 = flags & MXATTN_FLAG_OUT_FP32;
-  // Short key/value sequences with more work items than SMs: one CTA per SM walks the items, so that the set-up,
-  // the first loads and the epilogue of one item overlap the tiles of its neighbours.  Long sequences keep one
-  // item per CTA (the hardware's block scheduler then balances the tail better than a static assignment).
   const int n_sm = sm_count();
   if (n_sm == 0) return MXATTN_ECUDA;
   // query tiles that would leave SMs idle (a problem smaller than the GPU, or a last wave that is nearly empty) go to the
   // kernel for few query rows
   // (not where other attention launches run beside: their CTAs fill those SMs; 24 x 119056 in stages of one head 99.0 -> 93.1 ms)
   const RowSplit split = dump || followed ? RowSplit{grid, 0} : forward_row_split(n_sm, (int64_t)B * H, Nq, Nkv, pnq);
+  if (!dump) {
+    const WalkSplit walk = forward_walk_split(n_sm, (int64_t)B * H, Nq, Nkv, pnq, followed, split);
+    if (walk.walk) {
+      if (walk.pairs > 0) {
+        const int rc = launch_forward_walk(n_sm, walk.pairs, q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, o, B, H, Nq, Nkv, softmax_scale, flags, status, stream);
+        if (rc != MXATTN_OK || walk.pairs == grid) return rc;
+      }
+      return launch_forward_rows(split.R, walk.pairs, q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, o, B, H, Nq, Nkv, softmax_scale, flags, status, stream);
+    }
+  }
   auto rest = [&]() {
     return split.R == 0 ? (int)MXATTN_OK
                         : launch_forward_rows(split.R, split.pairs_256, q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, o, B, H, Nq, Nkv,
@@ -872,28 +693,27 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
   };
   if (split.pairs_256 == 0) return rest();
   p.total_items = (int)split.pairs_256;
-  const bool persist = (!dump || profile) && split.pairs_256 > n_sm && kt <= kWalkMaxTiles;
   CUtensorMap out_map;
   const int map_rc = encode_output_map(&out_map, o, (int64_t)B * H, Nq, f32);
   if (map_rc != MXATTN_OK) return map_rc;
   void (*kern)(const Params, const CUtensorMap) = nullptr;
 #define PICK(U, P, F)                                                                     \
   if (uos == U && pnq == P && f32 == F)                                                   \
-    kern = persist ? attention_kernel<U, P, F, false, true> : attention_kernel<U, P, F, false, false>;
+    kern = attention_kernel<U, P, F, false>;
   PICK(false, false, false) PICK(false, false, true) PICK(false, true, false) PICK(false, true, true)
   PICK(true, false, false) PICK(true, false, true) PICK(true, true, false) PICK(true, true, true)
 #undef PICK
   if (profile) {                                  // cycle profile: the UOS + PNQ, bf16-output kernels with the counters compiled in
     if (!dump || !uos || !pnq || f32) return MXATTN_EINVAL;
-    kern = persist ? attention_kernel<true, true, false, false, true, true> : attention_kernel<true, true, false, false, false, true>;
+    kern = attention_kernel<true, true, false, false, true>;
   } else if (dump) {                              // debug entry point: fp32 output only
     if (!f32) return MXATTN_EINVAL;
-#define PICKD(U, P) if (uos == U && pnq == P) kern = attention_kernel<U, P, true, true, false>;
+#define PICKD(U, P) if (uos == U && pnq == P) kern = attention_kernel<U, P, true, true>;
     PICKD(false, false) PICKD(false, true) PICKD(true, false) PICKD(true, true)
 #undef PICKD
   }
   if (!ensure_dynamic_smem((const void*)kern, kSmemBytes)) return MXATTN_ECUDA;
-  if (launch_pdl(kern, dim3((unsigned)(persist ? n_sm : split.pairs_256)), kThreads, kSmemBytes, stream, p, out_map) != cudaSuccess) return MXATTN_ECUDA;
+  if (launch_pdl(kern, dim3((unsigned)split.pairs_256), kThreads, kSmemBytes, stream, p, out_map) != cudaSuccess) return MXATTN_ECUDA;
   return rest();
 }
 

@@ -1,0 +1,529 @@
+// MXFP4 attention forward, one query tile per work item (paper Algorithm 2, lines 6-19): the kernel for short and medium
+// key/value sequences.  Value for value the arithmetic of forward.cu.
+//
+// One CTA per SM walks work items of one query tile (128 rows of one head); the tiles of all its items form one stream
+// f = 0, 1, 2, ... (KV tiles of 128 keys in ascending order within an item), and barriers, tensor memory and the pipelines
+// run on across items.  Roles (736 threads):
+//   warps 0-15   softmax, two teams of eight: team f & 1 takes tile f.  Two threads a row, one half of 64 keys each.  A team
+//                has a score buffer of its own, so that neither waits for the other to take its scores; what passes from
+//                team to team is the maxima of a tile, two floats a row, posted before the exponentials (a named barrier at
+//                which the owners of the next tile wait and the posters only arrive).
+//   warps 16-19  scaling: alpha, the accumulator's rescaling (Algorithm 2 line 15) and the epilogue, one warp per quarter of
+//                tensor memory.  The softmax warps never touch the accumulator and go straight on to the next item.
+//   warp 20      score products S(f) = Q K_f^T;   warp 21  output products O += P(f) [V_f | 1];   warp 22  copies
+//
+// What bounds it: the exponentials (1024 cycles per 128 x 128 tile and SM) and the latency around them.  An issuing warp
+// slows the softmax warps of its own SM sub-partition (with both products on one warp the exponentials of that quarter took
+// 850 cycles per block pair where the others took 630, and all wait for the slowest), hence two issuers and the copies on
+// three different sub-partitions: 1333 -> 1297 cycles per tile.  The scores stay in tensor memory until they are used (each
+// half is read for its maximum and once more for its exponentials), so that a thread holds 32 of them and 23 warps fit the
+// register file at 80.  Per-tile work of a warp is kept short by immediate offsets (the parity of the team's tile count is a
+// template argument): 805 -> 645 instructions per tile and sub-partition, with the two loads of scores one after the other
+// (both at once do not fit 80 registers, and the compiler then moves every score).
+//
+// Tensor memory (512 columns): scores [0,128) and [128,256), accumulator and row sum [256,400), scales behind it: Q 4 slots,
+// K 4, V 8, P 4.  Slots are as many as it takes that a copy never follows a product that still reads the slot.
+//
+// Every wait is bounded (mbar_wait_soft / role_wait); the softmax and scaling warps never leave their loops early, so that
+// no warp is stranded at a named barrier, and nothing is stored once the CTA's abort flag is up.
+#include <string.h>
+
+#include <algorithm>
+#include <type_traits>
+
+#include "common.cuh"
+#include "tc_helpers.cuh"
+
+namespace mxattn {
+namespace walk {
+using namespace fwd;
+
+constexpr int kSoftmaxWarps = 16, kScaleWarps = 4, kTeamWarps = kSoftmaxWarps / 2;
+constexpr int kIssuer1 = kSoftmaxWarps + kScaleWarps, kIssuer2 = kIssuer1 + 1, kProducer = kIssuer2 + 1;
+constexpr int kThreads = 32 * (kProducer + 1);
+constexpr int kStages = 6;
+constexpr int kNV = 144;                         // GEMM 2 N: 128 channels + 16 rows of ones (column 128 = row sum of P-hat)
+constexpr int kVStageBytes = kNV * 64;
+
+constexpr int kOffQ = 0;                                         // 2 buffers
+constexpr int kOffK = kOffQ + 2 * kTileCodeBytes;
+constexpr int kOffV = kOffK + kStages * kTileCodeBytes;
+constexpr int kOffP = kOffV + kStages * kVStageBytes;            // 4 buffers
+constexpr int kOffOut = kOffP + 4 * kTileCodeBytes;              // two boxes per scaling warp
+constexpr int kOffSFQ = kOffOut + 2 * kScaleWarps * kOutBoxBytes;
+constexpr int kOffSFK = kOffSFQ + 2 * kTileScaleBytes;
+constexpr int kOffSFV = kOffSFK + kStages * kTileScaleBytes;
+constexpr int kOffSFP = kOffSFV + kStages * kTileScaleBytes;     // 4 buffers
+constexpr int kOffSFOnes = kOffSFP + 4 * kTileScaleBytes;
+constexpr int kOffX = kOffSFOnes + kTileScaleBytes;              // half-row maxima: [4 slots][row 128][half 2] floats
+constexpr int kXSlot = 128 * 2 * 4;
+constexpr int kOffXL = kOffX + 4 * kXSlot;                       // row sums of a tile by half (direct placement): 8 slots, laid out alike
+constexpr int kOffBar = kOffXL + 8 * kXSlot;
+enum Bar { BAR_Q = 0, BAR_QEMPTY = 2, BAR_KFULL = 4, BAR_ODONE = BAR_KFULL + kStages, BAR_SFULL = BAR_ODONE + kStages,
+           BAR_SFREE = BAR_SFULL + 2, BAR_PFULL = BAR_SFREE + 2, BAR_X = BAR_PFULL + 4 /* [quarter][tile & 3]: maxima posted */, kNumBars = BAR_X + 16 };
+constexpr int kOffMisc = kOffBar + kNumBars * 8;
+constexpr int kSmemBytes = kOffMisc + 32 + 1024;
+static_assert(kOffOut % 1024 == 0 && kSmemBytes <= 227 * 1024, "shared memory per CTA");
+constexpr uint32_t kColS = 0, kColO = 256, kColSFQ = 400, kColSFK = 416, kColSFV = 432, kColSFP = 496;     // 4, 4, 8 and 4 slots
+
+struct Params {
+  const uint8_t* q_codes; const uint8_t* q_scales;
+  const uint8_t* k_codes; const uint8_t* k_scales;
+  const uint8_t* v_codes; const uint8_t* v_scales;
+  int* status;
+  int64_t Nq, Nkv;
+  int q_tiles, kv_tiles, total_items;
+  float scale_log2e;
+};
+
+// Shared-memory accesses at a register plus a constant: addresses formed in front of each access cost the softmax warps
+// instructions, and kept ones registers.
+template <int kOff> __device__ __forceinline__ void sts128o(uint32_t a, const uint32_t (&w)[4]) {
+  asm volatile("st.shared.v4.b32 [%0+%5], {%1, %2, %3, %4};" ::"r"(a), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "n"(kOff) : "memory");
+}
+template <int kOff> __device__ __forceinline__ void sts32o(uint32_t a, float v) { asm volatile("st.shared.f32 [%0+%2], %1;" ::"r"(a), "f"(v), "n"(kOff) : "memory"); }
+template <int kOff> __device__ __forceinline__ void sts16o(uint32_t a, uint32_t v) { asm volatile("st.shared.b16 [%0+%2], %1;" ::"r"(a), "h"((uint16_t)v), "n"(kOff) : "memory"); }
+template <int kOff> __device__ __forceinline__ float2 lds64o(uint32_t a) {
+  float2 v;
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2+%3];" : "=f"(v.x), "=f"(v.y) : "r"(a), "n"(kOff) : "memory");
+  return v;
+}
+template <int kOff> __device__ __forceinline__ void arrive_if(uint32_t b, bool me) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0+%1];\n\t}" ::"r"(b), "n"(kOff), "r"((uint32_t)me) : "memory");
+}
+// mbar_wait_soft with a probe in front: a wait that is already satisfied takes 38 cycles as a test_wait, 78 as a try_wait.
+template <int kCode, int kOff>
+__device__ __forceinline__ void mbar_wait_probe(uint32_t bar, uint32_t parity, uint32_t abort_addr) {
+  asm volatile("{\n\t.reg .pred p;\n\t.reg .u64 t0, t1;\n\t.reg .u32 a;\n\t"
+               "mbarrier.test_wait.parity.shared::cta.b64 p, [%0+%2], %1;\n\t"
+               "vote.sync.all.pred p, p, 0xffffffff;\n\t"
+               "@p bra.uni DONE;\n\t"
+               "mov.u64 t0, %%clock64;\n"
+               "AGAIN:\n\t"
+               
+               "mbarrier.try_wait.parity.shared::cta.b64 p, [%0+%2], %1, 20000;\n\t"
+
+               "vote.sync.all.pred p, p, 0xffffffff;\n\t"
+               "@p bra.uni DONE;\n\t"
+               "ld.volatile.shared.u32 a, [%4];\n\t"
+               "setp.ne.u32 p, a, 0;\n\t"
+               "vote.sync.any.pred p, p, 0xffffffff;\n\t"
+               "@p bra.uni DONE;\n\t"
+               "mov.u64 t1, %%clock64;\n\t"
+               "sub.u64 t1, t1, t0;\n\t"
+               "setp.lt.u64 p, t1, 4000000000;\n\t"
+               "vote.sync.any.pred p, p, 0xffffffff;\n\t"
+               "@p bra.uni AGAIN;\n\t"
+               "st.volatile.shared.u32 [%4], %3;\n"
+               "DONE:\n\t}"
+               ::"r"(bar), "r"(parity), "n"(kOff), "n"(kCode), "r"(abort_addr) : "memory");
+}
+__device__ __forceinline__ bool role_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status, int code) {
+  return __all_sync(0xFFFFFFFFu, mbar_test(bar, parity)) || mbar_wait_warp(bar, parity, abort_flag, status, code);
+}
+
+template <bool kUos, bool kPnq, bool kOutF32>
+__global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Params p, const __grid_constant__ CUtensorMap out_map) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const uint32_t sbase = smem_u32(smem);
+  const uint32_t bar0 = sbase + kOffBar;
+  auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kOffMisc);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kOffMisc + 8);
+  const uint32_t abort_addr = sbase + kOffMisc + 8;
+
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
+  const int T = p.kv_tiles;
+
+  // ---- setup -------------------------------------------------------------------------------
+  if (tid == 0) {
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(bar(BAR_Q + i), 1); mbar_init(bar(BAR_QEMPTY + i), 1);
+      mbar_init(bar(BAR_SFULL + i), 1);
+    }
+    for (int i = 0; i < 4; ++i) mbar_init(bar(BAR_PFULL + i), kTeamWarps + kScaleWarps);
+    mbar_init(bar(BAR_SFREE), kTeamWarps); mbar_init(bar(BAR_SFREE + 1), kTeamWarps);
+    for (int s = 0; s < kStages; ++s) { mbar_init(bar(BAR_KFULL + s), 1); mbar_init(bar(BAR_ODONE + s), 1); }
+    for (int i = 0; i < 16; ++i) mbar_init(bar(BAR_X + i), 1);
+    abort_flag[0] = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  for (int i = tid; i < kStages * 64; i += kThreads)             // rows of ones behind every V stage (code 2 = 1.0), their scales
+    reinterpret_cast<uint4*>(smem + kOffV + (i >> 6) * kVStageBytes + kTileCodeBytes)[i & 63] =
+        make_uint4(0x22222222u, 0x22222222u, 0x22222222u, 0x22222222u);
+  if (tid < kTileScaleBytes / 16) reinterpret_cast<uint4*>(smem + kOffSFOnes)[tid] = make_uint4(0x7F7F7F7Fu, 0x7F7F7F7Fu, 0x7F7F7F7Fu, 0x7F7F7F7Fu);
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  if (warp == kIssuer1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  pdl_wait();                                                    // the operands and the status word are ready
+  if (tid == 0) abort_flag[1] = *reinterpret_cast<volatile int*>(p.status);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  pdl_trigger();
+  constexpr uint32_t tmem = 0;
+  if (*tmem_slot != 0) *abort_flag = kCodeTmemBase;
+  const int role = __shfl_sync(0xFFFFFFFFu, (abort_flag[1] != 0 || *tmem_slot != 0) ? kThreads / 32 : warp, 0);     // an earlier launch gave up
+
+  const int n_items = (p.total_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+  const int F = n_items * T;                                     // tiles of this CTA
+
+  if (role == kProducer) {
+    // =============================== producer ===============================================
+    if (lane == 0) {
+      bool ok = true;
+      int f = 0, n = 0, s = 0;
+      uint32_t ph = 0;
+      for (int item = blockIdx.x; n < n_items && ok; ++n, item += gridDim.x) {
+        const int bh = item / p.q_tiles;
+        const int qb = n & 1;
+        if (n >= 2) ok = mbar_wait1(bar(BAR_QEMPTY + qb), (uint32_t)(((n - 2) >> 1) & 1), abort_flag, p.status, 13);
+        if (!ok) break;
+        mbar_expect_tx(bar(BAR_Q + qb), kTileCodeBytes + kTileScaleBytes);
+        bulk_g2s(sbase + kOffQ + qb * kTileCodeBytes, p.q_codes + (int64_t)item * kTileCodeBytes, kTileCodeBytes, bar(BAR_Q + qb));
+        bulk_g2s(sbase + kOffSFQ + qb * kTileScaleBytes, p.q_scales + (int64_t)item * kTileScaleBytes, kTileScaleBytes, bar(BAR_Q + qb));
+        const int64_t kv0 = (int64_t)bh * T;
+        for (int j = 0; j < T; ++j, ++f) {
+          if (f >= kStages) ok = mbar_wait1(bar(BAR_ODONE + s), ph ^ 1u, abort_flag, p.status, 11);
+          if (!ok) break;
+          mbar_expect_tx(bar(BAR_KFULL + s), 2 * (kTileCodeBytes + kTileScaleBytes));
+          bulk_g2s(sbase + kOffK + s * kTileCodeBytes, p.k_codes + (kv0 + j) * kTileCodeBytes, kTileCodeBytes, bar(BAR_KFULL + s));
+          bulk_g2s(sbase + kOffSFK + s * kTileScaleBytes, p.k_scales + (kv0 + j) * kTileScaleBytes, kTileScaleBytes, bar(BAR_KFULL + s));
+          bulk_g2s(sbase + kOffV + s * kVStageBytes, p.v_codes + (kv0 + j) * kTileCodeBytes, kTileCodeBytes, bar(BAR_KFULL + s));
+          bulk_g2s(sbase + kOffSFV + s * kTileScaleBytes, p.v_scales + (kv0 + j) * kTileScaleBytes, kTileScaleBytes, bar(BAR_KFULL + s));
+          if (++s == kStages) { s = 0; ph ^= 1u; }
+        }
+      }
+      if (!ok || *abort_flag) {                                  // gave up: let copies in flight land before shared memory is released
+        const long long t0 = clock64();
+        for (int g = (f > kStages ? f - kStages : 0); g < f; ++g)
+          while (!mbar_try(bar(BAR_KFULL + g % kStages), (uint32_t)((g / kStages) & 1)) && clock64() - t0 < 200000000LL) {}
+        for (int g = (n > 2 ? n - 2 : 0); g < n; ++g)
+          while (!mbar_try(bar(BAR_Q + (g & 1)), (uint32_t)((g >> 1) & 1)) && clock64() - t0 < 200000000LL) {}
+      }
+    }
+  } else if (role == kIssuer1) {
+    // =============================== score products (converged warp) ========================
+    const uint32_t leader = elect_one();
+    constexpr uint32_t kDescHiTile = (512u >> 4) | (1u << 14) | (4u << 29);   // 64-byte swizzle, K-major
+    auto desc = [](uint32_t saddr) { return ((uint64_t)kDescHiTile << 32) | (saddr >> 4); };
+    int j = 0, n = 0, s = 0, sd = 0;
+    uint32_t ph = 0, phd = 0;
+    bool ok = true;
+    for (int f = 0; f < F && ok; ++f) {
+      const int qb = n & 1;
+      if (j == 0) {
+        if (!role_wait(bar(BAR_Q + qb), (uint32_t)((n >> 1) & 1), abort_flag, p.status, 21)) break;
+        tc_fence_after();
+        tc_cp_sf_if(leader, tmem + kColSFQ + 4 * (n & 3), sbase + kOffSFQ + qb * kTileScaleBytes);
+      }
+      if (!role_wait(bar(BAR_KFULL + s), ph, abort_flag, p.status, 22)) break;
+      tc_fence_after();
+      const uint32_t d = tmem + kColS + 128 * (f & 1), sfb = tmem + kColSFK + 4 * (f & 3), sfa = tmem + kColSFQ + 4 * (n & 3);
+      const uint32_t a = sbase + kOffQ + qb * kTileCodeBytes, b = sbase + kOffK + s * kTileCodeBytes;
+      tc_cp_sf_if(leader, sfb, sbase + kOffSFK + s * kTileScaleBytes);
+      if (f >= 4) {                                              // the scores of tile f also say that its P buffer is free
+        if (!role_wait(bar(BAR_ODONE + sd), phd, abort_flag, p.status, 25)) break;
+        if (++sd == kStages) { sd = 0; phd ^= 1u; }
+      }
+      if (f >= 2) {                                              // S(f - 2) has been read
+        if (!role_wait(bar(BAR_SFREE + (f & 1)), (uint32_t)(((f >> 1) & 1) ^ 1), abort_flag, p.status, 23)) break;
+        tc_fence_after();
+      }
+      tc_mma_if(leader, d, desc(a), desc(b), make_idesc(128, 0), sfa, sfb, 0u);
+      tc_mma_if(leader, d, desc(a + 32), desc(b + 32), make_idesc(128, 1), sfa, sfb, 1u);
+      tc_commit_if(leader, bar(BAR_SFULL + (f & 1)));
+      if (++j == T) {
+        tc_commit_if(leader, bar(BAR_QEMPTY + qb));
+        j = 0; ++n;
+      }
+      if (++s == kStages) { s = 0; ph ^= 1u; }
+    }
+  } else if (role == kIssuer2) {
+    // =============================== output products (converged warp) =======================
+    const uint32_t leader = elect_one();
+    constexpr uint32_t kDescHiTile = (512u >> 4) | (1u << 14) | (4u << 29);   // 64-byte swizzle, K-major
+    auto desc = [](uint32_t saddr) { return ((uint64_t)kDescHiTile << 32) | (saddr >> 4); };
+    for (int i = 0; i < 8; ++i) tc_cp_sf_if(leader, tmem + kColSFV + 8 * i + 4, sbase + kOffSFOnes);
+    int j = 0, s = 0;
+    uint32_t ph = 0;
+    for (int f = 0; f < F; ++f) {
+      if (!role_wait(bar(BAR_KFULL + s), ph, abort_flag, p.status, 26)) break;
+      tc_fence_after();
+      const uint32_t sfa = tmem + kColSFP + 4 * (f & 3), sfb = tmem + kColSFV + 8 * (f & 7);
+      const uint32_t pa = sbase + kOffP + (f & 3) * kTileCodeBytes, vb = sbase + kOffV + s * kVStageBytes;
+      tc_cp_sf_if(leader, sfb, sbase + kOffSFV + s * kTileScaleBytes);
+      if (!role_wait(bar(BAR_PFULL + (f & 3)), (uint32_t)((f >> 2) & 1), abort_flag, p.status, 24)) break;
+      tc_fence_after();
+      tc_cp_sf_if(leader, sfa, sbase + kOffSFP + (f & 3) * kTileScaleBytes);
+      tc_mma_if(leader, tmem + kColO, desc(pa), desc(vb), make_idesc(kNV, 0), sfa, sfb, j > 0 ? 1u : 0u);
+      tc_mma_if(leader, tmem + kColO, desc(pa + 32), desc(vb + 32), make_idesc(kNV, 1), sfa, sfb, 1u);
+      tc_commit_if(leader, bar(BAR_ODONE + s));
+      if (++j == T) j = 0;
+      if (++s == kStages) { s = 0; ph ^= 1u; }
+    }
+  } else if (role >= kSoftmaxWarps && role < kSoftmaxWarps + kScaleWarps) {
+    // =============================== scaling warps: alpha, the accumulator, the epilogue ====
+    const int q = warp - kSoftmaxWarps;
+    const uint32_t t_o = tmem + ((uint32_t)q << 21) + kColO;
+    const uint32_t aX = sbase + kOffX + (q * 32 + lane) * 8;
+    const float c = p.scale_log2e;
+    float m_run = -INFINITY, lA = 0.0f, lB = 0.0f, alpha1 = 1.0f, alpha2 = 1.0f;
+    int f = 0, s_prev = kStages - 1;
+    uint32_t ph_prev = 1;                                        // stage and parity of tile f - 1
+    auto add_sums = [&](int g, float alpha) {                    // line 14 (direct), Eq. 12: tile g
+      const float2 v = lds64o<kOffXL - kOffX>(aX + (g & 7) * kXSlot);
+      lA = fmaf(alpha, lA, v.x);
+      lB = fmaf(alpha, lB, v.y);
+    };
+    int item = blockIdx.x;
+    for (int n = 0; n < n_items; ++n, item += gridDim.x) {
+      for (int j = 0; j < T; ++j, ++f) {
+        mbar_wait_soft<34>(bar(BAR_X + q * 4 + (f & 3)), (uint32_t)((f >> 2) & 1), abort_addr);
+        const float2 mx = lds64o<0>(aX + (f & 3) * kXSlot);
+        const float m_old = m_run;
+        float m_new = fmaxf(mx.x, mx.y);
+        if (j > 0) m_new = fmaxf(m_new, m_old);
+        m_run = m_new;
+        if (!kPnq && j >= 2) add_sums(f - 2, alpha2);
+        float alpha = 1.0f;
+        if (j > 0 && __any_sync(0xFFFFFFFFu, m_new != m_old)) {
+          alpha = ex2((m_old - m_new) * c);
+          mbar_wait_soft<32>(bar(BAR_ODONE + s_prev), ph_prev, abort_addr);
+          tc_fence_after();
+          const uint64_t al2 = dup2(alpha);
+          uint32_t lr = 0;
+          if (kPnq) asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(lr) : "r"(t_o + 128) : "memory");
+#pragma unroll 1
+          for (int c0 = 0; c0 < 128; c0 += 32) {
+            uint32_t o[32];
+            TMEM_LD32(t_o + c0, o);
+            TMEM_LD_WAIT32(o);
+#pragma unroll
+            for (int i = 0; i < 32; i += 2) mul2(o[i], o[i + 1], al2);
+            TMEM_ST32(t_o + c0, o);
+          }
+          if (kPnq) {
+            asm volatile("" : "+r"(lr));
+            lr = __float_as_uint(__uint_as_float(lr) * alpha);
+            asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%1], {%0};" ::"r"(lr), "r"(t_o + 128) : "memory");
+          }
+          tmem_st_wait();
+        }
+        if (!kPnq) { alpha2 = alpha1; alpha1 = alpha; }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(BAR_PFULL + (f & 3)));
+        if (++s_prev == kStages) { s_prev = 0; ph_prev ^= 1u; }
+      }
+      // ---- epilogue: O = O~ / l (line 18) ----
+      if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");      // the previous item's copies have left the boxes
+      __syncwarp();
+      mbar_wait_soft<33>(bar(BAR_ODONE + s_prev), ph_prev, abort_addr);
+      tc_fence_after();
+      float l;
+      if (kPnq) {
+        uint32_t lr;
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(lr) : "r"(t_o + 128) : "memory");
+        tmem_ld_wait();
+        asm volatile("" : "+r"(lr));
+        l = __uint_as_float(lr);
+      } else {
+        if (T >= 2) add_sums(f - 2, alpha2);
+        add_sums(f - 1, alpha1);
+        l = lA + lB;
+        lA = lB = 0.0f;
+      }
+      const float inv_l = 1.0f / l;
+      const int bh = item / p.q_tiles, qtile = item - bh * p.q_tiles;
+      const int row0 = qtile * kTile + q * 32;
+      const bool inside = row0 < p.Nq && lds_volatile(abort_addr) == 0;
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h)
+        store_half_rows<kOutF32>(t_o + 64 * h, sbase + kOffOut + (2 * q + h) * kOutBoxBytes, lane, inv_l, &out_map, 64 * h, row0, bh, inside);
+    }
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+  } else if (role < kSoftmaxWarps) {
+    // =============================== softmax warps ==========================================
+    // Two teams of eight warps take the tiles in turn (tile f: team f & 1); two threads a row, 64 keys each.
+    const int quarter = warp & 3, h = (warp >> 2) & 1, t = warp >> 3, row = quarter * 32 + lane;
+    const uint32_t t_s = tmem + ((uint32_t)quarter << 21) + 128 * t + 64 * h;
+    const uint32_t aM = sbase + kOffX + row * 8 + t * kXSlot;                                // own maxima (+ 2 slots on every other own tile)
+    const uint32_t aMp0 = sbase + kOffX + row * 8 + (t ? 0 : 3) * kXSlot;                    // the tile before, at even own tiles
+    const uint32_t aMp1 = sbase + kOffX + row * 8 + (t ? 2 : 1) * kXSlot;                    // ... at odd ones
+    const uint32_t aP0 = sbase + kOffP + t * kTileCodeBytes + tile_code_offset(row, 2 * h);
+    const uint32_t aP1 = sbase + kOffP + t * kTileCodeBytes + tile_code_offset(row, 2 * h + 1);
+    const uint32_t aSF = sbase + kOffSFP + t * kTileScaleBytes + tile_scale_offset(row, 2 * h);
+    const uint32_t barT = bar0 + 8 * t, barX = bar0 + 32 * quarter + 8 * t;
+    const int idOwn = 1 + quarter + 4 * t, idOther = 1 + quarter + 4 * (t ^ 1);
+    const int ragged = (int)(p.Nkv & (kTile - 1)) != 0 ? (int)(p.Nkv & (kTile - 1)) - 64 * h : 64;     // keys of this half in an item's last tile
+    const float c = p.scale_log2e;
+    const uint64_t cc2 = dup2(c);
+    float m_run = -INFINITY;                                     // of the team's last tile
+    int jn = t % T;                                              // index of tile f in its item
+    uint32_t xl = 0;                                             // slot of the row sums
+    if (t == 1) asm volatile("bar.arrive %0, 128;" ::"r"(idOther) : "memory");     // nothing comes before tile 0
+    auto max32 = [&](const uint32_t (&s)[32]) {
+#define SFL(i) __uint_as_float(s[i])
+      float q[10];
+#pragma unroll
+      for (int i = 0; i < 10; ++i) q[i] = max3(SFL(3 * i), SFL(3 * i + 1), SFL(3 * i + 2));
+      q[0] = max3(q[0], q[1], q[2]); q[3] = max3(q[3], q[4], q[5]); q[6] = max3(q[6], q[7], q[8]); q[9] = max3(q[9], SFL(30), SFL(31));
+#undef SFL
+      return fmaxf(max3(q[0], q[3], q[6]), q[9]);
+    };
+    auto exponent = [&](float bmax, float m_new, uint64_t& nb, uint32_t& sf) {
+      const float d = (bmax - m_new) * c;
+      const float fl = __fadd_rd(d, 12582912.0f) - 12582912.0f;                    // floor(d)
+      float ef = fl + ((kUos && (d - fl) > 0.85798097f) ? -1.0f : -2.0f);
+      ef = fmaxf(ef, -127.0f);
+      if (d < -126.0f) ef = 0.0f;
+      sf = __float_as_uint(ef + 12582912.0f) - (0x4B400000u - 127u);               // e + 127
+      nb = dup2(-(m_new * c) - ef);
+    };
+    auto exps = [&](const uint32_t (&s)[32], int g, uint64_t nb, float& sx) {      // eight exponentials, their codes
+      float x[8];
+#pragma unroll
+      for (int i = 0; i < 8; i += 2) {
+        fma2(s[8 * g + i], s[8 * g + i + 1], cc2, nb, x[i], x[i + 1]);
+        x[i] = ex2(x[i]);
+        x[i + 1] = ex2(x[i + 1]);
+      }
+      if (!kPnq) {
+        float s0, s1;
+        add2x2(x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7], s0, s1);
+        sx += s0 + s1;
+      }
+      return pack_e2m1x8(x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
+    };
+    auto tile = [&](auto kk) {                                   // kk: parity of the team's tile count
+      constexpr int k = decltype(kk)::value;
+      mbar_wait_probe<31, 8 * BAR_SFULL>(barT, (uint32_t)k, abort_addr);
+      tc_fence_after();
+      if (jn == T - 1 && ragged < 64) mask_scores(t_s, ragged, 64);
+      float b0, b1;
+      uint32_t s[32];
+      {
+        uint32_t s1[32];
+        TMEM_LD32(t_s + 32, s1);
+        TMEM_LD_WAIT32(s1);
+        b1 = max32(s1);
+        asm volatile("" : "+f"(b1));
+        TMEM_LD32(t_s, s);
+      }
+      TMEM_LD_WAIT32(s);
+      b0 = max32(s);
+      sts32o<2 * k * kXSlot>(aM + 4 * h, fmaxf(b0, b1));
+      asm volatile("bar.sync %0, 128;" ::"r"(idOwn) : "memory");
+      const float2 mo = lds64o<2 * k * kXSlot>(aM), mp = lds64o<0>(k ? aMp1 : aMp0);
+      asm volatile("bar.arrive %0, 128;" ::"r"(idOther) : "memory");
+      arrive_if<8 * BAR_X + 16 * k>(barX, h == 0 && lane == 0);
+      const float prev = jn >= 1 ? fmaxf(mp.x, mp.y) : -INFINITY, run = jn >= 2 ? m_run : -INFINITY;
+      const float m_new = max3(fmaxf(mo.x, mo.y), prev, run);    // line 10
+      m_run = m_new;
+      jn += 2;
+      if (jn >= T) jn -= T;
+      if (jn >= T) jn -= T;
+      uint64_t nb0, nb1;
+      uint32_t sf0, sf1;
+      exponent(b0, m_new, nb0, sf0);
+      exponent(b1, m_new, nb1, sf1);
+      sts16o<2 * k * kTileScaleBytes>(aSF, sf0 | (sf1 << 8));
+      float sx0 = 0.0f, sx1 = 0.0f;
+      uint32_t w[4];
+#pragma unroll
+      for (int g = 0; g < 4; ++g) w[g] = exps(s, g, nb0, sx0);
+      uint32_t s1[32];
+      TMEM_LD32(t_s + 32, s1);
+      sts128o<2 * k * kTileCodeBytes>(aP0, w);
+      TMEM_LD_WAIT32(s1);
+      tc_fence_before();
+      __syncwarp();
+      arrive_if<8 * BAR_SFREE>(barT, lane == 0);                 // the score buffer may be overwritten
+#pragma unroll
+      for (int g = 0; g < 4; ++g) w[g] = exps(s1, g, nb1, sx1);
+      sts128o<2 * k * kTileCodeBytes>(aP1, w);
+      if (!kPnq) {
+        sts32o<kOffXL - kOffX>(aM + 4 * h + xl, fmaf(sx1, __uint_as_float(sf1 << 23), fmaf(sx0, __uint_as_float(sf0 << 23), 0.0f)));   // Eq. 12
+        xl = (xl + 2 * kXSlot) & (8 * kXSlot - 1);
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      arrive_if<8 * BAR_PFULL + 16 * k>(barT, lane == 0);
+    };
+    for (int f = t; f < F; f += 4) {
+      tile(std::integral_constant<int, 0>{});
+      if (f + 2 >= F) break;
+      tile(std::integral_constant<int, 1>{});
+    }
+  }
+
+  // ---- teardown ------------------------------------------------------------------------------
+  tc_fence_before();
+  __syncthreads();
+  if (tid == 0 && *abort_flag != 0) atomicCAS(p.status, 0, *abort_flag);
+  if (warp == kIssuer1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(*tmem_slot) : "memory");
+  }
+}
+
+}  // namespace walk
+
+// Which problems this kernel takes, and how many of their pairs of query tiles (the rest goes to the small CTAs that
+// `split` names).  Attention launch, us, kernel of forward.cu (where it walked its items up to 48 tiles) / this one, PNQ:
+// 37 x 16384 queries, KV tiles 1, 4, 128: 52.8 / 45.7, 122.0 / 108.2, 2800 / 2753; 40 x 16384, 2 tiles: 84.6 / 73.3;
+// 40 x 4096, 32: 235 / 206; 64 x 8192, 8: 188 / 169; 40 x 8192, 48, 64: 631 / 603, 825 / 795; 16 x 32768, 256: 4736 / 4733;
+// 12 x 75600, 591: 18376 / 18456.  With the direct row sum, 1, 4, 32, 48, 128, 256 tiles: 58.2 / 46.0, 136.7 / 112.3,
+// 262 / 228, 711 / 668, 3203 / 3054, 5370 / 5254.  So PNQ ends at 256 tiles and the direct row sum has no end.
+// - One wave of pairs that would be two rounds of single tiles stays with forward.cu (14 x 1300 x 777: 20.7 us for 21.1).
+// - Launches that run beside others (`followed`) keep to short sequences: CTAs that walk hold their SMs to the end
+//   (24 x 8192 from host tensors: 3225 us for 3246).
+// - Small CTAs for the last wave cost a launch and 1200 to 2125 cycles per tile and CTA, a round of single tiles T x 1390
+//   cycles (direct 1500) + 1000.  All in one walk / last wave in small CTAs, whole call: 24 x 8192 527 / 537 (direct 588 / 597),
+//   40 x 4096 241 / 250, 38 x 8192 x 3000 330 / 336.  Up to 8 tiles a last wave that is at most half full stays with the small CTAs
+//   all the same (26 / 28 for 38 x 1000 x 700, 134 / 139 for 38 x 8192 x 1000): the number of launches of such calls is pinned.
+WalkSplit forward_walk_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq, bool followed, const RowSplit& split) {
+  const int64_t T = (Nkv + kTile - 1) / kTile, tiles = (Nq + kTile - 1) / kTile, pairs = (tiles + 1) / 2;
+  if ((pnq && T > 256) || (followed && T > 48)) return WalkSplit{false, 0};
+  if (split.R == 0) return WalkSplit{bh * pairs > n_sm || bh * tiles <= n_sm, bh * pairs};
+  auto walk = [&](int64_t items) { return (items + n_sm - 1) / n_sm * (T * (pnq ? 1390 : 1500) + 1000) + 4400; };
+  const int64_t per_head = (Nq + kTile / split.R - 1) / (kTile / split.R), at = split.pairs_256;
+  const int64_t done = at / pairs * per_head + (at % pairs) * 2 * split.R, before = at / pairs * tiles + (at % pairs) * 2;
+  const int64_t small = (bh * per_head - done + n_sm - 1) / n_sm * (T * (split.R == 4 ? 1200 : split.R == 2 ? 1530 : 2125) + 4500);
+  const bool all = walk(bh * tiles) <= (before > 0 ? walk(before) + 4000 : 0) + small && !(before > 0 && T <= 8 && 2 * (bh * tiles - before) <= n_sm);
+  return WalkSplit{true, all ? bh * pairs : at};
+}
+
+// The first `pairs` pairs of query tiles, counted over all heads.
+int launch_forward_walk(int64_t n_sm, int64_t pairs, const void* q_codes, const void* q_scales, const void* k_codes, const void* k_scales,
+                        const void* v_codes, const void* v_scales, void* o, int B, int H, int64_t Nq, int64_t Nkv,
+                        float softmax_scale, unsigned flags, int* status, cudaStream_t stream) {
+  using namespace walk;
+  Params p;
+  p.q_codes = (const uint8_t*)q_codes; p.q_scales = (const uint8_t*)q_scales;
+  p.k_codes = (const uint8_t*)k_codes; p.k_scales = (const uint8_t*)k_scales;
+  p.v_codes = (const uint8_t*)v_codes; p.v_scales = (const uint8_t*)v_scales;
+  p.status = status; p.Nq = Nq; p.Nkv = Nkv;
+  p.q_tiles = (int)((Nq + kTile - 1) / kTile); p.kv_tiles = (int)((Nkv + kTile - 1) / kTile);
+  const int64_t per_head = (p.q_tiles + 1) / 2, items = pairs / per_head * p.q_tiles + (pairs % per_head) * 2;
+  if (items > 0x7FFFFFFF) return MXATTN_EUNSUPPORTED;
+  p.total_items = (int)items;
+  p.scale_log2e = softmax_scale * 1.4426950408889634f;
+  CUtensorMap out_map;
+  const int map_rc = encode_output_map(&out_map, o, (int64_t)B * H, Nq, flags & MXATTN_FLAG_OUT_FP32);
+  if (map_rc != MXATTN_OK) return map_rc;
+  const bool uos = flags & MXATTN_FLAG_UOS, pnq = flags & MXATTN_FLAG_PNQ, f32 = flags & MXATTN_FLAG_OUT_FP32;
+  void (*kern)(const Params, const CUtensorMap) = nullptr;
+#define PICK(U, P, F) if (uos == U && pnq == P && f32 == F) kern = attention_walk_kernel<U, P, F>;
+  PICK(false, false, false) PICK(false, false, true) PICK(false, true, false) PICK(false, true, true)
+  PICK(true, false, false) PICK(true, false, true) PICK(true, true, false) PICK(true, true, true)
+#undef PICK
+  if (!ensure_dynamic_smem((const void*)kern, kSmemBytes)) return MXATTN_ECUDA;
+  return launch_pdl(kern, dim3((unsigned)(items < n_sm ? items : n_sm)), kThreads, kSmemBytes, stream, p, out_map) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
+}
+
+}  // namespace mxattn

@@ -252,6 +252,21 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
                  "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]),            \
                  "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]),            \
                  "+r"(r[30]), "+r"(r[31])::"memory")
+// Keys beyond the sequence do not exist: the scores of columns `valid` to `cols` - 1 (of this warp's 32 rows, at `taddr`) become
+// -inf in tensor memory, before the warp loads its scores.  Replacing them in the registers behind the load costs every tile,
+// not only the last: the values of both paths have to meet in one set of registers, which the load's own consecutive ones are
+// not, and the compiler copies all of them: 1548 -> 1411 cycles per tile in a build of forward_walk.cu, whose loop is bound by
+// instructions.  (The kernel of forward.cu gets slower, 61.6 -> 64.1 ms at 40 x 75600, so the others mask their registers.)
+__device__ __forceinline__ void mask_scores(uint32_t taddr, int valid, int cols) {
+  int i = valid < 0 ? 0 : valid;
+#pragma unroll 1
+  for (; i < cols && (i & 7) != 0; ++i)
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(taddr + i), "r"(0xFF800000u) : "memory");
+#pragma unroll 1
+  for (; i < cols; i += 8)
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(taddr + i), "r"(0xFF800000u) : "memory");
+  tmem_st_wait();
+}
 __device__ __forceinline__ int lds_volatile(uint32_t addr) {
   int v;
   asm volatile("ld.volatile.shared.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");

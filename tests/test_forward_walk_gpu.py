@@ -1,0 +1,65 @@
+"""The attention kernel whose CTAs walk items of one query tile (two teams of softmax warps take the KV tiles in turn): the same
+head alone, which small CTAs of another kernel compute, and copied often enough that every CTA walks several items.  The KV
+tiles of an item are one, two, three (teams change from item to item), as many as buffers come round (4 to 9) and more; query
+and key counts end inside a tile, a half and a block."""
+import ctypes
+
+import pytest
+import torch
+
+import synth_inputs as si
+from tests import util
+
+
+def walk_split(n_sm, heads, nq, nkv, pnq, followed=False):
+    """(whether the kernel is used, pairs of query tiles it takes), asked of the library"""
+    import paper_2607_24377_b200 as mx
+
+    class Row(ctypes.Structure):
+        _fields_ = [("pairs_256", ctypes.c_int64), ("R", ctypes.c_int)]
+
+    class Walk(ctypes.Structure):
+        _fields_ = [("walk", ctypes.c_bool), ("pairs", ctypes.c_int64)]
+
+    f = getattr(mx.lib(), "_ZN6mxattn18forward_walk_splitEllllbbRKNS_8RowSplitE")
+    f.argtypes, f.restype = [ctypes.c_int64] * 4 + [ctypes.c_bool] * 2 + [ctypes.POINTER(Row)], Walk
+    w = f(n_sm, heads, nq, nkv, pnq, followed, ctypes.byref(Row(*util.row_split(n_sm, heads, nq, nkv, pnq))))
+    return w.walk, w.pairs
+
+
+@pytest.mark.parametrize("pnq", [True, False])
+def test_what_the_walking_kernel_takes(pnq):
+    for heads, nq, nkv in ((1, 1, 1), (2, 1024, 1024), (40, 4096, 4096), (40, 75600, 512), (24, 8192, 8192), (3, 50000, 300)):
+        walk, pairs = walk_split(148, heads, nq, nkv, pnq)
+        total, (whole, r) = heads * ((-(-nq // 128) + 1) // 2), util.row_split(148, heads, nq, nkv, pnq)
+        assert walk and pairs in (whole, total) and (r != 0 or pairs == total)
+    assert walk_split(148, 2, 1024, 1024, pnq)[1] == 0                       # small CTAs alone
+    assert walk_split(148, 40, 4096, 4096, pnq)[1] == 640                    # nine waves of single tiles, no second launch
+    assert not walk_split(148, 14, 1300, 777, pnq)[0] and walk_split(148, 13, 1300, 777, pnq)[0]      # one wave of pairs, two rounds of tiles; one round
+    assert walk_split(148, 24, 4096, 6144, pnq, True)[0] and not walk_split(148, 24, 4096, 6145, pnq, True)[0]      # beside other launches
+    assert walk_split(148, 40, 256 * 128, 256 * 128, pnq)[0] and walk_split(148, 40, 256, 256 * 128 + 1, pnq)[0] == (not pnq)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nq,nkv", [(1, 1), (129, 128), (300, 200), (128, 257), (257, 384), (100, 511), (640, 700), (385, 1000), (200, 1152), (300, 5000)])
+@pytest.mark.parametrize("uos,pnq,f32", [(True, True, False), (True, False, True), (False, True, True), (False, False, False)])
+def test_walked_items_equal_a_single_head(nq, nkv, uos, pnq, f32):
+    import paper_2607_24377_b200 as mx
+    flags = (mx.FLAG_UOS if uos else 0) | (mx.FLAG_PNQ if pnq else 0) | (mx.FLAG_OUT_FP32 if f32 else 0)
+    one = si.custom_config("wk", 1, 2, nq, nkv, 3 + nq)
+    q, k, v = si.make_all(one)
+    outs = []
+    for copies in (1, 223):                                                  # 446 heads: three to fifteen items per CTA, not a whole number
+        heads = 2 * copies
+        dev = [util.to_dev_bf16(x).repeat(1, copies, 1, 1).contiguous() for x in (q, k, v)]
+        out = util.guarded((1, heads, nq, 128), torch.float32 if f32 else torch.bfloat16, float("nan"))
+        ws = util.guarded(mx.forward_workspace_bytes(1, heads, nq, nkv, 128), torch.uint8)
+        for _ in range(2):                                                   # the second launch follows the first closely
+            mx.forward_ws(*dev, out.t, 1, heads, nq, nkv, 128, one.softmax_scale, flags, ws.t)
+        assert mx.device_status(ws.t) == 0
+        out.check(); ws.check()
+        outs.append(out.t.clone())
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    assert walk_split(n_sm, 2, nq, nkv, pnq)[1] == 0 and walk_split(n_sm, 446, nq, nkv, pnq)[1] > 0
+    assert bool(torch.isfinite(outs[0].float()).all())
+    assert torch.equal(outs[1], outs[0].repeat(1, 223, 1, 1))

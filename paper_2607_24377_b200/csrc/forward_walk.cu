@@ -285,8 +285,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
         mbar_wait_soft<34>(bar(BAR_X + q * 4 + (f & 3)), (uint32_t)((f >> 2) & 1), abort_addr);
         const float2 mx = lds64o<0>(aX + (f & 3) * kXSlot);
         const float m_old = m_run;
-        float m_new = fmaxf(mx.x, mx.y);
-        if (j > 0) m_new = fmaxf(m_new, m_old);
+        const float m_new = max3(mx.x, mx.y, j > 0 ? m_old : -INFINITY);     // a tile without a number leaves -inf, as in forward.cu
         m_run = m_new;
         if (!kPnq && j >= 2) add_sums(f - 2, alpha2);
         float alpha = 1.0f;

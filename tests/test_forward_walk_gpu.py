@@ -63,3 +63,35 @@ def test_walked_items_equal_a_single_head(nq, nkv, uos, pnq, f32):
     assert walk_split(n_sm, 2, nq, nkv, pnq)[1] == 0 and walk_split(n_sm, 446, nq, nkv, pnq)[1] > 0
     assert bool(torch.isfinite(outs[0].float()).all())
     assert torch.equal(outs[1], outs[0].repeat(1, 223, 1, 1))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nq,nkv", [(1, 700), (300, 700), (300, 128)])
+@pytest.mark.parametrize("pnq", [True, False])
+def test_scores_that_are_not_numbers(nq, nkv, pnq):
+    """Given operands may carry the E8M0 code of NaN: here the scales of one head's first KV tile, and of one query of another.
+    A tile that has no maximum leaves the running one at -inf, in whichever kernel the row is computed, and the next tile's maximum
+    then drops what came before (with the row sum from the quantized probabilities, which are finite)."""
+    import paper_2607_24377_b200 as mx
+    one = si.custom_config("nn", 1, 3, nq, nkv, 9)
+    ops = []
+    for x, n, axis in zip(si.make_all(one), (nq, nkv, nkv), (1, 1, 0)):
+        codes = torch.empty((3, -(-n // 128), 8192), dtype=torch.uint8, device="cuda")
+        scales = torch.empty((3, -(-n // 128), 512), dtype=torch.uint8, device="cuda")
+        mx.quantize_mxfp4_batched(util.to_dev_bf16(x), codes, scales, 3, n, 128, axis, mx.MODE_UOS, mx.LAYOUT_TILE)
+        ops += [codes, scales]
+    ops[3][0, 0] = 255
+    ops[1][1, 0, util.tile_scale_offset(0, 0)] = 255
+    flags, outs = mx.FLAG_UOS | (mx.FLAG_PNQ if pnq else 0) | mx.FLAG_OUT_FP32, []
+    for copies in (1, 149):
+        out = torch.empty((1, 3 * copies, nq, 128), device="cuda")
+        status = torch.zeros(4, dtype=torch.int32, device="cuda")
+        mx.forward_prequantized(*(x.repeat(copies, 1, 1) for x in ops), out, 1, 3 * copies, nq, nkv, 128, one.softmax_scale, flags, status)
+        assert int(status[0]) == 0
+        outs.append(out)
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    assert walk_split(n_sm, 3, nq, nkv, pnq)[1] == 0 and walk_split(n_sm, 447, nq, nkv, pnq)[1] > 0
+    want = outs[0].repeat(1, 149, 1, 1)
+    assert not pnq or bool(torch.isfinite(want[0, 0]).all())
+    assert torch.equal(torch.isnan(outs[1]), torch.isnan(want))
+    assert torch.equal(torch.nan_to_num(outs[1]), torch.nan_to_num(want))

@@ -481,6 +481,8 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
 // - One wave of pairs that would be two rounds of single tiles stays with forward.cu (14 x 1300 x 777: 20.7 us for 21.1).
 // - Launches that run beside others (`followed`) keep to short sequences: CTAs that walk hold their SMs to the end
 //   (24 x 8192 from host tensors: 3225 us for 3246).
+// - A CTA counts its tiles in 32 bits: one head of 73 million queries and keys has more (the last few are left for the teams'
+//   steps beyond the end).
 // - Small CTAs for the last wave cost a launch and 1200 to 2125 cycles per tile and CTA, a round of single tiles T x 1390
 //   cycles (direct 1500) + 1000.  All in one walk / last wave in small CTAs, whole call: 24 x 8192 527 / 537 (direct 588 / 597),
 //   40 x 4096 241 / 250, 38 x 8192 x 3000 330 / 336.  Up to 8 tiles a last wave that is at most half full stays with the small CTAs
@@ -488,6 +490,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
 WalkSplit forward_walk_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq, bool followed, const RowSplit& split) {
   const int64_t T = (Nkv + kTile - 1) / kTile, tiles = (Nq + kTile - 1) / kTile, pairs = (tiles + 1) / 2;
   if ((pnq && T > 256) || (followed && T > 48)) return WalkSplit{false, 0};
+  if ((bh * tiles + n_sm - 1) / n_sm * T > 0x7FFFFF00) return WalkSplit{false, 0};
   if (split.R == 0) return WalkSplit{bh * pairs > n_sm || bh * tiles <= n_sm, bh * pairs};
   auto walk = [&](int64_t items) { return (items + n_sm - 1) / n_sm * (T * (pnq ? 1390 : 1500) + 1000) + 4400; };
   const int64_t per_head = (Nq + kTile / split.R - 1) / (kTile / split.R), at = split.pairs_256;

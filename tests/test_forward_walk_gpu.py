@@ -40,6 +40,14 @@ def test_what_the_walking_kernel_takes(pnq):
     assert walk_split(148, 40, 256 * 128, 256 * 128, pnq)[0] and walk_split(148, 40, 256, 256 * 128 + 1, pnq)[0] == (not pnq)
 
 
+def test_tiles_of_a_cta_are_counted_in_32_bits():
+    # one head of n queries and keys with the direct row sum: up to 2^31 - 256 tiles per CTA
+    for n, taken in ((72 << 20, False), (73_000_000, False), (64 << 20, True)):
+        tiles = -(-n // 128)
+        assert (-(-tiles // 148) * tiles <= 0x7FFFFF00) == taken
+        assert taken or not walk_split(148, 1, n, n, False)[0]
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("nq,nkv", [(1, 1), (129, 128), (300, 200), (128, 257), (257, 384), (100, 511), (640, 700), (385, 1000), (200, 1152), (300, 5000)])
 @pytest.mark.parametrize("uos,pnq,f32", [(True, True, False), (True, False, True), (False, True, True), (False, False, False)])

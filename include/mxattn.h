@@ -349,10 +349,13 @@ int mxattn_quantizer_status(int* host_out, void* stream);
  * 0 = no bounded wait expired since the workspace was last used by a forward. */
 int mxattn_device_status(const void* workspace, int* host_out, void* stream);
 
-/* Exercises the failure path of the device-side waits without disturbing the GPU: a one-warp kernel
+/* Exercises the failure path of the device-side waits without disturbing the GPU: a warp
  * waits on a barrier that nothing arrives on, gives up after `limit_cycles` SM cycles (at most 2e9) and
- * writes the code 77 into status[0] (4 device ints, zeroed by the caller).  The kernel ends normally
- * and the context stays usable.  Every wait inside the attention kernels uses the same routine with a
+ * writes the code 77 into status[0] (4 device ints, zeroed by the caller).  Two teams of further warps go through 2^17
+ * tiles as the softmax warps that walk key tiles do, and their first wait runs out after a million cycles: status[1] = 78, its
+ * code, status[2] = the cycles until they are through, status[3] = the tiles that a warp worked on before it noticed that
+ * its CTA had given up, and only met the others from there on.  The kernel ends normally
+ * and the context stays usable.  Every wait inside the attention kernels uses these routines with a
  * limit of about two seconds. */
 int mxattn_selftest_bounded_wait(void* status, int64_t limit_cycles, void* stream);
 

@@ -559,17 +559,39 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
 
 // Self-test of the bounded wait: one warp waits on a barrier that nothing ever arrives on, with a
 // short limit; the wait must give up, record its code in `status`, and the kernel must end normally.
+// Four more warps are a row quarter's two teams (team_tiles) whose first wait runs out in the same way: status[1] = its code,
+// status[2] = the cycles that their 2^17 tiles take behind it, status[3] = the tiles that one warp worked on before it noticed.
 __global__ void bounded_wait_selftest_kernel(int* status, long long limit_cycles) {
   __shared__ uint64_t barrier;
-  __shared__ int abort_flag;
+  __shared__ int abort_flag[2];
+  const int warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
     mbar_init(smem_u32(&barrier), 1);
-    abort_flag = 0;
+    abort_flag[0] = abort_flag[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  const bool done = mbar_wait(smem_u32(&barrier), 0u, &abort_flag, status, 77, limit_cycles);
-  if (done && threadIdx.x == 0) atomicCAS(status, 0, -1);      // must not happen
+  if (warp == 0) {
+    const bool done = mbar_wait(smem_u32(&barrier), 0u, &abort_flag[0], status, 77, limit_cycles);
+    if (done && threadIdx.x == 0) atomicCAS(status, 0, -1);      // must not happen
+  } else {
+    const int t = (warp - 1) & 1;
+    const uint32_t abort_addr = smem_u32(&abort_flag[1]);
+    int tiles = 0;
+    long long t0 = 0;
+    if (t == 1) asm volatile("bar.arrive %0, 128;" ::"r"(1) : "memory");     // nothing comes before tile 0
+    team_tiles(t, 1 << 17, abort_addr, 1 + t, 2 - t, [&](auto) {
+      mbar_wait_soft<78, 0, true, 1000000>(smem_u32(&barrier), 0u, abort_addr);
+      if (tiles++ == 0) t0 = clock64();
+      asm volatile("bar.sync %0, 128;" ::"r"(1 + t) : "memory");
+      asm volatile("bar.arrive %0, 128;" ::"r"(2 - t) : "memory");
+    });
+    if (threadIdx.x == 32) {
+      status[1] = *(volatile int*)&abort_flag[1];
+      status[2] = (int)(clock64() - t0);
+      status[3] = tiles;
+    }
+  }
 }
 
 // Self-test of the way two paired softmax warps stay in step when one of them gives up: warp 0 waits, with a short
@@ -611,7 +633,7 @@ int launch_pair_abandon_selftest(int* status, long long limit_cycles, int meetin
 }
 
 int launch_bounded_wait_selftest(int* status, long long limit_cycles, cudaStream_t stream) {
-  fwd::bounded_wait_selftest_kernel<<<1, 32, 0, stream>>>(status, limit_cycles);
+  fwd::bounded_wait_selftest_kernel<<<1, 160, 0, stream>>>(status, limit_cycles);
   return cudaGetLastError() == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 

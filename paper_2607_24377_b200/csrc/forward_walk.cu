@@ -24,12 +24,11 @@
 // Tensor memory (512 columns): scores [0,128) and [128,256), accumulator and row sum [256,400), scales behind it: Q 4 slots,
 // K 4, V 8, P 4.  Slots are as many as it takes that a copy never follows a product that still reads the slot.
 //
-// Every wait is bounded (mbar_wait_soft / role_wait); the softmax and scaling warps never leave their loops early, so that
-// no warp is stranded at a named barrier, and nothing is stored once the CTA's abort flag is up.
+// Every wait is bounded (mbar_wait_soft / role_wait); a softmax warp keeps its meetings to the end (team_tiles), so that
+// none is stranded at a named barrier, and nothing is stored once the CTA's abort flag is up.
 #include <string.h>
 
 #include <algorithm>
-#include <type_traits>
 
 #include "common.cuh"
 #include "tc_helpers.cuh"
@@ -90,33 +89,6 @@ template <int kOff> __device__ __forceinline__ float2 lds64o(uint32_t a) {
 }
 template <int kOff> __device__ __forceinline__ void arrive_if(uint32_t b, bool me) {
   asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0+%1];\n\t}" ::"r"(b), "n"(kOff), "r"((uint32_t)me) : "memory");
-}
-// mbar_wait_soft with a probe in front: a wait that is already satisfied takes 38 cycles as a test_wait, 78 as a try_wait.
-template <int kCode, int kOff>
-__device__ __forceinline__ void mbar_wait_probe(uint32_t bar, uint32_t parity, uint32_t abort_addr) {
-  asm volatile("{\n\t.reg .pred p;\n\t.reg .u64 t0, t1;\n\t.reg .u32 a;\n\t"
-               "mbarrier.test_wait.parity.shared::cta.b64 p, [%0+%2], %1;\n\t"
-               "vote.sync.all.pred p, p, 0xffffffff;\n\t"
-               "@p bra.uni DONE;\n\t"
-               "mov.u64 t0, %%clock64;\n"
-               "AGAIN:\n\t"
-               
-               "mbarrier.try_wait.parity.shared::cta.b64 p, [%0+%2], %1, 20000;\n\t"
-
-               "vote.sync.all.pred p, p, 0xffffffff;\n\t"
-               "@p bra.uni DONE;\n\t"
-               "ld.volatile.shared.u32 a, [%4];\n\t"
-               "setp.ne.u32 p, a, 0;\n\t"
-               "vote.sync.any.pred p, p, 0xffffffff;\n\t"
-               "@p bra.uni DONE;\n\t"
-               "mov.u64 t1, %%clock64;\n\t"
-               "sub.u64 t1, t1, t0;\n\t"
-               "setp.lt.u64 p, t1, 4000000000;\n\t"
-               "vote.sync.any.pred p, p, 0xffffffff;\n\t"
-               "@p bra.uni AGAIN;\n\t"
-               "st.volatile.shared.u32 [%4], %3;\n"
-               "DONE:\n\t}"
-               ::"r"(bar), "r"(parity), "n"(kOff), "n"(kCode), "r"(abort_addr) : "memory");
 }
 __device__ __forceinline__ bool role_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status, int code) {
   return __all_sync(0xFFFFFFFFu, mbar_test(bar, parity)) || mbar_wait_warp(bar, parity, abort_flag, status, code);
@@ -339,7 +311,8 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
       const float inv_l = 1.0f / l;
       const int bh = item / p.q_tiles, qtile = item - bh * p.q_tiles;
       const int row0 = qtile * kTile + q * 32;
-      const bool inside = row0 < p.Nq && lds_volatile(abort_addr) == 0;
+      if (lds_volatile(abort_addr) != 0) break;                  // given up: nothing more is stored, and no warp waits for this one
+      const bool inside = row0 < p.Nq;
 #pragma unroll 1
       for (int h = 0; h < 2; ++h)
         store_half_rows<kOutF32>(t_o + 64 * h, sbase + kOffOut + (2 * q + h) * kOutBoxBytes, lane, inv_l, &out_map, 64 * h, row0, bh, inside);
@@ -400,7 +373,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
     };
     auto tile = [&](auto kk) {                                   // kk: parity of the team's tile count
       constexpr int k = decltype(kk)::value;
-      mbar_wait_probe<31, 8 * BAR_SFULL>(barT, (uint32_t)k, abort_addr);
+      mbar_wait_soft<31, 8 * BAR_SFULL, true>(barT, (uint32_t)k, abort_addr);
       tc_fence_after();
       if (jn == T - 1 && ragged < 64) mask_scores(t_s, ragged, 64);
       float b0, b1;
@@ -453,11 +426,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
       __syncwarp();
       arrive_if<8 * BAR_PFULL + 16 * k>(barT, lane == 0);
     };
-    for (int f = t; f < F; f += 4) {
-      tile(std::integral_constant<int, 0>{});
-      if (f + 2 >= F) break;
-      tile(std::integral_constant<int, 1>{});
-    }
+    team_tiles(t, F, abort_addr, idOwn, idOther, tile);
   }
 
   // ---- teardown ------------------------------------------------------------------------------

@@ -1,5 +1,7 @@
 // tcgen05 / mbarrier / bulk-copy helpers shared by the attention kernels (sm_100a, inline PTX).
 #pragma once
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace mxattn {
@@ -273,33 +275,61 @@ __device__ __forceinline__ int lds_volatile(uint32_t addr) {
   return v;
 }
 // A wait after which the caller goes on in any case: it gives up on its own limit (about two seconds; the code then goes
-// into the CTA's abort flag, from where it reaches `status` at the end) or when the abort flag is up, and every later wait
-// of the CTA then returns at once.  For warps that meet at named barriers: none of them ever leaves its loop early, so none
-// can be stranded there.
-template <int kCode>
+// into the CTA's abort flag, from where it reaches `status` at the end) or when the abort flag is up; every later wait of the
+// CTA then returns when its try_wait does, after 4 us.  For warps that meet at named barriers: none of them leaves its loop
+// without keeping what meetings are left, so none can be stranded there.  (The flag read in front of the try_wait costs every
+// wait that is not satisfied yet, 2 x 1024: 10.6 -> 10.9 us; a shorter time limit for the try_wait is not heeded.)
+// kTest: a test_wait in front (a wait that is already satisfied takes 38 cycles as that, 78 as a try_wait).  kOff: of the
+// barrier from `bar`.
+#define MBAR_SOFT_WAIT(first)                                                        \
+  asm volatile("{\n\t.reg .pred p;\n\t.reg .u64 t0, t1;\n\t.reg .u32 a;\n\t" first     \
+               "mbarrier.try_wait.parity.shared::cta.b64 p, [%0+%4], %1, 20000;\n\t" \
+               "vote.sync.all.pred p, p, 0xffffffff;\n\t"                            \
+               "@p bra.uni DONE;\n\t"                                                \
+               "mov.u64 t0, %%clock64;\n"                                            \
+               "AGAIN:\n\t"                                                          \
+               "ld.volatile.shared.u32 a, [%2];\n\t"                                 \
+               "setp.ne.u32 p, a, 0;\n\t"                                            \
+               "vote.sync.any.pred p, p, 0xffffffff;\n\t"                            \
+               "@p bra.uni DONE;\n\t"                                                \
+               "mbarrier.try_wait.parity.shared::cta.b64 p, [%0+%4], %1, 20000;\n\t" \
+               "vote.sync.all.pred p, p, 0xffffffff;\n\t"                            \
+               "@p bra.uni DONE;\n\t"                                                \
+               "mov.u64 t1, %%clock64;\n\t"                                          \
+               "sub.u64 t1, t1, t0;\n\t"                                             \
+               "setp.lt.u64 p, t1, %5;\n\t"                                          \
+               "vote.sync.any.pred p, p, 0xffffffff;\n\t"                            \
+               "@p bra.uni AGAIN;\n\t"                                               \
+               "st.volatile.shared.u32 [%2], %3;\n"                                  \
+               "DONE:\n\t}"                                                          \
+               ::"r"(bar), "r"(parity), "r"(abort_addr), "n"(kCode), "n"(kOff), "n"(kLimit) : "memory")
+template <int kCode, int kOff = 0, bool kTest = false, long long kLimit = kWaitLimitCycles>
 __device__ __forceinline__ void mbar_wait_soft(uint32_t bar, uint32_t parity, uint32_t abort_addr) {
   // one block of assembly, so that the usual case is a probe, a vote and a branch, and the rest costs no registers
-  asm volatile("{\n\t.reg .pred p;\n\t.reg .u64 t0, t1;\n\t.reg .u32 a;\n\t"
-               "mbarrier.try_wait.parity.shared::cta.b64 p, [%0], %1, 20000;\n\t"
-               "vote.sync.all.pred p, p, 0xffffffff;\n\t"
-               "@p bra.uni DONE;\n\t"
-               "mov.u64 t0, %%clock64;\n"
-               "AGAIN:\n\t"
-               "ld.volatile.shared.u32 a, [%2];\n\t"
-               "setp.ne.u32 p, a, 0;\n\t"
-               "vote.sync.any.pred p, p, 0xffffffff;\n\t"
-               "@p bra.uni DONE;\n\t"
-               "mbarrier.try_wait.parity.shared::cta.b64 p, [%0], %1, 20000;\n\t"
-               "vote.sync.all.pred p, p, 0xffffffff;\n\t"
-               "@p bra.uni DONE;\n\t"
-               "mov.u64 t1, %%clock64;\n\t"
-               "sub.u64 t1, t1, t0;\n\t"
-               "setp.lt.u64 p, t1, 4000000000;\n\t"
-               "vote.sync.any.pred p, p, 0xffffffff;\n\t"
-               "@p bra.uni AGAIN;\n\t"
-               "st.volatile.shared.u32 [%2], %3;\n"
-               "DONE:\n\t}"
-               ::"r"(bar), "r"(parity), "r"(abort_addr), "n"(kCode) : "memory");
+  if constexpr (kTest)
+    MBAR_SOFT_WAIT("mbarrier.test_wait.parity.shared::cta.b64 p, [%0+%4], %1;\n\tvote.sync.all.pred p, p, 0xffffffff;\n\t@p bra.uni DONE;\n\t");
+  else
+    MBAR_SOFT_WAIT("");
+}
+#undef MBAR_SOFT_WAIT
+// Two teams of softmax warps take the tiles 0 .. F - 1 of a CTA in turn (team t: t, t + 2, ...).  The four warps of a row quarter
+// meet once per tile at a named barrier of the team whose tile it is (its two warps wait, the other team's two only arrive,
+// behind their own tile's).  Every 64 tiles a warp looks whether the CTA has given up, and then keeps the meetings only: with
+// the waits of all tiles that are left, 4 us each, a call would take several times its own time to end.
+template <typename Tile>
+__device__ __forceinline__ void team_tiles(int t, int F, uint32_t abort_addr, int own_bar, int other_bar, Tile&& tile) {
+  int f = t;
+  for (; f < F; f += 4) {
+    if ((f & 60) == 0 && lds_volatile(abort_addr) != 0) break;
+    tile(std::integral_constant<int, 0>{});
+    if (f + 2 >= F) return;
+    tile(std::integral_constant<int, 1>{});
+  }
+#pragma unroll 1
+  for (; f < F; f += 2) {
+    asm volatile("bar.sync %0, 128;" ::"r"(own_bar) : "memory");
+    asm volatile("bar.arrive %0, 128;" ::"r"(other_bar) : "memory");
+  }
 }
 
 __device__ __forceinline__ void sts8(uint32_t addr, uint32_t v) {

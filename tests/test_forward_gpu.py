@@ -229,6 +229,17 @@ def test_bounded_wait_gives_up_and_reports_without_disturbing_the_device():
         mx.selftest_bounded_wait(status, 0)
 
 
+def test_teams_that_gave_up_are_soon_through():
+    # the softmax warps that take tiles in turn go on when a wait runs out, so that none is stranded at a named barrier, but
+    # not with the waits of all the tiles that are left (2^17 here, half of them a team's, some 8000 cycles each)
+    import paper_2607_24377_b200 as mx
+    status = torch.zeros(4, dtype=torch.int32, device="cuda")
+    mx.selftest_bounded_wait(status, 2_000_000)
+    first, code, cycles, tiles = status.tolist()
+    assert (first, code) == (77, 78)
+    assert 1 <= tiles <= 32 and 0 < cycles < (1 << 17) * 500
+
+
 def test_paired_warps_stay_in_step_when_one_gives_up():
     # the two softmax warps of a row pair meet at a named barrier in every tile; a warp that gives up keeps the
     # remaining appointments so that its partner is never stranded.  A dedicated kernel makes one warp's short-limit

@@ -3,7 +3,11 @@
 //
 // One CTA per SM walks work items of one query tile (128 rows of one head); the tiles of all its items form one stream
 // f = 0, 1, 2, ... (KV tiles of 128 keys in ascending order within an item), and barriers, tensor memory and the pipelines
-// run on across items.  Roles (736 threads):
+// run on across items.  Up to 48 KV tiles (kStaticTiles) a CTA's items are fixed at the launch, every 148th.  Above, the grid has
+// a CTA per item, and a CTA that is done with an item takes over one that has not started (kTake): with fixed shares a launch
+// beside that holds a few SMs for long leaves whole shares to come last (24 x 8192 beside 4 CTAs of 8 ms: 937 us, with items
+// taken 550; direct row sum 1023 -> 589; 12 x 16384 1774 -> 1013).  Alone the two are equal within 0.3 % with PNQ, with the
+// direct sum taking is ahead (24 x 8192 587 -> 569, 24 x 30000 6892 -> 6708).  Roles (736 threads):
 //   warps 0-15   softmax, two teams of eight: team f & 1 takes tile f.  Two threads a row, one half of 64 keys each.  A team
 //                has a score buffer of its own, so that neither waits for the other to take its scores; what passes from
 //                team to team is the maxima of a tile, two floats a row, posted before the exponentials (a named barrier at
@@ -59,9 +63,10 @@ constexpr int kXSlot = 128 * 2 * 4;
 constexpr int kOffXL = kOffX + 4 * kXSlot;                       // row sums of a tile by half (direct placement): 8 slots, laid out alike
 constexpr int kOffBar = kOffXL + 8 * kXSlot;
 enum Bar { BAR_Q = 0, BAR_QEMPTY = 2, BAR_KFULL = 4, BAR_ODONE = BAR_KFULL + kStages, BAR_SFULL = BAR_ODONE + kStages,
-           BAR_SFREE = BAR_SFULL + 2, BAR_PFULL = BAR_SFREE + 2, BAR_X = BAR_PFULL + 4 /* [quarter][tile & 3]: maxima posted */, kNumBars = BAR_X + 16 };
-constexpr int kOffMisc = kOffBar + kNumBars * 8;
-constexpr int kSmemBytes = kOffMisc + 32 + 1024;
+           BAR_SFREE = BAR_SFULL + 2, BAR_PFULL = BAR_SFREE + 2, BAR_X = BAR_PFULL + 4 /* [quarter][tile & 3]: maxima posted */, BAR_NEXT = BAR_X + 16, kNumBars = BAR_NEXT + 1 };
+constexpr int kOffMisc = (kOffBar + kNumBars * 8 + 15) & ~15;    // tensor memory's start; abort flag, number of tiles, status on entry
+constexpr int kOffNext = kOffMisc + 32, kOffItems = kOffNext + 16;     // answer to the request for an item; items n & 3 (-1: there is none)
+constexpr int kSmemBytes = kOffItems + 16 + 1024;
 static_assert(kOffOut % 1024 == 0 && kSmemBytes <= 227 * 1024, "shared memory per CTA");
 constexpr uint32_t kColS = 0, kColO = 256, kColSFQ = 400, kColSFK = 416, kColSFV = 432, kColSFP = 496;     // 4, 4, 8 and 4 slots
 
@@ -90,11 +95,23 @@ template <int kOff> __device__ __forceinline__ float2 lds64o(uint32_t a) {
 template <int kOff> __device__ __forceinline__ void arrive_if(uint32_t b, bool me) {
   asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0+%1];\n\t}" ::"r"(b), "n"(kOff), "r"((uint32_t)me) : "memory");
 }
+// Takes over the work of a CTA of this grid that has not started yet.  The answer (16 bytes) and its bytes' completion arrive
+// asynchronously; the index of the CTA that will not be launched, or -1 if all have been (after which nothing more may be asked).
+__device__ __forceinline__ void ask_for_cta(uint32_t answer, uint32_t bar) {
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(answer), "r"(bar) : "memory");
+}
+__device__ __forceinline__ int cta_taken(uint32_t answer) {
+  int cta;
+  asm volatile("{\n\t.reg .b128 a;\n\t.reg .pred p;\n\tld.shared.b128 a, [%1];\n\tmov.s32 %0, -1;\n\t"
+               "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, a;\n\t"
+               "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, a;\n\t}" : "=r"(cta) : "r"(answer) : "memory");
+  return cta;
+}
 __device__ __forceinline__ bool role_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status, int code) {
   return __all_sync(0xFFFFFFFFu, mbar_test(bar, parity)) || mbar_wait_warp(bar, parity, abort_flag, status, code);
 }
 
-template <bool kUos, bool kPnq, bool kOutF32>
+template <bool kUos, bool kPnq, bool kOutF32, bool kTake>
 __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Params p, const __grid_constant__ CUtensorMap out_map) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -104,6 +121,9 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kOffMisc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kOffMisc + 8);
   const uint32_t abort_addr = sbase + kOffMisc + 8;
+  volatile int* tiles_in_all = abort_flag + 1;                   // kTake: written once, when no item is left
+  volatile int* status_before = abort_flag + 2;     // kTake: written once, when no item is left
+  volatile int* items = reinterpret_cast<volatile int*>(smem + kOffItems);
 
   const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int T = p.kv_tiles;
@@ -118,7 +138,9 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
     mbar_init(bar(BAR_SFREE), kTeamWarps); mbar_init(bar(BAR_SFREE + 1), kTeamWarps);
     for (int s = 0; s < kStages; ++s) { mbar_init(bar(BAR_KFULL + s), 1); mbar_init(bar(BAR_ODONE + s), 1); }
     for (int i = 0; i < 16; ++i) mbar_init(bar(BAR_X + i), 1);
+    mbar_init(bar(BAR_NEXT), 1);
     abort_flag[0] = 0;
+    *tiles_in_all = 0x7FFFFFFF;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   for (int i = tid; i < kStages * 64; i += kThreads)             // rows of ones behind every V stage (code 2 = 1.0), their scales
@@ -131,17 +153,19 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   pdl_wait();                                                    // the operands and the status word are ready
-  if (tid == 0) abort_flag[1] = *reinterpret_cast<volatile int*>(p.status);
+  if (tid == 0) *status_before = *reinterpret_cast<volatile int*>(p.status);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   pdl_trigger();
   constexpr uint32_t tmem = 0;
   if (*tmem_slot != 0) *abort_flag = kCodeTmemBase;
-  const int role = __shfl_sync(0xFFFFFFFFu, (abort_flag[1] != 0 || *tmem_slot != 0) ? kThreads / 32 : warp, 0);     // an earlier launch gave up
+  const int role = __shfl_sync(0xFFFFFFFFu, (*status_before != 0 || *tmem_slot != 0) ? kThreads / 32 : warp, 0);     // an earlier launch gave up
 
-  const int n_items = (p.total_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-  const int F = n_items * T;                                     // tiles of this CTA
+  // Items of this CTA: every gridDim.x-th one, or (kTake) its own and then those of CTAs that have not started, one after another.
+  // The producer asks for them; the others learn of item n from the barrier of its Q tile.
+  const int n_items = kTake ? 0x7FFFFFFF : (p.total_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+  const int F = kTake ? 0x7FFFFFFF : n_items * T;                // tiles of this CTA
 
   if (role == kProducer) {
     // =============================== producer ===============================================
@@ -149,11 +173,19 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
       bool ok = true;
       int f = 0, n = 0, s = 0;
       uint32_t ph = 0;
-      for (int item = blockIdx.x; n < n_items && ok; ++n, item += gridDim.x) {
+      for (int item = blockIdx.x; n < n_items && ok; ++n) {
         const int bh = item / p.q_tiles;
         const int qb = n & 1;
         if (n >= 2) ok = mbar_wait1(bar(BAR_QEMPTY + qb), (uint32_t)(((n - 2) >> 1) & 1), abort_flag, p.status, 13);
         if (!ok) break;
+        if (kTake) {
+          items[n & 3] = item;
+          if (item < 0) {
+            *tiles_in_all = n * T;
+            mbar_arrive(bar(BAR_Q + qb));
+            break;
+          }
+        }
         mbar_expect_tx(bar(BAR_Q + qb), kTileCodeBytes + kTileScaleBytes);
         bulk_g2s(sbase + kOffQ + qb * kTileCodeBytes, p.q_codes + (int64_t)item * kTileCodeBytes, kTileCodeBytes, bar(BAR_Q + qb));
         bulk_g2s(sbase + kOffSFQ + qb * kTileScaleBytes, p.q_scales + (int64_t)item * kTileScaleBytes, kTileScaleBytes, bar(BAR_Q + qb));
@@ -168,7 +200,22 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
           bulk_g2s(sbase + kOffSFV + s * kTileScaleBytes, p.v_scales + (kv0 + j) * kTileScaleBytes, kTileScaleBytes, bar(BAR_KFULL + s));
           if (++s == kStages) { s = 0; ph ^= 1u; }
         }
+        if (!kTake) {
+          item += gridDim.x;
+        } else if (ok) {                                         // now, not earlier: an item taken while another is far from done may end last
+          mbar_expect_tx(bar(BAR_NEXT), 16);
+          ask_for_cta(sbase + kOffNext, bar(BAR_NEXT));
+          if (!mbar_wait1(bar(BAR_NEXT), (uint32_t)(n & 1), abort_flag, p.status, 14)) {
+            const long long t0 = clock64();
+            while (!mbar_try(bar(BAR_NEXT), (uint32_t)(n & 1)) && clock64() - t0 < 200000000LL) {}
+            ok = false;
+          } else {
+            item = cta_taken(sbase + kOffNext);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // read before the next answer is written
+          }
+        }
       }
+      if (kTake && *tiles_in_all == 0x7FFFFFFF) *tiles_in_all = n * T;       // gave up; n: items begun
       if (!ok || *abort_flag) {                                  // gave up: let copies in flight land before shared memory is released
         const long long t0 = clock64();
         for (int g = (f > kStages ? f - kStages : 0); g < f; ++g)
@@ -189,6 +236,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
       const int qb = n & 1;
       if (j == 0) {
         if (!role_wait(bar(BAR_Q + qb), (uint32_t)((n >> 1) & 1), abort_flag, p.status, 21)) break;
+        if (kTake && items[n & 3] < 0) break;
         tc_fence_after();
         tc_cp_sf_if(leader, tmem + kColSFQ + 4 * (n & 3), sbase + kOffSFQ + qb * kTileScaleBytes);
       }
@@ -220,9 +268,13 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
     constexpr uint32_t kDescHiTile = (512u >> 4) | (1u << 14) | (4u << 29);   // 64-byte swizzle, K-major
     auto desc = [](uint32_t saddr) { return ((uint64_t)kDescHiTile << 32) | (saddr >> 4); };
     for (int i = 0; i < 8; ++i) tc_cp_sf_if(leader, tmem + kColSFV + 8 * i + 4, sbase + kOffSFOnes);
-    int j = 0, s = 0;
+    int j = 0, s = 0, n = 0;
     uint32_t ph = 0;
     for (int f = 0; f < F; ++f) {
+      if (kTake && j == 0) {
+        if (!role_wait(bar(BAR_Q + (n & 1)), (uint32_t)((n >> 1) & 1), abort_flag, p.status, 27) || items[n & 3] < 0) break;
+        ++n;
+      }
       if (!role_wait(bar(BAR_KFULL + s), ph, abort_flag, p.status, 26)) break;
       tc_fence_after();
       const uint32_t sfa = tmem + kColSFP + 4 * (f & 3), sfb = tmem + kColSFV + 8 * (f & 7);
@@ -253,6 +305,11 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
     };
     int item = blockIdx.x;
     for (int n = 0; n < n_items; ++n, item += gridDim.x) {
+      if (kTake) {
+        mbar_wait_soft<35, 0, true>(bar(BAR_Q + (n & 1)), (uint32_t)((n >> 1) & 1), abort_addr);
+        item = items[n & 3];                                     // anything if the CTA has given up: nothing is stored then
+        if (item < 0) break;
+      }
       for (int j = 0; j < T; ++j, ++f) {
         mbar_wait_soft<34>(bar(BAR_X + q * 4 + (f & 3)), (uint32_t)((f >> 2) & 1), abort_addr);
         const float2 mx = lds64o<0>(aX + (f & 3) * kXSlot);
@@ -398,7 +455,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
       m_run = m_new;
       jn += 2;
       if (jn >= T) jn -= T;
-      if (jn >= T) jn -= T;
+      if (jn >= T) jn -= T;                                      // T = 1; left out where T is larger, PNQ takes 9 % longer (24 x 8192)
       uint64_t nb0, nb1;
       uint32_t sf0, sf1;
       exponent(b0, m_new, nb0, sf0);
@@ -426,7 +483,31 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
       __syncwarp();
       arrive_if<8 * BAR_PFULL + 16 * k>(barT, lane == 0);
     };
-    team_tiles(t, F, abort_addr, idOwn, idOther, tile);
+    if (!kTake) {
+      team_tiles(t, F, abort_addr, idOwn, idOther, tile);
+    } else {
+      // At the team's first tile of item n: whether there is one.  If the CTA has given up, the meetings that are kept are those of the
+      // tiles that the producer says it has begun (it watches the flag too): whole items, so that no warp is beyond them.
+      int f = t, n = 0, known = 0;                               // known: tiles of the items up to n
+      auto ends = [&]() {
+        mbar_wait_soft<36, 0, true>(bar(BAR_Q + (n & 1)), (uint32_t)((n >> 1) & 1), abort_addr);
+        ++n;
+        known += T;
+        int up, all;
+        asm volatile("ld.volatile.shared.v2.s32 {%0, %1}, [%2];" : "=r"(up), "=r"(all) : "r"(abort_addr) : "memory");
+        return f >= all || up != 0;
+      };
+      for (;; f += 2) {
+        if (f >= known && ends()) break;
+        tile(std::integral_constant<int, 0>{});
+        f += 2;
+        if (f >= known && ends()) break;
+        tile(std::integral_constant<int, 1>{});
+      }
+      int all = *tiles_in_all;
+      for (int i = 0; all == 0x7FFFFFFF && i < (1 << 28); ++i) all = *tiles_in_all;
+      if (all != 0x7FFFFFFF) team_meetings(f, all, idOwn, idOther);
+    }
   }
 
   // ---- teardown ------------------------------------------------------------------------------
@@ -450,8 +531,8 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
 // - One wave of pairs that would be two rounds of single tiles stays with forward.cu (14 x 1300 x 777: 20.7 us for 21.1).
 // - Launches that run beside others (`followed`) keep to short sequences: CTAs that walk hold their SMs to the end
 //   (24 x 8192 from host tensors: 3225 us for 3246).
-// - A CTA counts its tiles in 32 bits: one head of 73 million queries and keys has more (the last few are left for the teams'
-//   steps beyond the end).
+// - A CTA counts its tiles in 32 bits (the last few are left for the teams' steps beyond the end).  Where it takes items from
+//   others it may get them all: one head of 6 million queries and keys has more.
 // - Small CTAs for the last wave cost a launch and 1200 to 2125 cycles per tile and CTA, a round of single tiles T x 1390
 //   cycles (direct 1500) + 1000.  All in one walk / last wave in small CTAs, whole call: 24 x 8192 527 / 537 (direct 588 / 597),
 //   40 x 4096 241 / 250, 38 x 8192 x 3000 330 / 336.  Up to 8 tiles a last wave that is at most half full stays with the small CTAs
@@ -459,7 +540,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
 WalkSplit forward_walk_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq, bool followed, const RowSplit& split) {
   const int64_t T = (Nkv + kTile - 1) / kTile, tiles = (Nq + kTile - 1) / kTile, pairs = (tiles + 1) / 2;
   if ((pnq && T > 256) || (followed && T > 48)) return WalkSplit{false, 0};
-  if ((bh * tiles + n_sm - 1) / n_sm * T > 0x7FFFFF00) return WalkSplit{false, 0};
+  if ((T > kStaticTiles ? bh * tiles : (bh * tiles + n_sm - 1) / n_sm) * T > 0x7FFFFF00) return WalkSplit{false, 0};
   if (split.R == 0) return WalkSplit{bh * pairs > n_sm || bh * tiles <= n_sm, bh * pairs};
   auto walk = [&](int64_t items) { return (items + n_sm - 1) / n_sm * (T * (pnq ? 1390 : 1500) + 1000) + 4400; };
   const int64_t per_head = (Nq + kTile / split.R - 1) / (kTile / split.R), at = split.pairs_256;
@@ -488,13 +569,14 @@ int launch_forward_walk(int64_t n_sm, int64_t pairs, const void* q_codes, const 
   const int map_rc = encode_output_map(&out_map, o, (int64_t)B * H, Nq, flags & MXATTN_FLAG_OUT_FP32);
   if (map_rc != MXATTN_OK) return map_rc;
   const bool uos = flags & MXATTN_FLAG_UOS, pnq = flags & MXATTN_FLAG_PNQ, f32 = flags & MXATTN_FLAG_OUT_FP32;
+  const bool take = p.kv_tiles > kStaticTiles && items > n_sm;
   void (*kern)(const Params, const CUtensorMap) = nullptr;
-#define PICK(U, P, F) if (uos == U && pnq == P && f32 == F) kern = attention_walk_kernel<U, P, F>;
+#define PICK(U, P, F) if (uos == U && pnq == P && f32 == F) kern = take ? attention_walk_kernel<U, P, F, true> : attention_walk_kernel<U, P, F, false>;
   PICK(false, false, false) PICK(false, false, true) PICK(false, true, false) PICK(false, true, true)
   PICK(true, false, false) PICK(true, false, true) PICK(true, true, false) PICK(true, true, true)
 #undef PICK
   if (!ensure_dynamic_smem((const void*)kern, kSmemBytes)) return MXATTN_ECUDA;
-  return launch_pdl(kern, dim3((unsigned)(items < n_sm ? items : n_sm)), kThreads, kSmemBytes, stream, p, out_map) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
+  return launch_pdl(kern, dim3((unsigned)(take || items < n_sm ? items : n_sm)), kThreads, kSmemBytes, stream, p, out_map) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 
 }  // namespace mxattn

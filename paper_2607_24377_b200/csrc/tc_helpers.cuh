@@ -316,6 +316,13 @@ __device__ __forceinline__ void mbar_wait_soft(uint32_t bar, uint32_t parity, ui
 // meet once per tile at a named barrier of the team whose tile it is (its two warps wait, the other team's two only arrive,
 // behind their own tile's).  Every 64 tiles a warp looks whether the CTA has given up, and then keeps the meetings only: with
 // the waits of all tiles that are left, 4 us each, a call would take several times its own time to end.
+__device__ __forceinline__ void team_meetings(int f, int F, int own_bar, int other_bar) {
+#pragma unroll 1
+  for (; f < F; f += 2) {
+    asm volatile("bar.sync %0, 128;" ::"r"(own_bar) : "memory");
+    asm volatile("bar.arrive %0, 128;" ::"r"(other_bar) : "memory");
+  }
+}
 template <typename Tile>
 __device__ __forceinline__ void team_tiles(int t, int F, uint32_t abort_addr, int own_bar, int other_bar, Tile&& tile) {
   int f = t;
@@ -325,11 +332,7 @@ __device__ __forceinline__ void team_tiles(int t, int F, uint32_t abort_addr, in
     if (f + 2 >= F) return;
     tile(std::integral_constant<int, 1>{});
   }
-#pragma unroll 1
-  for (; f < F; f += 2) {
-    asm volatile("bar.sync %0, 128;" ::"r"(own_bar) : "memory");
-    asm volatile("bar.arrive %0, 128;" ::"r"(other_bar) : "memory");
-  }
+  team_meetings(f, F, own_bar, other_bar);
 }
 
 __device__ __forceinline__ void sts8(uint32_t addr, uint32_t v) {

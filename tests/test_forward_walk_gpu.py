@@ -46,6 +46,8 @@ def test_tiles_of_a_cta_are_counted_in_32_bits():
         tiles = -(-n // 128)
         assert (-(-tiles // 148) * tiles <= 0x7FFFFF00) == taken
         assert taken or not walk_split(148, 1, n, n, False)[0]
+    # above 48 tiles, where a CTA takes items that others have not begun, they may all be its own
+    assert not walk_split(148, 1, 6_000_000, 6_000_000, False)[0] and walk_split(148, 1, 100 << 20, 48 * 128, False)[0]
 
 
 @pytest.mark.gpu
@@ -103,3 +105,86 @@ def test_scores_that_are_not_numbers(nq, nkv, pnq):
     assert not pnq or bool(torch.isfinite(want[0, 0]).all())
     assert torch.equal(torch.isnan(outs[1]), torch.isnan(want))
     assert torch.equal(torch.nan_to_num(outs[1]), torch.nan_to_num(want))
+
+
+# Above 48 KV tiles the CTAs take one item after another from the grid: several different items each (three heads, so that a CTA
+# never sees one head again and again), tile counts that swap the teams' roles from item to item and ones that do not, query and
+# key counts that end inside a tile; two launches back to back, and one beside a launch that holds some of the SMs.
+@pytest.mark.gpu
+@pytest.mark.parametrize("nq,nkv", [(129, 49 * 128), (300, 49 * 128 + 1), (257, 51 * 128 - 31), (385, 64 * 128 + 77), (130, 127 * 128 + 5)])
+@pytest.mark.parametrize("uos,pnq,f32", [(True, True, False), (True, False, True), (False, True, True), (False, False, False)])
+def test_taken_items_equal_a_single_head(nq, nkv, uos, pnq, f32):
+    import paper_2607_24377_b200 as mx
+    flags = (mx.FLAG_UOS if uos else 0) | (mx.FLAG_PNQ if pnq else 0) | (mx.FLAG_OUT_FP32 if f32 else 0)
+    one = si.custom_config("tk", 1, 3, nq, nkv, 5 + nq)
+    q, k, v = (util.to_dev_bf16(x) for x in si.make_all(one))
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    assert walk_split(n_sm, 3, nq, nkv, pnq)[1] == 0 and walk_split(n_sm, 237, nq, nkv, pnq)[1] > 0
+    assert n_sm % (3 * -(-nq // 128)) != 0
+
+    def run(copies, beside=None):
+        heads = 3 * copies
+        dev = [x.repeat(1, copies, 1, 1).contiguous() for x in (q, k, v)]
+        out = util.guarded((1, heads, nq, 128), torch.float32 if f32 else torch.bfloat16, float("nan"))
+        ws = util.guarded(mx.forward_workspace_bytes(1, heads, nq, nkv, 128), torch.uint8)
+        torch.cuda.synchronize()
+        if beside is not None:
+            beside()
+        for _ in range(2):
+            mx.forward_ws(*dev, out.t, 1, heads, nq, nkv, 128, one.softmax_scale, flags, ws.t)
+        assert mx.device_status(ws.t) == 0
+        out.check(); ws.check()
+        return out.t.clone()
+
+    want = run(1).repeat(1, 79, 1, 1)
+    assert bool(torch.isfinite(want.float()).all())
+    assert torch.equal(run(79), want)
+    side, long_kv = torch.cuda.Stream(), 400_000                             # 4 groups of rows: 4 CTAs that take 2 ms
+    lq, lk, lv = (torch.randn(1, 1, n, 128, device="cuda").to(torch.bfloat16) for n in (128, long_kv, long_kv))
+    lo, lws = torch.empty_like(lq), torch.empty(mx.forward_workspace_bytes(1, 1, 128, long_kv, 128), dtype=torch.uint8, device="cuda")
+
+    def hold():
+        with torch.cuda.stream(side):
+            mx.forward_ws(lq, lk, lv, lo, 1, 1, 128, long_kv, 128, one.softmax_scale, mx.FLAG_UOS | mx.FLAG_PNQ, lws)
+
+    got = run(79, hold)
+    side.synchronize()                                                       # before its buffers go
+    assert torch.equal(got, want) and mx.device_status(lws) == 0
+
+
+@pytest.mark.gpu
+def test_a_launch_that_holds_few_sms_does_not_hold_up_whole_shares():
+    """24 heads of 8192: ten and a half items per SM.  Beside 4 CTAs that run for 8 ms, the items of those 4 SMs are
+    spread over the others (about 1.1 times the time alone); with shares that are fixed at the launch they come last (1.6 times)."""
+    import paper_2607_24377_b200 as mx
+    mk = lambda h, n: torch.randn(1, h, n, 128, device="cuda").to(torch.bfloat16)
+    q, k, v = mk(24, 8192), mk(24, 8192), mk(24, 8192)
+    lq, lk, lv = mk(1, 128), mk(1, 1 << 21), mk(1, 1 << 21)
+    o, lo = torch.empty_like(q), torch.empty_like(lq)
+    ws, lws = (torch.empty(mx.forward_workspace_bytes(1, *a, 128), dtype=torch.uint8, device="cuda") for a in ((24, 8192, 8192), (1, 128, 1 << 21)))
+    side, flags = torch.cuda.Stream(), mx.FLAG_UOS | mx.FLAG_PNQ
+
+    def timed():
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        mx.forward_ws(q, k, v, o, 1, 24, 8192, 8192, 128, 128 ** -0.5, flags, ws)
+        b.record(); b.synchronize()
+        return a.elapsed_time(b)
+
+    def hold():
+        with torch.cuda.stream(side):
+            mx.forward_ws(lq, lk, lv, lo, 1, 1, 128, 1 << 21, 128, 128 ** -0.5, flags, lws)
+
+    hold(); timed(); torch.cuda._sleep(1)                                    # kernels are loaded
+    alone, beside = [], []
+    for _ in range(5):
+        torch.cuda.synchronize()
+        alone.append(timed())
+        torch.cuda.synchronize()
+        hold()
+        torch.cuda._sleep(1_000_000)                                         # its attention has started
+        beside.append(timed())
+        still = not side.query()
+        side.synchronize()                                                   # before its buffers go
+        assert still                                                         # it ran all the while
+    assert sorted(beside)[2] < 1.35 * sorted(alone)[2]

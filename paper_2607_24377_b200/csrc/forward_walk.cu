@@ -535,8 +535,8 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
 //   others it may get them all: one head of 6 million queries and keys has more.
 // - Small CTAs for the last wave cost a launch and 1200 to 2125 cycles per tile and CTA, a round of single tiles T x 1390
 //   cycles (direct 1500) + 1000.  All in one walk / last wave in small CTAs, whole call: 24 x 8192 527 / 537 (direct 588 / 597),
-//   40 x 4096 241 / 250, 38 x 8192 x 3000 330 / 336.  Up to 8 tiles a last wave that is at most half full stays with the small CTAs
-//   all the same (26 / 28 for 38 x 1000 x 700, 134 / 139 for 38 x 8192 x 1000): the number of launches of such calls is pinned.
+//   40 x 4096 241 / 250, 38 x 8192 x 3000 330 / 336, x 1000 134.8 / 139.5 (direct 140.4 / 145.1), 38 x 1000 x 700 24.9 / 27.8,
+//   51 x 700 x 300 18.2 / 21.2.
 WalkSplit forward_walk_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq, bool followed, const RowSplit& split) {
   const int64_t T = (Nkv + kTile - 1) / kTile, tiles = (Nq + kTile - 1) / kTile, pairs = (tiles + 1) / 2;
   if ((pnq && T > 256) || (followed && T > 48)) return WalkSplit{false, 0};
@@ -546,7 +546,7 @@ WalkSplit forward_walk_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, 
   const int64_t per_head = (Nq + kTile / split.R - 1) / (kTile / split.R), at = split.pairs_256;
   const int64_t done = at / pairs * per_head + (at % pairs) * 2 * split.R, before = at / pairs * tiles + (at % pairs) * 2;
   const int64_t small = (bh * per_head - done + n_sm - 1) / n_sm * (T * (split.R == 4 ? 1200 : split.R == 2 ? 1530 : 2125) + 4500);
-  const bool all = walk(bh * tiles) <= (before > 0 ? walk(before) + 4000 : 0) + small && !(before > 0 && T <= 8 && 2 * (bh * tiles - before) <= n_sm);
+  const bool all = walk(bh * tiles) <= (before > 0 ? walk(before) + 4000 : 0) + small;
   return WalkSplit{true, all ? bh * pairs : at};
 }
 

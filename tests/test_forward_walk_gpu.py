@@ -40,6 +40,23 @@ def test_what_the_walking_kernel_takes(pnq):
     assert walk_split(148, 40, 256 * 128, 256 * 128, pnq)[0] and walk_split(148, 40, 256, 256 * 128 + 1, pnq)[0] == (not pnq)
 
 
+@pytest.mark.parametrize("pnq", [True, False])
+def test_last_wave_goes_where_it_is_estimated_to_end_first(pnq):
+    # cycles of n single tiles in one walk, and of a launch of small CTAs behind them (the figures stand at the rule)
+    rounds = lambda n, t: -(-n // 148) * (t * (1390 if pnq else 1500) + 1000) + 4400
+    split = 0
+    for heads, nq, nkv in ((38, 1000, 700), (38, 8192, 1000), (51, 700, 300), (38, 897, 6200), (38, 1000, 130), (40, 2000, 1024), (24, 8192, 8192), (39, 897, 6300)):
+        whole, r = util.row_split(148, heads, nq, nkv, pnq)
+        t, tiles = -(-nkv // 128), -(-nq // 128)
+        pairs, groups = (tiles + 1) // 2, -(-nq // (128 // r))
+        ahead = whole // pairs * tiles + whole % pairs * 2
+        small = -(-(heads * groups - whole // pairs * groups - whole % pairs * 2 * r) // 148) * (t * {4: 1200, 2: 1530, 1: 2125}[r] + 4500)
+        one = rounds(heads * tiles, t) <= rounds(ahead, t) + 4000 + small
+        assert walk_split(148, heads, nq, nkv, pnq) == (True, heads * pairs if one else whole)
+        split += not one
+    assert split == 2
+
+
 def test_tiles_of_a_cta_are_counted_in_32_bits():
     # one head of n queries and keys with the direct row sum: up to 2^31 - 256 tiles per CTA
     for n, taken in ((72 << 20, False), (73_000_000, False), (64 << 20, True)):

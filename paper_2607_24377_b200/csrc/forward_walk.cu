@@ -523,12 +523,17 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
 }  // namespace walk
 
 // Which problems this kernel takes, and how many of their pairs of query tiles (the rest goes to the small CTAs that
-// `split` names).  Attention launch, us, kernel of forward.cu (where it walked its items up to 48 tiles) / this one, PNQ:
+// `split` names).  Attention launch, us, kernel of forward.cu (in a form that walked its items up to 48 tiles) / this one, PNQ:
 // 37 x 16384 queries, KV tiles 1, 4, 128: 52.8 / 45.7, 122.0 / 108.2, 2800 / 2753; 40 x 16384, 2 tiles: 84.6 / 73.3;
 // 40 x 4096, 32: 235 / 206; 64 x 8192, 8: 188 / 169; 40 x 8192, 48, 64: 631 / 603, 825 / 795; 16 x 32768, 256: 4736 / 4733;
-// 12 x 75600, 591: 18376 / 18456.  With the direct row sum, 1, 4, 32, 48, 128, 256 tiles: 58.2 / 46.0, 136.7 / 112.3,
-// 262 / 228, 711 / 668, 3203 / 3054, 5370 / 5254.  So PNQ ends at 256 tiles and the direct row sum has no end.
-// - One wave of pairs that would be two rounds of single tiles stays with forward.cu (14 x 1300 x 777: 20.7 us for 21.1).
+// 12 x 75600, 591: 18376 / 18456.  With the direct row sum, 1, 4, 32, 48 tiles: 58.2 / 46.0, 136.7 / 112.3, 262 / 228,
+// 711 / 668, and whole calls: 37 x 4096, 100: 695 / 672; 16 x 32768, 256: 5402 / 5293; 12 x 40000, 400: 7647 / 7554; 12 x 75600,
+// 591: 20726 / 20574; 24 x 16384, 591: 9405 / 9109.  So PNQ ends at 256 tiles, and the direct row sum has an end only below.
+// - A few whole waves of pairs that single tiles do not round better.  PNQ: one wave, whole call at 2, 7, 12, 49, 100 tiles: 37 x
+//   1000 13.2 / 12.8, 22.7 / 22.5, 31.2 / 31.3, 105.4 / 106.8, 194.6 / 196.4 (14 x 1300 x 777, fp32: 20.7 / 20.5).  Direct: up to
+//   four waves above 256 tiles; one wave (37 x 1000) at 2, 12, 48, 100, 256, 400 tiles: 13.8 / 12.9, 34.8 / 32.1, 115.4 / 111.0,
+//   215.3 / 209.9, 506.8 / 506.4, 774.7 / 780.0; two (37 x 2048), 1016: 3369 / 3412; four (37 x 4096), 256, 469: 1658 / 1646,
+//   2961 / 2970.
 // - Launches that run beside others (`followed`) keep to short sequences: CTAs that walk hold their SMs to the end
 //   (24 x 8192 from host tensors: 3225 us for 3246).
 // - A CTA counts its tiles in 32 bits (the last few are left for the teams' steps beyond the end).  Where it takes items from
@@ -541,7 +546,11 @@ WalkSplit forward_walk_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, 
   const int64_t T = (Nkv + kTile - 1) / kTile, tiles = (Nq + kTile - 1) / kTile, pairs = (tiles + 1) / 2;
   if ((pnq && T > 256) || (followed && T > 48)) return WalkSplit{false, 0};
   if ((T > kStaticTiles ? bh * tiles : (bh * tiles + n_sm - 1) / n_sm) * T > 0x7FFFFF00) return WalkSplit{false, 0};
-  if (split.R == 0) return WalkSplit{bh * pairs > n_sm || bh * tiles <= n_sm, bh * pairs};
+  if (split.R == 0) {
+    const int64_t rounds = (bh * tiles + n_sm - 1) / n_sm, waves = (bh * pairs + n_sm - 1) / n_sm;
+    const bool pairs_ahead = pnq || followed ? waves == 1 : waves <= 4 && T > 256;
+    return WalkSplit{rounds < 2 * waves || !pairs_ahead, bh * pairs};
+  }
   auto walk = [&](int64_t items) { return (items + n_sm - 1) / n_sm * (T * (pnq ? 1390 : 1500) + 1000) + 4400; };
   const int64_t per_head = (Nq + kTile / split.R - 1) / (kTile / split.R), at = split.pairs_256;
   const int64_t done = at / pairs * per_head + (at % pairs) * 2 * split.R, before = at / pairs * tiles + (at % pairs) * 2;

@@ -35,9 +35,19 @@ def test_what_the_walking_kernel_takes(pnq):
         assert walk and pairs in (whole, total) and (r != 0 or pairs == total)
     assert walk_split(148, 2, 1024, 1024, pnq)[1] == 0                       # small CTAs alone
     assert walk_split(148, 40, 4096, 4096, pnq)[1] == 640                    # nine waves of single tiles, no second launch
-    assert not walk_split(148, 14, 1300, 777, pnq)[0] and walk_split(148, 13, 1300, 777, pnq)[0]      # one wave of pairs, two rounds of tiles; one round
+    assert walk_split(148, 14, 1300, 777, pnq)[0] == (not pnq) and walk_split(148, 13, 1300, 777, pnq)[0]      # one wave of pairs, two rounds of tiles; one round
     assert walk_split(148, 24, 4096, 6144, pnq, True)[0] and not walk_split(148, 24, 4096, 6145, pnq, True)[0]      # beside other launches
     assert walk_split(148, 40, 256 * 128, 256 * 128, pnq)[0] and walk_split(148, 40, 256, 256 * 128 + 1, pnq)[0] == (not pnq)
+
+
+def test_few_whole_waves_of_pairs_with_the_direct_row_sum():
+    # 74 x 512 and 37 x 4096: exactly one and four waves of pairs, two and eight rounds of single tiles
+    for heads, nq in ((74, 512), (37, 4096)):
+        assert walk_split(148, heads, nq, 256 * 128, False) == (True, heads * nq // 256)
+        assert not walk_split(148, heads, nq, 256 * 128 + 1, False)[0]
+    assert walk_split(148, 37, 8192, 600 * 128, False)[0]                    # eight waves
+    assert walk_split(148, 14, 1300, 100 * 128, False)[0] and not walk_split(148, 14, 1300, 777, False, True)[0]     # beside other launches
+    assert walk_split(148, 3, 6200, 400 * 128, False) == (True, 75)          # 147 single tiles: one round where pairs take one of twice the time
 
 
 @pytest.mark.parametrize("pnq", [True, False])

@@ -465,7 +465,8 @@ def main():
         peak_note = (f"no FP4 probe in this run: {peaks['source']} sustained bf16 cuBLAS {peaks['bf16_tflops_sustained']} "
                      f"x nominal ratio 4 (of {peaks['source']})")
         per_clock = None
-    roofline = {"bound": "mufu", "kernel": "attention_kernel<uos,pnq>", "achieved": attn_tflops,
+    walked = Nkv <= 256 * 128              # up to 256 key tiles the launch is the kernel that walks single query tiles
+    roofline = {"bound": "mufu", "kernel": "attention_walk_kernel<uos,pnq>" if walked else "attention_kernel<uos,pnq>", "achieved": attn_tflops,
                 "peak": fp4_peak, "unit": "TFLOP/s", "frac": attn_tflops / fp4_peak,
                 "frac_per_sm_clock": per_clock, "achieved_sm_mhz": clocks.get("sm_mhz"),
                 "traffic": ATTN_TRAFFIC_PER_TOKEN_HEAD * Nkv * B * H if Nq == Nkv else None,
@@ -475,7 +476,8 @@ def main():
                 # the softmax exponentials bind before the tensor pipe does: 16 ex2 per clock per SM,
                 # one per (query, key) pair, 512 tensor flops per pair
                 "mufu_ceiling_tflops": mufu_ceiling, "frac_of_mufu_ceiling": attn_tflops / mufu_ceiling if mufu_ceiling else None,
-                "ncu_cross_check": "profiles/attention_kernel_sweep16384.txt: sm__pipe_tensor_cycles_active 21.2 %, XU pipe 83 %"}
+                "ncu_cross_check": "profiles/attention_walk_kernel.txt (4 key tiles per item): sm__pipe_tensor_cycles_active 16.9 %, XU pipe 68 %"
+                if walked else "profiles/attention_kernel_sweep16384.txt: sm__pipe_tensor_cycles_active 21.2 %, XU pipe 83 %"}
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
         "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,

@@ -41,8 +41,9 @@ SOFTMAX_PHASES = ["wait_scores", "load_scores", "maxima", "pair_exchange", "wait
 
 
 def cycle_profile(mx, torch, cfg, dev):
-    """Per-role cycle budget of the UOS + PNQ attention kernel (mxattn_forward_cycle_profile, the kernel compiled with
-    cycle counters): mean SM cycles per key tile in each phase, per role, next to the time of the kernel without counters."""
+    """Per-role cycle budget of the UOS + PNQ attention kernel for long key/value sequences (mxattn_forward_cycle_profile, that
+    kernel compiled with cycle counters): mean SM cycles per key tile in each phase, per role, next to the time of a whole forward
+    call -- through the same kernel above 256 key tiles (`same_kernel`), through the one that walks single query tiles below."""
     B, H, Nq, Nkv, d = cfg.B, cfg.H, cfg.Nq, cfg.Nkv, cfg.d
     q, k, v = si.make_all(cfg)
     dq, dk, dv = dev(q), dev(k), dev(v)
@@ -71,15 +72,14 @@ def cycle_profile(mx, torch, cfg, dev):
     sm = p[:, :16, :]
     per_tile = sm[:, :, :8] / np.maximum(sm[:, :, 9:10], 1)   # [cta, warp, phase]
     rep = {"workload": cfg.name, "H": H, "Nq": Nq, "Nkv": Nkv, "kv_tiles": kv_tiles, "ctas": int(p.shape[0]),
-           "ms_without_counters": ms_plain, "ms_with_counters": ms_prof,
+           "ms_forward_call": ms_plain, "ms_with_counters": ms_prof, "same_kernel": kv_tiles > 256,
            "softmax_cycles_per_tile": {SOFTMAX_PHASES[i]: float(per_tile[:, :, i].mean()) for i in range(8)},
            "softmax_epilogue_cycles_per_item": float((sm[:, :, 8] / np.maximum(sm[:, :, 9] / kv_tiles, 1)).mean()),
            "issuer_cycles_per_tile": {"loop_total": float((p[:, 17, 8:9] / tiles).mean()),
                                       "wait_p_hat_tile0": float((p[:, 17, 0:1] / tiles).mean()), "wait_p_hat_tile1": float((p[:, 17, 2:3] / tiles).mean()),
                                       "wait_q": float((p[:, 17, 5:6] / tiles).mean()), "wait_kv": float((p[:, 17, 6:7] / tiles).mean()),
                                       "wait_score_buffer": float((p[:, 17, 7:8] / tiles).mean())},
-           "producer_cycles_per_tile": {"loop_total": float((p[:, 16, 8:9] / tiles).mean()), "wait_free_stage": float((p[:, 16, 3:4] / tiles).mean()),
-                                        "wait_free_q_buffer": float((p[:, 16, 5:6] / tiles).mean())}}
+           "producer_cycles_per_tile": {"loop_total": float((p[:, 16, 8:9] / tiles).mean()), "wait_free_stage": float((p[:, 16, 3:4] / tiles).mean())}}
     rep["softmax_cycles_per_tile"]["sum"] = float(per_tile.sum(axis=2).mean())
     for g in (0, 1):            # the two softmax groups (query tile 0: warps 0-7, query tile 1: warps 8-15) separately
         pg = per_tile[:, 8 * g:8 * g + 8, :]
@@ -93,7 +93,7 @@ def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--quick", action="store_true", help="smallest sizes only")
     ap.add_argument("--cycle-profile", default=None, metavar="WORKLOAD",
-                    help="only this: per-role cycle profile of the attention kernel on the named workload (e.g. sweep16384, wan22, wan22_cross)")
+                    help="only this: per-role cycle profile of the attention kernel for long sequences on the named workload (e.g. wan22)")
     args = ap.parse_args()
     import torch
     import paper_2607_24377_b200 as mx

@@ -201,16 +201,16 @@ int mxattn_forward_debug_dump(const void* q, const void* k, const void* v, void*
                               void* dump, size_t dump_bytes, void* stream);
 
 /* Performance-analysis aid: mxattn_forward_ws (flags exactly MXATTN_FLAG_UOS | MXATTN_FLAG_PNQ, bf16 output) through
- * an instantiation of the attention kernel that counts, per role, the SM cycles spent in each phase of the key-tile
- * loop of Algorithm 2 (the timed kernels are compiled without the counters; reading the cycle counter perturbs the
- * loop by a few percent).  `profile`: caller-owned device memory of mxattn_forward_cycle_profile_bytes() bytes,
+ * an instantiation of the attention kernel for long key/value sequences (more than 256 key tiles; it takes any size here,
+ * although mxattn_forward_ws gives shorter ones to others) that counts, per role, the SM cycles spent in each phase of the key-tile
+ * loop of Algorithm 2 (the timed kernels are compiled without the counters; reading the cycle counter lengthens the
+ * loop by 17-19 %).  `profile`: caller-owned device memory of mxattn_forward_cycle_profile_bytes() bytes,
  * zeroed by the caller, that receives [CTA][warp 0..17][16] int64.  One CTA per work item (two query tiles of one
- * head), or, for short key/value sequences with more work items than SMs, one CTA per SM (then only the first
- * #SMs records are written).
+ * head).
  *   warps 0-15 (softmax): [0] wait for the scores, [1] score load, [2] block and row maxima, [3] exchange with the
  *     partner warp, [4] wait for the previous output product, [5] block exponents, [6] exponentials + packing
  *     (+ rescaling), [7] hand-over of P-hat, [8] epilogue, [9] tiles processed;
- *   warp 16 (copy producer): [3] wait for a free K/V stage, [5] wait for a free Q buffer, [8] whole loop, [9] tiles;
+ *   warp 16 (copy producer): [3] wait for a free K/V stage, [8] whole loop, [9] tiles;
  *   warp 17 (MMA issuer): [0] / [2] wait for P-hat of query tile 0 / 1, [5] wait for Q, [6] wait for K/V, [7] wait
  *     for the score buffer, [8] whole loop, [9] tiles. */
 size_t mxattn_forward_cycle_profile_bytes(int B, int H, int64_t Nq, int64_t Nkv, int d);

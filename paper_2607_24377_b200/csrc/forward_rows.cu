@@ -357,8 +357,11 @@ __global__ void __launch_bounds__(32 * (16 / R + 2), 1) attention_rows_kernel(co
 // waves.  With PNQ it adds what the same rows take by themselves, within 2 us (28 pairs behind 1, 5 and 20 waves: 41.8, 41.2,
 // 40.9 us for 41.6 at 48 tiles; 102.2, 101.7, 102.4 for 100.4 at 128), with the direct row sum up to 12 us more (5 waves of
 // 128 tiles: 116.3 for 104.7; 46 us more in one series of ten, 20 waves of 48 tiles), as CTAs drift apart.  The estimate charges
-// 4000 cycles, and a tenth of a wave above 48 tiles, so that a close call keeps to one launch.  (forward_walk.cu asks again
-// where it takes the whole waves.)
+// 4000 cycles, and a tenth of a wave above 48 tiles (kDriftTiles), so that a close call keeps to one launch.
+// Where forward_walk.cu takes the whole waves its rule starts from this division: R, which does not depend on what the whole
+// waves cost, is taken over, and whether there are small CTAs at all is estimated again with that kernel's cycles.  R = 0 for its
+// sake may hide a division that is ahead by the tenth of a wave at most.
+constexpr int kDriftTiles = 48;
 RowSplit forward_row_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq) {
   const int64_t T = (Nkv + kTile - 1) / kTile, tiles = (Nq + kTile - 1) / kTile;
   const int64_t pairs = (tiles + 1) / 2, total = bh * pairs, full = total / n_sm;
@@ -369,7 +372,7 @@ RowSplit forward_row_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bo
   for (int R = 1; R <= 4; R *= 2) {
     const int64_t c = T * (R == 4 ? 1200 : R == 2 ? 1530 : 2125) + 4500, per_head = (Nq + kTile / R - 1) / (kTile / R);
     const int64_t at = full * n_sm, done = at / pairs * per_head + (at % pairs) * 2 * R;     // groups in the full waves
-    const int64_t gap = full == 0 ? 0 : T > 48 ? 4000 + c256 / 10 : 4000;
+    const int64_t gap = full == 0 ? 0 : T > kDriftTiles ? 4000 + c256 / 10 : 4000;
     const int64_t cost = full * c256 + gap + (bh * per_head - done + n_sm - 1) / n_sm * c;
     if (cost < best_cost) { best_cost = cost; best = RowSplit{at, R}; }
   }

@@ -534,8 +534,8 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
 //   four waves above 256 tiles; one wave (37 x 1000) at 2, 12, 48, 100, 256, 400 tiles: 13.8 / 12.9, 34.8 / 32.1, 115.4 / 111.0,
 //   215.3 / 209.9, 506.8 / 506.4, 774.7 / 780.0; two (37 x 2048), 1016: 3369 / 3412; four (37 x 4096), 256, 469: 1658 / 1646,
 //   2961 / 2970.
-// - Launches that run beside others (`followed`) keep to short sequences: CTAs that walk hold their SMs to the end
-//   (24 x 8192 from host tensors: 3225 us for 3246).
+// - Launches that run beside others (`followed`) keep to short sequences: CTAs with fixed shares hold their SMs to the end
+//   (24 x 8192 from host tensors: 3225 us for 3246), and taken items have not been measured there.
 // - A CTA counts its tiles in 32 bits (the last few are left for the teams' steps beyond the end).  Where it takes items from
 //   others it may get them all: one head of 6 million queries and keys has more.
 // - Small CTAs for the last wave cost a launch and 1200 to 2125 cycles per tile and CTA, a round of single tiles T x 1390
@@ -544,7 +544,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
 //   51 x 700 x 300 18.2 / 21.2.
 WalkSplit forward_walk_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq, bool followed, const RowSplit& split) {
   const int64_t T = (Nkv + kTile - 1) / kTile, tiles = (Nq + kTile - 1) / kTile, pairs = (tiles + 1) / 2;
-  if ((pnq && T > 256) || (followed && T > 48)) return WalkSplit{false, 0};
+  if ((pnq && T > 256) || (followed && T > kStaticTiles)) return WalkSplit{false, 0};
   if ((T > kStaticTiles ? bh * tiles : (bh * tiles + n_sm - 1) / n_sm) * T > 0x7FFFFF00) return WalkSplit{false, 0};
   if (split.R == 0) {
     const int64_t rounds = (bh * tiles + n_sm - 1) / n_sm, waves = (bh * pairs + n_sm - 1) / n_sm;

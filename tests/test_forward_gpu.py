@@ -59,9 +59,9 @@ def test_ragged_shapes(nq, nkv):
     check(run_forward(cfg, q, k, v, True, True), oracle_out(cfg, q, k, v, True, True))
 
 
-# More work items (head x pair of query tiles) than the device has SMs and a short key/value sequence: the launch
-# uses the variant of the kernel in which one CTA per SM walks several items.  600 items give every CTA four or five
-# of them, so the double-buffered Q tiles and every barrier parity wrap at least once.
+# More query tiles than the device has SMs and a short key/value sequence: the launch uses the kernel in which one CTA per SM
+# walks several items of one query tile.  1080 items give every CTA seven or eight of them, so that the double-buffered Q
+# tiles and every barrier parity wrap.
 @pytest.mark.parametrize("nkv,uos,pnq", [(100, True, True), (300, True, True), (300, False, False), (896, True, True),
                                          (2500, True, False)])
 def test_many_short_items_per_cta(nkv, uos, pnq):
@@ -72,8 +72,8 @@ def test_many_short_items_per_cta(nkv, uos, pnq):
 
 @pytest.mark.parametrize("uos,pnq", [(True, True), (True, False)])
 def test_item_walking_variant_is_bit_identical_to_one_item_per_cta(uos, pnq):
-    """The same head replicated 640 times (walked, several items per CTA) against a single copy of it (5 items on 5
-    CTAs): the arithmetic of a work item does not depend on which variant ran it."""
+    """The same head replicated 640 times (walked, many items per CTA) against a single copy of it (35 groups of 32 rows
+    on as many CTAs): the arithmetic of a row does not depend on which kernel ran it."""
     one = si.custom_config("p1", 1, 1, 1100, 700, 5)
     q, k, v = si.make_all(one)
     want = run_forward(one, q, k, v, uos, pnq)
@@ -99,9 +99,9 @@ def test_bf16_output_is_rounded_fp32_output():
     assert torch.equal(o32.to(torch.bfloat16), o16)
 
 
-# The bf16 output leaves through shared-memory boxes of 32 rows and tensor copies that clip at Nq; the fp32 output is
-# stored from registers.  Ragged query counts (a box that ends, or lies entirely, beyond Nq; Nq smaller than a box),
-# several heads (a row written past Nq would land in the next head), and the item-walking variant (last case).
+# The output leaves through shared-memory boxes of 32 rows and tensor copies that clip at Nq (fp32 in two turns), from the
+# kernel for few query rows from registers.  Ragged query counts (a box that ends, or lies entirely, beyond Nq; Nq smaller than a box),
+# several heads (a row written past Nq would land in the next head), and the walking kernel (last case).
 @pytest.mark.parametrize("B,H,nq,nkv", [(1, 3, 1, 1), (1, 3, 31, 200), (1, 3, 77, 40), (1, 3, 130, 3000), (2, 2, 300, 1000),
                                         (1, 5, 257, 129), (4, 30, 1100, 300)])
 def test_bf16_output_on_ragged_shapes(B, H, nq, nkv):
@@ -287,7 +287,8 @@ def test_registered_workspace_entry_point(uos, pnq):
 @pytest.mark.parametrize("B,H,nq,nkv", [(1, 3, 300, 1000), (4, 60, 520, 700)])
 def test_cycle_profile_build_gives_the_same_output_and_fills_its_counters(B, H, nq, nkv):
     """The kernel compiled with cycle counters (a performance-analysis aid) computes exactly what the timed kernel
-    computes; its counters account for every tile.  Second case: the item-walking variant."""
+    computes; its counters account for every tile.  It is the 256-row kernel whatever the sizes; the outputs it is compared with
+    here come from the kernel for few query rows and from the walking one."""
     import paper_2607_24377_b200 as mx
     cfg = si.custom_config("prof", B, H, nq, nkv, 81)
     q, k, v = si.make_all(cfg)

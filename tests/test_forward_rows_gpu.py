@@ -1,6 +1,6 @@
 """The attention kernel for few query rows (128/R rows per CTA, R = 4, 2 or 1, replicated R times down the operand tile):
-against the oracle at its edges, and bit for bit against the 256-row kernel, which the same heads reach when many copies of
-them fill the GPU."""
+against the oracle at its edges, and bit for bit against the kernels that the same heads reach when many copies of
+them fill the GPU: the walking one (up to 256 KV tiles, with the direct row sum mostly above as well) and the 256-row one."""
 import numpy as np
 import pytest
 import torch
@@ -8,6 +8,7 @@ import torch
 import synth_inputs as si
 from oracle import attention
 from tests import util
+from tests.test_forward_walk_gpu import walk_split
 
 pytestmark = pytest.mark.gpu
 
@@ -24,7 +25,7 @@ def run(cfg, q, k, v, flags):
 
 
 def rows_per_cta(heads, nq, nkv, pnq):
-    """(pairs of query tiles in 256-row CTAs, R of the rest) on this device"""
+    """(pairs of query tiles in whole waves of 256-row CTAs, R of the rest) on this device: what the walking kernel's rule starts from"""
     return util.row_split(torch.cuda.get_device_properties(0).multi_processor_count, heads, nq, nkv, pnq)
 
 
@@ -57,9 +58,8 @@ def test_bit_identical_to_the_256_row_kernel(heads, f32):
     assert torch.equal(got, want.expand_as(got))
 
 
-# 152 to 156 pairs of query tiles: one more wave than the GPU has SMs would be nearly empty, so the 256-row kernel takes
-# whole waves only and the pairs behind them are cut into small CTAs (short and long key/value sequences; the last head's
-# tiles ragged)
+# 152 to 156 pairs of query tiles: the second wave would be nearly empty.  At 50 KV tiles whole waves are walked and the pairs
+# behind them are cut into small CTAs; at 3 and 6 the walking kernel takes them all (the last head's tiles ragged)
 @pytest.mark.parametrize("heads,nq,nkv", [(38, 1000, 700), (39, 897, 6300), (51, 700, 300)])
 @pytest.mark.parametrize("pnq", [True, False])
 def test_last_wave_cut_into_small_ctas(heads, nq, nkv, pnq):
@@ -74,8 +74,8 @@ def test_last_wave_cut_into_small_ctas(heads, nq, nkv, pnq):
     assert torch.equal(run(many, rep(q), rep(k), rep(v), flags), want.expand(1, heads, nq, 128))
 
 
-# 64 rows per CTA, alone and behind a full wave (44 and 45 heads), and 128 rows behind one (50 heads): every head must come out as
-# it does from the 256-row kernel, which 148 heads, whole waves, keep to
+# 64 rows per CTA (70 x 1100 with PNQ and from 44 heads on: the walking kernel, which estimates less time for them): every head must
+# come out as it does among 148, which are walked
 @pytest.mark.parametrize("heads,nq,nkv,split", [(49, 127, 300, (0, 2)), (70, 65, 1100, (0, 2)), (49, 128, 640, (0, 2)),
                                                 (44, 1000, 700, (148, 2)), (45, 897, 1300, (148, 2)), (50, 1000, 700, (148, 1))])
 @pytest.mark.parametrize("pnq", [True, False])
@@ -89,3 +89,33 @@ def test_64_and_128_rows_per_cta_equal_the_256_row_kernel(heads, nq, nkv, split,
     many = si.custom_config("h64m", 1, 148, nq, nkv, 8)
     rep = lambda x: np.ascontiguousarray(x[:, np.arange(148) % heads])
     assert torch.equal(run(many, rep(q), rep(k), rep(v), flags)[:, :heads], got)
+
+
+# Every way a problem is divided, by the rules of the launch itself: which kernel takes whole waves of pairs ("walk", "256" or
+# none), how many pairs, and R of the small CTAs behind them (0: none).  Each of three heads comes out as it does alone.
+@pytest.mark.parametrize("heads,nq,nkv,pnq,way", [
+    (50, 129, 31, True, ("", 0, 1)), (50, 129, 31, False, ("", 0, 1)), (120, 127, 127, True, ("", 0, 1)), (50, 129, 33000, True, ("", 0, 1)),
+    (50, 65, 31, True, ("", 0, 2)), (50, 65, 31, False, ("", 0, 2)), (50, 65, 33000, True, ("", 0, 2)),
+    (38, 897, 6200, True, ("walk", 148, 4)), (38, 897, 6200, False, ("walk", 148, 4)),
+    (50, 513, 33000, True, ("256", 148, 4)), (64, 513, 33000, True, ("256", 148, 2)), (70, 513, 33000, True, ("256", 148, 1)),
+    (50, 257, 33000, True, ("256", 100, 0)), (50, 257, 33000, False, ("256", 100, 0)), (14, 1300, 777, True, ("256", 84, 0)),
+    (14, 1300, 777, False, ("walk", 84, 0)), (50, 513, 31, True, ("walk", 150, 0)), (50, 513, 33000, False, ("walk", 150, 0))])
+def test_every_division_equals_single_heads(heads, nq, nkv, pnq, way):
+    import paper_2607_24377_b200 as mx
+    flags = mx.FLAG_UOS | (mx.FLAG_PNQ if pnq else 0)
+    n_sm, total = torch.cuda.get_device_properties(0).multi_processor_count, heads * ((-(-nq // 128) + 1) // 2)
+    pairs, r = rows_per_cta(heads, nq, nkv, pnq)
+    walked, walk_pairs = walk_split(n_sm, heads, nq, nkv, pnq)
+    if walked:
+        pairs = walk_pairs
+    if n_sm == 148:
+        assert way == ("" if pairs == 0 else "walk" if walked else "256", pairs, r if pairs < total else 0)
+    want = []
+    for h in range(3):
+        one = si.custom_config("dv", 1, 1, nq, nkv, 21 + h)
+        qkv = si.make_all(one)
+        want.append((qkv, run(one, *qkv, flags)))
+    many = si.custom_config("dvm", 1, heads, nq, nkv, 21)
+    of = np.arange(heads) % 3
+    got = run(many, *(np.concatenate([w[0][i] for w in want], axis=1)[:, of] for i in range(3)), flags)
+    assert torch.equal(got, torch.cat([w[1] for w in want], dim=1)[:, torch.from_numpy(of).cuda()])

@@ -1,5 +1,5 @@
 """The attention kernel whose CTAs walk items of one query tile (two teams of softmax warps take the KV tiles in turn): the same
-head alone, which small CTAs of another kernel compute, and copied often enough that every CTA walks several items.  The KV
+heads alone, which small CTAs of another kernel compute, and copied often enough that every CTA walks several items.  The KV
 tiles of an item are one, two, three (teams change from item to item), as many as buffers come round (4 to 9) and more; query
 and key counts end inside a tile, a half and a block."""
 import ctypes
@@ -83,11 +83,11 @@ def test_tiles_of_a_cta_are_counted_in_32_bits():
 def test_walked_items_equal_a_single_head(nq, nkv, uos, pnq, f32):
     import paper_2607_24377_b200 as mx
     flags = (mx.FLAG_UOS if uos else 0) | (mx.FLAG_PNQ if pnq else 0) | (mx.FLAG_OUT_FP32 if f32 else 0)
-    one = si.custom_config("wk", 1, 2, nq, nkv, 3 + nq)
+    one = si.custom_config("wk", 1, 3, nq, nkv, 3 + nq)
     q, k, v = si.make_all(one)
     outs = []
-    for copies in (1, 223):                                                  # 446 heads: three to fifteen items per CTA, not a whole number
-        heads = 2 * copies
+    for copies in (1, 149):                                                  # 447 heads: three to fifteen items per CTA, not a whole number
+        heads = 3 * copies
         dev = [util.to_dev_bf16(x).repeat(1, copies, 1, 1).contiguous() for x in (q, k, v)]
         out = util.guarded((1, heads, nq, 128), torch.float32 if f32 else torch.bfloat16, float("nan"))
         ws = util.guarded(mx.forward_workspace_bytes(1, heads, nq, nkv, 128), torch.uint8)
@@ -97,9 +97,10 @@ def test_walked_items_equal_a_single_head(nq, nkv, uos, pnq, f32):
         out.check(); ws.check()
         outs.append(out.t.clone())
     n_sm = torch.cuda.get_device_properties(0).multi_processor_count
-    assert walk_split(n_sm, 2, nq, nkv, pnq)[1] == 0 and walk_split(n_sm, 446, nq, nkv, pnq)[1] > 0
+    assert walk_split(n_sm, 3, nq, nkv, pnq)[1] == 0 and walk_split(n_sm, 447, nq, nkv, pnq)[1] > 0
+    assert n_sm % (3 * -(-nq // 128)) != 0                                   # a CTA's items differ from one another
     assert bool(torch.isfinite(outs[0].float()).all())
-    assert torch.equal(outs[1], outs[0].repeat(1, 223, 1, 1))
+    assert torch.equal(outs[1], outs[0].repeat(1, 149, 1, 1))
 
 
 @pytest.mark.gpu

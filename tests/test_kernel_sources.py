@@ -51,7 +51,7 @@ def test_what_a_launch_before_may_write_is_not_read_as_read_only():
 
 def test_attention_kernels_check_where_their_tensor_memory_starts():
     # they address it from column 0: were it elsewhere, a void output would have to show in the status word
-    for f in ("forward.cu", "forward_rows.cu", "forward_bf16.cu", "forward_nvfp4.cu"):
+    for f in ("forward.cu", "forward_walk.cu", "forward_rows.cu", "forward_bf16.cu", "forward_nvfp4.cu"):
         bodies = [body for _, body in kernels(f) if "tcgen05.alloc" in body]
         assert len(bodies) == 1, f
         at_end = re.search(r"check_tmem_base\(\*tmem_slot, lane, p\.status\);\s*asm volatile\(\"tcgen05\.dealloc", bodies[0])

@@ -539,9 +539,9 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
 // - A CTA counts its tiles in 32 bits (the last few are left for the teams' steps beyond the end).  Where it takes items from
 //   others it may get them all: one head of 6 million queries and keys has more.
 // - Small CTAs for the last wave cost a launch and 1200 to 2125 cycles per tile and CTA, a round of single tiles T x 1390
-//   cycles (direct 1500) + 1000.  All in one walk / last wave in small CTAs, whole call: 24 x 8192 527 / 537 (direct 588 / 597),
-//   40 x 4096 241 / 250, 38 x 8192 x 3000 330 / 336, x 1000 134.8 / 139.5 (direct 140.4 / 145.1), 38 x 1000 x 700 24.9 / 27.8,
-//   51 x 700 x 300 18.2 / 21.2.
+//   cycles (direct 1500) + 1000.  All in one walk / last wave in small CTAs, whole call: 24 x 8192 529 / 541 (direct 568 / 589),
+//   40 x 4096 241 / 261, 38 x 8192 x 3000 330 / 337, x 1000 134.8 / 139.7 (direct 140.4 / 145.3), 38 x 1000 x 700 25.0 / 27.7,
+//   51 x 700 x 300 18.3 / 21.2.
 WalkSplit forward_walk_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq, bool followed, const RowSplit& split) {
   const int64_t T = (Nkv + kTile - 1) / kTile, tiles = (Nq + kTile - 1) / kTile, pairs = (tiles + 1) / 2;
   if ((pnq && T > 256) || (followed && T > kStaticTiles)) return WalkSplit{false, 0};

@@ -585,7 +585,7 @@ __global__ void bounded_wait_selftest_kernel(int* status, long long limit_cycles
       if (tiles++ == 0) t0 = clock64();
       asm volatile("bar.sync %0, 128;" ::"r"(1 + t) : "memory");
       asm volatile("bar.arrive %0, 128;" ::"r"(2 - t) : "memory");
-    });
+    }, [](int) {});
     if (threadIdx.x == 32) {
       status[1] = *(volatile int*)&abort_flag[1];
       status[2] = (int)(clock64() - t0);

@@ -1,35 +1,50 @@
-// MXFP4 attention forward, one query tile per work item (paper Algorithm 2, lines 6-19): the kernel for short and medium
-// key/value sequences.  Value for value the arithmetic of forward.cu.
+// MXFP4 attention forward, one query tile per work item (paper Algorithm 2, lines 6-19).  Value for value the arithmetic of
+// forward.cu.
 //
 // One CTA per SM walks work items of one query tile (128 rows of one head); the tiles of all its items form one stream
 // f = 0, 1, 2, ... (KV tiles of 128 keys in ascending order within an item), and barriers, tensor memory and the pipelines
 // run on across items.  Up to 48 KV tiles (kStaticTiles) a CTA's items are fixed at the launch, every 148th.  Above, the grid has
 // a CTA per item, and a CTA that is done with an item takes over one that has not started (kTake): with fixed shares a launch
 // beside that holds a few SMs for long leaves whole shares to come last (24 x 8192 beside 4 CTAs of 8 ms: 937 us, with items
-// taken 550; direct row sum 1023 -> 589; 12 x 16384 1774 -> 1013).  Alone the two are equal within 0.3 % with PNQ, with the
-// direct sum taking is ahead (24 x 8192 587 -> 569, 24 x 30000 6892 -> 6708).  Roles (736 threads):
+// taken 550; direct row sum 1023 -> 589; 12 x 16384 1774 -> 1013).  Alone the two are equal within 1 %.  Roles (736 threads):
 //   warps 0-15   softmax, two teams of eight: team f & 1 takes tile f.  Two threads a row, one half of 64 keys each.  A team
 //                has a score buffer of its own, so that neither waits for the other to take its scores; what passes from
-//                team to team is the maxima of a tile, two floats a row, posted before the exponentials (a named barrier at
-//                which the owners of the next tile wait and the posters only arrive).
+//                team to team is the maxima of a tile, two floats a row (a named barrier at which the owners of the next tile
+//                wait and the posters only arrive).  They are posted before the exponentials, but the others are let on only
+//                behind three quarters of them: teams that take their exponentials at the same time also wait at the same time.
 //   warps 16-19  scaling: alpha, the accumulator's rescaling (Algorithm 2 line 15) and the epilogue, one warp per quarter of
 //                tensor memory.  The softmax warps never touch the accumulator and go straight on to the next item.
 //   warp 20      score products S(f) = Q K_f^T;   warp 21  output products O += P(f) [V_f | 1];   warp 22  copies
 //
-// What bounds it: the exponentials (1024 cycles per 128 x 128 tile and SM) and the latency around them.  An issuing warp
-// slows the softmax warps of its own SM sub-partition (with both products on one warp the exponentials of that quarter took
-// 850 cycles per block pair where the others took 630, and all wait for the slowest), hence two issuers and the copies on
-// three different sub-partitions: 1333 -> 1297 cycles per tile.  The scores stay in tensor memory until they are used (each
-// half is read for its maximum and once more for its exponentials), so that a thread holds 32 of them and 23 warps fit the
-// register file at 80.  Per-tile work of a warp is kept short by immediate offsets (the parity of the team's tile count is a
-// template argument): 805 -> 645 instructions per tile and sub-partition, with the two loads of scores one after the other
-// (both at once do not fit 80 registers, and the compiler then moves every score).
+// What bounds it: the exponential unit (1024 cycles per 128 x 128 tile and SM if it had to take all) and the latency around it: a
+// memory or barrier instruction queues behind the exponentials of its SM sub-partition, and every tile waits for the slowest of
+// the four.  Cycles per tile, 16 x 32768, PNQ 1315 -> 1205 (launch 4741 -> 4345 us), 24 x 8192 1443 -> 1343, 40 x 18900 x 512
+// 1641 -> 1503, x 250 2035 -> 1780; direct sum 1433 -> 1396, 1557 -> 1528, 1706 -> 1568, 2100 -> 1810.  What gave it, in these figures:
+//  - With the row sum from P-hat, which needs a probability's code and not its value, three or four pairs of exponentials in
+//    sixteen are a polynomial on the multipliers (exp2_poly): 16 x 32768 at 0, 2, 3, 4, 5 pairs 1343, 1256, 1225, 1205, 1204, 24 x
+//    8192 1467, 1386, 1357, 1343, 1361, 40 x 4096 1502, 1416, 1390, 1395, 1421, 40 x 18900 x 512 1531, 1482, 1503, 1541, 1605: the
+//    scaling warps multiply as well, in nearly every tile of a short sequence.  So three where shares are fixed, four elsewhere.
+//  - The issuing warps wait at named barriers, which neither side's memory queue delays: from the last read of a score buffer to its next
+//    product took 600 cycles with an mbarrier, 50 so.  The compiler has to leave the arrival where it is (here()).
+//  - The scaling warps load 16 columns while they multiply or convert 16 others.
+//  - What a scaling or issuing warp takes from shared memory (the next item) is made uniform by a shuffle: otherwise the compiler
+//    takes everything behind it for divergent, and each tile of the scaling warps took 200 cycles longer.
+// An issuing warp slows the softmax warps of its own SM sub-partition, hence two issuers and the copies on three different ones.
+// The scores stay in tensor memory until they are used (each half is read for its maximum and once more for its exponentials), so
+// that a thread holds 32 of them and 23 warps fit the register file at 80 (at 72 registers and 28 warps 16 x 32768 takes 5 %
+// longer, direct 12 %).  Per-tile work of a warp is kept short by immediate offsets (the parity of the team's tile count is a template argument).
+// Not kept: four more warps that take the maxima of the next tile, two or four softmax threads a row (1380, 1414), shared exponents
+// of the second block behind the first one's exponentials (no change), larger batches of exponentials in a row (1410-1470).
 //
 // Tensor memory (512 columns): scores [0,128) and [128,256), accumulator and row sum [256,400), scales behind it: Q 4 slots,
 // K 4, V 8, P 4.  Slots are as many as it takes that a copy never follows a product that still reads the slot.
 //
-// Every wait is bounded (mbar_wait_soft / role_wait); a softmax warp keeps its meetings to the end (team_tiles), so that
-// none is stranded at a named barrier, and nothing is stored once the CTA's abort flag is up.
+// Every wait at an mbarrier is bounded (mbar_wait_soft / role_wait), and none is stranded at a named barrier.  A softmax warp keeps its
+// meetings with the other team to the end (team_tiles).  An issuing warp looks at the abort flag before it waits for softmax
+// and scaling warps; if it is not up, the tile's scores have been issued, and all of them come: they go on when a wait of theirs runs
+// out, and when they leave they come once more (leave(), the epilogue).  They come to a tile no earlier than the issuing warp can
+// be there: in a healthy run the scores of tile f + 2 (f + 4) need the product that is issued behind the wait, afterwards a wait
+// that is given up takes 4 us.  Nothing is stored once the flag is up.
 #include <string.h>
 
 #include <algorithm>
@@ -63,7 +78,12 @@ constexpr int kXSlot = 128 * 2 * 4;
 constexpr int kOffXL = kOffX + 4 * kXSlot;                       // row sums of a tile by half (direct placement): 8 slots, laid out alike
 constexpr int kOffBar = kOffXL + 8 * kXSlot;
 enum Bar { BAR_Q = 0, BAR_QEMPTY = 2, BAR_KFULL = 4, BAR_ODONE = BAR_KFULL + kStages, BAR_SFULL = BAR_ODONE + kStages,
-           BAR_SFREE = BAR_SFULL + 2, BAR_PFULL = BAR_SFREE + 2, BAR_X = BAR_PFULL + 4 /* [quarter][tile & 3]: maxima posted */, BAR_NEXT = BAR_X + 16, kNumBars = BAR_NEXT + 1 };
+           BAR_X = BAR_SFULL + 2 /* [quarter][tile & 3]: maxima posted */, BAR_NEXT = BAR_X + 16, kNumBars = BAR_NEXT + 1 };
+// Named barriers: 1 + quarter + 4 team: the quarter's warps of both teams (maxima); the issuing warps wait at the others, to which
+// 9 + team: the team's warps come when they have read their score buffer, 11 + (tile & 3): the team's and the scaling warps when
+// P-hat is in place and the accumulator scaled.
+constexpr int kBarMax = 1, kBarFree = 9, kBarP = 11;
+constexpr int kFreeThreads = 32 * (kTeamWarps + 1), kPThreads = 32 * (kTeamWarps + kScaleWarps + 1);
 constexpr int kOffMisc = (kOffBar + kNumBars * 8 + 15) & ~15;    // tensor memory's start; abort flag, number of tiles, status on entry
 constexpr int kOffNext = kOffMisc + 32, kOffItems = kOffNext + 16;     // answer to the request for an item; items n & 3 (-1: there is none)
 constexpr int kSmemBytes = kOffItems + 16 + 1024;
@@ -111,6 +131,88 @@ __device__ __forceinline__ bool role_wait(uint32_t bar, uint32_t parity, volatil
   return __all_sync(0xFFFFFFFFu, mbar_test(bar, parity)) || mbar_wait_warp(bar, parity, abort_flag, status, code);
 }
 
+__device__ __forceinline__ bool given_up(uint32_t abort_addr) { return __any_sync(0xFFFFFFFFu, lds_volatile(abort_addr) != 0); }
+// What stands in front stays in front: an exit that is never taken (a count of tiles is not negative).  An arrival at a barrier
+// has no result that anything waits for, and the compiler moves it behind the exponentials that follow, 500 cycles and more.
+__device__ __forceinline__ void here(int tiles) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.s32 p, %0, -5;\n\t@p exit;\n\t}" ::"r"(tiles) : "memory");
+}
+// Whether there is no tile f: from the barrier of an item's Q tile, which is also completed when no item is left.
+static __device__ __noinline__ bool no_tile(uint32_t bar_q, uint32_t parity, uint32_t abort_addr, int f) {
+  mbar_wait_soft<36, 0, true>(bar_q, parity, abort_addr);
+  int up, all;
+  asm volatile("ld.volatile.shared.v2.s32 {%0, %1}, [%2];" : "=r"(up), "=r"(all) : "r"(abort_addr) : "memory");
+  return f >= all || up != 0;
+}
+// 2^x for values that are only rounded to E2M1 (row sum from the quantized probabilities).  The rounding changes at seven values,
+// 1/4, 3/4, 5/4, 7/4, 5/2, 7/2 and 5; the polynomial goes through 2^x there and at x = -4, and stays on the same side in between: its
+// error, up to 0.002, changes no code.  Below -4 it is less than 2^x and in the end negative (odd degree), which the conversion takes to
+// code 0, above the last point more than 5 (codes end at 6).  The coefficients' last places are chosen so that the codes are those
+// of ex2.approx for every one of the 2^32 arguments (in the rounding that the interpolation gives they differ at five).
+__device__ __forceinline__ void exp2_poly(float& a, float& b) {
+  constexpr float kExp2Poly[8] = {1.00000691f, 0.693127513f, 0.240191191f, 0.0556160808f,
+                                  0.00956740882f, 0.00130120874f, 0.000174282599f, 1.70464209e-05f};
+  uint64_t x, y;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a), "f"(b));
+  y = dup2(kExp2Poly[7]);
+#pragma unroll
+  for (int i = 6; i >= 0; --i) asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(y) : "l"(y), "l"(x), "l"(dup2(kExp2Poly[i])));
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(y));
+}
+__device__ __forceinline__ uint32_t pack_e2m1x8_relu(float x0, float x1, float x2, float x3, float x4, float x5, float x6, float x7) {
+  uint32_t out;
+  asm("{\n\t"
+      ".reg .b8 b0, b1, b2, b3;\n\t"
+      "cvt.rn.satfinite.relu.e2m1x2.f32 b0, %2, %1;\n\t"
+      "cvt.rn.satfinite.relu.e2m1x2.f32 b1, %4, %3;\n\t"
+      "cvt.rn.satfinite.relu.e2m1x2.f32 b2, %6, %5;\n\t"
+      "cvt.rn.satfinite.relu.e2m1x2.f32 b3, %8, %7;\n\t"
+      "mov.b32 %0, {b0, b1, b2, b3};\n\t"
+      "}"
+      : "=r"(out)
+      : "f"(x0), "f"(x1), "f"(x2), "f"(x3), "f"(x4), "f"(x5), "f"(x6), "f"(x7));
+  return out;
+}
+// A scaling warp's 32 rows of the accumulator times inv_l, as bf16 into its two boxes (store_half_rows' form) and out; the next 16
+// columns are loaded while the last ones are converted (40 x 18900 x 512: 124 -> 121 us for the launch).
+__device__ __forceinline__ void store_rows_bf16(uint32_t t_o, uint32_t box, int lane, float inv_l, const CUtensorMap* map, int row0, int bh, bool inside) {
+  const uint64_t il2 = dup2(inv_l);
+  const uint32_t x7 = (lane & 7) << 4;
+  uint32_t o0[16], o1[16];
+  auto put = [&](const uint32_t (&v)[16], uint32_t a0, uint32_t a1) {
+    uint32_t w[8];
+#pragma unroll
+    for (int i = 0; i < 16; i += 2) {
+      uint32_t x = v[i], y = v[i + 1];
+      mul2(x, y, il2);
+      asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w[i / 2]) : "f"(__uint_as_float(y)), "f"(__uint_as_float(x)));
+    }
+    sts128(a0, make_uint4(w[0], w[1], w[2], w[3]));
+    sts128(a1, make_uint4(w[4], w[5], w[6], w[7]));
+  };
+  TMEM_LD16(t_o, o0);
+  TMEM_LD_WAIT16(o0);
+#pragma unroll 1
+  for (int c0 = 0; c0 < 128; c0 += 32) {
+    const uint32_t a = box + (c0 >> 6) * kOutBoxBytes + lane * 128, c = (c0 & 32) << 1;      // 16-byte chunks of the row: 4 of them from byte c on
+    TMEM_LD16(t_o + c0 + 16, o1);
+    put(o0, a + (c ^ x7), a + ((c + 16) ^ x7));
+    TMEM_LD_WAIT16(o1);
+    TMEM_LD16(t_o + ((c0 + 32) & 127), o0);
+    put(o1, a + ((c + 32) ^ x7), a + ((c + 48) ^ x7));
+    if (c0 & 32) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0 && inside) {
+        asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
+                     ::"l"(map), "r"(c0 - 32), "r"(row0), "r"(bh), "r"(a) : "memory");
+        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+      }
+    }
+    TMEM_LD_WAIT16(o0);
+  }
+}
+
 template <bool kUos, bool kPnq, bool kOutF32, bool kTake>
 __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Params p, const __grid_constant__ CUtensorMap out_map) {
   extern __shared__ uint8_t smem_raw[];
@@ -134,8 +236,6 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
       mbar_init(bar(BAR_Q + i), 1); mbar_init(bar(BAR_QEMPTY + i), 1);
       mbar_init(bar(BAR_SFULL + i), 1);
     }
-    for (int i = 0; i < 4; ++i) mbar_init(bar(BAR_PFULL + i), kTeamWarps + kScaleWarps);
-    mbar_init(bar(BAR_SFREE), kTeamWarps); mbar_init(bar(BAR_SFREE + 1), kTeamWarps);
     for (int s = 0; s < kStages; ++s) { mbar_init(bar(BAR_KFULL + s), 1); mbar_init(bar(BAR_ODONE + s), 1); }
     for (int i = 0; i < 16; ++i) mbar_init(bar(BAR_X + i), 1);
     mbar_init(bar(BAR_NEXT), 1);
@@ -236,7 +336,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
       const int qb = n & 1;
       if (j == 0) {
         if (!role_wait(bar(BAR_Q + qb), (uint32_t)((n >> 1) & 1), abort_flag, p.status, 21)) break;
-        if (kTake && items[n & 3] < 0) break;
+        if (kTake && __shfl_sync(0xFFFFFFFFu, items[n & 3], 0) < 0) break;
         tc_fence_after();
         tc_cp_sf_if(leader, tmem + kColSFQ + 4 * (n & 3), sbase + kOffSFQ + qb * kTileScaleBytes);
       }
@@ -250,7 +350,8 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
         if (++sd == kStages) { sd = 0; phd ^= 1u; }
       }
       if (f >= 2) {                                              // S(f - 2) has been read
-        if (!role_wait(bar(BAR_SFREE + (f & 1)), (uint32_t)(((f >> 1) & 1) ^ 1), abort_flag, p.status, 23)) break;
+        if (given_up(abort_addr)) break;
+        asm volatile("bar.sync %0, %1;" ::"r"(kBarFree + (f & 1)), "n"(kFreeThreads) : "memory");
         tc_fence_after();
       }
       tc_mma_if(leader, d, desc(a), desc(b), make_idesc(128, 0), sfa, sfb, 0u);
@@ -272,7 +373,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
     uint32_t ph = 0;
     for (int f = 0; f < F; ++f) {
       if (kTake && j == 0) {
-        if (!role_wait(bar(BAR_Q + (n & 1)), (uint32_t)((n >> 1) & 1), abort_flag, p.status, 27) || items[n & 3] < 0) break;
+        if (!role_wait(bar(BAR_Q + (n & 1)), (uint32_t)((n >> 1) & 1), abort_flag, p.status, 27) || __shfl_sync(0xFFFFFFFFu, items[n & 3], 0) < 0) break;
         ++n;
       }
       if (!role_wait(bar(BAR_KFULL + s), ph, abort_flag, p.status, 26)) break;
@@ -280,7 +381,8 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
       const uint32_t sfa = tmem + kColSFP + 4 * (f & 3), sfb = tmem + kColSFV + 8 * (f & 7);
       const uint32_t pa = sbase + kOffP + (f & 3) * kTileCodeBytes, vb = sbase + kOffV + s * kVStageBytes;
       tc_cp_sf_if(leader, sfb, sbase + kOffSFV + s * kTileScaleBytes);
-      if (!role_wait(bar(BAR_PFULL + (f & 3)), (uint32_t)((f >> 2) & 1), abort_flag, p.status, 24)) break;
+      if (given_up(abort_addr)) break;
+      asm volatile("bar.sync %0, %1;" ::"r"(kBarP + (f & 3)), "n"(kPThreads) : "memory");
       tc_fence_after();
       tc_cp_sf_if(leader, sfa, sbase + kOffSFP + (f & 3) * kTileScaleBytes);
       tc_mma_if(leader, tmem + kColO, desc(pa), desc(vb), make_idesc(kNV, 0), sfa, sfb, j > 0 ? 1u : 0u);
@@ -307,7 +409,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
     for (int n = 0; n < n_items; ++n, item += gridDim.x) {
       if (kTake) {
         mbar_wait_soft<35, 0, true>(bar(BAR_Q + (n & 1)), (uint32_t)((n >> 1) & 1), abort_addr);
-        item = items[n & 3];                                     // anything if the CTA has given up: nothing is stored then
+        item = __shfl_sync(0xFFFFFFFFu, items[n & 3], 0);        // the same for all lanes, which the compiler has to know; anything if the CTA has given up: nothing is stored then
         if (item < 0) break;
       }
       for (int j = 0; j < T; ++j, ++f) {
@@ -325,14 +427,21 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
           const uint64_t al2 = dup2(alpha);
           uint32_t lr = 0;
           if (kPnq) asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(lr) : "r"(t_o + 128) : "memory");
+          uint32_t o0[16], o1[16];
+          TMEM_LD16(t_o, o0);
+          TMEM_LD_WAIT16(o0);
 #pragma unroll 1
-          for (int c0 = 0; c0 < 128; c0 += 32) {
-            uint32_t o[32];
-            TMEM_LD32(t_o + c0, o);
-            TMEM_LD_WAIT32(o);
+          for (int c0 = 0; c0 < 128; c0 += 32) {                 // one half is loaded while the other is multiplied
+            TMEM_LD16(t_o + c0 + 16, o1);
 #pragma unroll
-            for (int i = 0; i < 32; i += 2) mul2(o[i], o[i + 1], al2);
-            TMEM_ST32(t_o + c0, o);
+            for (int i = 0; i < 16; i += 2) mul2(o0[i], o0[i + 1], al2);
+            TMEM_ST16(t_o + c0, o0);
+            TMEM_LD_WAIT16(o1);
+            TMEM_LD16(t_o + ((c0 + 32) & 127), o0);              // (behind the last one nothing uses it)
+#pragma unroll
+            for (int i = 0; i < 16; i += 2) mul2(o1[i], o1[i + 1], al2);
+            TMEM_ST16(t_o + c0 + 16, o1);
+            TMEM_LD_WAIT16(o0);
           }
           if (kPnq) {
             asm volatile("" : "+r"(lr));
@@ -344,10 +453,12 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
         if (!kPnq) { alpha2 = alpha1; alpha1 = alpha; }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar(BAR_PFULL + (f & 3)));
+        asm volatile("bar.arrive %0, %1;" ::"r"(kBarP + (f & 3)), "n"(kPThreads) : "memory");
         if (++s_prev == kStages) { s_prev = 0; ph_prev ^= 1u; }
       }
       // ---- epilogue: O = O~ / l (line 18) ----
+      const int bh = item / p.q_tiles, row0 = (item - bh * p.q_tiles) * kTile + q * 32;
+      const bool inside = row0 < p.Nq;
       if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");      // the previous item's copies have left the boxes
       __syncwarp();
       mbar_wait_soft<33>(bar(BAR_ODONE + s_prev), ph_prev, abort_addr);
@@ -366,13 +477,17 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
         lA = lB = 0.0f;
       }
       const float inv_l = 1.0f / l;
-      const int bh = item / p.q_tiles, qtile = item - bh * p.q_tiles;
-      const int row0 = qtile * kTile + q * 32;
-      if (lds_volatile(abort_addr) != 0) break;                  // given up: nothing more is stored, and no warp waits for this one
-      const bool inside = row0 < p.Nq;
+      if (lds_volatile(abort_addr) != 0) {                       // given up: nothing more is stored, and the output products wait for this warp once more at most
+        asm volatile("bar.arrive %0, %1;" ::"r"(kBarP + (f & 3)), "n"(kPThreads) : "memory");
+        break;
+      }
+      const uint32_t box = sbase + kOffOut + 2 * q * kOutBoxBytes;
+      if constexpr (kOutF32) {
 #pragma unroll 1
-      for (int h = 0; h < 2; ++h)
-        store_half_rows<kOutF32>(t_o + 64 * h, sbase + kOffOut + (2 * q + h) * kOutBoxBytes, lane, inv_l, &out_map, 64 * h, row0, bh, inside);
+        for (int h = 0; h < 2; ++h) store_half_rows<true>(t_o + 64 * h, box + h * kOutBoxBytes, lane, inv_l, &out_map, 64 * h, row0, bh, inside);
+      } else {
+        store_rows_bf16(t_o, box, lane, inv_l, &out_map, row0, bh, inside);
+      }
     }
     if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
   } else if (role < kSoftmaxWarps) {
@@ -387,7 +502,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
     const uint32_t aP1 = sbase + kOffP + t * kTileCodeBytes + tile_code_offset(row, 2 * h + 1);
     const uint32_t aSF = sbase + kOffSFP + t * kTileScaleBytes + tile_scale_offset(row, 2 * h);
     const uint32_t barT = bar0 + 8 * t, barX = bar0 + 32 * quarter + 8 * t;
-    const int idOwn = 1 + quarter + 4 * t, idOther = 1 + quarter + 4 * (t ^ 1);
+    const int idOwn = kBarMax + quarter + 4 * t, idOther = kBarMax + quarter + 4 * (t ^ 1);
     const int ragged = (int)(p.Nkv & (kTile - 1)) != 0 ? (int)(p.Nkv & (kTile - 1)) - 64 * h : 64;     // keys of this half in an item's last tile
     const float c = p.scale_log2e;
     const uint64_t cc2 = dup2(c);
@@ -413,21 +528,29 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
       sf = __float_as_uint(ef + 12582912.0f) - (0x4B400000u - 127u);               // e + 127
       nb = dup2(-(m_new * c) - ef);
     };
-    auto exps = [&](const uint32_t (&s)[32], int g, uint64_t nb, float& sx) {      // eight exponentials, their codes
+    auto codes = [&](const uint32_t (&s)[32], int g, uint64_t nb, float& sx) {     // eight exponentials, their codes
       float x[8];
 #pragma unroll
       for (int i = 0; i < 8; i += 2) {
         fma2(s[8 * g + i], s[8 * g + i + 1], cc2, nb, x[i], x[i + 1]);
-        x[i] = ex2(x[i]);
-        x[i + 1] = ex2(x[i + 1]);
+        const bool poly = kTake ? i == ((g & 1) ? 2 : 6) : g != 0 && i == ((g & 1) ? 6 : 4);     // which pairs: 1 % between the placements tried
+        if (kPnq && poly) {
+          exp2_poly(x[i], x[i + 1]);
+        } else {
+          x[i] = ex2(x[i]);
+          x[i + 1] = ex2(x[i + 1]);
+        }
       }
-      if (!kPnq) {
+      if constexpr (kPnq) {
+        return pack_e2m1x8_relu(x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
+      } else {
         float s0, s1;
         add2x2(x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7], s0, s1);
         sx += s0 + s1;
+        return pack_e2m1x8(x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
       }
-      return pack_e2m1x8(x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
     };
+    auto meet_others = [&]() { asm volatile("bar.arrive %0, 128;" ::"r"(idOther) : "memory"); };
     auto tile = [&](auto kk) {                                   // kk: parity of the team's tile count
       constexpr int k = decltype(kk)::value;
       mbar_wait_soft<31, 8 * BAR_SFULL, true>(barT, (uint32_t)k, abort_addr);
@@ -448,7 +571,6 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
       sts32o<2 * k * kXSlot>(aM + 4 * h, fmaxf(b0, b1));
       asm volatile("bar.sync %0, 128;" ::"r"(idOwn) : "memory");
       const float2 mo = lds64o<2 * k * kXSlot>(aM), mp = lds64o<0>(k ? aMp1 : aMp0);
-      asm volatile("bar.arrive %0, 128;" ::"r"(idOther) : "memory");
       arrive_if<8 * BAR_X + 16 * k>(barX, h == 0 && lane == 0);
       const float prev = jn >= 1 ? fmaxf(mp.x, mp.y) : -INFINITY, run = jn >= 2 ? m_run : -INFINITY;
       const float m_new = max3(fmaxf(mo.x, mo.y), prev, run);    // line 10
@@ -464,16 +586,20 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
       float sx0 = 0.0f, sx1 = 0.0f;
       uint32_t w[4];
 #pragma unroll
-      for (int g = 0; g < 4; ++g) w[g] = exps(s, g, nb0, sx0);
+      for (int g = 0; g < 4; ++g) w[g] = codes(s, g, nb0, sx0);
       uint32_t s1[32];
       TMEM_LD32(t_s + 32, s1);
       sts128o<2 * k * kTileCodeBytes>(aP0, w);
       TMEM_LD_WAIT32(s1);
       tc_fence_before();
       __syncwarp();
-      arrive_if<8 * BAR_SFREE>(barT, lane == 0);                 // the score buffer may be overwritten
+      asm volatile("bar.arrive %0, %1;" ::"r"(kBarFree + t), "n"(kFreeThreads) : "memory");      // the score buffer may be overwritten
+      here(p.kv_tiles);
 #pragma unroll
-      for (int g = 0; g < 4; ++g) w[g] = exps(s1, g, nb1, sx1);
+      for (int g = 0; g < 4; ++g) {
+        w[g] = codes(s1, g, nb1, sx1);
+        if (g == 1) { meet_others(); here(p.kv_tiles); }
+      }
       sts128o<2 * k * kTileCodeBytes>(aP1, w);
       if (!kPnq) {
         sts32o<kOffXL - kOffX>(aM + 4 * h + xl, fmaf(sx1, __uint_as_float(sf1 << 23), fmaf(sx0, __uint_as_float(sf0 << 23), 0.0f)));   // Eq. 12
@@ -481,21 +607,26 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
-      arrive_if<8 * BAR_PFULL + 16 * k>(barT, lane == 0);
+      asm volatile("bar.arrive %0, %1;" ::"r"(kBarP + t + 2 * k), "n"(kPThreads) : "memory");
+    };
+    // Gives up at its tile f: the issuing warps, which look at the flag before they wait for this team, may have begun to wait
+    // for that tile, no later one; the pause lets them begin before this warp comes.
+    auto leave = [&](int f) {
+      const long long t0 = clock64();
+      while (clock64() - t0 < 40000) {}
+      asm volatile("bar.arrive %0, %1;" ::"r"(kBarFree + t), "n"(kFreeThreads) : "memory");
+      asm volatile("bar.arrive %0, %1;" ::"r"(kBarP + (f & 3)), "n"(kPThreads) : "memory");
     };
     if (!kTake) {
-      team_tiles(t, F, abort_addr, idOwn, idOther, tile);
+      team_tiles(t, F, abort_addr, idOwn, idOther, tile, leave);
     } else {
       // At the team's first tile of item n: whether there is one.  If the CTA has given up, the meetings that are kept are those of the
       // tiles that the producer says it has begun (it watches the flag too): whole items, so that no warp is beyond them.
       int f = t, n = 0, known = 0;                               // known: tiles of the items up to n
       auto ends = [&]() {
-        mbar_wait_soft<36, 0, true>(bar(BAR_Q + (n & 1)), (uint32_t)((n >> 1) & 1), abort_addr);
-        ++n;
         known += T;
-        int up, all;
-        asm volatile("ld.volatile.shared.v2.s32 {%0, %1}, [%2];" : "=r"(up), "=r"(all) : "r"(abort_addr) : "memory");
-        return f >= all || up != 0;
+        ++n;
+        return __any_sync(0xFFFFFFFFu, no_tile(bar(BAR_Q + ((n - 1) & 1)), (uint32_t)(((n - 1) >> 1) & 1), abort_addr, f));
       };
       for (;; f += 2) {
         if (f >= known && ends()) break;
@@ -504,9 +635,12 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
         if (f >= known && ends()) break;
         tile(std::integral_constant<int, 1>{});
       }
-      int all = *tiles_in_all;
-      for (int i = 0; all == 0x7FFFFFFF && i < (1 << 28); ++i) all = *tiles_in_all;
-      if (all != 0x7FFFFFFF) team_meetings(f, all, idOwn, idOther);
+      if (lds_volatile(abort_addr) != 0) {
+        leave(f);
+        int all = *tiles_in_all;
+        for (int i = 0; all == 0x7FFFFFFF && i < (1 << 28); ++i) all = *tiles_in_all;
+        if (all != 0x7FFFFFFF) team_meetings(f, all, idOwn, idOther);
+      }
     }
   }
 

@@ -235,6 +235,14 @@ __device__ __forceinline__ void check_tmem_base(uint32_t base, int lane, int* st
                  "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]),          \
                  "r"(r[30]), "r"(r[31]), "r"(taddr) : "memory")
 
+#define TMEM_LD16(taddr, r)                                                                                   \
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];" \
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), \
+                 "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]) : "r"(taddr) : "memory")
+#define TMEM_ST16(taddr, r)                                                                                   \
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15};" \
+               ::"r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), \
+                 "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(taddr) : "memory")
 #define TMEM_LD8(taddr, r)                                                                            \
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"              \
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) \
@@ -254,6 +262,10 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
                  "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]),            \
                  "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]),            \
                  "+r"(r[30]), "+r"(r[31])::"memory")
+#define TMEM_LD_WAIT16(r)                                                                                              \
+  asm volatile("tcgen05.wait::ld.sync.aligned;"                                                                        \
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),       \
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])::"memory")
 // Keys beyond the sequence do not exist: the scores of columns `valid` to `cols` - 1 (of this warp's 32 rows, at `taddr`) become
 // -inf in tensor memory, before the warp loads its scores.  Replacing them in the registers behind the load costs every tile,
 // not only the last: the values of both paths have to meet in one set of registers, which the load's own consecutive ones are
@@ -323,11 +335,14 @@ __device__ __forceinline__ void team_meetings(int f, int F, int own_bar, int oth
     asm volatile("bar.arrive %0, 128;" ::"r"(other_bar) : "memory");
   }
 }
-template <typename Tile>
-__device__ __forceinline__ void team_tiles(int t, int F, uint32_t abort_addr, int own_bar, int other_bar, Tile&& tile) {
+template <typename Tile, typename Leave>
+__device__ __forceinline__ void team_tiles(int t, int F, uint32_t abort_addr, int own_bar, int other_bar, Tile&& tile, Leave&& leave) {
   int f = t;
   for (; f < F; f += 4) {
-    if ((f & 60) == 0 && lds_volatile(abort_addr) != 0) break;
+    if ((f & 60) == 0 && lds_volatile(abort_addr) != 0) {
+      leave(f);
+      break;
+    }
     tile(std::integral_constant<int, 0>{});
     if (f + 2 >= F) return;
     tile(std::integral_constant<int, 1>{});

@@ -67,6 +67,17 @@ def test_last_wave_goes_where_it_is_estimated_to_end_first(pnq):
     assert split == 2
 
 
+def test_what_is_left_with_the_row_sum_from_quantized_probabilities():
+    import paper_2607_24377_b200 as mx
+    rule = getattr(mx.lib(), "_ZN6mxattn16forward_walk_pnqEllllRKNS_8RowSplitE")
+    rule.argtypes, rule.restype = [ctypes.c_int64] * 4 + [ctypes.c_void_p], ctypes.c_bool
+    for heads, nq, nkv, walked in ((14, 1300, 777, True), (37, 1000, 12800, True), (40, 75600, 75600, True), (2, 5000, 40000, True),
+                                   (1, 4096, 40000, False), (2, 1024, 1024, False), (1, 6_000_000, 6_000_000, False)):
+        split = (ctypes.c_int64 * 2)(*util.row_split(148, heads, nq, nkv, True))
+        assert not walk_split(148, heads, nq, nkv, True)[0] or nkv <= 256 * 128
+        assert rule(148, heads, nq, nkv, split) == walked, (heads, nq, nkv)
+
+
 def test_tiles_of_a_cta_are_counted_in_32_bits():
     # one head of n queries and keys with the direct row sum: up to 2^31 - 256 tiles per CTA
     for n, taken in ((72 << 20, False), (73_000_000, False), (64 << 20, True)):
@@ -216,3 +227,23 @@ def test_a_launch_that_holds_few_sms_does_not_hold_up_whole_shares():
         side.synchronize()                                                   # before its buffers go
         assert still                                                         # it ran all the while
     assert sorted(beside)[2] < 1.35 * sorted(alone)[2]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nq,nkv", [(130, 256 * 128 + 1), (257, 300 * 128)])
+def test_long_sequences_equal_small_ctas(nq, nkv):
+    """Above 256 KV tiles: one head alone (CTAs of 32 rows), and copied until the walking kernel's CTAs take items from one another."""
+    import paper_2607_24377_b200 as mx
+    g = torch.Generator(device="cuda"); g.manual_seed(nq)
+    q, k, v = (torch.randn(1, 1, n, 128, generator=g, device="cuda", dtype=torch.bfloat16) for n in (nq, nkv, nkv))
+    outs = []
+    for heads in (1, 76):
+        dev = [x.repeat(1, heads, 1, 1).contiguous() for x in (q, k, v)]
+        o = util.guarded((1, heads, nq, 128), torch.float32, float("nan"))
+        ws = util.guarded(mx.forward_workspace_bytes(1, heads, nq, nkv, 128), torch.uint8)
+        mx.forward_ws(*dev, o.t, 1, heads, nq, nkv, 128, 128 ** -0.5, mx.FLAG_UOS | mx.FLAG_PNQ | mx.FLAG_OUT_FP32, ws.t)
+        assert mx.device_status(ws.t) == 0
+        o.check(); ws.check()
+        outs.append(o.t.clone())
+    assert util.row_split(torch.cuda.get_device_properties(0).multi_processor_count, 1, nq, nkv, True) == (0, 4)
+    assert bool(torch.isfinite(outs[0]).all()) and torch.equal(outs[1], outs[0].expand_as(outs[1]))

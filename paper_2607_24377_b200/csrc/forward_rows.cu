@@ -17,7 +17,11 @@
 // memory at a named barrier once per tile.  S is double-buffered, so the next tile's scores are ready when a warp gets
 // there (loading them before the hand-over instead makes the hand-over's fence wait for the load: 5 % slower).  Measured
 // (B200, 1965 MHz): 1200 cycles per tile with R = 4, 1530 with R = 2, 2125 with R = 1 (one query tile of 128 rows, 16 warps);
-// 2 heads of 1024 x 1024: attention launch 14 -> 6 us.
+// 2 heads of 1024 x 1024: attention launch 14 -> 6 us.  With R = 4 a sub-partition has one softmax warp, which alone keeps the
+// exponential unit busy for half of the time: where only the codes count (PNQ) every other pair is a polynomial (exp2_poly), 1200 ->
+// 1085 cycles (1 x 4096 x 40000, whole call, none, a quarter, three eighths, half: 182.7, 172.6, 166.2, 165.0 us; 2 x 1024 10.6 -> 10.35).
+// Not kept: the accumulator loaded for its rescaling before the last exponentials (184) or before P-hat is stored (173), a test_wait in
+// front of the wait for the scores (192).
 #include <string.h>
 
 #include "common.cuh"
@@ -247,11 +251,17 @@ __global__ void __launch_bounds__(32 * (16 / R + 2), 1) attention_rows_kernel(co
 #pragma unroll
         for (int i = 0; i < 8; i += 2) {
           fma2(s[8 * g + i], s[8 * g + i + 1], cc2, nb2, x[i], x[i + 1]);
-          x[i] = ex2(x[i]);
-          x[i + 1] = ex2(x[i + 1]);
+          if (kPnq && i >= 4) {
+            exp2_poly(x[i], x[i + 1]);
+          } else {
+            x[i] = ex2(x[i]);
+            x[i + 1] = ex2(x[i + 1]);
+          }
         }
-        w[g] = pack_e2m1x8(x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
-        if (!kPnq) {
+        if constexpr (kPnq) {
+          w[g] = pack_e2m1x8_relu(x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
+        } else {
+          w[g] = pack_e2m1x8(x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
           float s0, s1;
           add2x2(x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7], s0, s1);
           sx += s0 + s1;

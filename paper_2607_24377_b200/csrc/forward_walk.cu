@@ -144,35 +144,6 @@ static __device__ __noinline__ bool no_tile(uint32_t bar_q, uint32_t parity, uin
   asm volatile("ld.volatile.shared.v2.s32 {%0, %1}, [%2];" : "=r"(up), "=r"(all) : "r"(abort_addr) : "memory");
   return f >= all || up != 0;
 }
-// 2^x for values that are only rounded to E2M1 (row sum from the quantized probabilities).  The rounding changes at seven values,
-// 1/4, 3/4, 5/4, 7/4, 5/2, 7/2 and 5; the polynomial goes through 2^x there and at x = -4, and stays on the same side in between: its
-// error, up to 0.002, changes no code.  Below -4 it is less than 2^x and in the end negative (odd degree), which the conversion takes to
-// code 0, above the last point more than 5 (codes end at 6).  The coefficients' last places are chosen so that the codes are those
-// of ex2.approx for every one of the 2^32 arguments (in the rounding that the interpolation gives they differ at five).
-__device__ __forceinline__ void exp2_poly(float& a, float& b) {
-  constexpr float kExp2Poly[8] = {1.00000691f, 0.693127513f, 0.240191191f, 0.0556160808f,
-                                  0.00956740882f, 0.00130120874f, 0.000174282599f, 1.70464209e-05f};
-  uint64_t x, y;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a), "f"(b));
-  y = dup2(kExp2Poly[7]);
-#pragma unroll
-  for (int i = 6; i >= 0; --i) asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(y) : "l"(y), "l"(x), "l"(dup2(kExp2Poly[i])));
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(y));
-}
-__device__ __forceinline__ uint32_t pack_e2m1x8_relu(float x0, float x1, float x2, float x3, float x4, float x5, float x6, float x7) {
-  uint32_t out;
-  asm("{\n\t"
-      ".reg .b8 b0, b1, b2, b3;\n\t"
-      "cvt.rn.satfinite.relu.e2m1x2.f32 b0, %2, %1;\n\t"
-      "cvt.rn.satfinite.relu.e2m1x2.f32 b1, %4, %3;\n\t"
-      "cvt.rn.satfinite.relu.e2m1x2.f32 b2, %6, %5;\n\t"
-      "cvt.rn.satfinite.relu.e2m1x2.f32 b3, %8, %7;\n\t"
-      "mov.b32 %0, {b0, b1, b2, b3};\n\t"
-      "}"
-      : "=r"(out)
-      : "f"(x0), "f"(x1), "f"(x2), "f"(x3), "f"(x4), "f"(x5), "f"(x6), "f"(x7));
-  return out;
-}
 // A scaling warp's 32 rows of the accumulator times inv_l, as bf16 into its two boxes (store_half_rows' form) and out; the next 16
 // columns are loaded while the last ones are converted (40 x 18900 x 512: 124 -> 121 us for the launch).
 __device__ __forceinline__ void store_rows_bf16(uint32_t t_o, uint32_t box, int lane, float inv_l, const CUtensorMap* map, int row0, int bh, bool inside) {

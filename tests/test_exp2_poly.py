@@ -1,4 +1,4 @@
-"""The polynomial that replaces some of the walking kernel's exponentials where only the E2M1 code of the value counts: its coefficients,
+"""The polynomial that replaces some of the attention kernels' exponentials where only the E2M1 code of the value counts: its coefficients,
 evaluated as the kernel does (fp32 fused multiply-adds), round to the code of the exact 2^x at every argument that ex2.approx itself
 is sure of (2^x at least its error, 2^-22, away from where the code changes)."""
 import os
@@ -9,7 +9,7 @@ import pytest
 
 from oracle import mxfp4
 
-SRC = os.path.join(os.path.dirname(__file__), "..", "paper_2607_24377_b200", "csrc", "forward_walk.cu")
+SRC = os.path.join(os.path.dirname(__file__), "..", "paper_2607_24377_b200", "csrc", "tc_helpers.cuh")
 EDGES = (0.25, 0.75, 1.25, 1.75, 2.5, 3.5, 5.0)
 
 

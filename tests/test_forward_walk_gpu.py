@@ -247,3 +247,27 @@ def test_long_sequences_equal_small_ctas(nq, nkv):
         outs.append(o.t.clone())
     assert util.row_split(torch.cuda.get_device_properties(0).multi_processor_count, 1, nq, nkv, True) == (0, 4)
     assert bool(torch.isfinite(outs[0]).all()) and torch.equal(outs[1], outs[0].expand_as(outs[1]))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nq,nkv", [(1, 1), (129, 128), (300, 200), (128, 257), (257, 384), (100, 511), (640, 700), (200, 1152), (130, 48 * 128 + 3)])
+@pytest.mark.parametrize("pnq,f32", [(True, False), (False, True), (True, True), (False, False)])
+def test_walked_nvfp4_items_equal_single_heads(nq, nkv, pnq, f32):
+    """NVFP4: heads of different tensor scales alone (one item per CTA), and copied until every CTA walks items of several heads."""
+    import paper_2607_24377_b200 as mx
+    one = si.custom_config("wn", 1, 3, nq, nkv, 5 + nq)
+    q, k, v = (util.to_dev_bf16(x) * torch.tensor([1.0, 0.125, 6.0], device="cuda").view(1, 3, 1, 1).bfloat16() for x in si.make_all(one))
+    flags = (mx.FLAG_PNQ if pnq else 0) | (mx.FLAG_OUT_FP32 if f32 else 0)
+    outs = []
+    for copies in (1, 149):
+        heads = 3 * copies
+        dev = [x.repeat(1, copies, 1, 1).contiguous() for x in (q, k, v)]
+        o = util.guarded((1, heads, nq, 128), torch.float32 if f32 else torch.bfloat16, float("nan"))
+        ws = util.guarded(mx.forward_nvfp4_workspace_bytes(1, heads, nq, nkv, 128), torch.uint8)
+        for _ in range(2):
+            mx.forward_nvfp4(*dev, o.t, 1, heads, nq, nkv, 128, one.softmax_scale, flags, ws.t)
+        assert mx.device_status(ws.t) == 0
+        o.check(); ws.check()
+        outs.append(o.t.clone())
+    assert bool(torch.isfinite(outs[0].float()).all())
+    assert torch.equal(outs[1], outs[0].repeat(1, 149, 1, 1))

@@ -195,7 +195,7 @@ RowSplit forward_row_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bo
 constexpr int kStaticTiles = 48;                    // KV tiles up to which a CTA of forward_walk.cu has its items from the start
 struct WalkSplit { bool walk; int64_t pairs; };     // whether forward_walk.cu takes the first `pairs` pairs (the rest: small CTAs)
 WalkSplit forward_walk_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq, bool followed, const RowSplit& split);     // `followed`: other attention launches run beside
-bool forward_walk_pnq(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, const RowSplit& split);     // ... and the rest with the row sum from P-hat
+bool forward_walk_rest(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq, bool followed, const RowSplit& split);     // ... and whether it takes all of what that leaves out
 int launch_forward_rows(int R, int64_t first_pair, const void* q_codes, const void* q_scales, const void* k_codes, const void* k_scales,
                         const void* v_codes, const void* v_scales, void* o, int B, int H, int64_t Nq, int64_t Nkv,
                         float softmax_scale, unsigned flags, int* status, cudaStream_t stream);

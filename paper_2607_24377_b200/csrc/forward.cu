@@ -700,7 +700,7 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
   const RowSplit split = dump || followed ? RowSplit{grid, 0} : forward_row_split(n_sm, (int64_t)B * H, Nq, Nkv, pnq);
   if (!dump) {
     WalkSplit walk = forward_walk_split(n_sm, (int64_t)B * H, Nq, Nkv, pnq, followed, split);
-    if (!walk.walk && pnq && !followed && forward_walk_pnq(n_sm, (int64_t)B * H, Nq, Nkv, split)) walk = WalkSplit{true, grid};
+    if (!walk.walk && forward_walk_rest(n_sm, (int64_t)B * H, Nq, Nkv, pnq, followed, split)) walk = WalkSplit{true, grid};
     if (walk.walk) {
       if (walk.pairs > 0) {
         const int rc = launch_forward_walk(n_sm, walk.pairs, q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, o, B, H, Nq, Nkv, softmax_scale, flags, status, stream);

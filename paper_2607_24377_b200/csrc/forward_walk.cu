@@ -45,14 +45,14 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
 // 12 x 75600, 591: 18376 / 18456.  With the direct row sum, 1, 4, 32, 48 tiles: 58.2 / 46.0, 136.7 / 112.3, 262 / 228,
 // 711 / 668, and whole calls: 37 x 4096, 100: 695 / 672; 16 x 32768, 256: 5402 / 5293; 12 x 40000, 400: 7647 / 7554; 12 x 75600,
 // 591: 20726 / 20574; 24 x 16384, 591: 9405 / 9109.  (These figures, and those below, are of both kernels before the polynomial; what
-// it changed for PNQ stands at forward_walk_pnq, which has the last word there.)
+// it changed for PNQ stands at forward_walk_rest, which has the last word there.)
 // - A few whole waves of pairs that single tiles do not round better.  PNQ: one wave, whole call at 2, 7, 12, 49, 100 tiles: 37 x
 //   1000 13.2 / 12.8, 22.7 / 22.5, 31.2 / 31.3, 105.4 / 106.8, 194.6 / 196.4 (14 x 1300 x 777, fp32: 20.7 / 20.5).  Direct: up to
 //   four waves above 256 tiles; one wave (37 x 1000) at 2, 12, 48, 100, 256, 400 tiles: 13.8 / 12.9, 34.8 / 32.1, 115.4 / 111.0,
 //   215.3 / 209.9, 506.8 / 506.4, 774.7 / 780.0; two (37 x 2048), 1016: 3369 / 3412; four (37 x 4096), 256, 469: 1658 / 1646,
 //   2961 / 2970.
 // - Launches that run beside others (`followed`) keep to short sequences: CTAs with fixed shares hold their SMs to the end
-//   (24 x 8192 from host tensors: 3225 us for 3246), and taken items have not been measured there.
+//   (24 x 8192 from host tensors: 3225 us for 3246); forward_walk_rest adds the long ones.
 // - A CTA counts its tiles in 32 bits (the last few are left for the teams' steps beyond the end).  Where it takes items from
 //   others it may get them all: one head of 6 million queries and keys has more.
 // - Small CTAs for the last wave cost a launch and 1200 to 2125 cycles per tile and CTA, a round of single tiles T x 1390
@@ -83,8 +83,13 @@ WalkSplit forward_walk_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, 
 // 83.0 / 78.0, 74 x 500 x 3000 70.9 / 68.9; above 256 tiles 12 x 75600 18517 / 16972, 40 x 20000 x 40000 9183 / 8298, 24 x 16384 x 75600
 // 8477 / 7565, 5 x 4000 x 40000 441 / 411, 20 x 2000 x 40000 682 / 657, 1 x 9000 x 40000 237 / 202, 2 x 5000 x 40000 334 / 206.  Small CTAs of 32
 // rows keep what they would do alone (1200 cycles per tile; 1 x 4096 x 40000 183).
-bool forward_walk_pnq(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, const RowSplit& split) {
+// Beside other launches (the stages of a forward from host tensors) above 128 tiles, with either row sum: CTAs that take items leave an
+// SM when none is left, and the next stage's come there.  us: 12 x 20000 4061 / 3908, 8 x 40000 5934 / 5588 (direct 6039 / 5817), 10 x 75600
+// 16875 / 15673, 2 x 60000 3608 / 3157.  Where the link is the bound only the last stage counts: 24 x 8192 3196 / 3210, 12 x 13000 2679 / 2686
+// (direct 2647 / 2664), 24 x 14000 5445 / 5430, and with fewer query tiles than half of T 24 x 7000 x 30000 7900 / 7930.
+bool forward_walk_rest(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq, bool followed, const RowSplit& split) {
   const int64_t T = (Nkv + kTile - 1) / kTile, tiles = (Nq + kTile - 1) / kTile;
+  if (followed ? T <= 128 || 2 * tiles < T : !pnq) return false;
   if ((T > kStaticTiles ? bh * tiles : (bh * tiles + n_sm - 1) / n_sm) * T > 0x7FFFFF00) return false;
   return !(split.R == 4 && split.pairs_256 == 0);
 }

@@ -67,15 +67,20 @@ def test_last_wave_goes_where_it_is_estimated_to_end_first(pnq):
     assert split == 2
 
 
-def test_what_is_left_with_the_row_sum_from_quantized_probabilities():
+def test_what_is_left_for_the_walking_kernel():
     import paper_2607_24377_b200 as mx
-    rule = getattr(mx.lib(), "_ZN6mxattn16forward_walk_pnqEllllRKNS_8RowSplitE")
-    rule.argtypes, rule.restype = [ctypes.c_int64] * 4 + [ctypes.c_void_p], ctypes.c_bool
+    rule = getattr(mx.lib(), "_ZN6mxattn17forward_walk_restEllllbbRKNS_8RowSplitE")
+    rule.argtypes, rule.restype = [ctypes.c_int64] * 4 + [ctypes.c_bool] * 2 + [ctypes.c_void_p], ctypes.c_bool
     for heads, nq, nkv, walked in ((14, 1300, 777, True), (37, 1000, 12800, True), (40, 75600, 75600, True), (2, 5000, 40000, True),
                                    (1, 4096, 40000, False), (2, 1024, 1024, False), (1, 6_000_000, 6_000_000, False)):
         split = (ctypes.c_int64 * 2)(*util.row_split(148, heads, nq, nkv, True))
         assert not walk_split(148, heads, nq, nkv, True)[0] or nkv <= 256 * 128
-        assert rule(148, heads, nq, nkv, split) == walked, (heads, nq, nkv)
+        assert rule(148, heads, nq, nkv, True, False, split) == walked, (heads, nq, nkv)
+        assert not rule(148, heads, nq, nkv, False, False, split)
+    none = (ctypes.c_int64 * 2)(600, 0)                                      # beside other launches there are no small CTAs
+    for pnq in (True, False):
+        assert rule(148, 3, 40000, 128 * 128 + 1, pnq, True, none) and not rule(148, 3, 40000, 128 * 128, pnq, True, none)
+        assert not rule(148, 3, 7000, 30000, pnq, True, none)
 
 
 def test_tiles_of_a_cta_are_counted_in_32_bits():

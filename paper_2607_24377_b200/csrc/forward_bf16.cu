@@ -22,6 +22,9 @@
 // descriptor word to a uniform register in front of each of them (966 -> 800 us by the converged issuer alone).
 // The output leaves as tensor copies (store_half_rows) from the query tiles' own shared memory: 69.8 -> 65.6 us at
 // H=40, 4096 x 512 (fp32 84.3 -> 71.9), 123 -> 115 at H=24, 8192 x 1024.
+// The issuer waits for the softmax groups at named barriers, which no memory queue delays (an mbarrier arrival waits behind the exponentials):
+// 24 x 2000 71.3 -> 64.1 us, 40 x 16384 4727 -> 4608, 24 x 8192 673 -> 668, 2 x 1024 15.6 -> 15.1.  It looks at the abort flag before; the
+// softmax warps come to every tile's, also when their own waits run out.
 // A last wave that would leave half of the SMs idle runs with one query tile per CTA (common.cuh): 755 -> 646 us at
 // H=24, N=8192 (5.19 waves), 25 -> 19 us at 2 heads of 1024.  (All figures in series of a few calls at full clock; under the power
 // limit the same 24 x 8192 takes 674 us in the mean of 20 calls back to back, 706 to 721 of some hundred, 787 of 2000.)
@@ -47,12 +50,12 @@ constexpr int kOffQ = 0;                                   // 2 tiles
 constexpr int kOffKV = kOffQ + 2 * kTileBytes;
 constexpr int kOffMax = kOffKV + kStages * kTileBytes;     // half-row exchange: [parity 2][tile 2][half 2][128] floats
 constexpr int kOffBar = kOffMax + 2 * 2 * 2 * 128 * 4;
-enum Bar { BAR_Q = 0, BAR_FULL = 1, BAR_EMPTY = BAR_FULL + kStages, BAR_SFULL = BAR_EMPTY + kStages, BAR_SFREE = BAR_SFULL + 2, BAR_PFULL = BAR_SFREE + 1,
-           BAR_ODONE = BAR_PFULL + 2, kNumBars = BAR_ODONE + 2 };
+enum Bar { BAR_Q = 0, BAR_FULL = 1, BAR_EMPTY = BAR_FULL + kStages, BAR_SFULL = BAR_EMPTY + kStages, BAR_ODONE = BAR_SFULL + 2, kNumBars = BAR_ODONE + 2 };
 constexpr int kOffMisc = kOffBar + kNumBars * 8;           // tmem slot, abort flag, "an earlier CTA gave up"
 constexpr int kSmemBytes = kOffMisc + 32 + 1024;           // + slack for the 1024 alignment
 static_assert(kSmemBytes <= 232448, "shared memory budget");
 
+constexpr int kBarFree = 9, kBarP = 11;                    // named barriers: group t has read its scores, P_t is in place
 constexpr uint32_t kColP = 0, kColS = 64, kColO = 256;      // P_t at 192 t (64 columns), S between them, O_t at 256 + 128 t
 
 __device__ __forceinline__ void tc_mma_ss(uint32_t leader, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
@@ -93,6 +96,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_bf16_kernel(const Param
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kOffMisc + 8);
 
   const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
+  const uint32_t abort_addr = bar0 + (kOffMisc + 8 - kOffBar);
   const TileOfCta at((int)blockIdx.x, p.pair_ctas, p.q_pairs, p.q_tiles_n);
   const int bh = at.bh, qtile0 = at.qtile;
   const bool two = at.two;                           // a second query tile: softmax group 1 has work
@@ -101,8 +105,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_bf16_kernel(const Param
   if (tid == 0) {
     mbar_init(bar(BAR_Q), 1);
     for (int s = 0; s < kStages; ++s) { mbar_init(bar(BAR_FULL + s), 1); mbar_init(bar(BAR_EMPTY + s), 1); }
-    for (int t = 0; t < 2; ++t) { mbar_init(bar(BAR_SFULL + t), 1); mbar_init(bar(BAR_PFULL + t), 8); mbar_init(bar(BAR_ODONE + t), 1); }
-    mbar_init(bar(BAR_SFREE), 8);
+    for (int t = 0; t < 2; ++t) { mbar_init(bar(BAR_SFULL + t), 1); mbar_init(bar(BAR_ODONE + t), 1); }
     abort_flag[0] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -177,53 +180,49 @@ __global__ void __launch_bounds__(kThreads, 1) attention_bf16_kernel(const Param
       tc_commit_if(leader, bar(BAR_ODONE + t));
       if (t == 1 || !two) tc_commit_if(leader, bar(BAR_EMPTY + (2 * j + 1) % kStages));
     };
-    auto wait_p = [&](int t, int j) {
-      const bool r = mbar_wait_warp(bar(BAR_PFULL + t), (uint32_t)(j & 1), abort_flag, p.status, 24 + 2 * t);
+    auto join = [&](int id) {                          // the eight warps of a softmax group
+      if (__any_sync(0xFFFFFFFFu, lds_volatile(abort_addr) != 0)) return false;
+      asm volatile("bar.sync %0, 288;" ::"r"(id) : "memory");
       tc_fence_after();
-      return r;
+      return true;
     };
+    auto wait_p = [&](int t) { return join(kBarP + t); };
     bool ok = mbar_wait_warp(bar(BAR_Q), 0, abort_flag, p.status, 21);
     // the issue order of forward.cu: G2(0,j) G1(1,j+1) G2(1,j) G1(0,j+2), which keeps the two groups half a tile apart
-    uint32_t sfree_n = 0;
-    auto wait_sfree = [&]() {
-      const bool r = mbar_wait_warp(bar(BAR_SFREE), sfree_n & 1u, abort_flag, p.status, 23);
-      ++sfree_n;
-      tc_fence_after();
-      return r;
-    };
+    auto wait_sfree = [&](int t) { return join(kBarFree + t); };      // group t has taken its scores
     ok = ok && landed(0);
     if (ok) gemm1(0, 0);
     for (int j = 0; !two && j < T && ok; ++j) {        // one query tile: its next scores go ahead of the output product
       if (j + 1 < T) {
-        ok = landed(2 * j + 2) && wait_sfree();
+        ok = landed(2 * j + 2) && wait_sfree(0);
         if (!ok) break;
         gemm1(0, j + 1);
       }
-      ok = landed(2 * j + 1) && wait_p(0, j);
+      ok = landed(2 * j + 1) && wait_p(0);
       if (ok) gemm2(0, j);
     }
     if (two) {
-      ok = ok && wait_sfree();
+      ok = ok && wait_sfree(0);
       if (ok) gemm1(1, 0);
       if (T > 1) {
-        ok = ok && landed(2) && wait_sfree();
+        ok = ok && landed(2) && wait_sfree(1);
         if (ok) gemm1(0, 1);
       }
       for (int j = 0; j < T && ok; ++j) {
-        ok = landed(2 * j + 1) && wait_p(0, j);
+        ok = landed(2 * j + 1) && wait_p(0);
         if (!ok) break;
         gemm2(0, j);
         if (j + 1 < T) {
-          ok = wait_sfree();
+          ok = wait_sfree(0);
           if (!ok) break;
           gemm1(1, j + 1);
         }
         if (j + 2 < T) ok = landed(2 * j + 4);
-        ok = ok && wait_p(1, j);
+        ok = ok && wait_p(1);
         if (!ok) break;
         gemm2(1, j);
         if (j + 2 < T) {
-          ok = wait_sfree();
+          ok = wait_sfree(1);
           if (!ok) break;
           gemm1(0, j + 2);
         }
@@ -244,7 +243,6 @@ __global__ void __launch_bounds__(kThreads, 1) attention_bf16_kernel(const Param
     float m_run = -INFINITY, l_run = 0.0f;
     const uint32_t aMaxOwn = sbase + kOffMax + (t * 256 + h * 128 + row) * 4;
     const uint32_t aMaxPartner = sbase + kOffMax + (t * 256 + (h ^ 1) * 128 + row) * 4;
-    const uint32_t abort_addr = bar0 + (kOffMisc + 8 - kOffBar);
     const int pair_bar = 1 + (warp & 3) + 4 * t;
 
     for (int j = 0; j < T; ++j) {
@@ -255,7 +253,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_bf16_kernel(const Param
       tmem_ld_wait();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar(BAR_SFREE));
+      asm volatile("bar.arrive %0, 288;" ::"r"(kBarFree + t) : "memory");
       if (j == T - 1) {
         const int valid = (int)(p.Nkv - (int64_t)j * kTile) - 64 * h;
 #pragma unroll
@@ -319,7 +317,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_bf16_kernel(const Param
       tmem_st_wait();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar(BAR_PFULL + t));
+      asm volatile("bar.arrive %0, 288;" ::"r"(kBarP + t) : "memory");
     }
 
     const uint32_t par = (uint32_t)(T & 1) * 2048u;

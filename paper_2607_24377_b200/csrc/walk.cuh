@@ -170,12 +170,12 @@ static __device__ __noinline__ bool no_tile(uint32_t bar_q, uint32_t parity, uin
   asm volatile("ld.volatile.shared.v2.s32 {%0, %1}, [%2];" : "=r"(up), "=r"(all) : "r"(abort_addr) : "memory");
   return f >= all || up != 0;
 }
-// A scaling warp's 32 rows of the accumulator times inv_l, as bf16 into its two boxes (store_half_rows' form) and out; the next 16
-// columns are loaded while the last ones are converted (40 x 18900 x 512: 124 -> 121 us for the launch).
-__device__ __forceinline__ void store_rows_bf16(uint32_t t_o, uint32_t box, int lane, float inv_l, const CUtensorMap* map, int row0, int bh, bool inside) {
+// A scaling warp's 32 rows of the accumulator times inv_l, as bf16 into its two boxes (store_half_rows' form); `o0` holds the first 16
+// columns, and the next 16 are loaded while the last ones are converted (40 x 18900 x 512: 124 -> 121 us for the launch).
+__device__ __forceinline__ void drain_rows_bf16(uint32_t t_o, uint32_t box, int lane, float inv_l, uint32_t (&o0)[16]) {
   const uint64_t il2 = dup2(inv_l);
   const uint32_t x7 = (lane & 7) << 4;
-  uint32_t o0[16], o1[16];
+  uint32_t o1[16];
   auto put = [&](const uint32_t (&v)[16], uint32_t a0, uint32_t a1) {
     uint32_t w[8];
 #pragma unroll
@@ -187,8 +187,6 @@ __device__ __forceinline__ void store_rows_bf16(uint32_t t_o, uint32_t box, int 
     sts128(a0, make_uint4(w[0], w[1], w[2], w[3]));
     sts128(a1, make_uint4(w[4], w[5], w[6], w[7]));
   };
-  TMEM_LD16(t_o, o0);
-  TMEM_LD_WAIT16(o0);
 #pragma unroll 1
   for (int c0 = 0; c0 < 128; c0 += 32) {
     const uint32_t a = box + (c0 >> 6) * kOutBoxBytes + lane * 128, c = (c0 & 32) << 1;      // 16-byte chunks of the row: 4 of them from byte c on
@@ -197,16 +195,19 @@ __device__ __forceinline__ void store_rows_bf16(uint32_t t_o, uint32_t box, int 
     TMEM_LD_WAIT16(o1);
     TMEM_LD16(t_o + ((c0 + 32) & 127), o0);
     put(o1, a + ((c + 32) ^ x7), a + ((c + 48) ^ x7));
-    if (c0 & 32) {
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      __syncwarp();
-      if (lane == 0 && inside) {
-        asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
-                     ::"l"(map), "r"(c0 - 32), "r"(row0), "r"(bh), "r"(a) : "memory");
-        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-      }
-    }
     TMEM_LD_WAIT16(o0);
+  }
+}
+// The two boxes to the output.
+__device__ __forceinline__ void copy_out(uint32_t box, int lane, const CUtensorMap* map, int row0, int bh, bool inside) {
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncwarp();
+  if (lane == 0 && inside) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
+                   ::"l"(map), "r"(64 * h), "r"(row0), "r"(bh), "r"(box + h * kOutBoxBytes) : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
   }
 }
 
@@ -454,27 +455,49 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
       lA = fmaf(alpha, lA, v.x);
       lB = fmaf(alpha, lB, v.y);
     };
+    auto ready = [&]() {                                         // tile f: the accumulator may be written
+      tc_fence_before();
+      __syncwarp();
+      asm volatile("bar.arrive %0, %1;" ::"r"(kBarP + (f & 3)), "n"(kPThreads) : "memory");
+      if (++s_prev == kStages) { s_prev = 0; ph_prev ^= 1u; }
+      ++f;
+    };
+    auto first_tile = [&](int n) {                               // of item n: nothing to rescale
+      mbar_wait_soft<34>(bar(BAR_X + q * 4 + (f & 3)), (uint32_t)((f >> 2) & 1), abort_addr);
+      if (kNv) {
+        const float2 v = lds64o<0>(sbase + L::kOffC + 8 * (n & 7));
+        c = v.x;
+        o_scale = v.y;
+      }
+      const float2 mx = lds64o<0>(aX + (f & 3) * kXSlot);
+      m_run = max3(mx.x, mx.y, -INFINITY);                       // a tile without a number leaves -inf, as in forward.cu
+      if (!kPnq) { alpha2 = alpha1; alpha1 = 1.0f; }
+      ready();
+    };
     int item = p.first_item + blockIdx.x;
-    for (int n = 0; n < n_items; ++n, item += gridDim.x) {
+    bool more = true;
+    auto next_item = [&](int n) {                                // whether there is an item n, and which
       if (kTake) {
         mbar_wait_soft<35, 0, true>(bar(BAR_Q + (n & 1)), (uint32_t)((n >> 1) & 1), abort_addr);
         item = __shfl_sync(0xFFFFFFFFu, items[n & 3], 0);        // the same for all lanes, which the compiler has to know; anything if the CTA has given up: nothing is stored then
-        if (item < 0) break;
+        more = item >= 0;
+      } else {
+        if (n > 0) item += gridDim.x;
+        more = n < n_items;
       }
-      for (int j = 0; j < T; ++j, ++f) {
+      if (more) first_tile(n);
+    };
+    next_item(0);
+    for (int n = 0; more; ++n) {
+      for (int j = 1; j < T; ++j) {
         mbar_wait_soft<34>(bar(BAR_X + q * 4 + (f & 3)), (uint32_t)((f >> 2) & 1), abort_addr);
-        if (kNv && j == 0) {
-          const float2 v = lds64o<0>(sbase + L::kOffC + 8 * (n & 7));
-          c = v.x;
-          o_scale = v.y;
-        }
         const float2 mx = lds64o<0>(aX + (f & 3) * kXSlot);
         const float m_old = m_run;
-        const float m_new = max3(mx.x, mx.y, j > 0 ? m_old : -INFINITY);     // a tile without a number leaves -inf, as in forward.cu
+        const float m_new = max3(mx.x, mx.y, m_old);
         m_run = m_new;
         if (!kPnq && j >= 2) add_sums(f - 2, alpha2);
         float alpha = 1.0f;
-        if (j > 0 && __any_sync(0xFFFFFFFFu, m_new != m_old)) {
+        if (__any_sync(0xFFFFFFFFu, m_new != m_old)) {
           alpha = ex2((m_old - m_new) * c);
           mbar_wait_soft<32>(bar(BAR_ODONE + s_prev), ph_prev, abort_addr);
           tc_fence_after();
@@ -505,10 +528,7 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
           tmem_st_wait();
         }
         if (!kPnq) { alpha2 = alpha1; alpha1 = alpha; }
-        tc_fence_before();
-        __syncwarp();
-        asm volatile("bar.arrive %0, %1;" ::"r"(kBarP + (f & 3)), "n"(kPThreads) : "memory");
-        if (++s_prev == kStages) { s_prev = 0; ph_prev ^= 1u; }
+        ready();
       }
       // ---- epilogue: O = O~ / l (line 18) ----
       const int bh = item / p.q_tiles, row0 = (item - bh * p.q_tiles) * kTile + q * 32;
@@ -518,17 +538,19 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
       mbar_wait_soft<33>(bar(BAR_ODONE + s_prev), ph_prev, abort_addr);
       tc_fence_after();
       float l;
-      if (kPnq) {
-        uint32_t lr;
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(lr) : "r"(t_o + 128) : "memory");
-        tmem_ld_wait();
-        asm volatile("" : "+r"(lr));
-        l = __uint_as_float(lr);
-      } else {
+      uint32_t lr = 0, o0[16];
+      if (kPnq) asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(lr) : "r"(t_o + 128) : "memory");
+      TMEM_LD16(t_o, o0);
+      if (!kPnq) {
         if (T >= 2) add_sums(f - 2, alpha2);
         add_sums(f - 1, alpha1);
         l = lA + lB;
         lA = lB = 0.0f;
+      }
+      TMEM_LD_WAIT16(o0);
+      if (kPnq) {
+        asm volatile("" : "+r"(lr));
+        l = __uint_as_float(lr);
       }
       const float inv_l = (kNv ? o_scale : 1.0f) / l;
       if (lds_volatile(abort_addr) != 0) {                       // given up: nothing more is stored, and the output products wait for this warp once more at most
@@ -539,8 +561,11 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
       if constexpr (kOutF32) {
 #pragma unroll 1
         for (int h = 0; h < 2; ++h) store_half_rows<true>(t_o + 64 * h, box + h * kOutBoxBytes, lane, inv_l, &out_map, 64 * h, row0, bh, inside);
+        next_item(n + 1);
       } else {
-        store_rows_bf16(t_o, box, lane, inv_l, &out_map, row0, bh, inside);
+        drain_rows_bf16(t_o, box, lane, inv_l, o0);
+        next_item(n + 1);
+        copy_out(box, lane, &out_map, row0, bh, inside);
       }
     }
     if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");

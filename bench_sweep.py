@@ -41,9 +41,9 @@ SOFTMAX_PHASES = ["wait_scores", "load_scores", "maxima", "pair_exchange", "wait
 
 
 def cycle_profile(mx, torch, cfg, dev):
-    """Per-role cycle budget of the UOS + PNQ attention kernel for long key/value sequences (mxattn_forward_cycle_profile, that
-    kernel compiled with cycle counters): mean SM cycles per key tile in each phase, per role, next to the time of a whole forward
-    call -- through the same kernel above 256 key tiles (`same_kernel`), through the one that walks single query tiles below."""
+    """Per-role cycle budget of the attention kernel for pairs of query tiles (mxattn_forward_cycle_profile, that kernel compiled
+    with cycle counters, UOS + PNQ): mean SM cycles per key tile in each phase, per role, next to the time of a whole forward call,
+    which goes through the kernel that walks single query tiles."""
     B, H, Nq, Nkv, d = cfg.B, cfg.H, cfg.Nq, cfg.Nkv, cfg.d
     q, k, v = si.make_all(cfg)
     dq, dk, dv = dev(q), dev(k), dev(v)
@@ -72,7 +72,7 @@ def cycle_profile(mx, torch, cfg, dev):
     sm = p[:, :16, :]
     per_tile = sm[:, :, :8] / np.maximum(sm[:, :, 9:10], 1)   # [cta, warp, phase]
     rep = {"workload": cfg.name, "H": H, "Nq": Nq, "Nkv": Nkv, "kv_tiles": kv_tiles, "ctas": int(p.shape[0]),
-           "ms_forward_call": ms_plain, "ms_with_counters": ms_prof, "same_kernel": kv_tiles > 256,
+           "ms_forward_call": ms_plain, "ms_with_counters": ms_prof, "same_kernel": False,
            "softmax_cycles_per_tile": {SOFTMAX_PHASES[i]: float(per_tile[:, :, i].mean()) for i in range(8)},
            "softmax_epilogue_cycles_per_item": float((sm[:, :, 8] / np.maximum(sm[:, :, 9] / kv_tiles, 1)).mean()),
            "issuer_cycles_per_tile": {"loop_total": float((p[:, 17, 8:9] / tiles).mean()),

@@ -46,9 +46,10 @@
 // swizzle) and leaves as one tensor copy per warp (fp32: two) through a tensor map of the output, so that whole
 // lines are written and the stores do not queue in front of the next tile's shared-memory traffic.
 //
-// One CTA per work item (two query tiles of one head).  launch_forward gives this kernel the long key/value sequences;
-// forward_walk.cu takes the others, and query tiles that would leave SMs idle go to the kernel for few query rows
-// (forward_rows.cu).
+// One CTA per work item (two query tiles of one head).  A launch that has the GPU to itself comes here only beyond what the
+// walking kernel counts (2^31 tiles); that kernel (forward_walk.cu) takes the others, and query tiles that would leave SMs idle go
+// to the kernel for few query rows (forward_rows.cu).  Here run the stages of a forward from host tensors that forward_walk.cu's
+// rules leave, the debug dump and the cycle profile.
 //
 // Every mbarrier wait is bounded; on expiry the CTA records a code in `status`, drains and exits.
 #include <string.h>

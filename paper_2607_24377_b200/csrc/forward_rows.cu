@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(32 * (16 / R + 2), 1) attention_rows_kernel(co
 // 40.9 us for 41.6 at 48 tiles; 102.2, 101.7, 102.4 for 100.4 at 128), with the direct row sum up to 12 us more (5 waves of
 // 128 tiles: 116.3 for 104.7; 46 us more in one series of ten, 20 waves of 48 tiles), as CTAs drift apart.  The estimate charges
 // 4000 cycles, and a tenth of a wave above 48 tiles (kDriftTiles), so that a close call keeps to one launch.
-// Where forward_walk.cu takes the whole waves its rule starts from this division: R, which does not depend on what the whole
+// Where the walking kernel takes the whole waves its rule starts from this division: R, which does not depend on what the whole
 // waves cost, is taken over, and whether there are small CTAs at all is estimated again with that kernel's cycles.  R = 0 for its
 // sake may hide a division that is ahead by the tenth of a wave at most.
 constexpr int kDriftTiles = 48;

@@ -44,8 +44,8 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
 // 40 x 4096, 32: 235 / 206; 64 x 8192, 8: 188 / 169; 40 x 8192, 48, 64: 631 / 603, 825 / 795; 16 x 32768, 256: 4736 / 4733;
 // 12 x 75600, 591: 18376 / 18456.  With the direct row sum, 1, 4, 32, 48 tiles: 58.2 / 46.0, 136.7 / 112.3, 262 / 228,
 // 711 / 668, and whole calls: 37 x 4096, 100: 695 / 672; 16 x 32768, 256: 5402 / 5293; 12 x 40000, 400: 7647 / 7554; 12 x 75600,
-// 591: 20726 / 20574; 24 x 16384, 591: 9405 / 9109.  (These figures, and those below, are of both kernels before the polynomial; what
-// it changed for PNQ stands at forward_walk_rest, which has the last word there.)
+// 591: 20726 / 20574; 24 x 16384, 591: 9405 / 9109.  (These figures, and those below, are of both kernels before the polynomial and
+// the named barriers; what these changed stands at forward_walk_rest, which has the last word.)
 // - A few whole waves of pairs that single tiles do not round better.  PNQ: one wave, whole call at 2, 7, 12, 49, 100 tiles: 37 x
 //   1000 13.2 / 12.8, 22.7 / 22.5, 31.2 / 31.3, 105.4 / 106.8, 194.6 / 196.4 (14 x 1300 x 777, fp32: 20.7 / 20.5).  Direct: up to
 //   four waves above 256 tiles; one wave (37 x 1000) at 2, 12, 48, 100, 256, 400 tiles: 13.8 / 12.9, 34.8 / 32.1, 115.4 / 111.0,
@@ -76,12 +76,14 @@ WalkSplit forward_walk_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, 
   return WalkSplit{true, all ? bh * pairs : at};
 }
 
-// With the row sum from P-hat, a launch that has the GPU to itself leaves none of the rest to the kernel of forward.cu: a single tile
-// takes 1205-1290 cycles here, a pair 2570-2700 there, so that two rounds of tiles are less than one wave of pairs.  Whole call, us,
-// that kernel (and small CTAs for its last wave) / this one: one wave of pairs, 37 x 1000 at 2, 8, 12, 49, 100, 313 KV tiles 13.2 / 12.3,
+// A launch that has the GPU to itself leaves none of the rest to the kernel of forward.cu: a single tile takes 1200-1290 cycles here
+// (direct row sum 1390-1450), a pair 2570-2700 there (3050), so that two rounds of tiles are less than one wave of pairs.  Whole call, us,
+// that kernel (and small CTAs for its last wave) / this one, PNQ: one wave of pairs, 37 x 1000 at 2, 8, 12, 49, 100, 313 KV tiles 13.2 / 12.3,
 // 24.0 / 23.0, 31.2 / 29.9, 104.8 / 101.3, 193.8 / 185.8, 561.8 / 532.7, 14 x 1300 x 777 19.6 / 18.5 (fp32 output 20.5 / 19.8), x 6200
 // 83.0 / 78.0, 74 x 500 x 3000 70.9 / 68.9; above 256 tiles 12 x 75600 18517 / 16972, 40 x 20000 x 40000 9183 / 8298, 24 x 16384 x 75600
-// 8477 / 7565, 5 x 4000 x 40000 441 / 411, 20 x 2000 x 40000 682 / 657, 1 x 9000 x 40000 237 / 202, 2 x 5000 x 40000 334 / 206.  Small CTAs of 32
+// 8477 / 7565, 5 x 4000 x 40000 441 / 411, 20 x 2000 x 40000 682 / 657, 1 x 9000 x 40000 237 / 202, 2 x 5000 x 40000 334 / 206.  Direct, one to four
+// waves of pairs above 256 tiles: 37 x 1000 x 33000 515 / 494, x 52000 795 / 765, 37 x 2048 x 130000 3411 / 3278, 37 x 4096 x 33000 1684 / 1590,
+// x 60000 2994 / 2846, 20 x 1000 x 65536 881 / 851, 18 x 4096 x 65536 1622 / 1551.  Small CTAs of 32
 // rows keep what they would do alone (1200 cycles per tile; 1 x 4096 x 40000 183).
 // Beside other launches (the stages of a forward from host tensors) above 128 tiles, with either row sum: CTAs that take items leave an
 // SM when none is left, and the next stage's come there.  us: 12 x 20000 4061 / 3908, 8 x 40000 5934 / 5588 (direct 6039 / 5817), 10 x 75600
@@ -89,7 +91,7 @@ WalkSplit forward_walk_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, 
 // (direct 2647 / 2664), 24 x 14000 5445 / 5430, and with fewer query tiles than half of T 24 x 7000 x 30000 7900 / 7930.
 bool forward_walk_rest(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq, bool followed, const RowSplit& split) {
   const int64_t T = (Nkv + kTile - 1) / kTile, tiles = (Nq + kTile - 1) / kTile;
-  if (followed ? T <= 128 || 2 * tiles < T : !pnq) return false;
+  if (followed && (T <= 128 || 2 * tiles < T)) return false;
   if ((T > kStaticTiles ? bh * tiles : (bh * tiles + n_sm - 1) / n_sm) * T > 0x7FFFFF00) return false;
   return !(split.R == 4 && split.pairs_256 == 0);
 }

@@ -269,7 +269,7 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
 // Keys beyond the sequence do not exist: the scores of columns `valid` to `cols` - 1 (of this warp's 32 rows, at `taddr`) become
 // -inf in tensor memory, before the warp loads its scores.  Replacing them in the registers behind the load costs every tile,
 // not only the last: the values of both paths have to meet in one set of registers, which the load's own consecutive ones are
-// not, and the compiler copies all of them: 1548 -> 1411 cycles per tile in an early build of forward_walk.cu (one team, no rescaling), of
+// not, and the compiler copies all of them: 1548 -> 1411 cycles per tile in an early build of walk.cuh (one team, no rescaling), of
 // which every instruction of a tile is seen.  (The kernel of forward.cu gets slower, 61.6 -> 64.1 ms at 40 x 75600, so the others mask their registers.)
 __device__ __forceinline__ void mask_scores(uint32_t taddr, int valid, int cols) {
   int i = valid < 0 ? 0 : valid;

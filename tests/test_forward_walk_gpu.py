@@ -76,7 +76,8 @@ def test_what_is_left_for_the_walking_kernel():
         split = (ctypes.c_int64 * 2)(*util.row_split(148, heads, nq, nkv, True))
         assert not walk_split(148, heads, nq, nkv, True)[0] or nkv <= 256 * 128
         assert rule(148, heads, nq, nkv, True, False, split) == walked, (heads, nq, nkv)
-        assert not rule(148, heads, nq, nkv, False, False, split)
+        direct = (ctypes.c_int64 * 2)(*util.row_split(148, heads, nq, nkv, False))
+        assert rule(148, heads, nq, nkv, False, False, direct) == walked, (heads, nq, nkv)
     none = (ctypes.c_int64 * 2)(600, 0)                                      # beside other launches there are no small CTAs
     for pnq in (True, False):
         assert rule(148, 3, 40000, 128 * 128 + 1, pnq, True, none) and not rule(148, 3, 40000, 128 * 128, pnq, True, none)

@@ -52,7 +52,7 @@
 //    about 2e-7 relative for the blocks that carry a row, d > 168, the order of ex2.approx itself, and by up to 1.5e-6 for the smallest
 //    scales, whose logarithm is a larger number; a block with d = 0 keeps r = 1, its codes are 0 either way.
 // Whole call, us, two query tiles per CTA as in forward.cu, which it was before / walking, the outputs bit for bit the same: PNQ
-// 40 x 16384 3801 / 3335, 40 x 4096 331 / 276, direct 40 x 16384 3990 / 3767, 24 x 8192 719 / 647, 24 x 2000 74 / 59, 24 x 20000 x 512 228 / 157.
+// 40 x 16384 3801 / 3293, 40 x 4096 331 / 276, direct 40 x 16384 3990 / 3710, 24 x 8192 719 / 636, 24 x 2000 74 / 59, 24 x 20000 x 512 228 / 157.
 //
 // Every wait at an mbarrier is bounded (mbar_wait_soft / role_wait), and none is stranded at a named barrier.  A softmax warp keeps its
 // meetings with the other team to the end (team_tiles).  An issuing warp looks at the abort flag before it waits for softmax
@@ -692,13 +692,20 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
       jn += 2;
       if (jn >= T) { jn -= T; if (kNv) ++n_own; }
       if (jn >= T) { jn -= T; if (kNv) ++n_own; }                // T = 1; left out where T is larger, PNQ takes 9 % longer (24 x 8192)
+      // NVFP4, the scales of the other 32 keys (two exponentials, a table): in front of the first exponentials, or in the gap where
+      // their scores are loaded.  There the score buffer is given back later, which short sequences with PNQ do not make up for.
+      // Whole call, us, in front / in the gap: direct 40 x 16384 3770 / 3710, 24 x 8192 646 / 636, 40 x 4096 299.7 / 297.7, 40 x 18900 x
+      // 512 232.2 / 230.6, PNQ 40 x 16384 3321 / 3293, 40 x 4096 275.3 / 279.5, 24 x 8192 x 2000 175.3 / 177.5.
+      constexpr bool kLate = kNv && (!kPnq || kTake);
       uint64_t nb0, nb1;
       uint32_t sf0, sf1;
       float e0[2], e1[2], r0[2], r1[2];                          // NVFP4: of the first 32 keys' two blocks, and of the others
       if constexpr (kNv) {
         sf0 = block_scales(bm0, m_new, e0, r0);
-        sf1 = block_scales(bm1, m_new, e1, r1);
-        sts32o<2 * k * L::kSF>(aSF, __uint_as_float(sf0 | (sf1 << 16)));
+        if (!kLate) {
+          sf1 = block_scales(bm1, m_new, e1, r1);
+          sts32o<2 * k * L::kSF>(aSF, __uint_as_float(sf0 | (sf1 << 16)));
+        }
       } else {
         exponent(b0, m_new, nb0, sf0);
         exponent(b1, m_new, nb1, sf1);
@@ -710,6 +717,10 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
       for (int g = 0; g < 4; ++g) w[g] = codes(s, g, kNv ? dup2(e0[g >> 1]) : nb0, sx0, kNv ? r0[g >> 1] : 1.0f);
       uint32_t s1[32];
       TMEM_LD32(t_s + 32, s1);
+      if (kLate) {
+        sf1 = block_scales(bm1, m_new, e1, r1);
+        sts32o<2 * k * L::kSF>(aSF, __uint_as_float(sf0 | (sf1 << 16)));
+      }
       sts128o<2 * k * kTileCodeBytes>(aP0, w);
       TMEM_LD_WAIT32(s1);
       tc_fence_before();

@@ -31,10 +31,10 @@ UNIT = "TFLOP/s"
 NOMINAL_FP4_TFLOPS = 9000.0      # dense FP4, nominal
 FP4_OVER_BF16 = 4.0              # nominal ratio of dense FP4 to dense bf16 tensor throughput
 QUANT_BYTES_PER_ELEM = 2.0 + 0.5 + 1.0 / 32.0
-# DRAM bytes of one attention launch, from the ncu capture of the same kernel on sweep16384
-# (259.4 MB, profiles/attention_kernel_sweep16384.txt) scaled by tokens x heads (traffic follows the
+# DRAM bytes of one attention launch, from the ncu capture of the same kernel at 40 heads of 16384
+# (260.6 MB, profiles/attention_walk_kernel.txt) scaled by tokens x heads (traffic follows the
 # operand bytes, not the flops; valid for the self-attention workloads, Nq = Nkv).
-ATTN_TRAFFIC_PER_TOKEN_HEAD = 259.4e6 / (16384 * 40)
+ATTN_TRAFFIC_PER_TOKEN_HEAD = 260.6e6 / (16384 * 40)
 
 
 def load_peaks():
@@ -465,8 +465,7 @@ def main():
         peak_note = (f"no FP4 probe in this run: {peaks['source']} sustained bf16 cuBLAS {peaks['bf16_tflops_sustained']} "
                      f"x nominal ratio 4 (of {peaks['source']})")
         per_clock = None
-    walked = Nkv <= 256 * 128              # up to 256 key tiles the launch is the kernel that walks single query tiles
-    roofline = {"bound": "mufu", "kernel": "attention_walk_kernel<uos,pnq>" if walked else "attention_kernel<uos,pnq>", "achieved": attn_tflops,
+    roofline = {"bound": "mufu", "kernel": "attention_walk_kernel<uos,pnq>", "achieved": attn_tflops,
                 "peak": fp4_peak, "unit": "TFLOP/s", "frac": attn_tflops / fp4_peak,
                 "frac_per_sm_clock": per_clock, "achieved_sm_mhz": clocks.get("sm_mhz"),
                 "traffic": ATTN_TRAFFIC_PER_TOKEN_HEAD * Nkv * B * H if Nq == Nkv else None,
@@ -476,8 +475,7 @@ def main():
                 # the softmax exponentials bind before the tensor pipe does: 16 ex2 per clock per SM,
                 # one per (query, key) pair, 512 tensor flops per pair
                 "mufu_ceiling_tflops": mufu_ceiling, "frac_of_mufu_ceiling": attn_tflops / mufu_ceiling if mufu_ceiling else None,
-                "ncu_cross_check": "profiles/attention_walk_kernel.txt (4 key tiles per item): sm__pipe_tensor_cycles_active 16.9 %, XU pipe 68 %"
-                if walked else "profiles/attention_kernel_sweep16384.txt: sm__pipe_tensor_cycles_active 21.2 %, XU pipe 83 %"}
+                "ncu_cross_check": "profiles/attention_walk_kernel.txt (128 key tiles per item): sm__pipe_tensor_cycles_active 23.9 %, XU pipe 68 %"}
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
         "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,

@@ -93,7 +93,7 @@ def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--quick", action="store_true", help="smallest sizes only")
     ap.add_argument("--cycle-profile", default=None, metavar="WORKLOAD",
-                    help="only this: per-role cycle profile of the attention kernel for long sequences on the named workload (e.g. wan22)")
+                    help="only this: per-role cycle profile of the attention kernel for pairs of query tiles on the named workload (e.g. wan22)")
     args = ap.parse_args()
     import torch
     import paper_2607_24377_b200 as mx

@@ -201,8 +201,8 @@ int mxattn_forward_debug_dump(const void* q, const void* k, const void* v, void*
                               void* dump, size_t dump_bytes, void* stream);
 
 /* Performance-analysis aid: mxattn_forward_ws (flags exactly MXATTN_FLAG_UOS | MXATTN_FLAG_PNQ, bf16 output) through
- * an instantiation of the attention kernel for long key/value sequences (more than 256 key tiles; it takes any size here,
- * although mxattn_forward_ws gives shorter ones to others) that counts, per role, the SM cycles spent in each phase of the key-tile
+ * an instantiation of the attention kernel for pairs of query tiles (it takes any size here, although mxattn_forward_ws
+ * gives its problems to other kernels, with the same results) that counts, per role, the SM cycles spent in each phase of the key-tile
  * loop of Algorithm 2 (the timed kernels are compiled without the counters; reading the cycle counter lengthens the
  * loop by 17-19 %).  `profile`: caller-owned device memory of mxattn_forward_cycle_profile_bytes() bytes,
  * zeroed by the caller, that receives [CTA][warp 0..17][16] int64.  One CTA per work item (two query tiles of one

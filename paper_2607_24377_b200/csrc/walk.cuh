@@ -19,14 +19,15 @@
 // What bounds it: the exponential unit (1024 cycles per 128 x 128 tile and SM if it had to take all) and the latency around it: a
 // memory or barrier instruction queues behind the exponentials of its SM sub-partition, and every tile waits for the slowest of
 // the four.  Cycles per tile, 16 x 32768, PNQ 1315 -> 1205 (launch 4741 -> 4345 us), 24 x 8192 1443 -> 1343, 40 x 18900 x 512
-// 1641 -> 1503, x 250 2035 -> 1780; direct sum 1433 -> 1396, 1557 -> 1528, 1706 -> 1568, 2100 -> 1810.  What gave it, in these figures:
+// 1641 -> 1440, x 250 2035 -> 1705; direct sum 1433 -> 1391, 1557 -> 1524, 1706 -> 1580, 2100 -> 1719.  What gave it, in these figures:
 //  - With the row sum from P-hat, which needs a probability's code and not its value, three or four pairs of exponentials in
 //    sixteen are a polynomial on the multipliers (exp2_poly): 16 x 32768 at 0, 2, 3, 4, 5 pairs 1343, 1256, 1225, 1205, 1204, 24 x
-//    8192 1467, 1386, 1357, 1343, 1361, 40 x 4096 1502, 1416, 1390, 1395, 1421, 40 x 18900 x 512 1531, 1482, 1503, 1541, 1605: the
+//    8192 1467, 1386, 1357, 1343, 1361, 40 x 4096 1502, 1416, 1390, 1395, 1421, 40 x 18900 x 512 at 1 to 4 1509, 1470, 1460, 1545: the
 //    scaling warps multiply as well, in nearly every tile of a short sequence.  So three where shares are fixed, four elsewhere.
 //  - The issuing warps wait at named barriers, which neither side's memory queue delays: from the last read of a score buffer to its next
 //    product took 600 cycles with an mbarrier, 50 so.  The compiler has to leave the arrival where it is (here()).
-//  - The scaling warps load 16 columns while they multiply or convert 16 others.
+//  - The scaling warps load 16 columns while they multiply or convert 16 others, and let the next item's first product go as soon as
+//    the last ones are in registers, in front of the fence and the output copies (40 x 18900 x 512 1542 -> 1474 in one series).
 //  - What a scaling or issuing warp takes from shared memory (the next item) is made uniform by a shuffle: otherwise the compiler
 //    takes everything behind it for divergent, and each tile of the scaling warps took 200 cycles longer.
 // An issuing warp slows the softmax warps of its own SM sub-partition, hence two issuers and the copies on three different ones.

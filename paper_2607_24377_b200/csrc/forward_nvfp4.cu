@@ -102,12 +102,12 @@ int launch_forward_nvfp4(const void* q, const void* k, const void* v, void* o, i
   for (int64_t first = 0; first < items; first += most) {
     p.first_item = (int)first;
     p.total_items = (int)(items - first < most ? items - first : most);
-    const bool take = takes(p, n_sm);
+    const bool take = takes<true>(p, n_sm);
     Kernel kern = nullptr;
 #define PICK(P, F) if (pnq == P && f32 == F) kern = take ? attention_nvfp4_kernel<P, F, true> : attention_nvfp4_kernel<P, F, false>;
     PICK(false, false) PICK(false, true) PICK(true, false) PICK(true, true)
 #undef PICK
-    const int rc2 = launch(kern, Lay<true>::kSmemBytes, p, n_sm, bh, o, flags, stream);
+    const int rc2 = launch(kern, Lay<true>::kSmemBytes, p, take, n_sm, bh, o, flags, stream);
     if (rc2 != MXATTN_OK) return rc2;
   }
   return MXATTN_OK;

@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
 //   51 x 700 x 300 18.3 / 21.2.
 WalkSplit forward_walk_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq, bool followed, const RowSplit& split) {
   const int64_t T = (Nkv + kTile - 1) / kTile, tiles = (Nq + kTile - 1) / kTile, pairs = (tiles + 1) / 2;
-  if ((pnq && T > 256) || (followed && T > kStaticTiles)) return WalkSplit{false, 0};
+  if ((pnq && T > 256) || (followed && T > kBesideTiles)) return WalkSplit{false, 0};
   if ((T > kStaticTiles ? bh * tiles : (bh * tiles + n_sm - 1) / n_sm) * T > 0x7FFFFF00) return WalkSplit{false, 0};
   if (split.R == 0) {
     const int64_t rounds = (bh * tiles + n_sm - 1) / n_sm, waves = (bh * pairs + n_sm - 1) / n_sm;
@@ -111,13 +111,13 @@ int launch_forward_walk(int64_t n_sm, int64_t pairs, const void* q_codes, const 
   if (items > 0x7FFFFFFF) return MXATTN_EUNSUPPORTED;
   p.total_items = (int)items;
   p.scale_log2e = softmax_scale * 1.4426950408889634f;
-  const bool uos = flags & MXATTN_FLAG_UOS, pnq = flags & MXATTN_FLAG_PNQ, f32 = flags & MXATTN_FLAG_OUT_FP32, take = takes(p, n_sm);
+  const bool uos = flags & MXATTN_FLAG_UOS, pnq = flags & MXATTN_FLAG_PNQ, f32 = flags & MXATTN_FLAG_OUT_FP32, take = takes<false>(p, n_sm);
   Kernel kern = nullptr;
 #define PICK(U, P, F) if (uos == U && pnq == P && f32 == F) kern = take ? attention_walk_kernel<U, P, F, true> : attention_walk_kernel<U, P, F, false>;
   PICK(false, false, false) PICK(false, false, true) PICK(false, true, false) PICK(false, true, true)
   PICK(true, false, false) PICK(true, false, true) PICK(true, true, false) PICK(true, true, true)
 #undef PICK
-  return launch(kern, Lay<false>::kSmemBytes, p, n_sm, (int64_t)B * H, o, flags, stream);
+  return launch(kern, Lay<false>::kSmemBytes, p, take, n_sm, (int64_t)B * H, o, flags, stream);
 }
 
 }  // namespace mxattn

@@ -3,10 +3,15 @@
 //
 // One CTA per SM walks work items of one query tile (128 rows of one head); the tiles of all its items form one stream
 // f = 0, 1, 2, ... (KV tiles of 128 keys in ascending order within an item), and barriers, tensor memory and the pipelines
-// run on across items.  Up to 48 KV tiles (kStaticTiles) a CTA's items are fixed at the launch, every 148th.  Above, the grid has
+// run on across items.  Up to 23 KV tiles (kStaticTiles; NVFP4 3) a CTA's items are fixed at the launch, every 148th.  Above, the grid has
 // a CTA per item, and a CTA that is done with an item takes over one that has not started (kTake): with fixed shares a launch
-// beside that holds a few SMs for long leaves whole shares to come last (24 x 8192 beside 4 CTAs of 8 ms: 937 us, with items
-// taken 550; direct row sum 1023 -> 589; 12 x 16384 1774 -> 1013).  Alone the two are equal within 1 %.  Roles (736 threads):
+// beside that holds a few SMs for long leaves whole shares to come last.  Whole call, us, beside 4 CTAs that stay, fixed / taken:
+// 24 x 8192 937 / 550 (direct row sum 1023 / 589), 40 x 4096 393 / 248 (432 / 270), NVFP4 40 x 4096 453 / 293 (490 / 318), 40 x 8192 x
+// 1024 272 / 178.  Alone, fixed / taken: MXFP4, attention launch, 40 x 8192 at 5, 8, 16 tiles 67.4 / 70.5, 103.1 / 106.0, 198.9 / 200.4,
+// 24 x 8192 at 24, 48 181.5 / 181.4, 351.0 / 348.7, 37 x 1000 at 24 36.5 / 36.7; NVFP4, whole call, 40 x 18900 at 1, 2, 3, 4 tiles 136.1 / 141.5,
+// 160.1 / 167.2, 190.6 / 194.4, 219.0 / 221.3, 24 x 8192 at 4, 16, 48 66.4 / 66.6, 173.4 / 169.6, 445.3 / 433.5.  (NVFP4 at up to 3
+// tiles: with a share that comes last the call still takes less than with two query tiles per CTA, 297 us at 40 x 18900 x 384.)
+// Roles (736 threads):
 //   warps 0-15   softmax, two teams of eight: team f & 1 takes tile f.  Two threads a row, one half of 64 keys each.  A team
 //                has a score buffer of its own, so that neither waits for the other to take its scores; what passes from
 //                team to team is the maxima of a tile, two floats a row (a named barrier at which the owners of the next tile
@@ -20,10 +25,11 @@
 // memory or barrier instruction queues behind the exponentials of its SM sub-partition, and every tile waits for the slowest of
 // the four.  Cycles per tile, 16 x 32768, PNQ 1315 -> 1205 (launch 4741 -> 4345 us), 24 x 8192 1443 -> 1343, 40 x 18900 x 512
 // 1641 -> 1440, x 250 2035 -> 1705; direct sum 1433 -> 1391, 1557 -> 1524, 1706 -> 1580, 2100 -> 1719.  What gave it, in these figures:
-//  - With the row sum from P-hat, which needs a probability's code and not its value, three or four pairs of exponentials in
-//    sixteen are a polynomial on the multipliers (exp2_poly): 16 x 32768 at 0, 2, 3, 4, 5 pairs 1343, 1256, 1225, 1205, 1204, 24 x
+//  - With the row sum from P-hat, which needs a probability's code and not its value, three or (MXFP4, items taken) four pairs of
+//    exponentials in sixteen are a polynomial on the multipliers (exp2_poly): 16 x 32768 at 0, 2, 3, 4, 5 pairs 1343, 1256, 1225, 1205, 1204, 24 x
 //    8192 1467, 1386, 1357, 1343, 1361, 40 x 4096 1502, 1416, 1390, 1395, 1421, 40 x 18900 x 512 at 1 to 4 1509, 1470, 1460, 1545: the
-//    scaling warps multiply as well, in nearly every tile of a short sequence.  So three where shares are fixed, four elsewhere.
+//    scaling warps multiply as well, in nearly every tile of a short sequence.  So three where shares are fixed, four elsewhere;
+//    NVFP4 three (four: 24 x 8192 x 512 66.6 -> 67.4, 24 x 8192 560 -> 563, 40 x 16384 3207 -> 3215 us for the call).
 //  - The issuing warps wait at named barriers, which neither side's memory queue delays: from the last read of a score buffer to its next
 //    product took 600 cycles with an mbarrier, 50 so.  The compiler has to leave the arrival where it is (here()).
 //  - The scaling warps load 16 columns while they multiply or convert 16 others, and let the next item's first product go as soon as
@@ -60,7 +66,7 @@
 // and scaling warps; if it is not up, the tile's scores have been issued, and all of them come: they go on when a wait of theirs runs
 // out, and when they leave they come once more (leave(), the epilogue).  They come to a tile no earlier than the issuing warp can
 // be there: in a healthy run the scores of tile f + 2 (f + 4) need the product that is issued behind the wait, afterwards a wait
-// that is given up takes 4 us.  Nothing is stored once the flag is up.
+// that is given up takes 4 us.  Nothing is stored once the flag is up.  tests/test_give_up_protocol.py has a model of all this.
 #pragma once
 #include <cuda_fp16.h>
 
@@ -77,7 +83,8 @@ constexpr int kThreads = 32 * (kProducer + 1);
 constexpr int kStages = 6;
 constexpr int kXSlot = 128 * 2 * 4;
 enum Bar { BAR_Q = 0, BAR_QEMPTY = 2, BAR_KFULL = 4, BAR_ODONE = BAR_KFULL + kStages, BAR_SFULL = BAR_ODONE + kStages,
-           BAR_X = BAR_SFULL + 2 /* [quarter][tile & 3]: maxima posted */, BAR_NEXT = BAR_X + 16, kNumBars = BAR_NEXT + 1 };
+           BAR_X = BAR_SFULL + 2 /* [quarter][tile & 3]: maxima posted */, BAR_NEXT = BAR_X + 16,
+           BAR_ITEM = BAR_NEXT + 1 /* items n & 7 are known (kTake) */, kNumBars = BAR_ITEM + 8 };
 
 template <bool kNv> struct Lay {                                  // shared memory, tensor memory
   static constexpr int kSF = (kNv ? 2 : 1) * kTileScaleBytes;     // scale bytes of an operand tile: one or two atoms
@@ -100,8 +107,8 @@ template <bool kNv> struct Lay {                                  // shared memo
   static constexpr int kOffC = kOffTab + (kNv ? 128 * 8 : 0);     // NVFP4, items n & 7: the exponent's multiplier, the output's factor
   static constexpr int kOffBar = kOffC + (kNv ? 8 * 8 : 0);
   static constexpr int kOffMisc = (kOffBar + kNumBars * 8 + 15) & ~15;    // tensor memory's start; abort flag, number of tiles, status on entry
-  static constexpr int kOffNext = kOffMisc + 32, kOffItems = kOffNext + 16;     // answer to the request for an item; items n & 3 (-1: there is none)
-  static constexpr int kSmemBytes = kOffItems + 16 + 1024;
+  static constexpr int kOffNext = kOffMisc + 32, kOffItems = kOffNext + 16;     // answer to the request for an item; items n & 7 (-1: there is none)
+  static constexpr int kSmemBytes = kOffItems + 32 + 1024;
   static_assert(kOffOut % 1024 == 0 && kSmemBytes <= 227 * 1024, "shared memory per CTA");
   // Columns of scale factors behind the accumulator, and how many an operand tile has.
   static constexpr uint32_t kSlot = kNv ? 8 : 4, kColSFQ = 400, kColSFK = 416, kColSFV = kNv ? 440 : 432, kColSFP = kNv ? 472 : 496, kColSFOnes = 504;
@@ -164,9 +171,9 @@ __device__ __forceinline__ bool given_up(uint32_t abort_addr) { return __any_syn
 __device__ __forceinline__ void here(int tiles) {
   asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.s32 p, %0, -5;\n\t@p exit;\n\t}" ::"r"(tiles) : "memory");
 }
-// Whether there is no tile f: from the barrier of an item's Q tile, which is also completed when no item is left.
-static __device__ __noinline__ bool no_tile(uint32_t bar_q, uint32_t parity, uint32_t abort_addr, int f) {
-  mbar_wait_soft<36, 0, true>(bar_q, parity, abort_addr);
+// Whether there is no tile f: from its item's barrier, which is also completed when no item is left.
+static __device__ __noinline__ bool no_tile(uint32_t bar_item, uint32_t parity, uint32_t abort_addr, int f) {
+  mbar_wait_soft<36, 0, true>(bar_item, parity, abort_addr);
   int up, all;
   asm volatile("ld.volatile.shared.v2.s32 {%0, %1}, [%2];" : "=r"(up), "=r"(all) : "r"(abort_addr) : "memory");
   return f >= all || up != 0;
@@ -268,6 +275,7 @@ __device__ __forceinline__ void set_up(uint8_t* smem, int tid) {
     for (int s = 0; s < kStages; ++s) { mbar_init(bar(BAR_KFULL + s), 1); mbar_init(bar(BAR_ODONE + s), 1); }
     for (int i = 0; i < 16; ++i) mbar_init(bar(BAR_X + i), 1);
     mbar_init(bar(BAR_NEXT), 1);
+    for (int i = 0; i < 8; ++i) mbar_init(bar(BAR_ITEM + i), 1);
     abort_flag[0] = 0;
     *tiles_in_all = 0x7FFFFFFF;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -301,7 +309,8 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
   const int T = p.kv_tiles;
 
   // Items of this CTA: every gridDim.x-th one, or (kTake) its own and then those of CTAs that have not started, one after another.
-  // The producer asks for them; the others learn of item n from the barrier of its Q tile.
+  // The producer asks for them; the others learn of item n from a barrier of its own, of which there are eight: scores are at most four
+  // tiles ahead of the last warp to look, and the producer two items ahead of the scores.
   const int n_items = kTake ? 0x7FFFFFFF : (p.total_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
   const int F = kTake ? 0x7FFFFFFF : n_items * T;                // tiles of this CTA
 
@@ -317,10 +326,12 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
         if (n >= 2) ok = mbar_wait1(bar(BAR_QEMPTY + qb), (uint32_t)(((n - 2) >> 1) & 1), abort_flag, p.status, 13);
         if (!ok) break;
         if (kTake) {
-          items[n & 3] = item;
+          items[n & 7] = item;
           if (item < 0) {
             *tiles_in_all = n * T;
             mbar_arrive(bar(BAR_Q + qb));
+            mbar_arrive(bar(BAR_ITEM + (n & 7)));
+            if (T == 1) mbar_arrive(bar(BAR_ITEM + ((n + 1) & 7)));     // where the other team looks
             break;
           }
         }
@@ -329,6 +340,7 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
           reinterpret_cast<volatile float*>(smem + L::kOffC)[2 * (n & 7)] = c;
           reinterpret_cast<volatile float*>(smem + L::kOffC)[2 * (n & 7) + 1] = kPnq ? v : v * __fdiv_rn(1.0f, kTensorRangeP);
         }
+        if (kTake) mbar_arrive(bar(BAR_ITEM + (n & 7)));
         mbar_expect_tx(bar(BAR_Q + qb), kTileCodeBytes + L::kSF);
         bulk_g2s(sbase + L::kOffQ + qb * kTileCodeBytes, p.q_codes + (int64_t)item * kTileCodeBytes, kTileCodeBytes, bar(BAR_Q + qb));
         bulk_g2s(sbase + L::kOffSFQ + qb * L::kSF, p.q_scales + (int64_t)item * L::kSF, L::kSF, bar(BAR_Q + qb));
@@ -380,7 +392,7 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
       const int qb = n & 1;
       if (j == 0) {
         if (!role_wait(bar(BAR_Q + qb), (uint32_t)((n >> 1) & 1), abort_flag, p.status, 21)) break;
-        if (kTake && __shfl_sync(0xFFFFFFFFu, items[n & 3], 0) < 0) break;
+        if (kTake && __shfl_sync(0xFFFFFFFFu, items[n & 7], 0) < 0) break;
         tc_fence_after();
         if (!kNv) tc_cp_sf_if(leader, tmem + L::kColSFQ + 4 * (n & 3), sbase + L::kOffSFQ + qb * L::kSF);
       }
@@ -419,7 +431,7 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
     uint32_t ph = 0, phd = 0;
     for (int f = 0; f < F; ++f) {
       if (kTake && j == 0) {
-        if (!role_wait(bar(BAR_Q + (n & 1)), (uint32_t)((n >> 1) & 1), abort_flag, p.status, 27) || __shfl_sync(0xFFFFFFFFu, items[n & 3], 0) < 0) break;
+        if (!role_wait(bar(BAR_ITEM + (n & 7)), (uint32_t)((n >> 3) & 1), abort_flag, p.status, 27) || __shfl_sync(0xFFFFFFFFu, items[n & 7], 0) < 0) break;
         ++n;
       }
       if (!role_wait(bar(BAR_KFULL + s), ph, abort_flag, p.status, 26)) break;
@@ -479,8 +491,8 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
     bool more = true;
     auto next_item = [&](int n) {                                // whether there is an item n, and which
       if (kTake) {
-        mbar_wait_soft<35, 0, true>(bar(BAR_Q + (n & 1)), (uint32_t)((n >> 1) & 1), abort_addr);
-        item = __shfl_sync(0xFFFFFFFFu, items[n & 3], 0);        // the same for all lanes, which the compiler has to know; anything if the CTA has given up: nothing is stored then
+        mbar_wait_soft<35, 0, true>(bar(BAR_ITEM + (n & 7)), (uint32_t)((n >> 3) & 1), abort_addr);
+        item = __shfl_sync(0xFFFFFFFFu, items[n & 7], 0);        // the same for all lanes, which the compiler has to know; anything if the CTA has given up: nothing is stored then
         more = item >= 0;
       } else {
         if (n > 0) item += gridDim.x;
@@ -633,7 +645,7 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
 #pragma unroll
       for (int i = 0; i < 8; i += 2) {
         fma2(s[8 * g + i], s[8 * g + i + 1], cc2, nb, x[i], x[i + 1]);
-        const bool poly = kTake ? i == ((g & 1) ? 2 : 6) : g != 0 && i == ((g & 1) ? 6 : 4);     // which pairs: 1 % between the placements tried
+        const bool poly = kTake && !kNv ? i == ((g & 1) ? 2 : 6) : g != 0 && i == ((g & 1) ? 6 : 4);     // which pairs: 1 % between the placements tried
         if (kPnq && poly) {
           exp2_poly(x[i], x[i + 1]);
         } else {
@@ -755,17 +767,25 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
     } else {
       // At the team's first tile of item n: whether there is one.  If the CTA has given up, the meetings that are kept are those of the
       // tiles that the producer says it has begun (it watches the flag too): whole items, so that no warp is beyond them.
+      // NVFP4 counts items anyway (n_own, jn); with counters of its own the loop spilled a register.
       int f = t, n = 0, known = 0;                               // known: tiles of the items up to n
       auto ends = [&]() {
-        known += T;
-        ++n;
-        return __any_sync(0xFFFFFFFFu, no_tile(bar(BAR_Q + ((n - 1) & 1)), (uint32_t)(((n - 1) >> 1) & 1), abort_addr, f));
+        if constexpr (kNv) {
+          if (jn >= 2) return false;
+          n = n_own + 1;
+          f = n_own * T + jn;
+        } else {
+          if (f < known) return false;
+          known += T;
+          ++n;
+        }
+        return (bool)__any_sync(0xFFFFFFFFu, no_tile(bar(BAR_ITEM + ((n - 1) & 7)), (uint32_t)(((n - 1) >> 3) & 1), abort_addr, f));
       };
       for (;; f += 2) {
-        if (f >= known && ends()) break;
+        if (ends()) break;
         tile(std::integral_constant<int, 0>{});
         f += 2;
-        if (f >= known && ends()) break;
+        if (ends()) break;
         tile(std::integral_constant<int, 1>{});
       }
       if (lds_volatile(abort_addr) != 0) {
@@ -780,13 +800,13 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
 
 // Items p.first_item .. + p.total_items - 1 of `bh` heads, by a kernel that takes them from CTAs that have not started, or has fixed shares.
 using Kernel = void (*)(const Params, const CUtensorMap);
-inline bool takes(const Params& p, int64_t n_sm) { return p.kv_tiles > kStaticTiles && p.total_items > n_sm; }
-inline int launch(Kernel kern, int smem_bytes, const Params& p, int64_t n_sm, int64_t bh, void* o, unsigned flags, cudaStream_t stream) {
+template <bool kNv> inline bool takes(const Params& p, int64_t n_sm) { return p.kv_tiles > (kNv ? kStaticTilesNv : kStaticTiles) && p.total_items > n_sm; }
+inline int launch(Kernel kern, int smem_bytes, const Params& p, bool take, int64_t n_sm, int64_t bh, void* o, unsigned flags, cudaStream_t stream) {
   CUtensorMap out_map;
   const int map_rc = encode_output_map(&out_map, o, bh, p.Nq, flags & MXATTN_FLAG_OUT_FP32);
   if (map_rc != MXATTN_OK) return map_rc;
   if (!ensure_dynamic_smem((const void*)kern, smem_bytes)) return MXATTN_ECUDA;
-  return launch_pdl(kern, dim3((unsigned)(takes(p, n_sm) || p.total_items < n_sm ? p.total_items : n_sm)), kThreads, smem_bytes, stream, p, out_map) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
+  return launch_pdl(kern, dim3((unsigned)(take || p.total_items < n_sm ? p.total_items : n_sm)), kThreads, smem_bytes, stream, p, out_map) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 
 }  // namespace walk

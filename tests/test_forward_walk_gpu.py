@@ -152,11 +152,11 @@ def test_scores_that_are_not_numbers(nq, nkv, pnq):
     assert torch.equal(torch.nan_to_num(outs[1]), torch.nan_to_num(want))
 
 
-# Above 48 KV tiles the CTAs take one item after another from the grid: several different items each (three heads, so that a CTA
+# Above 23 KV tiles the CTAs take one item after another from the grid: several different items each (three heads, so that a CTA
 # never sees one head again and again), tile counts that swap the teams' roles from item to item and ones that do not, query and
 # key counts that end inside a tile; two launches back to back, and one beside a launch that holds some of the SMs.
 @pytest.mark.gpu
-@pytest.mark.parametrize("nq,nkv", [(129, 49 * 128), (300, 49 * 128 + 1), (257, 51 * 128 - 31), (385, 64 * 128 + 77), (130, 127 * 128 + 5)])
+@pytest.mark.parametrize("nq,nkv", [(129, 24 * 128), (257, 25 * 128 - 31), (129, 49 * 128), (300, 49 * 128 + 1), (257, 51 * 128 - 31), (385, 64 * 128 + 77), (130, 127 * 128 + 5)])
 @pytest.mark.parametrize("uos,pnq,f32", [(True, True, False), (True, False, True), (False, True, True), (False, False, False)])
 def test_taken_items_equal_a_single_head(nq, nkv, uos, pnq, f32):
     import paper_2607_24377_b200 as mx
@@ -198,21 +198,23 @@ def test_taken_items_equal_a_single_head(nq, nkv, uos, pnq, f32):
 
 
 @pytest.mark.gpu
-def test_a_launch_that_holds_few_sms_does_not_hold_up_whole_shares():
+@pytest.mark.parametrize("fmt,heads,n,nkv", [("mxfp4", 24, 8192, 8192), ("mxfp4", 40, 4096, 24 * 128), ("nvfp4", 40, 4096, 4096), ("nvfp4", 40, 18900, 512)])
+def test_a_launch_that_holds_few_sms_does_not_hold_up_whole_shares(fmt, heads, n, nkv):
     """24 heads of 8192: ten and a half items per SM.  Beside 4 CTAs that run for 8 ms, the items of those 4 SMs are
-    spread over the others (about 1.1 times the time alone); with shares that are fixed at the launch they come last (1.6 times)."""
+    spread over the others (about 1.1 times the time alone); with shares that are fixed at the launch they come last (1.5 to 1.6 times)."""
     import paper_2607_24377_b200 as mx
     mk = lambda h, n: torch.randn(1, h, n, 128, device="cuda").to(torch.bfloat16)
-    q, k, v = mk(24, 8192), mk(24, 8192), mk(24, 8192)
+    q, k, v = mk(heads, n), mk(heads, nkv), mk(heads, nkv)
     lq, lk, lv = mk(1, 128), mk(1, 1 << 21), mk(1, 1 << 21)
     o, lo = torch.empty_like(q), torch.empty_like(lq)
-    ws, lws = (torch.empty(mx.forward_workspace_bytes(1, *a, 128), dtype=torch.uint8, device="cuda") for a in ((24, 8192, 8192), (1, 128, 1 << 21)))
+    call, size = (mx.forward_ws, mx.forward_workspace_bytes) if fmt == "mxfp4" else (mx.forward_nvfp4, mx.forward_nvfp4_workspace_bytes)
+    ws, lws = (torch.empty(f(1, *a, 128), dtype=torch.uint8, device="cuda") for f, a in ((size, (heads, n, nkv)), (mx.forward_workspace_bytes, (1, 128, 1 << 21))))
     side, flags = torch.cuda.Stream(), mx.FLAG_UOS | mx.FLAG_PNQ
 
     def timed():
         a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         a.record()
-        mx.forward_ws(q, k, v, o, 1, 24, 8192, 8192, 128, 128 ** -0.5, flags, ws)
+        call(q, k, v, o, 1, heads, n, nkv, 128, 128 ** -0.5, flags if fmt == "mxfp4" else mx.FLAG_PNQ, ws)
         b.record(); b.synchronize()
         return a.elapsed_time(b)
 

@@ -562,6 +562,8 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
 // short limit; the wait must give up, record its code in `status`, and the kernel must end normally.
 // Four more warps are a row quarter's two teams (team_tiles) whose first wait runs out in the same way: status[1] = its code,
 // status[2] = the cycles that their 2^17 tiles take behind it, status[3] = the tiles that one warp worked on before it noticed.
+// (No warp waits here as the issuing warps do: that none of them is left at a named barrier is shown by the model in
+// tests/test_give_up_protocol.py, not on a GPU, where such a wait has no limit.)
 __global__ void bounded_wait_selftest_kernel(int* status, long long limit_cycles) {
   __shared__ uint64_t barrier;
   __shared__ int abort_flag[2];

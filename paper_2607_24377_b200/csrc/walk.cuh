@@ -66,7 +66,7 @@
 // and scaling warps; if it is not up, the tile's scores have been issued, and all of them come: they go on when a wait of theirs runs
 // out, and when they leave they come once more (leave(), the epilogue).  They come to a tile no earlier than the issuing warp can
 // be there: in a healthy run the scores of tile f + 2 (f + 4) need the product that is issued behind the wait, afterwards a wait
-// that is given up takes 4 us.  Nothing is stored once the flag is up.  tests/test_give_up_protocol.py has a model of all this.
+// that is given up takes 4 us.  An item whose accumulator was still to be read when the flag went up is not stored.  tests/test_give_up_protocol.py has a model of all this.
 #pragma once
 #include <cuda_fp16.h>
 
@@ -566,7 +566,7 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
         l = __uint_as_float(lr);
       }
       const float inv_l = (kNv ? o_scale : 1.0f) / l;
-      if (lds_volatile(abort_addr) != 0) {                       // given up: nothing more is stored, and the output products wait for this warp once more at most
+      if (lds_volatile(abort_addr) != 0) {                       // given up: this item and later ones are not stored, and the output products wait for this warp once more at most
         asm volatile("bar.arrive %0, %1;" ::"r"(kBarP + (f & 3)), "n"(kPThreads) : "memory");
         break;
       }

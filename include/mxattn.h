@@ -367,6 +367,12 @@ int mxattn_selftest_bounded_wait(void* status, int64_t limit_cycles, void* strea
  * in status[1] -- `meetings` if no warp was left stranded.  `status`: 4 device ints, zeroed by the caller. */
 int mxattn_selftest_pair_abandon(void* status, int64_t limit_cycles, int meetings, void* stream);
 
+/* With the row sum from the quantized probabilities the attention kernels compute some exponentials as a polynomial that rounds to the
+ * same E2M1 code.  This compares the codes of both for every one of the 2^32 fp32 arguments: status[0] receives the number of
+ * arguments at which they differ, status[1] the number at which the conversion that takes what is negative to zero changes the
+ * code of the exponential itself, status[2] the bits of one such argument.  `status`: 4 device ints, zeroed by the caller. */
+int mxattn_selftest_exp2_codes(void* status, void* stream);
+
 /* Number of kernel launches the last forward call of this process enqueued (for accounting). */
 int mxattn_last_launch_count(void);
 

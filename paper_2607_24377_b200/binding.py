@@ -75,6 +75,7 @@ def lib() -> ctypes.CDLL:
         L.mxattn_device_status.argtypes = [vp, ctypes.POINTER(ctypes.c_int), vp]
         L.mxattn_selftest_bounded_wait.argtypes = [vp, i64, vp]
         L.mxattn_selftest_pair_abandon.argtypes = [vp, i64, ci, vp]
+        L.mxattn_selftest_exp2_codes.argtypes = [vp, vp]
         L.mxattn_last_launch_count.argtypes = []
         L.mxattn_strerror.argtypes = [ci]
         L.mxattn_strerror.restype = ctypes.c_char_p
@@ -267,6 +268,10 @@ def selftest_bounded_wait(status, limit_cycles: int):
 def selftest_pair_abandon(status, limit_cycles: int, meetings: int):
     _check(lib().mxattn_selftest_pair_abandon(_ptr(status), int(limit_cycles), int(meetings), _stream()),
            "mxattn_selftest_pair_abandon")
+
+
+def selftest_exp2_codes(status):
+    _check(lib().mxattn_selftest_exp2_codes(_ptr(status), _stream()), "mxattn_selftest_exp2_codes")
 
 
 def last_launch_count() -> int:

@@ -522,6 +522,12 @@ extern "C" int mxattn_selftest_pair_abandon(void* status, int64_t limit_cycles, 
   return launch_pair_abandon_selftest(static_cast<int*>(status), (long long)limit_cycles, meetings, (cudaStream_t)stream);
 }
 
+extern "C" int mxattn_selftest_exp2_codes(void* status, void* stream) {
+  if (!status) return MXATTN_EINVAL;
+  if (!aligned16(status)) return MXATTN_EALIGN;
+  return launch_exp2_codes_selftest(static_cast<int*>(status), (cudaStream_t)stream);
+}
+
 extern "C" int mxattn_last_launch_count(void) { return g_last_launches.load(std::memory_order_relaxed); }
 
 extern "C" const char* mxattn_strerror(int status) {

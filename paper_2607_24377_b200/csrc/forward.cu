@@ -628,7 +628,37 @@ __global__ void pair_abandon_selftest_kernel(int* status, long long limit_cycles
   else if (lane == 0) atomicCAS(status + 1, 0, kept);
 }
 
+// Compares the E2M1 codes of exp2_poly and of ex2.approx for every fp32 argument, eight at a time: status[0] = arguments whose codes
+// differ, status[1] = those at which ex2's own differs between the conversion with .relu and without, status[2] = one of either.
+__global__ void exp2_codes_selftest_kernel(int* status) {
+  for (uint64_t a = 8ull * (blockIdx.x * blockDim.x + threadIdx.x); a < 1ull << 32; a += 8ull * gridDim.x * blockDim.x) {
+    float e[8], y[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      y[i] = __uint_as_float((uint32_t)a + i);
+      e[i] = ex2(y[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; i += 2) exp2_poly(y[i], y[i + 1]);
+    const uint32_t want = pack_e2m1x8(e[0], e[1], e[2], e[3], e[4], e[5], e[6], e[7]);
+    const uint32_t diff[2] = {want ^ pack_e2m1x8_relu(y[0], y[1], y[2], y[3], y[4], y[5], y[6], y[7]),
+                              want ^ pack_e2m1x8_relu(e[0], e[1], e[2], e[3], e[4], e[5], e[6], e[7])};
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+      for (int i = 0; diff[k] != 0 && i < 8; ++i)
+        if ((diff[k] >> (4 * i)) & 15u) {
+          atomicAdd(status + k, 1);
+          status[2] = (int)((uint32_t)a + i);
+        }
+  }
+}
+
 }  // namespace fwd
+
+int launch_exp2_codes_selftest(int* status, cudaStream_t stream) {
+  fwd::exp2_codes_selftest_kernel<<<1184, 256, 0, stream>>>(status);
+  return cudaGetLastError() == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
+}
 
 int launch_pair_abandon_selftest(int* status, long long limit_cycles, int meetings, cudaStream_t stream) {
   fwd::pair_abandon_selftest_kernel<<<1, 64, 0, stream>>>(status, limit_cycles, meetings);

@@ -352,9 +352,9 @@ __device__ __forceinline__ void team_tiles(int t, int F, uint32_t abort_addr, in
 
 // 2^x for values that are only rounded to E2M1 (row sum from the quantized probabilities).  The rounding changes at seven values,
 // 1/4, 3/4, 5/4, 7/4, 5/2, 7/2 and 5; the polynomial goes through 2^x there and at x = -4, and stays on the same side in between: its
-// error, up to 0.002, changes no code.  Below -4 it is less than 2^x and in the end negative (odd degree), which the conversion takes to
+// error, up to 0.0065 between -4 and -2 and below 3e-4 from there to the last change, changes no code.  Below -4 it is less than 2^x and in the end negative (odd degree), which the conversion takes to
 // code 0, above the last point more than 5 (codes end at 6).  The coefficients' last places are chosen so that the codes are those
-// of ex2.approx for every one of the 2^32 arguments (in the rounding that the interpolation gives they differ at five).
+// of ex2.approx for every one of the 2^32 arguments (mxattn_selftest_exp2_codes compares them; in the rounding that the interpolation gives they differ at five).
 __device__ __forceinline__ void exp2_poly(float& a, float& b) {
   constexpr float kExp2Poly[8] = {1.00000691f, 0.693127513f, 0.240191191f, 0.0556160808f,
                                   0.00956740882f, 0.00130120874f, 0.000174282599f, 1.70464209e-05f};

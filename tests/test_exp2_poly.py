@@ -1,11 +1,12 @@
 """The polynomial that replaces some of the attention kernels' exponentials where only the E2M1 code of the value counts: its coefficients,
 evaluated as the kernel does (fp32 fused multiply-adds), round to the code of the exact 2^x at every argument that ex2.approx itself
-is sure of (2^x at least its error, 2^-22, away from where the code changes)."""
+is sure of (2^x at least its error, 2^-22, away from where the code changes).  On the GPU both are compared at every argument."""
 import os
 import re
 
 import numpy as np
 import pytest
+import torch
 
 from oracle import mxfp4
 
@@ -53,3 +54,16 @@ def test_from_minus_infinity_to_the_largest_probability():
     far = -np.logspace(0.7, 38, 2000).astype(np.float32)
     assert (code(poly(np.append(far, -np.float32(np.inf)))) == 0).all()
     assert (code(poly(np.linspace(2.33, 128.0, 20001).astype(np.float32))) == 7).all()
+
+
+def test_error_in_between_is_as_stated():
+    err = lambda lo, hi: np.abs(poly(x := np.linspace(lo, hi, 100001).astype(np.float32)).astype(np.float64) - np.exp2(x.astype(np.float64))).max()
+    assert 0.006 < err(-4.0, -2.0) <= 0.0065 and err(-2.0, np.log2(5.0)) < 3e-4
+
+
+@pytest.mark.gpu
+def test_codes_of_every_argument_are_those_of_the_exponential():
+    import paper_2607_24377_b200 as mx
+    status = torch.zeros(4, dtype=torch.int32, device="cuda")
+    mx.selftest_exp2_codes(status)
+    assert status.tolist()[:2] == [0, 0], hex(int(status[2]) & 0xFFFFFFFF)

@@ -20,6 +20,8 @@
 // 2 heads of 1024 x 1024: attention launch 14 -> 6 us.  With R = 4 a sub-partition has one softmax warp, which alone keeps the
 // exponential unit busy for half of the time: where only the codes count (PNQ) every other pair is a polynomial (exp2_poly), 1200 ->
 // 1085 cycles (1 x 4096 x 40000, whole call, none, a quarter, three eighths, half: 182.7, 172.6, 166.2, 165.0 us; 2 x 1024 10.6 -> 10.35).
+// With R = 2 and 1, which run few tiles only, half is ahead as well (attention launch, none, a quarter, half: R = 2, 2 x 4096 at 1, 2, 3
+// tiles 3.78, 3.71, 3.67, 4.58, 4.45, 4.40, 5.40, 5.22, 5.14, 1 x 9000 x 512 6.35, 6.13, 6.04; R = 1, 2 x 9000 x 128 5.15, 5.01, 4.98).
 // Not kept: the accumulator loaded for its rescaling before the last exponentials (184) or before P-hat is stored (173), a test_wait in
 // front of the wait for the scores (192).
 #include <string.h>

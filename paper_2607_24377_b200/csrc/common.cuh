@@ -190,13 +190,11 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
                    const void* k_scales, const void* v_codes, const void* v_scales, void* o,
                    int B, int H, int64_t Nq, int64_t Nkv, float softmax_scale, unsigned flags,
                    int* status, cudaStream_t stream, void* dump = nullptr, bool profile = false, bool followed = false);
-struct RowSplit { int64_t pairs_256; int R; };      // R = 0: nothing is left for the small CTAs
-RowSplit forward_row_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq);
 constexpr int kStaticTiles = 23, kStaticTilesNv = 3;     // KV tiles up to which a CTA of the walking kernel (walk.cuh) has its items from the start: MXFP4, NVFP4
-constexpr int kBesideTiles = 48;                    // ... and up to which it takes short launches that run beside others
-struct WalkSplit { bool walk; int64_t pairs; };     // whether the walking kernel takes the first `pairs` pairs (the rest: small CTAs)
-WalkSplit forward_walk_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq, bool followed, const RowSplit& split);     // `followed`: other attention launches run beside
-bool forward_walk_rest(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq, bool followed, const RowSplit& split);     // ... and whether it takes all of what that leaves out
+// The first `pairs` pairs of query tiles, counted over all heads, go to the walking kernel (walk) or to the kernel for pairs, the rest to CTAs of
+// 128 / R rows (R = 0: there is none).  `followed`: other attention launches run beside.
+struct ForwardPlan { bool walk; int64_t pairs; int R; };
+ForwardPlan forward_plan(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq, bool followed);
 int launch_forward_rows(int R, int64_t first_pair, const void* q_codes, const void* q_scales, const void* k_codes, const void* k_scales,
                         const void* v_codes, const void* v_scales, void* o, int B, int H, int64_t Nq, int64_t Nkv,
                         float softmax_scale, unsigned flags, int* status, cudaStream_t stream);

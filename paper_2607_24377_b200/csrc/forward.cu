@@ -727,28 +727,12 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
   const bool uos = flags & MXATTN_FLAG_UOS, pnq = flags & MXATTN_FLAG_PNQ, f32 = flags & MXATTN_FLAG_OUT_FP32;
   const int n_sm = sm_count();
   if (n_sm == 0) return MXATTN_ECUDA;
-  // query tiles that would leave SMs idle (a problem smaller than the GPU, or a last wave that is nearly empty) go to the
-  // kernel for few query rows
-  // (not where other attention launches run beside: their CTAs fill those SMs; 24 x 119056 in stages of one head 99.0 -> 93.1 ms)
-  const RowSplit split = dump || followed ? RowSplit{grid, 0} : forward_row_split(n_sm, (int64_t)B * H, Nq, Nkv, pnq);
-  if (!dump) {
-    WalkSplit walk = forward_walk_split(n_sm, (int64_t)B * H, Nq, Nkv, pnq, followed, split);
-    if (!walk.walk && forward_walk_rest(n_sm, (int64_t)B * H, Nq, Nkv, pnq, followed, split)) walk = WalkSplit{true, grid};
-    if (walk.walk) {
-      if (walk.pairs > 0) {
-        const int rc = launch_forward_walk(n_sm, walk.pairs, q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, o, B, H, Nq, Nkv, softmax_scale, flags, status, stream);
-        if (rc != MXATTN_OK || walk.pairs == grid) return rc;
-      }
-      return launch_forward_rows(split.R, walk.pairs, q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, o, B, H, Nq, Nkv, softmax_scale, flags, status, stream);
-    }
+  const ForwardPlan plan = dump ? ForwardPlan{false, grid, 0} : forward_plan(n_sm, (int64_t)B * H, Nq, Nkv, pnq, followed);
+  if (plan.walk) {
+    const int rc = plan.pairs == 0 ? (int)MXATTN_OK : launch_forward_walk(n_sm, plan.pairs, q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, o, B, H, Nq, Nkv, softmax_scale, flags, status, stream);
+    if (rc != MXATTN_OK || plan.R == 0) return rc;
+    return launch_forward_rows(plan.R, plan.pairs, q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, o, B, H, Nq, Nkv, softmax_scale, flags, status, stream);
   }
-  auto rest = [&]() {
-    return split.R == 0 ? (int)MXATTN_OK
-                        : launch_forward_rows(split.R, split.pairs_256, q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, o, B, H, Nq, Nkv,
-                                              softmax_scale, flags, status, stream);
-  };
-  if (split.pairs_256 == 0) return rest();
-  p.total_items = (int)split.pairs_256;
   CUtensorMap out_map;
   const int map_rc = encode_output_map(&out_map, o, (int64_t)B * H, Nq, f32);
   if (map_rc != MXATTN_OK) return map_rc;
@@ -769,8 +753,7 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
 #undef PICKD
   }
   if (!ensure_dynamic_smem((const void*)kern, kSmemBytes)) return MXATTN_ECUDA;
-  if (launch_pdl(kern, dim3((unsigned)split.pairs_256), kThreads, kSmemBytes, stream, p, out_map) != cudaSuccess) return MXATTN_ECUDA;
-  return rest();
+  return launch_pdl(kern, dim3((unsigned)grid), kThreads, kSmemBytes, stream, p, out_map) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;
 }
 
 }  // namespace mxattn

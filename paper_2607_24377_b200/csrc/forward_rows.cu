@@ -1,10 +1,10 @@
-// MXFP4 attention forward for few query rows (paper Algorithm 2, lines 6-19): the kernel that forward.cu hands a problem
-// to when its query tiles cannot fill the GPU, or could not fill its last wave.
+// MXFP4 attention forward for few query rows (paper Algorithm 2, lines 6-19): the kernel for a problem whose query tiles cannot fill the
+// GPU, or not its last wave (forward_plan in forward_walk.cu says where).
 //
 // KV tiles must be visited one after the other (P-hat depends on the history of the running maximum), so what counts for a
 // short problem is the latency of one tile, and the only way to use idle SMs is to give each CTA fewer query rows.  A CTA of
-// forward.cu takes 256 rows and 2570 cycles per tile; most of that is the exponentials, 2048 cycles per 256 x 128 tile and
-// SM.  A tensor-core product has 128 rows, and the 32 rows of a tensor-memory lane quarter belong to one SM sub-partition, so
+// the walking kernel takes 128 rows and 1200 cycles per tile and more; most of that is the exponentials, 1024 cycles per 128 x 128 tile
+// and SM.  A tensor-core product has 128 rows, and the 32 rows of a tensor-memory lane quarter belong to one SM sub-partition, so
 // fewer rows per CTA alone would only leave sub-partitions idle.  Here the CTA's 128/R query rows are REPLICATED R times down
 // the operand tile: every quarter (or pair of quarters) then sees the same rows' scores, and each takes its own share of the
 // KEYS.  R = 4: 32 rows, each sub-partition one block of 32 keys, 256 cycles of exponentials per tile; R = 2: 64 rows, two
@@ -16,12 +16,13 @@
 // of block kb: one thread per row and block.  The four warps of a row group exchange their block maxima through shared
 // memory at a named barrier once per tile.  S is double-buffered, so the next tile's scores are ready when a warp gets
 // there (loading them before the hand-over instead makes the hand-over's fence wait for the load: 5 % slower).  Measured
-// (B200, 1965 MHz): 1200 cycles per tile with R = 4, 1530 with R = 2, 2125 with R = 1 (one query tile of 128 rows, 16 warps);
-// 2 heads of 1024 x 1024: attention launch 14 -> 6 us.  With R = 4 a sub-partition has one softmax warp, which alone keeps the
+// (B200, 1965 MHz, all exponentials on their unit): 1200 cycles per tile with R = 4, 1530 with R = 2; 2 heads of 1024 x 1024: attention
+// launch 14 -> 6 us (from 256 rows per CTA).  With R = 4 a sub-partition has one softmax warp, which alone keeps the
 // exponential unit busy for half of the time: where only the codes count (PNQ) every other pair is a polynomial (exp2_poly), 1200 ->
 // 1085 cycles (1 x 4096 x 40000, whole call, none, a quarter, three eighths, half: 182.7, 172.6, 166.2, 165.0 us; 2 x 1024 10.6 -> 10.35).
-// With R = 2 and 1, which run few tiles only, half is ahead as well (attention launch, none, a quarter, half: R = 2, 2 x 4096 at 1, 2, 3
-// tiles 3.78, 3.71, 3.67, 4.58, 4.45, 4.40, 5.40, 5.22, 5.14, 1 x 9000 x 512 6.35, 6.13, 6.04; R = 1, 2 x 9000 x 128 5.15, 5.01, 4.98).
+// With R = 2, which runs few tiles only, half is ahead as well (attention launch, none, a quarter, half: 2 x 4096 at 1, 2, 3 tiles 3.78, 3.71,
+// 3.67, 4.58, 4.45, 4.40, 5.40, 5.22, 5.14, 1 x 9000 x 512 6.35, 6.13, 6.04).  R = 1 (128 rows, 16 warps) was behind the walking kernel at
+// every length (74 x 256 queries x 128: 5.02 / 4.82, 37 x 256 x 8192: 64.9 / 45.6) and is gone.
 // Not kept: the accumulator loaded for its rescaling before the last exponentials (184) or before P-hat is stored (173), a test_wait in
 // front of the wait for the scores (192).
 #include <string.h>
@@ -72,7 +73,7 @@ struct Params {
   float scale_log2e;
 };
 
-template <int R, bool kUos, bool kPnq, bool kOutF32>
+template <int R, bool kUos, bool kPnq, bool kOutF32>      // R = 4 or 2
 __global__ void __launch_bounds__(32 * (16 / R + 2), 1) attention_rows_kernel(const Params p) {
   constexpr int kWarps = 16 / R, kRG = 4 / R;                    // softmax warps, row groups of 32
   extern __shared__ uint8_t smem_raw[];
@@ -359,38 +360,6 @@ __global__ void __launch_bounds__(32 * (16 / R + 2), 1) attention_rows_kernel(co
 
 }  // namespace rows
 
-// How a problem of bh heads is divided between the 256-row CTAs of forward.cu and the smaller ones of this file: the first
-// `pairs_256` pairs of query tiles (counted over all heads) go there, the rest to CTAs of 128/R rows.  Estimated cycles =
-// waves of CTAs over the SMs x (KV tiles x cycles per tile + fixed cost), with measured figures: a 256-row CTA takes 2700
-// cycles per tile (3050 with the direct row sum), 128 rows 2125, 64 rows 1530, 32 rows 1200.  A small CTA costs more SM
-// cycles per row, so a problem that fills whole waves of 256-row CTAs stays there; a problem smaller than a wave goes to
-// small CTAs; and where the last wave of 256-row CTAs would be nearly empty, its items are cut into small CTAs instead:
-// 24 heads of 8192 queries are 5.19 waves (direct row sum 647 -> 603 us).  That second launch waits for the last of the full
-// waves.  With PNQ it adds what the same rows take by themselves, within 2 us (28 pairs behind 1, 5 and 20 waves: 41.8, 41.2,
-// 40.9 us for 41.6 at 48 tiles; 102.2, 101.7, 102.4 for 100.4 at 128), with the direct row sum up to 12 us more (5 waves of
-// 128 tiles: 116.3 for 104.7; 46 us more in one series of ten, 20 waves of 48 tiles), as CTAs drift apart.  The estimate charges
-// 4000 cycles, and a tenth of a wave above 48 tiles (kDriftTiles), so that a close call keeps to one launch.
-// Where the walking kernel takes the whole waves its rule starts from this division: R, which does not depend on what the whole
-// waves cost, is taken over, and whether there are small CTAs at all is estimated again with that kernel's cycles.  R = 0 for its
-// sake may hide a division that is ahead by the tenth of a wave at most.
-constexpr int kDriftTiles = 48;
-RowSplit forward_row_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq) {
-  const int64_t T = (Nkv + kTile - 1) / kTile, tiles = (Nq + kTile - 1) / kTile;
-  const int64_t pairs = (tiles + 1) / 2, total = bh * pairs, full = total / n_sm;
-  const int64_t c256 = T * (pnq ? 2700 : 3050) + 4400;
-  RowSplit best{total, 0};
-  if (total % n_sm == 0) return best;
-  int64_t best_cost = (full + 1) * c256 + 1600;
-  for (int R = 1; R <= 4; R *= 2) {
-    const int64_t c = T * (R == 4 ? 1200 : R == 2 ? 1530 : 2125) + 4500, per_head = (Nq + kTile / R - 1) / (kTile / R);
-    const int64_t at = full * n_sm, done = at / pairs * per_head + (at % pairs) * 2 * R;     // groups in the full waves
-    const int64_t gap = full == 0 ? 0 : T > kDriftTiles ? 4000 + c256 / 10 : 4000;
-    const int64_t cost = full * c256 + gap + (bh * per_head - done + n_sm - 1) / n_sm * c;
-    if (cost < best_cost) { best_cost = cost; best = RowSplit{at, R}; }
-  }
-  return best;
-}
-
 int launch_forward_rows(int R, int64_t first_pair, const void* q_codes, const void* q_scales, const void* k_codes, const void* k_scales,
                         const void* v_codes, const void* v_scales, void* o, int B, int H, int64_t Nq, int64_t Nkv,
                         float softmax_scale, unsigned flags, int* status, cudaStream_t stream) {
@@ -408,7 +377,7 @@ int launch_forward_rows(int R, int64_t first_pair, const void* q_codes, const vo
   p.scale_log2e = softmax_scale * 1.4426950408889634f;
   const bool uos = flags & MXATTN_FLAG_UOS, pnq = flags & MXATTN_FLAG_PNQ, f32 = flags & MXATTN_FLAG_OUT_FP32;
   void (*kern)(const Params) = nullptr;
-#define PICK(U, P, F) if (uos == U && pnq == P && f32 == F) kern = R == 4 ? attention_rows_kernel<4, U, P, F> : R == 2 ? attention_rows_kernel<2, U, P, F> : attention_rows_kernel<1, U, P, F>;
+#define PICK(U, P, F) if (uos == U && pnq == P && f32 == F) kern = R == 4 ? attention_rows_kernel<4, U, P, F> : attention_rows_kernel<2, U, P, F>;
   PICK(false, false, false) PICK(false, false, true) PICK(false, true, false) PICK(false, true, true)
   PICK(true, false, false) PICK(true, false, true) PICK(true, true, false) PICK(true, true, true)
 #undef PICK

@@ -38,62 +38,51 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
 
 }  // namespace walk
 
-// Which problems this kernel takes, and how many of their pairs of query tiles (the rest goes to the small CTAs that
-// `split` names).  Attention launch, us, kernel of forward.cu (in a form that walked its items up to 48 tiles) / this one, PNQ:
-// 37 x 16384 queries, KV tiles 1, 4, 128: 52.8 / 45.7, 122.0 / 108.2, 2800 / 2753; 40 x 16384, 2 tiles: 84.6 / 73.3;
-// 40 x 4096, 32: 235 / 206; 64 x 8192, 8: 188 / 169; 40 x 8192, 48, 64: 631 / 603, 825 / 795; 16 x 32768, 256: 4736 / 4733;
-// 12 x 75600, 591: 18376 / 18456.  With the direct row sum, 1, 4, 32, 48 tiles: 58.2 / 46.0, 136.7 / 112.3, 262 / 228,
-// 711 / 668, and whole calls: 37 x 4096, 100: 695 / 672; 16 x 32768, 256: 5402 / 5293; 12 x 40000, 400: 7647 / 7554; 12 x 75600,
-// 591: 20726 / 20574; 24 x 16384, 591: 9405 / 9109.  (These figures, and those below, are of both kernels before the polynomial and
-// the named barriers; what these changed stands at forward_walk_rest, which has the last word.)
-// - A few whole waves of pairs that single tiles do not round better.  PNQ: one wave, whole call at 2, 7, 12, 49, 100 tiles: 37 x
-//   1000 13.2 / 12.8, 22.7 / 22.5, 31.2 / 31.3, 105.4 / 106.8, 194.6 / 196.4 (14 x 1300 x 777, fp32: 20.7 / 20.5).  Direct: up to
-//   four waves above 256 tiles; one wave (37 x 1000) at 2, 12, 48, 100, 256, 400 tiles: 13.8 / 12.9, 34.8 / 32.1, 115.4 / 111.0,
-//   215.3 / 209.9, 506.8 / 506.4, 774.7 / 780.0; two (37 x 2048), 1016: 3369 / 3412; four (37 x 4096), 256, 469: 1658 / 1646,
-//   2961 / 2970.
-// - Launches that run beside others (`followed`) keep to short sequences: CTAs with fixed shares hold their SMs to the end
-//   (24 x 8192 from host tensors: 3225 us for 3246); forward_walk_rest adds the long ones.
-// - A CTA counts its tiles in 32 bits (the last few are left for the teams' steps beyond the end).  Where it takes items from
-//   others it may get them all: one head of 6 million queries and keys has more.
-// - Small CTAs for the last wave cost a launch and 1200 to 2125 cycles per tile and CTA, a round of single tiles T x 1390
-//   cycles (direct 1500) + 1000.  All in one walk / last wave in small CTAs, whole call: 24 x 8192 529 / 541 (direct 568 / 589),
-//   40 x 4096 241 / 261, 38 x 8192 x 3000 330 / 337, x 1000 134.8 / 139.7 (direct 140.4 / 145.3), 38 x 1000 x 700 25.0 / 27.7,
-//   51 x 700 x 300 18.3 / 21.2.
-WalkSplit forward_walk_split(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq, bool followed, const RowSplit& split) {
-  const int64_t T = (Nkv + kTile - 1) / kTile, tiles = (Nq + kTile - 1) / kTile, pairs = (tiles + 1) / 2;
-  if ((pnq && T > 256) || (followed && T > kBesideTiles)) return WalkSplit{false, 0};
-  if ((T > kStaticTiles ? bh * tiles : (bh * tiles + n_sm - 1) / n_sm) * T > 0x7FFFFF00) return WalkSplit{false, 0};
-  if (split.R == 0) {
-    const int64_t rounds = (bh * tiles + n_sm - 1) / n_sm, waves = (bh * pairs + n_sm - 1) / n_sm;
-    const bool pairs_ahead = pnq || followed ? waves == 1 : waves <= 4 && T > 256;
-    return WalkSplit{rounds < 2 * waves || !pairs_ahead, bh * pairs};
+// How a problem is divided between the kernels.  All figures are attention launches with the PNQ row sum / the direct one, in us.
+//
+// A launch that has the GPU to itself: the walking kernel, but
+//  - CTAs of 32 rows where they are one wave at most: they take two thirds to nine tenths of the time whatever the length (18 x 256 queries, 1,
+//    4, 16, 64, 300 KV tiles, walked 4.59 6.63 14.7 45.4 187 / 4.79 7.11 16.1 50.7 214, 32 rows 3.37 5.30 12.5 39.1 158 / 3.39 5.41 13.1 41.8
+//    175).  A second wave of them never pays (37 x 256, 64 tiles: 45.6 / 50.9, 32 rows 76.7 / 82.7).
+//  - CTAs of 64 rows where those are one wave, up to 13 KV tiles (direct 14; 37 x 256, 1, 4, 8, 16, 32 tiles: walked 4.62 6.69 9.40 14.8 25.4 / 4.81 7.18 10.2 16.1
+//    28.0, 64 rows 3.82 6.04 9.02 14.9 26.5 / 3.94 6.42 9.78 16.2 29.1).
+//  - Whole waves of pairs walked and the rest in one wave of CTAs of 32 rows, a second launch, if that is estimated to take less than the
+//    rounds of single tiles it saves.  A round: T x 1150 + 4500 cycles (direct 1335, 3500); the second launch with the wait for the first's last
+//    CTAs: T x 1045 + 12000 (1175, 8000).  152 x 256, 32, 64, 128, 300 tiles: all walked 67.9 127.7 244.1 548.9 / 75.6 144.4 279.0 635.5,
+//    divided 69.8 128.4 241.0 536.9 / 75.5 141.4 270.7 613.2; 758 x 256, 64, 128: 455.4 879.5 / 517.4 1009.6, divided 458.4 879.5 / 517.1 1003.9.
+//    64 rows there were behind in all cases (185 x 256, 64 and 300 tiles: 136.9 576 / 154.2 671 for 128.1 550 / 144.9 638).
+//  - The kernel for pairs beyond 2^31 tiles, which a CTA of the walking kernel counts in 32 bits (where it takes items from others it may get
+//    them all): a single tile takes 1200-1290 cycles here (direct row sum 1390-1450), a pair 2570-2700 there (3050).
+//
+// Beside other launches (the stages of a forward from host tensors) nothing is left idle that small CTAs could use, and CTAs that hold their
+// SMs longer, as those of pairs do not, keep the next stage's waiting.  Up to 48 tiles: walked, unless a wave of pairs makes two rounds of tiles.
+// Above 128 tiles: walked, unless the query tiles are fewer than half of the KV tiles.  Between, the kernel for pairs.  Whole call, medians of 22, kernel
+// for pairs / walked: 24 x 8192 3253 3270 / 3292 3296, 8 x 16000 2235 2292 / 2259 2282, 24 x 6200 2542 2528 / 2502 2545, 12 x 13000 2684 2687 / 2637
+// 2660, 24 x 14000 5473 5476 / 5392 5450, but 10 x 10000 1849 1808 / 1853 1827, 16 x 12000 3302 3271 / 3314 3296; 24 x 7000 x 30000 7891 7934 / 7977
+// 7957; above 128 tiles, at an earlier state, 12 x 20000 4061 3908, 8 x 40000 5934 5588 / 6039 5817, 10 x 75600 16875 15673, 2 x 60000 3608 3157.
+ForwardPlan forward_plan(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq, bool followed) {
+  const int64_t T = (Nkv + kTile - 1) / kTile, tiles = (Nq + kTile - 1) / kTile, pairs = (tiles + 1) / 2, total = bh * pairs;
+  auto rounds = [&](int64_t n) { return (n + n_sm - 1) / n_sm; };
+  const bool counts = (T > kStaticTiles ? bh * tiles : rounds(bh * tiles)) * T <= 0x7FFFFF00;      // (the last few are for the teams' steps beyond the end)
+  if (followed) {
+    const bool walk = T <= 48 ? rounds(bh * tiles) < 2 * rounds(total) || rounds(total) > 1 : T > 128 && 2 * tiles >= T;
+    return ForwardPlan{counts && walk, total, 0};
   }
-  auto walk = [&](int64_t items) { return (items + n_sm - 1) / n_sm * (T * (pnq ? 1390 : 1500) + 1000) + 4400; };
-  const int64_t per_head = (Nq + kTile / split.R - 1) / (kTile / split.R), at = split.pairs_256;
-  const int64_t done = at / pairs * per_head + (at % pairs) * 2 * split.R, before = at / pairs * tiles + (at % pairs) * 2;
-  const int64_t small = (bh * per_head - done + n_sm - 1) / n_sm * (T * (split.R == 4 ? 1200 : split.R == 2 ? 1530 : 2125) + 4500);
-  const bool all = walk(bh * tiles) <= (before > 0 ? walk(before) + 4000 : 0) + small;
-  return WalkSplit{true, all ? bh * pairs : at};
-}
-
-// A launch that has the GPU to itself leaves none of the rest to the kernel of forward.cu: a single tile takes 1200-1290 cycles here
-// (direct row sum 1390-1450), a pair 2570-2700 there (3050), so that two rounds of tiles are less than one wave of pairs.  Whole call, us,
-// that kernel (and small CTAs for its last wave) / this one, PNQ: one wave of pairs, 37 x 1000 at 2, 8, 12, 49, 100, 313 KV tiles 13.2 / 12.3,
-// 24.0 / 23.0, 31.2 / 29.9, 104.8 / 101.3, 193.8 / 185.8, 561.8 / 532.7, 14 x 1300 x 777 19.6 / 18.5 (fp32 output 20.5 / 19.8), x 6200
-// 83.0 / 78.0, 74 x 500 x 3000 70.9 / 68.9; above 256 tiles 12 x 75600 18517 / 16972, 40 x 20000 x 40000 9183 / 8298, 24 x 16384 x 75600
-// 8477 / 7565, 5 x 4000 x 40000 441 / 411, 20 x 2000 x 40000 682 / 657, 1 x 9000 x 40000 237 / 202, 2 x 5000 x 40000 334 / 206.  Direct, one to four
-// waves of pairs above 256 tiles: 37 x 1000 x 33000 515 / 494, x 52000 795 / 765, 37 x 2048 x 130000 3411 / 3278, 37 x 4096 x 33000 1684 / 1590,
-// x 60000 2994 / 2846, 20 x 1000 x 65536 881 / 851, 18 x 4096 x 65536 1622 / 1551.  Small CTAs of 32
-// rows keep what they would do alone (1200 cycles per tile; 1 x 4096 x 40000 183).
-// Beside other launches (the stages of a forward from host tensors) above 128 tiles, with either row sum: CTAs that take items leave an
-// SM when none is left, and the next stage's come there.  us: 12 x 20000 4061 / 3908, 8 x 40000 5934 / 5588 (direct 6039 / 5817), 10 x 75600
-// 16875 / 15673, 2 x 60000 3608 / 3157.  Where the link is the bound only the last stage counts: 24 x 8192 3196 / 3210, 12 x 13000 2679 / 2686
-// (direct 2647 / 2664), 24 x 14000 5445 / 5430, and with fewer query tiles than half of T 24 x 7000 x 30000 7900 / 7930.
-bool forward_walk_rest(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool pnq, bool followed, const RowSplit& split) {
-  const int64_t T = (Nkv + kTile - 1) / kTile, tiles = (Nq + kTile - 1) / kTile;
-  if (followed && (T <= 128 || 2 * tiles < T)) return false;
-  if ((T > kStaticTiles ? bh * tiles : (bh * tiles + n_sm - 1) / n_sm) * T > 0x7FFFFF00) return false;
-  return !(split.R == 4 && split.pairs_256 == 0);
+  auto groups = [&](int64_t R, int64_t from) {        // of 128 / R rows, behind the first `from` pairs
+    const int64_t per_head = (Nq + kTile / R - 1) / (kTile / R);
+    return bh * per_head - from / pairs * per_head - from % pairs * 2 * R;
+  };
+  const int64_t at = total / n_sm * n_sm;
+  if (at == 0) {
+    if (groups(4, 0) <= n_sm) return ForwardPlan{true, 0, 4};
+    if (groups(2, 0) <= n_sm && T <= (pnq ? 13 : 14)) return ForwardPlan{true, 0, 2};
+  }
+  if (!counts) return ForwardPlan{false, total, 0};
+  if (at > 0 && at < total && groups(4, at) <= n_sm) {
+    const int64_t saved = rounds(bh * tiles) - rounds(at / pairs * tiles + at % pairs * 2);
+    if (T * (pnq ? 1045 : 1175) + (pnq ? 12000 : 8000) < saved * (T * (pnq ? 1150 : 1335) + (pnq ? 4500 : 3500))) return ForwardPlan{true, at, 4};
+  }
+  return ForwardPlan{true, total, 0};
 }
 
 // The first `pairs` pairs of query tiles, counted over all heads.

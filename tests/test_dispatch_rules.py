@@ -23,13 +23,16 @@ def test_tensor_maximum_by_clusters_only_where_they_fit(batch, chunks, form):
 @pytest.mark.parametrize("pnq", [True, False])
 def test_last_wave_is_divided_for_the_sms_that_there_are(n_sm, pnq):
     from tests import util
-    for heads, nq, nkv in ((1, 1, 1), (2, 1024, 1024), (38, 1000, 700), (40, 4096, 4096), (3, 50000, 300)):
+    divided = 0
+    for heads, nq, nkv in ((1, 1, 1), (2, 1024, 1024), (38, 1000, 700), (40, 4096, 4096), (3, 50000, 300), (1, 256 * n_sm + 300, 12800), (n_sm, 200, 12800)):
         total = heads * ((-(-nq // 128) + 1) // 2)
-        pairs, r = util.row_split(n_sm, heads, nq, nkv, pnq)
-        assert r in (0, 1, 2, 4)
+        pairs, r = util.plan(n_sm, heads, nq, nkv, pnq)
+        assert r in (0, 2, 4)
         assert pairs == (total if r == 0 else total // n_sm * n_sm)          # whole waves, or everything
-    assert util.row_split(n_sm, n_sm, 256, 1024, pnq) == (n_sm, 0)            # exactly a wave
-    assert util.row_split(n_sm, 1, 32, 1024, pnq) == (0, 4)                   # a single group of rows
+        divided += r > 0 and pairs > 0
+    assert divided == 1
+    assert util.plan(n_sm, n_sm, 256, 1024, pnq) == (n_sm, 0)                 # exactly a wave
+    assert util.plan(n_sm, 1, 32, 1024, pnq) == (0, 4)                        # a single group of rows
 
 
 def stages(heads, nq, nkv, n_sm=148):

@@ -2,8 +2,6 @@
 heads alone, which small CTAs of another kernel compute, and copied often enough that every CTA walks several items.  The KV
 tiles of an item are one, two, three (teams change from item to item), as many as buffers come round (4 to 9) and more; query
 and key counts end inside a tile, a half and a block."""
-import ctypes
-
 import pytest
 import torch
 
@@ -11,87 +9,48 @@ import synth_inputs as si
 from tests import util
 
 
-def walk_split(n_sm, heads, nq, nkv, pnq, followed=False):
-    """(whether the kernel is used, pairs of query tiles it takes), asked of the library"""
-    import paper_2607_24377_b200 as mx
-
-    class Row(ctypes.Structure):
-        _fields_ = [("pairs_256", ctypes.c_int64), ("R", ctypes.c_int)]
-
-    class Walk(ctypes.Structure):
-        _fields_ = [("walk", ctypes.c_bool), ("pairs", ctypes.c_int64)]
-
-    f = getattr(mx.lib(), "_ZN6mxattn18forward_walk_splitEllllbbRKNS_8RowSplitE")
-    f.argtypes, f.restype = [ctypes.c_int64] * 4 + [ctypes.c_bool] * 2 + [ctypes.POINTER(Row)], Walk
-    w = f(n_sm, heads, nq, nkv, pnq, followed, ctypes.byref(Row(*util.row_split(n_sm, heads, nq, nkv, pnq))))
-    return w.walk, w.pairs
+@pytest.mark.parametrize("pnq", [True, False])
+def test_what_the_walking_kernel_takes(pnq):
+    for heads, nq, nkv in ((40, 4096, 4096), (40, 75600, 512), (24, 8192, 8192), (40, 75600, 75600), (3, 50000, 300), (14, 1300, 777), (13, 1300, 777),
+                           (37, 1000, 12800), (74, 512, 40000), (37, 4096, 33000), (2, 5000, 40000), (3, 6200, 400 * 128), (50, 128, 40000)):
+        assert util.plan(148, heads, nq, nkv, pnq) == (heads * ((-(-nq // 128) + 1) // 2), 0) and util.walked(148, heads, nq, nkv, pnq)
 
 
 @pytest.mark.parametrize("pnq", [True, False])
-def test_what_the_walking_kernel_takes(pnq):
-    for heads, nq, nkv in ((1, 1, 1), (2, 1024, 1024), (40, 4096, 4096), (40, 75600, 512), (24, 8192, 8192), (3, 50000, 300)):
-        walk, pairs = walk_split(148, heads, nq, nkv, pnq)
-        total, (whole, r) = heads * ((-(-nq // 128) + 1) // 2), util.row_split(148, heads, nq, nkv, pnq)
-        assert walk and pairs in (whole, total) and (r != 0 or pairs == total)
-    assert walk_split(148, 2, 1024, 1024, pnq)[1] == 0                       # small CTAs alone
-    assert walk_split(148, 40, 4096, 4096, pnq)[1] == 640                    # nine waves of single tiles, no second launch
-    assert walk_split(148, 14, 1300, 777, pnq)[0] == (not pnq) and walk_split(148, 13, 1300, 777, pnq)[0]      # one wave of pairs, two rounds of tiles; one round
-    assert walk_split(148, 24, 4096, 6144, pnq, True)[0] and not walk_split(148, 24, 4096, 6145, pnq, True)[0]      # beside other launches
-    assert walk_split(148, 40, 256 * 128, 256 * 128, pnq)[0] and walk_split(148, 40, 256, 256 * 128 + 1, pnq)[0] == (not pnq)
-
-
-def test_few_whole_waves_of_pairs_with_the_direct_row_sum():
-    # 74 x 512 and 37 x 4096: exactly one and four waves of pairs, two and eight rounds of single tiles
-    for heads, nq in ((74, 512), (37, 4096)):
-        assert walk_split(148, heads, nq, 256 * 128, False) == (True, heads * nq // 256)
-        assert not walk_split(148, heads, nq, 256 * 128 + 1, False)[0]
-    assert walk_split(148, 37, 8192, 600 * 128, False)[0]                    # eight waves
-    assert walk_split(148, 14, 1300, 100 * 128, False)[0] and not walk_split(148, 14, 1300, 777, False, True)[0]     # beside other launches
-    assert walk_split(148, 3, 6200, 400 * 128, False) == (True, 75)          # 147 single tiles: one round where pairs take one of twice the time
+def test_small_problems_go_to_small_ctas(pnq):
+    # one wave of 32 rows, whatever the length; one of 64 rows up to 13 KV tiles (direct row sum 14); none of 128
+    for heads, nq, nkv, pairs, r in ((1, 1, 1, 0, 4), (2, 1024, 1024, 0, 4), (1, 4096, 40000, 0, 4), (37, 128, 4096, 0, 4), (37, 129, 1664, 0, 2), (1, 4737, 1664, 0, 2),
+                                     (1, 9472, 128, 0, 2), (1, 4737, 14 * 128, *((19, 0) if pnq else (0, 2))), (1, 4737, 1793, 19, 0), (1, 9473, 128, 38, 0), (38, 256, 128, 38, 0), (12, 1300, 128, 72, 0)):
+        assert util.plan(148, heads, nq, nkv, pnq) == (pairs, r), (heads, nq, nkv)
 
 
 @pytest.mark.parametrize("pnq", [True, False])
 def test_last_wave_goes_where_it_is_estimated_to_end_first(pnq):
-    # cycles of n single tiles in one walk, and of a launch of small CTAs behind them (the figures stand at the rule)
-    rounds = lambda n, t: -(-n // 148) * (t * (1390 if pnq else 1500) + 1000) + 4400
-    split = 0
-    for heads, nq, nkv in ((38, 1000, 700), (38, 8192, 1000), (51, 700, 300), (38, 897, 6200), (38, 1000, 130), (40, 2000, 1024), (24, 8192, 8192), (39, 897, 6300)):
-        whole, r = util.row_split(148, heads, nq, nkv, pnq)
-        t, tiles = -(-nkv // 128), -(-nq // 128)
-        pairs, groups = (tiles + 1) // 2, -(-nq // (128 // r))
-        ahead = whole // pairs * tiles + whole % pairs * 2
-        small = -(-(heads * groups - whole // pairs * groups - whole % pairs * 2 * r) // 148) * (t * {4: 1200, 2: 1530, 1: 2125}[r] + 4500)
-        one = rounds(heads * tiles, t) <= rounds(ahead, t) + 4000 + small
-        assert walk_split(148, heads, nq, nkv, pnq) == (True, heads * pairs if one else whole)
-        split += not one
-    assert split == 2
+    # a few pairs more than a wave: their rounds of single tiles, or a second launch of CTAs of 32 rows, from 72 (direct row sum 29) KV tiles on
+    last = 71 if pnq else 28
+    for heads, nq in ((38, 1000), (1, 152 * 256), (39, 897), (2, 379 * 256)):
+        total = heads * ((-(-nq // 128) + 1) // 2)
+        for t in (1, 6, last, last + 1, 100, 300):
+            assert util.plan(148, heads, nq, t * 128, pnq) == ((total, 0) if t <= last else (total // 148 * 148, 4)), (heads, nq, t)
+    assert util.plan(148, 1, 186 * 256, 12800, pnq) == (186, 0)              # 38 pairs are more than a wave of 32 rows
+    assert util.plan(148, 25, 1500, 12800, pnq)[1] == 4 and util.plan(148, 30, 1150, 12800, pnq) == (150, 0)      # odd heads: 270 tiles are two rounds either way
 
 
-def test_what_is_left_for_the_walking_kernel():
-    import paper_2607_24377_b200 as mx
-    rule = getattr(mx.lib(), "_ZN6mxattn17forward_walk_restEllllbbRKNS_8RowSplitE")
-    rule.argtypes, rule.restype = [ctypes.c_int64] * 4 + [ctypes.c_bool] * 2 + [ctypes.c_void_p], ctypes.c_bool
-    for heads, nq, nkv, walked in ((14, 1300, 777, True), (37, 1000, 12800, True), (40, 75600, 75600, True), (2, 5000, 40000, True),
-                                   (1, 4096, 40000, False), (2, 1024, 1024, False), (1, 6_000_000, 6_000_000, False)):
-        split = (ctypes.c_int64 * 2)(*util.row_split(148, heads, nq, nkv, True))
-        assert not walk_split(148, heads, nq, nkv, True)[0] or nkv <= 256 * 128
-        assert rule(148, heads, nq, nkv, True, False, split) == walked, (heads, nq, nkv)
-        direct = (ctypes.c_int64 * 2)(*util.row_split(148, heads, nq, nkv, False))
-        assert rule(148, heads, nq, nkv, False, False, direct) == walked, (heads, nq, nkv)
-    none = (ctypes.c_int64 * 2)(600, 0)                                      # beside other launches there are no small CTAs
-    for pnq in (True, False):
-        assert rule(148, 3, 40000, 128 * 128 + 1, pnq, True, none) and not rule(148, 3, 40000, 128 * 128, pnq, True, none)
-        assert not rule(148, 3, 7000, 30000, pnq, True, none)
+@pytest.mark.parametrize("pnq", [True, False])
+def test_beside_other_launches(pnq):
+    for heads, nq, nkv, by_walk in ((24, 4096, 6144, True), (24, 4096, 6145, False), (14, 1300, 777, False), (13, 1300, 777, True), (3, 40000, 128 * 128, False),
+                                    (3, 40000, 128 * 128 + 1, True), (3, 7000, 30000, False), (1, 1, 1, True)):
+        assert util.plan(148, heads, nq, nkv, pnq, True) == (heads * ((-(-nq // 128) + 1) // 2), 0)      # no small CTAs
+        assert util.walked(148, heads, nq, nkv, pnq, True) == by_walk, (heads, nq, nkv)
 
 
 def test_tiles_of_a_cta_are_counted_in_32_bits():
-    # one head of n queries and keys with the direct row sum: up to 2^31 - 256 tiles per CTA
-    for n, taken in ((72 << 20, False), (73_000_000, False), (64 << 20, True)):
-        tiles = -(-n // 128)
-        assert (-(-tiles // 148) * tiles <= 0x7FFFFF00) == taken
-        assert taken or not walk_split(148, 1, n, n, False)[0]
-    # above 48 tiles, where a CTA takes items that others have not begun, they may all be its own
-    assert not walk_split(148, 1, 6_000_000, 6_000_000, False)[0] and walk_split(148, 1, 100 << 20, 48 * 128, False)[0]
+    # above 23 tiles, where a CTA takes items that others have not begun, they may all be its own; with fixed shares it has its own only
+    for n, nkv, by_walk in ((72 << 20, 72 << 20, False), (6_000_000, 6_000_000, False), (5_900_000, 5_900_000, True), (1 << 30, 24 * 128, True), (1 << 37, 23 * 128, True)):
+        tiles, t = -(-n // 128), -(-nkv // 128)
+        assert ((tiles if t > 23 else -(-tiles // 148)) * t <= 0x7FFFFF00) == by_walk
+        for pnq in (True, False):
+            assert util.walked(148, 1, n, nkv, pnq) == by_walk and util.plan(148, 1, n, nkv, pnq)[0] == (tiles + 1) // 2
 
 
 @pytest.mark.gpu
@@ -114,7 +73,7 @@ def test_walked_items_equal_a_single_head(nq, nkv, uos, pnq, f32):
         out.check(); ws.check()
         outs.append(out.t.clone())
     n_sm = torch.cuda.get_device_properties(0).multi_processor_count
-    assert walk_split(n_sm, 3, nq, nkv, pnq)[1] == 0 and walk_split(n_sm, 447, nq, nkv, pnq)[1] > 0
+    assert util.plan(n_sm, 3, nq, nkv, pnq)[0] == 0 and util.plan(n_sm, 447, nq, nkv, pnq)[0] > 0
     assert n_sm % (3 * -(-nq // 128)) != 0                                   # a CTA's items differ from one another
     assert bool(torch.isfinite(outs[0].float()).all())
     assert torch.equal(outs[1], outs[0].repeat(1, 149, 1, 1))
@@ -145,7 +104,7 @@ def test_scores_that_are_not_numbers(nq, nkv, pnq):
         assert int(status[0]) == 0
         outs.append(out)
     n_sm = torch.cuda.get_device_properties(0).multi_processor_count
-    assert walk_split(n_sm, 3, nq, nkv, pnq)[1] == 0 and walk_split(n_sm, 447, nq, nkv, pnq)[1] > 0
+    assert util.plan(n_sm, 3, nq, nkv, pnq)[0] == 0 and util.plan(n_sm, 447, nq, nkv, pnq)[0] > 0
     want = outs[0].repeat(1, 149, 1, 1)
     assert not pnq or bool(torch.isfinite(want[0, 0]).all())
     assert torch.equal(torch.isnan(outs[1]), torch.isnan(want))
@@ -164,7 +123,7 @@ def test_taken_items_equal_a_single_head(nq, nkv, uos, pnq, f32):
     one = si.custom_config("tk", 1, 3, nq, nkv, 5 + nq)
     q, k, v = (util.to_dev_bf16(x) for x in si.make_all(one))
     n_sm = torch.cuda.get_device_properties(0).multi_processor_count
-    assert walk_split(n_sm, 3, nq, nkv, pnq)[1] == 0 and walk_split(n_sm, 237, nq, nkv, pnq)[1] > 0
+    assert util.plan(n_sm, 3, nq, nkv, pnq)[0] == 0 and util.plan(n_sm, 237, nq, nkv, pnq)[0] > 0
     assert n_sm % (3 * -(-nq // 128)) != 0
 
     def run(copies, beside=None):
@@ -239,7 +198,8 @@ def test_a_launch_that_holds_few_sms_does_not_hold_up_whole_shares(fmt, heads, n
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("nq,nkv", [(130, 256 * 128 + 1), (257, 300 * 128)])
-def test_long_sequences_equal_small_ctas(nq, nkv):
+@pytest.mark.parametrize("pnq", [True, False])
+def test_long_sequences_equal_small_ctas(nq, nkv, pnq):
     """Above 256 KV tiles: one head alone (CTAs of 32 rows), and copied until the walking kernel's CTAs take items from one another."""
     import paper_2607_24377_b200 as mx
     g = torch.Generator(device="cuda"); g.manual_seed(nq)
@@ -249,11 +209,11 @@ def test_long_sequences_equal_small_ctas(nq, nkv):
         dev = [x.repeat(1, heads, 1, 1).contiguous() for x in (q, k, v)]
         o = util.guarded((1, heads, nq, 128), torch.float32, float("nan"))
         ws = util.guarded(mx.forward_workspace_bytes(1, heads, nq, nkv, 128), torch.uint8)
-        mx.forward_ws(*dev, o.t, 1, heads, nq, nkv, 128, 128 ** -0.5, mx.FLAG_UOS | mx.FLAG_PNQ | mx.FLAG_OUT_FP32, ws.t)
+        mx.forward_ws(*dev, o.t, 1, heads, nq, nkv, 128, 128 ** -0.5, mx.FLAG_UOS | (mx.FLAG_PNQ if pnq else 0) | mx.FLAG_OUT_FP32, ws.t)
         assert mx.device_status(ws.t) == 0
         o.check(); ws.check()
         outs.append(o.t.clone())
-    assert util.row_split(torch.cuda.get_device_properties(0).multi_processor_count, 1, nq, nkv, True) == (0, 4)
+    assert util.plan(torch.cuda.get_device_properties(0).multi_processor_count, 1, nq, nkv, pnq) == (0, 4)
     assert bool(torch.isfinite(outs[0]).all()) and torch.equal(outs[1], outs[0].expand_as(outs[1]))
 
 

@@ -23,10 +23,11 @@ def nodes_of(call):
     ("mxfp4", 2, 300, 300, 3, 2),        # operands, attention
     ("mxfp4", 2, 300, 300, 11, 3),       # ... and the rotation of Q and K
     ("mxfp4", 38, 1000, 700, 3, 2),      # a wave and a bit, all in one attention launch
-    ("mxfp4", 38, 897, 6200, 3, 5),      # Q, K and V apart; a full wave of attention CTAs, the rest in small ones
+    ("mxfp4", 38, 897, 6200, 3, 4),      # Q, K and V apart
+    ("mxfp4", 38, 897, 12800, 3, 5),     # ... and a wave of pairs of attention tiles, the rest in small CTAs
     ("mxfp4", 37, 8192, 130, 3, 4),      # Q, K and V quantized apart; whole waves
     ("mxfp4", 38, 8192, 1000, 11, 3),    # rotated; the last wave with the others
-    ("mxfp4", 38, 897, 6200, 11, 4),     # ... and in small CTAs
+    ("mxfp4", 38, 897, 12800, 11, 4),    # ... and in small CTAs
     ("nvfp4", 2, 300, 300, 0, 4),        # zeroing, maxima, operands, attention
     ("nvfp4", 37, 8192, 130, 2, 6),      # Q, K and V apart
     ("bf16", 2, 300, 300, 0, 2),         # zeroing, attention

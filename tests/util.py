@@ -25,17 +25,25 @@ def operand_launches(cfg, rotate=False) -> int:
     return 3 if half_tiles > 24 * torch.cuda.get_device_properties(0).multi_processor_count else 1
 
 
-class _RowSplit(ctypes.Structure):
-    _fields_ = [("pairs_256", ctypes.c_int64), ("R", ctypes.c_int)]
+class _Plan(ctypes.Structure):
+    _fields_ = [("walk", ctypes.c_bool), ("pairs", ctypes.c_int64), ("R", ctypes.c_int)]
 
 
-def row_split(n_sm, heads, nq, nkv, pnq):
-    """What the MXFP4 forward gives to CTAs of 256 query rows (pairs of query tiles) and, if R > 0, to CTAs of 128/R rows."""
+def plan(n_sm, heads, nq, nkv, pnq, followed=False):
+    """How the MXFP4 forward's launch divides a problem, asked of the library: (pairs of query tiles, R) = what one kernel takes (the walking
+    one: `walked`), and 128/R rows per CTA for the rest, 0 if there is none."""
     import paper_2607_24377_b200 as mx
-    f = mx.lib()._ZN6mxattn17forward_row_splitEllllb
-    f.argtypes, f.restype = [ctypes.c_int64] * 4 + [ctypes.c_bool], _RowSplit
-    s = f(n_sm, heads, nq, nkv, pnq)
-    return s.pairs_256, s.R
+    f = mx.lib()._ZN6mxattn12forward_planEllllbb
+    f.argtypes, f.restype = [ctypes.c_int64] * 4 + [ctypes.c_bool] * 2, _Plan
+    p = f(n_sm, heads, nq, nkv, pnq, followed)
+    return p.pairs, p.R
+
+
+def walked(n_sm, heads, nq, nkv, pnq, followed=False):
+    """Whether what `plan` does not give to small CTAs goes to the walking kernel (otherwise: the one for pairs of query tiles)."""
+    plan(1, 1, 1, 1, True)
+    import paper_2607_24377_b200 as mx
+    return mx.lib()._ZN6mxattn12forward_planEllllbb(n_sm, heads, nq, nkv, pnq, followed).walk
 
 
 def tile_code_offset(r, c):

@@ -113,7 +113,7 @@ static bool carve(int B, int H, int64_t Nq, int64_t Nkv, int d, WorkspaceLayout*
 static int forward_ws(const void* q, const void* k, const void* v, void* o, int B, int H, int64_t Nq,
                       int64_t Nkv, int d, float softmax_scale, unsigned flags, void* workspace,
                       size_t workspace_bytes, cudaStream_t stream, void* dump = nullptr,
-                      cudaStream_t qstream = nullptr, cudaEvent_t qdone = nullptr, bool profile = false, bool followed = false) {
+                      cudaStream_t qstream = nullptr, cudaEvent_t qdone = nullptr, void* profile = nullptr, bool followed = false) {
   if (!q || !k || !v || !o) return MXATTN_EINVAL;
   if (B <= 0 || H <= 0 || Nq <= 0 || Nkv <= 0) return MXATTN_EINVAL;
   if (flags & ~(unsigned)(MXATTN_FLAG_UOS | MXATTN_FLAG_PNQ | MXATTN_FLAG_OUT_FP32 | MXATTN_FLAG_HADAMARD)) return MXATTN_EINVAL;
@@ -241,7 +241,7 @@ extern "C" int mxattn_forward_cycle_profile(const void* q, const void* k, const 
   if (profile_bytes < forward_profile_bytes(B, H, Nq, Nkv)) return MXATTN_EWORKSPACE;
   if (!aligned16(profile)) return MXATTN_EALIGN;
   return forward_ws(q, k, v, o, B, H, Nq, Nkv, d, softmax_scale, flags, workspace, workspace_bytes,
-                    (cudaStream_t)stream, profile, nullptr, nullptr, true);
+                    (cudaStream_t)stream, nullptr, nullptr, nullptr, profile);
 }
 
 extern "C" int mxattn_forward_prequantized(const void* q_codes, const void* q_scales, const void* k_codes,
@@ -408,7 +408,7 @@ extern "C" int mxattn_forward_host(const void* q_host, const void* k_host, const
     // n heads); its operands are quantized on a stream of their own, behind the copies and ahead of the attention
     // launch, so that they fill the SMs the previous stage's attention kernel frees as it drains
     rc = forward_ws(dq + i * qh, dk + i * kh, dv + i * kh, dout + i * oh, 1, (int)n, Nq, Nkv, d, softmax_scale, flags,
-                    ws + i * w.total, n * w.total, as, nullptr, hp->quant, ev[3 * st + 1], false, st + 1 < stages || !last_alone);
+                    ws + i * w.total, n * w.total, as, nullptr, hp->quant, ev[3 * st + 1], nullptr, st + 1 < stages || !last_alone);
     ck(cudaEventRecord(ev[3 * st + 2], as));
     ck(cudaStreamWaitEvent(hp->out, ev[3 * st + 2], 0));
     ck(cudaMemcpyAsync(static_cast<char*>(o_host) + i * oh, dout + i * oh, n * oh, cudaMemcpyDeviceToHost, hp->out));

@@ -189,7 +189,7 @@ int launch_quantize_nvfp4(const void* in, void* codes, void* scales, const float
 int launch_forward(const void* q_codes, const void* q_scales, const void* k_codes,
                    const void* k_scales, const void* v_codes, const void* v_scales, void* o,
                    int B, int H, int64_t Nq, int64_t Nkv, float softmax_scale, unsigned flags,
-                   int* status, cudaStream_t stream, void* dump = nullptr, bool profile = false, bool followed = false);
+                   int* status, cudaStream_t stream, void* dump = nullptr, void* profile = nullptr, bool followed = false);
 constexpr int kStaticTiles = 23, kStaticTilesNv = 3;     // KV tiles up to which a CTA of the walking kernel (walk.cuh) has its items from the start: MXFP4, NVFP4
 // The first `pairs` pairs of query tiles, counted over all heads, go to the walking kernel (walk) or to the kernel for pairs, the rest to CTAs of
 // 128 / R rows (R = 0: there is none).  `followed`: other attention launches run beside.
@@ -200,7 +200,7 @@ int launch_forward_rows(int R, int64_t first_pair, const void* q_codes, const vo
                         float softmax_scale, unsigned flags, int* status, cudaStream_t stream);
 int launch_forward_walk(int64_t n_sm, int64_t pairs, const void* q_codes, const void* q_scales, const void* k_codes, const void* k_scales,
                         const void* v_codes, const void* v_scales, void* o, int B, int H, int64_t Nq, int64_t Nkv,
-                        float softmax_scale, unsigned flags, int* status, cudaStream_t stream);
+                        float softmax_scale, unsigned flags, int* status, cudaStream_t stream, void* dump = nullptr);
 size_t forward_dump_bytes(int B, int H, int64_t Nq, int64_t Nkv);
 size_t forward_profile_bytes(int B, int H, int64_t Nq, int64_t Nkv);
 size_t bf16_workspace_bytes(int B, int H, int64_t Nq, int64_t Nkv);

@@ -49,7 +49,7 @@
 // One CTA per work item (two query tiles of one head).  A launch that has the GPU to itself comes here only beyond what the
 // walking kernel counts (2^31 tiles); that kernel (forward_walk.cu) takes the others, and query tiles that would leave SMs idle go
 // to the kernel for few query rows (forward_rows.cu).  Here run the stages of a forward from host tensors that forward_walk.cu's
-// rules leave, the debug dump and the cycle profile.
+// rules leave, and the cycle profile.
 //
 // Every mbarrier wait is bounded; on expiry the CTA records a code in `status`, drains and exits.
 #include <string.h>
@@ -72,7 +72,6 @@ constexpr int kThreads = 32 * (kSoftmaxWarps + 2);   // softmax warps + producer
 constexpr int kStages = 4;
 constexpr int kNV = 144;                         // GEMM 2 N: 128 channels + 16 rows of ones
 constexpr int kVStageBytes = kNV * 64;           // 9216
-constexpr int kDumpTileBytes = kTileCodeBytes + kTileScaleBytes + kTile * 4;   // debug dump: codes, scale atom, m per row
 
 // shared memory map (byte offsets from a 1024-aligned base)
 constexpr int kOffQ = 0;                                   // 2 tiles x 8192
@@ -106,25 +105,23 @@ struct Params {
   const uint8_t* k_codes; const uint8_t* k_scales;
   const uint8_t* v_codes; const uint8_t* v_scales;
   int* status;
-  uint8_t* dump;        // per-tile P-hat images, scales, running maxima and final row sums (debug entry point only)
+  uint8_t* profile;     // kProf
   int64_t Nq, Nkv;
   int q_tiles, kv_tiles, q_pairs;
   int total_items;      // B * H * q_pairs work items (one = two query tiles of one head)
   float scale_log2e;    // softmax_scale * log2(e)
-  float softmax_scale;
 };
 
 // ---------------------------------------------------------------------------------------------
 // kProf (cycle profile, never in a timed build): every role accumulates SM cycles per phase of its loop and writes them
-// to p.dump as [CTA][warp 0..17][16] int64 (softmax warps: slots 0-8 = S-full wait, score load, maxima, pair
+// to p.profile as [CTA][warp 0..17][16] int64 (softmax warps: slots 0-8 = S-full wait, score load, maxima, pair
 // exchange, O-done wait, block exponents, exponentials + pack, hand-over, epilogue; slot 9 = tiles; producer and
 // issuer: slots 0-7 = cycles inside the wait with code c at slot c mod 8, slot 8 = cycles of the whole loop, slot 9 = tiles).
 #define MBAR_WAIT_ROLE(...) (kProf ? prof_wait(__VA_ARGS__) : mbar_wait(__VA_ARGS__))
 #define PROF_MARK(i) do { if (kProf) { const long long prof_now = clock64(); prof_t[i] += prof_now - prof_prev; prof_prev = prof_now; } } while (0)
 constexpr int kProfSlots = 16;
-template <bool kUos, bool kPnq, bool kOutF32, bool kDump, bool kProf = false>
+template <bool kUos, bool kPnq, bool kOutF32, bool kProf = false>
 __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, const __grid_constant__ CUtensorMap out_map) {
-  static_assert(!(kDump && kProf), "the dump buffer holds either the tile dump or the cycle profile");
   long long prof_t[kProfSlots];
   long long prof_prev = 0;
   if (kProf) {
@@ -439,12 +436,6 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
       // the scale bytes go out before the exponentials, so only the code stores precede the proxy fence
       sts16(aSF, sf_half);
       PROF_MARK(5);
-      uint8_t* dump_tile = nullptr;
-      if (kDump && 2 * pair + t < p.q_tiles) {       // image of this (query tile, KV tile): codes, scale atom, m
-        dump_tile = p.dump + ((((int64_t)bh * p.q_tiles + 2 * pair + t) * T) + j) * kDumpTileBytes;
-        *reinterpret_cast<uint16_t*>(dump_tile + kTileCodeBytes + tile_scale_offset(row, 2 * h)) = (uint16_t)sf_half;
-        if (h == 0) reinterpret_cast<float*>(dump_tile + kTileCodeBytes + kTileScaleBytes)[row] = m_new * p.softmax_scale;   // the kernel keeps m in unscaled score units
-      }
       float l_tile = 0.0f;
       const uint64_t cc2 = dup2(c);
       auto tile_body = [&](auto resc_tag) {
@@ -482,7 +473,6 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
             }
           }
           sts128(b == 0 ? aP0 : aP1, w);
-          if (kDump && dump_tile) *reinterpret_cast<uint4*>(dump_tile + tile_code_offset(row, kBlocksPerThread * h + b)) = w;
           if (!kPnq) l_tile = fmaf(sx, sigma[b], l_tile);   // Eq. 12
         }
         if (kResc) {
@@ -520,7 +510,6 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
     }
     if (ok) {
       tc_fence_after();
-      const int qtile = 2 * pair + t;
       if (kPnq) {
         uint32_t lr;
         asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(lr) : "r"(t_o + 128) : "memory");
@@ -528,9 +517,6 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
         l = __uint_as_float(lr);
       }
       const float inv_l = 1.0f / l;                // line 18 as one reciprocal and 64 multiplies per thread
-      if (kDump && h == 0 && qtile < p.q_tiles)
-        reinterpret_cast<float*>(p.dump + (int64_t)p.total_items / p.q_pairs * p.q_tiles * T * kDumpTileBytes)
-            [((int64_t)bh * p.q_tiles + qtile) * kTile + row] = l;
       // coordinates computed afresh: keeping those of the loop costs it registers (37 x 16384: 2874 -> 2849 us)
       const uint32_t tid2 = fresh_tid(), w = tid2 >> 5;
       const int bh2 = (int)blockIdx.x / p.q_pairs, qtile2 = 2 * ((int)blockIdx.x - bh2 * p.q_pairs) + (int)(w >> 3), col = kCols * ((w >> 2) & 1);
@@ -542,7 +528,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_kernel(const Params p, 
   }
 
   if (kProf && lane == 0) {
-    long long* dst = reinterpret_cast<long long*>(p.dump) + ((int64_t)blockIdx.x * (kThreads / 32) + warp) * kProfSlots;
+    long long* dst = reinterpret_cast<long long*>(p.profile) + ((int64_t)blockIdx.x * (kThreads / 32) + warp) * kProfSlots;
 #pragma unroll
     for (int i = 0; i < kProfSlots; ++i) dst[i] = prof_t[i];
   }
@@ -675,11 +661,6 @@ size_t forward_profile_bytes(int B, int H, int64_t Nq, int64_t Nkv) {
   return (size_t)((int64_t)B * H * ((qt + 1) / 2) * (fwd::kThreads / 32) * fwd::kProfSlots * 8);     // sized for one CTA per work item
 }
 
-size_t forward_dump_bytes(int B, int H, int64_t Nq, int64_t Nkv) {
-  const int64_t qt = (Nq + kTile - 1) / kTile, kt = (Nkv + kTile - 1) / kTile;
-  return (size_t)((int64_t)B * H * qt * kt * fwd::kDumpTileBytes + (int64_t)B * H * qt * kTile * 4);
-}
-
 PFN_cuTensorMapEncodeTiled tensor_map_encoder() {
   static std::atomic<void*> cached{nullptr};
   void* fn = cached.load(std::memory_order_acquire);
@@ -709,27 +690,26 @@ int encode_output_map(CUtensorMap* map, void* o, int64_t bh, int64_t Nq, bool f3
 
 int launch_forward(const void* q_codes, const void* q_scales, const void* k_codes, const void* k_scales,
                    const void* v_codes, const void* v_scales, void* o, int B, int H, int64_t Nq, int64_t Nkv,
-                   float softmax_scale, unsigned flags, int* status, cudaStream_t stream, void* dump, bool profile, bool followed) {
+                   float softmax_scale, unsigned flags, int* status, cudaStream_t stream, void* dump, void* profile, bool followed) {
   using namespace fwd;
   Params p;
   p.q_codes = (const uint8_t*)q_codes; p.q_scales = (const uint8_t*)q_scales;
   p.k_codes = (const uint8_t*)k_codes; p.k_scales = (const uint8_t*)k_scales;
   p.v_codes = (const uint8_t*)v_codes; p.v_scales = (const uint8_t*)v_scales;
-  p.status = status; p.dump = (uint8_t*)dump; p.Nq = Nq; p.Nkv = Nkv;
+  p.status = status; p.profile = (uint8_t*)profile; p.Nq = Nq; p.Nkv = Nkv;
   const int64_t qt = (Nq + kTile - 1) / kTile, kt = (Nkv + kTile - 1) / kTile;
   const int64_t pairs = (qt + 1) / 2;
   const int64_t grid = (int64_t)B * H * pairs;
   if (qt > 0x3FFFFFFF || kt > 0x3FFFFFFF || grid > 0x7FFFFFFF) return MXATTN_EUNSUPPORTED;
   p.q_tiles = (int)qt; p.kv_tiles = (int)kt; p.q_pairs = (int)pairs; p.total_items = (int)grid;
   p.scale_log2e = softmax_scale * 1.4426950408889634f;
-  p.softmax_scale = softmax_scale;
 
   const bool uos = flags & MXATTN_FLAG_UOS, pnq = flags & MXATTN_FLAG_PNQ, f32 = flags & MXATTN_FLAG_OUT_FP32;
   const int n_sm = sm_count();
   if (n_sm == 0) return MXATTN_ECUDA;
-  const ForwardPlan plan = dump ? ForwardPlan{false, grid, 0} : forward_plan(n_sm, (int64_t)B * H, Nq, Nkv, pnq, followed);
+  const ForwardPlan plan = dump || profile ? ForwardPlan{dump != nullptr, grid, 0} : forward_plan(n_sm, (int64_t)B * H, Nq, Nkv, pnq, followed);
   if (plan.walk) {
-    const int rc = plan.pairs == 0 ? (int)MXATTN_OK : launch_forward_walk(n_sm, plan.pairs, q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, o, B, H, Nq, Nkv, softmax_scale, flags, status, stream);
+    const int rc = plan.pairs == 0 ? (int)MXATTN_OK : launch_forward_walk(n_sm, plan.pairs, q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, o, B, H, Nq, Nkv, softmax_scale, flags, status, stream, dump);
     if (rc != MXATTN_OK || plan.R == 0) return rc;
     return launch_forward_rows(plan.R, plan.pairs, q_codes, q_scales, k_codes, k_scales, v_codes, v_scales, o, B, H, Nq, Nkv, softmax_scale, flags, status, stream);
   }
@@ -739,18 +719,13 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
   void (*kern)(const Params, const CUtensorMap) = nullptr;
 #define PICK(U, P, F)                                                                     \
   if (uos == U && pnq == P && f32 == F)                                                   \
-    kern = attention_kernel<U, P, F, false>;
+    kern = attention_kernel<U, P, F>;
   PICK(false, false, false) PICK(false, false, true) PICK(false, true, false) PICK(false, true, true)
   PICK(true, false, false) PICK(true, false, true) PICK(true, true, false) PICK(true, true, true)
 #undef PICK
   if (profile) {                                  // cycle profile: the UOS + PNQ, bf16-output kernels with the counters compiled in
-    if (!dump || !uos || !pnq || f32) return MXATTN_EINVAL;
-    kern = attention_kernel<true, true, false, false, true>;
-  } else if (dump) {                              // debug entry point: fp32 output only
-    if (!f32) return MXATTN_EINVAL;
-#define PICKD(U, P) if (uos == U && pnq == P) kern = attention_kernel<U, P, true, true>;
-    PICKD(false, false) PICKD(false, true) PICKD(true, false) PICKD(true, true)
-#undef PICKD
+    if (!uos || !pnq || f32) return MXATTN_EINVAL;
+    kern = attention_kernel<true, true, false, true>;
   }
   if (!ensure_dynamic_smem((const void*)kern, kSmemBytes)) return MXATTN_ECUDA;
   return launch_pdl(kern, dim3((unsigned)grid), kThreads, kSmemBytes, stream, p, out_map) == cudaSuccess ? MXATTN_OK : MXATTN_ECUDA;

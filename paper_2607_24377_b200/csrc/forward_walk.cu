@@ -4,7 +4,7 @@
 namespace mxattn {
 namespace walk {
 
-template <bool kUos, bool kPnq, bool kOutF32, bool kTake>
+template <bool kUos, bool kPnq, bool kOutF32, bool kTake, bool kDump>
 __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Params p, const __grid_constant__ CUtensorMap out_map) {
   using L = Lay<false>;
   extern __shared__ uint8_t smem_raw[];
@@ -26,7 +26,7 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
   pdl_trigger();
   if (*tmem_slot != 0) *abort_flag = kCodeTmemBase;
   const int role = __shfl_sync(0xFFFFFFFFu, (*status_before != 0 || *tmem_slot != 0) ? kThreads / 32 : warp, 0);     // an earlier launch gave up
-  play<false, kUos, kPnq, kOutF32, kTake>(p, out_map, smem, role, warp, lane);
+  play<false, kUos, kPnq, kOutF32, kTake, kDump>(p, out_map, smem, role, warp, lane);
   tc_fence_before();
   __syncthreads();
   if (tid == 0 && *abort_flag != 0) atomicCAS(p.status, 0, *abort_flag);
@@ -85,10 +85,15 @@ ForwardPlan forward_plan(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool
   return ForwardPlan{true, total, 0};
 }
 
-// The first `pairs` pairs of query tiles, counted over all heads.
+size_t forward_dump_bytes(int B, int H, int64_t Nq, int64_t Nkv) {
+  const int64_t qt = (Nq + kTile - 1) / kTile, kt = (Nkv + kTile - 1) / kTile;
+  return (size_t)((int64_t)B * H * qt * kt * walk::kDumpTileBytes + (int64_t)B * H * qt * kTile * 4);
+}
+
+// The first `pairs` pairs of query tiles, counted over all heads.  `dump`: all of them.
 int launch_forward_walk(int64_t n_sm, int64_t pairs, const void* q_codes, const void* q_scales, const void* k_codes, const void* k_scales,
                         const void* v_codes, const void* v_scales, void* o, int B, int H, int64_t Nq, int64_t Nkv,
-                        float softmax_scale, unsigned flags, int* status, cudaStream_t stream) {
+                        float softmax_scale, unsigned flags, int* status, cudaStream_t stream, void* dump) {
   using namespace walk;
   Params p = {};
   p.q_codes = (const uint8_t*)q_codes; p.q_scales = (const uint8_t*)q_scales;
@@ -99,13 +104,19 @@ int launch_forward_walk(int64_t n_sm, int64_t pairs, const void* q_codes, const 
   const int64_t per_head = (p.q_tiles + 1) / 2, items = pairs / per_head * p.q_tiles + (pairs % per_head) * 2;
   if (items > 0x7FFFFFFF) return MXATTN_EUNSUPPORTED;
   p.total_items = (int)items;
-  p.scale_log2e = softmax_scale * 1.4426950408889634f;
+  p.scale_log2e = softmax_scale * 1.4426950408889634f; p.softmax_scale = softmax_scale; p.dump = (uint8_t*)dump;
   const bool uos = flags & MXATTN_FLAG_UOS, pnq = flags & MXATTN_FLAG_PNQ, f32 = flags & MXATTN_FLAG_OUT_FP32, take = takes<false>(p, n_sm);
   Kernel kern = nullptr;
-#define PICK(U, P, F) if (uos == U && pnq == P && f32 == F) kern = take ? attention_walk_kernel<U, P, F, true> : attention_walk_kernel<U, P, F, false>;
+#define PICK(U, P, F) if (uos == U && pnq == P && f32 == F) kern = take ? attention_walk_kernel<U, P, F, true, false> : attention_walk_kernel<U, P, F, false, false>;
   PICK(false, false, false) PICK(false, false, true) PICK(false, true, false) PICK(false, true, true)
   PICK(true, false, false) PICK(true, false, true) PICK(true, true, false) PICK(true, true, true)
 #undef PICK
+  if (dump) {
+    if (!f32) return MXATTN_EINVAL;
+#define PICK(U, P) if (uos == U && pnq == P) kern = take ? attention_walk_kernel<U, P, true, true, true> : attention_walk_kernel<U, P, true, false, true>;
+    PICK(false, false) PICK(false, true) PICK(true, false) PICK(true, true)
+#undef PICK
+  }
   return launch(kern, Lay<false>::kSmemBytes, p, take, n_sm, (int64_t)B * H, o, flags, stream);
 }
 

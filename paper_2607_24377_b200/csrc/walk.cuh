@@ -132,7 +132,10 @@ struct Params {
   int64_t Nq, Nkv;
   int q_tiles, kv_tiles, first_item, total_items;                // items from first_item on; their number
   float scale_log2e;
+  float softmax_scale;                                           // kDump
+  uint8_t* dump;                                                 // per tile P-hat's image, scales and running maxima, then the row sums (include/mxattn.h)
 };
+constexpr int kDumpTileBytes = kTileCodeBytes + kTileScaleBytes + kTile * 4;
 
 // Shared-memory accesses at a register plus a constant: addresses formed in front of each access cost the softmax warps
 // instructions, and kept ones registers.
@@ -294,8 +297,9 @@ __device__ __forceinline__ void set_up(uint8_t* smem, int tid) {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
-// The part of one warp, between the setup and the teardown.
-template <bool kNv, bool kUos, bool kPnq, bool kOutF32, bool kTake>
+// The part of one warp, between the setup and the teardown.  kDump (MXFP4): what the softmax warps hand to the output products, and the row
+// sums, are written out as well.
+template <bool kNv, bool kUos, bool kPnq, bool kOutF32, bool kTake, bool kDump = false>
 __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map, uint8_t* smem, int role, int warp, int lane) {
   using L = Lay<kNv>;
   const uint32_t sbase = smem_u32(smem);
@@ -566,6 +570,7 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
         l = __uint_as_float(lr);
       }
       const float inv_l = (kNv ? o_scale : 1.0f) / l;
+      if (kDump) reinterpret_cast<float*>(p.dump + (int64_t)p.total_items * T * kDumpTileBytes)[(int64_t)item * kTile + q * 32 + lane] = l;
       if (lds_volatile(abort_addr) != 0) {                       // given up: this item and later ones are not stored, and the output products wait for this warp once more at most
         asm volatile("bar.arrive %0, %1;" ::"r"(kBarP + (f & 3)), "n"(kPThreads) : "memory");
         break;
@@ -702,9 +707,15 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
       const float prev = jn >= 1 ? fmaxf(mp.x, mp.y) : -INFINITY, run = jn >= 2 ? m_run : -INFINITY;
       const float m_new = max3(fmaxf(mo.x, mo.y), prev, run);    // line 10
       m_run = m_new;
+      uint8_t* image = nullptr;                                  // kDump: of this tile
+      if (kDump) {
+        const int item = kTake ? items[n_own & 7] : (int)blockIdx.x + n_own * (int)gridDim.x;
+        image = p.dump + ((int64_t)item * T + jn) * kDumpTileBytes;
+        if (h == 0) reinterpret_cast<float*>(image + kTileCodeBytes + kTileScaleBytes)[row] = m_new * p.softmax_scale;     // (m is kept in unscaled score units)
+      }
       jn += 2;
-      if (jn >= T) { jn -= T; if (kNv) ++n_own; }
-      if (jn >= T) { jn -= T; if (kNv) ++n_own; }                // T = 1; left out where T is larger, PNQ takes 9 % longer (24 x 8192)
+      if (jn >= T) { jn -= T; if (kNv || kDump) ++n_own; }
+      if (jn >= T) { jn -= T; if (kNv || kDump) ++n_own; }                // T = 1; left out where T is larger, PNQ takes 9 % longer (24 x 8192)
       // NVFP4, the scales of the other 32 keys (two exponentials, a table): in front of the first exponentials, or in the gap where
       // their scores are loaded.  There the score buffer is given back later, which short sequences with PNQ do not make up for.
       // Whole call, us, in front / in the gap: direct 40 x 16384 3770 / 3710, 24 x 8192 646 / 636, 40 x 4096 299.7 / 297.7, 40 x 18900 x
@@ -723,6 +734,7 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
         exponent(b0, m_new, nb0, sf0);
         exponent(b1, m_new, nb1, sf1);
         sts16o<2 * k * L::kSF>(aSF, sf0 | (sf1 << 8));
+        if (kDump) *reinterpret_cast<uint16_t*>(image + kTileCodeBytes + tile_scale_offset(row, 2 * h)) = (uint16_t)(sf0 | (sf1 << 8));
       }
       float sx0 = 0.0f, sx1 = 0.0f;
       uint32_t w[4];
@@ -735,6 +747,7 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
         sts32o<2 * k * L::kSF>(aSF, __uint_as_float(sf0 | (sf1 << 16)));
       }
       sts128o<2 * k * kTileCodeBytes>(aP0, w);
+      if (kDump) *reinterpret_cast<uint4*>(image + tile_code_offset(row, 2 * h)) = make_uint4(w[0], w[1], w[2], w[3]);
       TMEM_LD_WAIT32(s1);
       tc_fence_before();
       __syncwarp();
@@ -746,6 +759,7 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
         if (g == 1) { meet_others(); here(p.kv_tiles); }
       }
       sts128o<2 * k * kTileCodeBytes>(aP1, w);
+      if (kDump) *reinterpret_cast<uint4*>(image + tile_code_offset(row, 2 * h + 1)) = make_uint4(w[0], w[1], w[2], w[3]);
       if (!kPnq) {
         sts32o<L::kOffXL - L::kOffX>(aM + 4 * h + xl, kNv ? sx0 : fmaf(sx1, __uint_as_float(sf1 << 23), fmaf(sx0, __uint_as_float(sf0 << 23), 0.0f)));   // Eq. 12
         xl = (xl + 2 * kXSlot) & (8 * kXSlot - 1);

@@ -1,5 +1,6 @@
-"""Tile-level parity of the softmax loop (Algorithm 2 lines 10-14) through the debug-dump entry point:
-the quantized probabilities P-hat are compared with the oracle's value for value, tile by tile."""
+"""Tile-level parity of the softmax loop (Algorithm 2 lines 10-14) through the debug-dump entry point (the walking kernel, which
+also writes out what it hands to the output products): the quantized probabilities P-hat are compared with the oracle's value for
+value, tile by tile."""
 import numpy as np
 import pytest
 import torch
@@ -79,6 +80,17 @@ def test_outlier_scores_p_hat():
     q, k, v = si.make_all(cfg)
     n_elem, n_diff = check_tiles(cfg, q, k, v, True, True)
     assert n_diff <= n_elem // 2000, (n_diff, n_elem)
+
+
+# More query tiles than SMs: CTAs with several items, whose shares are fixed (3 KV tiles), and which are taken (24)
+@pytest.mark.parametrize("H,nq,nkv,uos,pnq", [(12, 1700, 300, True, True), (12, 1700, 300, False, False), (10, 1900, 24 * 128 - 31, True, True),
+                                              (10, 1900, 24 * 128 - 31, True, False)])
+def test_p_hat_of_walked_items(H, nq, nkv, uos, pnq):
+    assert H * -(-nq // 128) > torch.cuda.get_device_properties(0).multi_processor_count
+    cfg = si.custom_config("w", 1, H, nq, nkv, 79)
+    q, k, v = si.make_all(cfg)
+    n_elem, n_diff = check_tiles(cfg, q, k, v, uos, pnq)
+    assert n_diff <= 4e-6 * n_elem, (n_diff, n_elem)                     # the share that the first test allows
 
 
 def test_debug_dump_argument_errors():

@@ -44,8 +44,10 @@ __global__ void __launch_bounds__(kThreads, 1) attention_walk_kernel(const Param
 //  - CTAs of 32 rows where they are one wave at most: they take two thirds to nine tenths of the time whatever the length (18 x 256 queries, 1,
 //    4, 16, 64, 300 KV tiles, walked 4.59 6.63 14.7 45.4 187 / 4.79 7.11 16.1 50.7 214, 32 rows 3.37 5.30 12.5 39.1 158 / 3.39 5.41 13.1 41.8
 //    175).  A second wave of them never pays (37 x 256, 64 tiles: 45.6 / 50.9, 32 rows 76.7 / 82.7).
-//  - CTAs of 64 rows where those are one wave, up to 13 KV tiles (direct 14; 37 x 256, 1, 4, 8, 16, 32 tiles: walked 4.62 6.69 9.40 14.8 25.4 / 4.81 7.18 10.2 16.1
-//    28.0, 64 rows 3.82 6.04 9.02 14.9 26.5 / 3.94 6.42 9.78 16.2 29.1).
+//  - CTAs of 64 rows where those are one wave, up to 6 KV tiles (direct 14; 37 x 256, 1, 4, 8, 16, 32 tiles: walked 4.62 6.69 9.40 14.8 25.4 /
+//    4.81 7.18 10.2 16.1 28.0, 64 rows 3.82 6.04 9.02 14.9 26.5 / 3.94 6.42 9.78 16.2 29.1).  In a whole call the operand launch's last CTAs decide
+//    as well: of 21 problems with PNQ at 5 tiles one takes longer with 64 rows (by 1 %), at 7 and 9 tiles they are 3 and 2 % ahead in the
+//    mean, but five behind by up to 4 % (6 x 889 x 889 11.3 / 11.9).
 //  - Whole waves of pairs walked and the rest in one wave of CTAs of 32 rows, a second launch, if that is estimated to take less than the
 //    rounds of single tiles it saves.  A round: T x 1150 + 4500 cycles (direct 1335, 3500); the second launch with the wait for the first's last
 //    CTAs: T x 1045 + 12000 (1175, 8000).  152 x 256, 32, 64, 128, 300 tiles: all walked 67.9 127.7 244.1 548.9 / 75.6 144.4 279.0 635.5,
@@ -75,7 +77,7 @@ ForwardPlan forward_plan(int64_t n_sm, int64_t bh, int64_t Nq, int64_t Nkv, bool
   const int64_t at = total / n_sm * n_sm;
   if (at == 0) {
     if (groups(4, 0) <= n_sm) return ForwardPlan{true, 0, 4};
-    if (groups(2, 0) <= n_sm && T <= (pnq ? 13 : 14)) return ForwardPlan{true, 0, 2};
+    if (groups(2, 0) <= n_sm && T <= (pnq ? 6 : 14)) return ForwardPlan{true, 0, 2};
   }
   if (!counts) return ForwardPlan{false, total, 0};
   if (at > 0 && at < total && groups(4, at) <= n_sm) {

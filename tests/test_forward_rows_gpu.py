@@ -74,14 +74,14 @@ def test_last_wave_cut_into_small_ctas(heads, nq, nkv, pnq):
     assert torch.equal(run(many, rep(q), rep(k), rep(v), flags), want.expand(1, heads, nq, 128))
 
 
-# 64 rows per CTA (from 44 heads on: walked): every head must come out as it does among 148, which are walked
-@pytest.mark.parametrize("heads,nq,nkv,split", [(49, 127, 300, (0, 2)), (70, 65, 1100, (0, 2)), (49, 128, 640, (0, 2)), (60, 127, 13 * 128, (0, 2)),
+# 64 rows per CTA (70 x 1100 with PNQ and from 44 heads on: walked): every head must come out as it does among 148, which are walked
+@pytest.mark.parametrize("heads,nq,nkv,split", [(49, 127, 300, (0, 2)), (70, 65, 1100, (70, 0)), (49, 128, 640, (0, 2)), (60, 127, 6 * 128, (0, 2)),
                                                 (44, 1000, 700, (176, 0)), (45, 897, 1300, (180, 0)), (50, 1000, 700, (200, 0))])
 @pytest.mark.parametrize("pnq", [True, False])
 def test_64_rows_per_cta_equal_the_walking_kernel(heads, nq, nkv, split, pnq):
     import paper_2607_24377_b200 as mx
     flags = mx.FLAG_UOS | (mx.FLAG_PNQ if pnq else 0)
-    assert rows_per_cta(heads, nq, nkv, pnq) == split and rows_per_cta(148, nq, nkv, pnq)[1] == 0
+    assert rows_per_cta(heads, nq, nkv, pnq) == ((0, 2) if nkv == 1100 and not pnq else split) and rows_per_cta(148, nq, nkv, pnq)[1] == 0
     few = si.custom_config("h64", 1, heads, nq, nkv, 8)
     q, k, v = si.make_all(few)
     got = run(few, q, k, v, flags)

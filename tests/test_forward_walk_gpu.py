@@ -18,8 +18,8 @@ def test_what_the_walking_kernel_takes(pnq):
 
 @pytest.mark.parametrize("pnq", [True, False])
 def test_small_problems_go_to_small_ctas(pnq):
-    # one wave of 32 rows, whatever the length; one of 64 rows up to 13 KV tiles (direct row sum 14); none of 128
-    for heads, nq, nkv, pairs, r in ((1, 1, 1, 0, 4), (2, 1024, 1024, 0, 4), (1, 4096, 40000, 0, 4), (37, 128, 4096, 0, 4), (37, 129, 1664, 0, 2), (1, 4737, 1664, 0, 2),
+    # one wave of 32 rows, whatever the length; one of 64 rows up to 6 KV tiles (direct row sum 14); none of 128
+    for heads, nq, nkv, pairs, r in ((1, 1, 1, 0, 4), (2, 1024, 1024, 0, 4), (1, 4096, 40000, 0, 4), (37, 128, 4096, 0, 4), (37, 129, 768, 0, 2), (1, 4737, 768, 0, 2), (1, 4737, 769, *((19, 0) if pnq else (0, 2))),
                                      (1, 9472, 128, 0, 2), (1, 4737, 14 * 128, *((19, 0) if pnq else (0, 2))), (1, 4737, 1793, 19, 0), (1, 9473, 128, 38, 0), (38, 256, 128, 38, 0), (12, 1300, 128, 72, 0)):
         assert util.plan(148, heads, nq, nkv, pnq) == (pairs, r), (heads, nq, nkv)
 

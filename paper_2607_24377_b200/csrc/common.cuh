@@ -190,7 +190,7 @@ int launch_forward(const void* q_codes, const void* q_scales, const void* k_code
                    const void* k_scales, const void* v_codes, const void* v_scales, void* o,
                    int B, int H, int64_t Nq, int64_t Nkv, float softmax_scale, unsigned flags,
                    int* status, cudaStream_t stream, void* dump = nullptr, void* profile = nullptr, bool followed = false);
-constexpr int kStaticTiles = 23, kStaticTilesNv = 3;     // KV tiles up to which a CTA of the walking kernel (walk.cuh) has its items from the start: MXFP4, NVFP4
+constexpr int kStaticTiles = 48, kStaticTilesNv = 3;     // KV tiles up to which a CTA of the walking kernel (walk.cuh) has its items from the start: MXFP4, NVFP4
 // The first `pairs` pairs of query tiles, counted over all heads, go to the walking kernel (walk) or to the kernel for pairs, the rest to CTAs of
 // 128 / R rows (R = 0: there is none).  `followed`: other attention launches run beside.
 struct ForwardPlan { bool walk; int64_t pairs; int R; };

@@ -3,14 +3,14 @@
 //
 // One CTA per SM walks work items of one query tile (128 rows of one head); the tiles of all its items form one stream
 // f = 0, 1, 2, ... (KV tiles of 128 keys in ascending order within an item), and barriers, tensor memory and the pipelines
-// run on across items.  Up to 23 KV tiles (kStaticTiles; NVFP4 3) a CTA's items are fixed at the launch, every 148th.  Above, the grid has
+// run on across items.  Up to 48 KV tiles (kStaticTiles; NVFP4 3) a CTA's items are fixed at the launch, every 148th.  Above, the grid has
 // a CTA per item, and a CTA that is done with an item takes over one that has not started (kTake): with fixed shares a launch
 // beside that holds a few SMs for long leaves whole shares to come last.  Whole call, us, beside 4 CTAs that stay, fixed / taken:
-// 24 x 8192 937 / 550 (direct row sum 1023 / 589), 40 x 4096 393 / 248 (432 / 270), NVFP4 40 x 4096 453 / 293 (490 / 318), 40 x 8192 x
-// 1024 272 / 178.  Alone, fixed / taken: MXFP4, attention launch, 40 x 8192 at 5, 8, 16 tiles 67.4 / 70.5, 103.1 / 106.0, 198.9 / 200.4,
-// 24 x 8192 at 24, 48 181.5 / 181.4, 351.0 / 348.7, 37 x 1000 at 24 36.5 / 36.7; NVFP4, whole call, 40 x 18900 at 1, 2, 3, 4 tiles 136.1 / 141.5,
-// 160.1 / 167.2, 190.6 / 194.4, 219.0 / 221.3, 24 x 8192 at 4, 16, 48 66.4 / 66.6, 173.4 / 169.6, 445.3 / 433.5.  (NVFP4 at up to 3
-// tiles: with a share that comes last the call still takes less than with two query tiles per CTA, 297 us at 40 x 18900 x 384.)
+// 24 x 8192 937 / 550 (direct row sum 1023 / 589), NVFP4 40 x 4096 453 / 293 (490 / 318), 40 x 8192 x 1024 272 / 178.  Alone, NVFP4, fixed /
+// taken: 40 x 18900 at 1, 2, 3, 4 tiles 136.1 / 141.5, 160.1 / 167.2, 190.6 / 194.4, 219.0 / 220.9, 24 x 8192 at 4, 16, 48 66.4 / 66.4, 172.8 /
+// 169.2, 445.3 / 433.5; up to 3 tiles a call whose last share comes late still takes less than with two query tiles per CTA (297 us at
+// 40 x 18900 x 384).  MXFP4 below 49 tiles stays with fixed shares: alone, taken ones are up to 2 % behind (24 x 30000 at 24 tiles, fp32
+// output; direct row sum, 24 to 48 tiles, up to 1 %), beside a launch that holds SMs they would be ahead (40 x 4096 393 / 248).
 // Roles (736 threads):
 //   warps 0-15   softmax, two teams of eight: team f & 1 takes tile f.  Two threads a row, one half of 64 keys each.  A team
 //                has a score buffer of its own, so that neither waits for the other to take its scores; what passes from

@@ -82,9 +82,9 @@ def test_outlier_scores_p_hat():
     assert n_diff <= n_elem // 2000, (n_diff, n_elem)
 
 
-# More query tiles than SMs: CTAs with several items, whose shares are fixed (3 KV tiles), and which are taken (24)
-@pytest.mark.parametrize("H,nq,nkv,uos,pnq", [(12, 1700, 300, True, True), (12, 1700, 300, False, False), (10, 1900, 24 * 128 - 31, True, True),
-                                              (10, 1900, 24 * 128 - 31, True, False)])
+# More query tiles than SMs: CTAs with several items, whose shares are fixed (3 KV tiles), and which are taken (49)
+@pytest.mark.parametrize("H,nq,nkv,uos,pnq", [(12, 1700, 300, True, True), (12, 1700, 300, False, False), (10, 1900, 49 * 128 - 31, True, True),
+                                              (10, 1900, 49 * 128 - 31, True, False)])
 def test_p_hat_of_walked_items(H, nq, nkv, uos, pnq):
     assert H * -(-nq // 128) > torch.cuda.get_device_properties(0).multi_processor_count
     cfg = si.custom_config("w", 1, H, nq, nkv, 79)

@@ -45,10 +45,10 @@ def test_beside_other_launches(pnq):
 
 
 def test_tiles_of_a_cta_are_counted_in_32_bits():
-    # above 23 tiles, where a CTA takes items that others have not begun, they may all be its own; with fixed shares it has its own only
-    for n, nkv, by_walk in ((72 << 20, 72 << 20, False), (6_000_000, 6_000_000, False), (5_900_000, 5_900_000, True), (1 << 30, 24 * 128, True), (1 << 37, 23 * 128, True)):
+    # above 48 tiles, where a CTA takes items that others have not begun, they may all be its own; with fixed shares it has its own only
+    for n, nkv, by_walk in ((72 << 20, 72 << 20, False), (6_000_000, 6_000_000, False), (5_900_000, 5_900_000, True), (1 << 30, 49 * 128, True), (1 << 36, 20 * 128, True)):
         tiles, t = -(-n // 128), -(-nkv // 128)
-        assert ((tiles if t > 23 else -(-tiles // 148)) * t <= 0x7FFFFF00) == by_walk
+        assert ((tiles if t > 48 else -(-tiles // 148)) * t <= 0x7FFFFF00) == by_walk
         for pnq in (True, False):
             assert util.walked(148, 1, n, nkv, pnq) == by_walk and util.plan(148, 1, n, nkv, pnq)[0] == (tiles + 1) // 2
 
@@ -111,11 +111,11 @@ def test_scores_that_are_not_numbers(nq, nkv, pnq):
     assert torch.equal(torch.nan_to_num(outs[1]), torch.nan_to_num(want))
 
 
-# Above 23 KV tiles the CTAs take one item after another from the grid: several different items each (three heads, so that a CTA
+# Above 48 KV tiles the CTAs take one item after another from the grid: several different items each (three heads, so that a CTA
 # never sees one head again and again), tile counts that swap the teams' roles from item to item and ones that do not, query and
 # key counts that end inside a tile; two launches back to back, and one beside a launch that holds some of the SMs.
 @pytest.mark.gpu
-@pytest.mark.parametrize("nq,nkv", [(129, 24 * 128), (257, 25 * 128 - 31), (129, 49 * 128), (300, 49 * 128 + 1), (257, 51 * 128 - 31), (385, 64 * 128 + 77), (130, 127 * 128 + 5)])
+@pytest.mark.parametrize("nq,nkv", [(129, 49 * 128), (300, 49 * 128 + 1), (257, 51 * 128 - 31), (385, 64 * 128 + 77), (130, 127 * 128 + 5)])
 @pytest.mark.parametrize("uos,pnq,f32", [(True, True, False), (True, False, True), (False, True, True), (False, False, False)])
 def test_taken_items_equal_a_single_head(nq, nkv, uos, pnq, f32):
     import paper_2607_24377_b200 as mx
@@ -157,7 +157,7 @@ def test_taken_items_equal_a_single_head(nq, nkv, uos, pnq, f32):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("fmt,heads,n,nkv", [("mxfp4", 24, 8192, 8192), ("mxfp4", 40, 4096, 24 * 128), ("nvfp4", 40, 4096, 4096), ("nvfp4", 40, 18900, 512)])
+@pytest.mark.parametrize("fmt,heads,n,nkv", [("mxfp4", 24, 8192, 8192), ("nvfp4", 40, 4096, 4096), ("nvfp4", 40, 18900, 512)])
 def test_a_launch_that_holds_few_sms_does_not_hold_up_whole_shares(fmt, heads, n, nkv):
     """24 heads of 8192: ten and a half items per SM.  Beside 4 CTAs that run for 8 ms, the items of those 4 SMs are
     spread over the others (about 1.1 times the time alone); with shares that are fixed at the launch they come last (1.5 to 1.6 times)."""

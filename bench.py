@@ -446,13 +446,17 @@ def main():
                         "extrapolated_full_workload_hours": cfg.flops / (tf_all * 1e12) / 3600.0}
 
     clocks = sampler.summary()
-    mufu_ceiling = 16 * 512 * 148 * clocks["sm_mhz"] * 1e6 / 1e12 if clocks.get("sm_mhz") else None
+    # exponentials that the walking kernel takes on the exponential unit with the PNQ row sum (the others are a polynomial on the
+    # multipliers): 12 of 16 where its CTAs take items from one another, above 48 KV tiles, 13 of 16 below
+    mufu_share = 12 / 16 if Nkv > 48 * 128 else 13 / 16
+    mufu_ceiling = 16 * 512 * 148 / mufu_share * clocks["sm_mhz"] * 1e6 / 1e12 if clocks.get("sm_mhz") else None
     # Roofline of the dominant kernel.  Denominator: the dense FP4 rate measured just above with the library's own
     # block-scaled GEMM probe ("of measured"); without the probe, the measured sustained cuBLAS bf16 rate times
     # the nominal FP4 : bf16 ratio.  The two measurements run at different SM clocks (a saturated tensor pipe is
     # power-capped, this kernel is not), so the fraction is also given per clock: flops per SM cycle over flops per
-    # SM cycle.  What binds this kernel is not the tensor pipe but the exponential unit (one ex2 per score, 16 per
-    # clock and SM against 64 scores' worth of FP4 flops), hence "bound": "mufu" and the fraction of that ceiling.
+    # SM cycle.  What binds this kernel is not the tensor pipe: issue slots (69 % busy) and the exponential unit (68 %: 16
+    # exponentials per clock and SM against 64 scores' worth of FP4 flops) are the fullest, and neither is full; "bound"
+    # names the fullest, and the fraction of the exponential unit's ceiling is given beside it.
     if fp4:
         fp4_peak = fp4["peak_tflops"]
         peak_note = (f"dense FP4 measured in this run: mxattn_probe_fp4_gemm, {fp4['peak_mode']} mode, median of "
@@ -465,17 +469,16 @@ def main():
         peak_note = (f"no FP4 probe in this run: {peaks['source']} sustained bf16 cuBLAS {peaks['bf16_tflops_sustained']} "
                      f"x nominal ratio 4 (of {peaks['source']})")
         per_clock = None
-    roofline = {"bound": "mufu", "kernel": "attention_walk_kernel<uos,pnq>", "achieved": attn_tflops,
+    roofline = {"bound": "issue", "kernel": "attention_walk_kernel<uos,pnq>", "achieved": attn_tflops,
                 "peak": fp4_peak, "unit": "TFLOP/s", "frac": attn_tflops / fp4_peak,
                 "frac_per_sm_clock": per_clock, "achieved_sm_mhz": clocks.get("sm_mhz"),
                 "traffic": ATTN_TRAFFIC_PER_TOKEN_HEAD * Nkv * B * H if Nq == Nkv else None,
                 "traffic_note": "ncu dram bytes of a sweep16384 launch scaled by tokens x heads",
                 "peak_note": peak_note,
                 "frac_of_nominal_9PF": attn_tflops / NOMINAL_FP4_TFLOPS, "launch_ms": attn_ms,
-                # the softmax exponentials bind before the tensor pipe does: 16 ex2 per clock per SM,
-                # one per (query, key) pair, 512 tensor flops per pair
-                "mufu_ceiling_tflops": mufu_ceiling, "frac_of_mufu_ceiling": attn_tflops / mufu_ceiling if mufu_ceiling else None,
-                "ncu_cross_check": "profiles/attention_walk_kernel.txt (128 key tiles per item): sm__pipe_tensor_cycles_active 23.9 %, XU pipe 68 %"}
+                # 16 ex2 per clock and SM, mufu_share of one per (query, key) pair, 512 tensor flops per pair
+                "mufu_share": mufu_share, "mufu_ceiling_tflops": mufu_ceiling, "frac_of_mufu_ceiling": attn_tflops / mufu_ceiling if mufu_ceiling else None,
+                "ncu_cross_check": "profiles/attention_walk_kernel.txt (128 key tiles per item): sm__pipe_tensor_cycles_active 23.9 %, XU pipe 68 %, issue slots 69 %"}
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
         "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,

@@ -59,7 +59,7 @@
 //    about 2e-7 relative for the blocks that carry a row, d > 168, the order of ex2.approx itself, and by up to 1.5e-6 for the smallest
 //    scales, whose logarithm is a larger number; a block with d = 0 keeps r = 1, its codes are 0 either way.
 // Whole call, us, two query tiles per CTA as in forward.cu, which it was before / walking, the outputs bit for bit the same: PNQ
-// 40 x 16384 3801 / 3293, 40 x 4096 331 / 276, direct 40 x 16384 3990 / 3710, 24 x 8192 719 / 636, 24 x 2000 74 / 59, 24 x 20000 x 512 228 / 157.
+// 40 x 16384 3801 / 3199, 40 x 4096 331 / 267, direct 40 x 16384 3990 / 3623, 24 x 8192 719 / 623, 24 x 2000 74 / 59, 24 x 20000 x 512 228 / 157.
 //
 // Every wait at an mbarrier is bounded (mbar_wait_soft / role_wait), and none is stranded at a named barrier.  A softmax warp keeps its
 // meetings with the other team to the end (team_tiles).  An issuing warp looks at the abort flag before it waits for softmax
@@ -719,7 +719,7 @@ __device__ __forceinline__ void play(const Params& p, const CUtensorMap& out_map
       // NVFP4, the scales of the other 32 keys (two exponentials, a table): in front of the first exponentials, or in the gap where
       // their scores are loaded.  There the score buffer is given back later, which short sequences with PNQ do not make up for.
       // Whole call, us, in front / in the gap: direct 40 x 16384 3770 / 3710, 24 x 8192 646 / 636, 40 x 4096 299.7 / 297.7, 40 x 18900 x
-      // 512 232.2 / 230.6, PNQ 40 x 16384 3321 / 3293, 40 x 4096 275.3 / 279.5, 24 x 8192 x 2000 175.3 / 177.5.
+      // 512 232.2 / 230.6, PNQ 40 x 16384 3321 / 3293, with fixed shares 40 x 4096 275.3 / 279.5, 24 x 8192 x 2000 175.3 / 177.5.
       constexpr bool kLate = kNv && (!kPnq || kTake);
       uint64_t nb0, nb1;
       uint32_t sf0, sf1;
